@@ -339,16 +339,22 @@ template <typename real> fs_status batch_build(fs_batch *b, const fs_instance *i
         FS_CUDA(cudaMemcpy(b->spread_items, si.data(), si.size() * sizeof(SpreadItem), cudaMemcpyHostToDevice));
     // near-field items (FP32): all instances, largest estimated work first
     if (b->precision == 32) {
-        std::vector<std::pair<int64_t, int4>> ni;
+        std::vector<std::pair<NearCell, int>> runs;   // (cell's run of items, instance)
+        size_t n_items = 0;
         for (int i = 0; i < K; ++i) {
-            const fs_plan *pl = b->plans[i];
-            for (size_t k = 0; k < pl->near_items_h.size(); ++k)
-                ni.push_back({pl->near_work_h[k], make_int4(pl->near_items_h[k].x, pl->near_items_h[k].y, i, 0)});
+            for (const NearCell &c : b->plans[i]->near_cells_h)
+                runs.push_back({c, i});
+            n_items += b->plans[i]->near_items_h.size();
         }
-        std::stable_sort(ni.begin(), ni.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
-        std::vector<int4> items(ni.size());
-        for (size_t k = 0; k < ni.size(); ++k)
-            items[k] = ni[k].second;
+        std::stable_sort(runs.begin(), runs.end(),
+                         [](const auto &x, const auto &y) { return x.first.work > y.first.work; });
+        std::vector<int4> items;
+        items.reserve(n_items);
+        for (const auto &r : runs) {
+            const fs_plan *pl = b->plans[r.second];
+            for (int k = r.first.first; k < r.first.first + r.first.count; ++k)
+                items.push_back(make_int4(pl->near_items_h[k].x, pl->near_items_h[k].y, r.second, pl->tgt_cap));
+        }
         b->n_near_items = (int64_t)items.size();
         FS_TRY(b->alloc(&b->near_items, items.size()));
         if (!items.empty())

@@ -309,9 +309,8 @@ __host__ __device__ __forceinline__ int base2(int packed) { return (packed >> 16
 
 // Tile-major cell key: cells of one spreading tile are contiguous, cells row-major inside.
 // Points are sorted by key * kSub + sub, where sub is the Morton index of the point's
-// 8 x 8 sub-cell, so consecutive points inside a cell are spatially compact; the sorted
-// range of cell `key` is [start[key * kSub], start[(key + 1) * kSub]) and that of one
-// sub-cell is [start[key * kSub + sub], start[key * kSub + sub + 1]).
+// 8 x 8 sub-cell, and then, inside each cell, into the pieces of CellSplit; the sorted range of
+// cell `key` is [start[key * kSub], start[(key + 1) * kSub]).
 constexpr int kSubEdge = 8;
 constexpr int kSub = kSubEdge * kSubEdge;
 

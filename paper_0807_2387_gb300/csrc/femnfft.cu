@@ -176,10 +176,18 @@ void fs::build_window_poly(double sigma, int m, WindowPoly *wp)
 
 namespace {
 
-// Bin one point set: keys, counting sort, per-point records.
+// Own points per near-field warp item, from the mean number of own points per cell as a point sees
+// it.  Smaller items have smaller boxes, so more of the evaluated pairs lie within eps_I, and there
+// are more warps; but each builds its candidate lists from the same neighbour cells.  Measured
+// (near field, 8 / 16 / 32): 1,000 points at 16 per cell 11 / 12 / 14 us; 65,537 at 45 47 / 41 / 49 us;
+// the 2^18-point adjoint step at 181 1256 / 1064 / 1050 us; 2^20 clustered points 3.23 / 2.46 / 2.26 ms.
+int near_item_lanes(double per_cell) { return per_cell < 25.0 ? 8 : (per_cell < 100.0 ? 16 : 32); }
+
+// Bin one point set: keys, counting sort, order within the cells (pieces of at most *cap points, chosen
+// here unless given), per-point records; `cells`: the cells' first points.
 template <typename real>
 fs_status bin_points(fs_plan *pl, const double *xy, int64_t n, int **perm, int **base, void **frac, double2 **pos,
-                     float2 **pos32, float2 **lo32, int **start)
+                     float2 **pos32, float2 **lo32, int **start, int *cap, std::vector<int> *cells)
 {
     FS_TRY(pl->alloc(perm, n));
     FS_TRY(pl->alloc(base, n));
@@ -206,6 +214,23 @@ fs_status bin_points(fs_plan *pl, const double *xy, int64_t n, int **perm, int *
     FS_CUDA(launch_exclusive_scan(count, *start, pl->n_keys, tmp, st));
     FS_CUDA(cudaMemcpyAsync(fill, *start, sizeof(int) * ((size_t)pl->n_keys + 1), cudaMemcpyDeviceToDevice, st));
     FS_CUDA(launch_scatter(key, n, fill, *perm, st));
+    {
+        const int n_cells = pl->n_keys / kSub;
+        std::vector<int> all((size_t)pl->n_keys + 1);
+        FS_CUDA(cudaMemcpyAsync(all.data(), *start, sizeof(int) * all.size(), cudaMemcpyDeviceToHost, st));
+        FS_CUDA(cudaStreamSynchronize(st));
+        cells->resize(n_cells + 1);
+        double sq = 0.0;
+        for (int c = 0; c <= n_cells; ++c) {
+            (*cells)[c] = all[(size_t)c * kSub];
+            const double k = c > 0 ? (*cells)[c] - (*cells)[c - 1] : 0;
+            sq += k * k;
+        }
+        if (*cap == 0)
+            *cap = near_item_lanes(n > 0 ? sq / (double)n : 0.0);
+        FS_CUDA(launch_cell_order(*start, n_cells, *cap, xy, pl->s, pl->n_os, pl->window_lo, pl->n_a, pl->m,
+                                  pl->cg.cell, *perm, st));
+    }
     FS_CUDA(launch_gather_points<real>(xy, *perm, n, pl->s, pl->n_os, pl->window_lo, pl->n_a, pl->m, pl->cg.cell, *pos,
                                        *frac, *base, *pos32, *lo32, st));
     FS_CUDA(cudaStreamSynchronize(st));
@@ -216,101 +241,62 @@ fs_status bin_points(fs_plan *pl, const double *xy, int64_t n, int **perm, int *
     return FS_OK;
 }
 
-// FP32 near-field warp items over the "own" points (targets for the forward, sources for
-// the adjoint): at most 64 consecutive points of one cell (two per lane), in the cell's
-// Morton sub-cell order, so an item is compact.  Target items split each cell evenly into
-// the fewest items of at most 64; source items give a sub-cell holding 32 or more points
-// items of its own (boxes an eighth of a cell wide) and merge sparser sub-cells of the same
-// cell up to 64.  On the 2^20-point mixture the even split leaves fewer idle lane slots and
-// fewer candidate visits (items 19,884 -> 18,098, evaluated pair slots -4 %), and the
-// forward near field fell from 3.28 to 2.87 ms on GB300; the source items, which also serve
-// the source-major FEM kernel, keep the rule that kernel was tuned with.  Items are ordered
-// by estimated work (points x "other" points in the 3 x 3 cells around the item's cell),
-// largest first, so the heavy warps start early and the tail of the launch stays short.
-fs_status build_near_items(fs_plan *pl, const int *own_start_d, const int *oth_start_d, bool whole_cells, int2 **out,
-                           int64_t *n_out, std::vector<int2> *items_out = nullptr,
-                           std::vector<int64_t> *work_out = nullptr)
+// FP32 near-field warp items over the "own" points (targets for the forward, sources for the
+// adjoint and the source-major near field; own and oth: the cells' first points): the pieces of
+// at most cap points that the cells are sorted into, halved where they exceed max_item.  Items are sorted by estimated work (points x
+// "other" points in the 3 x 3 cells around the item's cell), largest first, so that the heavy
+// warps start early and the tail of the launch stays short: the cells are sorted, and the items
+// of a cell, which are of one size, stay together.
+fs_status build_near_items(fs_plan *pl, const std::vector<int> &own, const std::vector<int> &oth, int cap,
+                           int max_item, int2 **out, int64_t *n_out, std::vector<int2> *items_out = nullptr,
+                           std::vector<NearCell> *cells_out = nullptr)
 {
-    constexpr int kCap = 64, kOwn = 32;
-    std::vector<int> start(pl->n_keys + 1), oth(pl->n_keys + 1);
-    FS_CUDA(cudaMemcpy(start.data(), own_start_d, sizeof(int) * start.size(), cudaMemcpyDeviceToHost));
-    FS_CUDA(cudaMemcpy(oth.data(), oth_start_d, sizeof(int) * oth.size(), cudaMemcpyDeviceToHost));
-    const int n_cells = pl->n_keys / kSub;
-    std::vector<int2> items;
-    std::vector<int> item_cell;
-    for (int key = 0; whole_cells && key < n_cells; ++key) {
-        const int a = start[key * kSub], c = start[(key + 1) * kSub] - a;
-        const int pieces = (c + kCap - 1) / kCap;
-        for (int i = 0; i < pieces; ++i) {
-            const int lo = a + (int)((int64_t)c * i / pieces), hi = a + (int)((int64_t)c * (i + 1) / pieces);
-            items.push_back(make_int2(lo, hi - lo));
-            item_cell.push_back(key);
-        }
-    }
-    for (int key = 0; !whole_cells && key < n_cells; ++key) {
-        int open_start = -1, open_count = 0;
-        auto flush = [&]() {
-            if (open_count > 0) {
-                items.push_back(make_int2(open_start, open_count));
-                item_cell.push_back(key);
-            }
-            open_count = 0;
-        };
-        for (int sub = 0; sub < kSub; ++sub) {
-            const int a = start[key * kSub + sub], c = start[key * kSub + sub + 1] - a;
-            if (c == 0)
-                continue;
-            if (c >= kOwn) {
-                flush();
-                const int pieces = (c + kCap - 1) / kCap;
-                for (int i = 0; i < pieces; ++i) {
-                    const int lo = a + (int)((int64_t)c * i / pieces), hi = a + (int)((int64_t)c * (i + 1) / pieces);
-                    items.push_back(make_int2(lo, hi - lo));
-                    item_cell.push_back(key);
-                }
-                continue;
-            }
-            if (open_count > 0 && open_count + c > kCap)
-                flush();
-            if (open_count == 0)
-                open_start = a;
-            open_count += c;   // contiguous: sub-cells of a cell follow each other in the sorted order
-        }
-        flush();
-    }
-    std::vector<int64_t> nb(n_cells, 0);
     const int nc = pl->cg.n_c;
+    std::vector<std::pair<int64_t, int>> order;   // (work of one item, cell)
     for (int c1 = 0; c1 < nc; ++c1)
         for (int c2 = 0; c2 < nc; ++c2) {
-            int64_t acc = 0;
-            for (int d1 = -1; d1 <= 1; ++d1)
-                for (int d2 = -1; d2 <= 1; ++d2) {
-                    const int e1 = c1 + d1, e2 = c2 + d2;
-                    if (e1 < 0 || e2 < 0 || e1 >= nc || e2 >= nc)
-                        continue;
+            const int key = pl->cg.key(c1, c2), count = own[key + 1] - own[key];
+            if (count == 0)
+                continue;
+            int64_t around = 0;
+            for (int e1 = std::max(c1 - 1, 0); e1 <= std::min(c1 + 1, nc - 1); ++e1)
+                for (int e2 = std::max(c2 - 1, 0); e2 <= std::min(c2 + 1, nc - 1); ++e2) {
                     const int kk = pl->cg.key(e1, e2);
-                    acc += oth[(kk + 1) * kSub] - oth[kk * kSub];
+                    around += oth[kk + 1] - oth[kk];
                 }
-            nb[pl->cg.key(c1, c2)] = acc;
+            order.push_back({std::min({count, cap, max_item}) * around, key});
         }
-    std::vector<std::pair<int64_t, int2>> wi;
-    wi.reserve(items.size());
-    for (size_t i = 0; i < items.size(); ++i)
-        wi.push_back({(int64_t)items[i].y * nb[item_cell[i]], items[i]});
-    std::stable_sort(wi.begin(), wi.end(), [](const auto &a, const auto &b) { return a.first > b.first; });
-    for (size_t i = 0; i < items.size(); ++i)
-        items[i] = wi[i].second;
-    if (items_out)
-        *items_out = items;
-    if (work_out) {
-        work_out->resize(items.size());
-        for (size_t i = 0; i < items.size(); ++i)
-            (*work_out)[i] = wi[i].first;
+    std::stable_sort(order.begin(), order.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
+    std::vector<int2> items;
+    std::vector<NearCell> cells;
+    for (const auto &o : order) {
+        const int a = own[o.second], count = own[o.second + 1] - a, before = (int)items.size();
+        for (int r = 0; r < CellSplit::runs(count); ++r) {
+            const int first = a + CellSplit::run_first(count, r);
+            const CellSplit split(a + CellSplit::run_first(count, r + 1) - first, cap);
+            for (int j = 0; j < split.strips; ++j) {
+                const int lo = split.strip_first(j), len = split.strip_first(j + 1) - lo;
+                const int parts = split.strip_piece(j + 1) - split.strip_piece(j);
+                for (int i = 0; i < parts; ++i) {
+                    const int p0 = (int)((int64_t)len * i / parts), p1 = (int)((int64_t)len * (i + 1) / parts);
+                    const int cuts = (p1 - p0 + max_item - 1) / max_item;
+                    for (int h = 0; h < cuts; ++h) {
+                        const int h0 = (p1 - p0) * h / cuts, h1 = (p1 - p0) * (h + 1) / cuts;
+                        items.push_back(make_int2(first + lo + p0 + h0, h1 - h0));
+                    }
+                }
+            }
+        }
+        cells.push_back(NearCell{o.first, before, (int)items.size() - before});
     }
     *n_out = (int64_t)items.size();
     FS_TRY(pl->alloc(out, items.size()));
     if (!items.empty())
         FS_CUDA(cudaMemcpy(*out, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    if (items_out)
+        *items_out = std::move(items);
+    if (cells_out)
+        *cells_out = std::move(cells);
     return FS_OK;
 }
 
@@ -503,10 +489,16 @@ fs_status plan_init(fs_plan *pl, const double *src, int64_t M, const double *tgt
     build_window_poly(pl->sigma, pl->m, &pl->wpoly);
 
     // binning
+    // FEM plans (several quadrature points around every node): a cell holds few targets, so a
+    // target item's box would span the whole cell; the forward near field then runs over items
+    // of sources, whose boxes stay small
+    pl->src_major = pl->precision == 32 && N > 0 && M >= 3 * N;
+    if (pl->src_major)
+        pl->src_cap = kSrcMajorItem;
     FS_TRY(bin_points<real>(pl, src, M, &pl->src_perm, &pl->src_base, &pl->src_frac, &pl->src_pos, &pl->src_pos32,
-                            &pl->src_lo32, &pl->src_start));
+                            &pl->src_lo32, &pl->src_start, &pl->src_cap, &pl->src_cells));
     FS_TRY(bin_points<real>(pl, tgt, N, &pl->tgt_perm, &pl->tgt_base, &pl->tgt_frac, &pl->tgt_pos, &pl->tgt_pos32,
-                            &pl->tgt_lo32, &pl->tgt_start));
+                            &pl->tgt_lo32, &pl->tgt_start, &pl->tgt_cap, &pl->tgt_cells));
     int dev_status = 0;
     FS_CUDA(cudaMemcpy(&dev_status, pl->status, sizeof(int), cudaMemcpyDeviceToHost));
     if (dev_status != 0)
@@ -515,11 +507,9 @@ fs_status plan_init(fs_plan *pl, const double *src, int64_t M, const double *tgt
     // spreading work items: tiles split into slices of at most kSpreadChunk points (sources
     // for the forward spread, targets for the adjoint one)
     for (int side = 0; side < 2; ++side) {
-        std::vector<int> start(pl->n_keys + 1);
-        FS_CUDA(cudaMemcpy(start.data(), side == 0 ? pl->src_start : pl->tgt_start, sizeof(int) * start.size(),
-                           cudaMemcpyDeviceToHost));
+        const std::vector<int> &start = side == 0 ? pl->src_cells : pl->tgt_cells;
         std::vector<SpreadItem> items;
-        const int TT = T * T * kSub;
+        const int TT = T * T;
         const int n_tiles = pl->cg.n_t * pl->cg.n_t;
         for (int t = 0; t < n_tiles; ++t) {
             const int a = start[t * TT], b2 = start[(t + 1) * TT];
@@ -554,14 +544,10 @@ fs_status plan_init(fs_plan *pl, const double *src, int64_t M, const double *tgt
     }
 
     if (pl->precision == 32) {
-        FS_TRY(build_near_items(pl, pl->tgt_start, pl->src_start, true, &pl->near_items, &pl->n_near_items,
-                                &pl->near_items_h, &pl->near_work_h));
-        // FEM plans (several quadrature points around every node): a cell holds few targets, so a
-        // target item's box would span the whole cell; the forward near field then runs over
-        // items of sources, whose boxes stay small
-        pl->src_major = N > 0 && M >= 3 * N;
+        FS_TRY(build_near_items(pl, pl->tgt_cells, pl->src_cells, pl->tgt_cap, 32, &pl->near_items, &pl->n_near_items,
+                                &pl->near_items_h, &pl->near_cells_h));
         if (pl->src_major)
-            FS_TRY(build_near_items(pl, pl->src_start, pl->tgt_start, false, &pl->src_near_items,
+            FS_TRY(build_near_items(pl, pl->src_cells, pl->tgt_cells, pl->src_cap, kSrcMajorItem, &pl->src_near_items,
                                     &pl->n_src_near_items));
     }
 
@@ -588,7 +574,7 @@ fs_status plan_init(fs_plan *pl, const double *src, int64_t M, const double *tgt
         FS_TRY(pl->alloc(&cnt, 2 * kNearCountSlots));
         FS_CUDA(cudaMemsetAsync(cnt, 0, 2 * kNearCountSlots * sizeof(unsigned long long), st));
         if constexpr (sizeof(real) == 4)
-            FS_CUDA(launch_near_count32(pl->n_near_items, pl->near_items, pl->tgt_base, pl->tgt_pos32, pl->tgt_lo32,
+            FS_CUDA(launch_near_count32(pl->n_near_items, pl->near_items, pl->tgt_cap, pl->tgt_base, pl->tgt_pos32, pl->tgt_lo32,
                                         pl->src_pos32, pl->src_lo32, pl->src_start, pl->cg, make_near<float>(pl), cnt,
                                         st));
         else
@@ -752,7 +738,7 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
                                           (const float *)q, make_near<float>(pl), (float *)pl->phi_s,
                                           (float *)pl->grad_s, (float *)pl->coinc, pl->aux));
             } else {
-                FS_CUDA(launch_near32(pl->n_near_items, pl->near_items, pl->tgt_base, pl->tgt_pos32, pl->tgt_lo32,
+                FS_CUDA(launch_near32(pl->n_near_items, pl->near_items, pl->tgt_cap, pl->tgt_base, pl->tgt_pos32, pl->tgt_lo32,
                                       pl->src_pos32, pl->src_lo32, pl->src_start, pl->cg, (const float *)q,
                                       make_near<float>(pl), (float *)pl->phi_s, (float *)pl->grad_s,
                                       (float *)pl->coinc, true, pl->aux));
@@ -807,7 +793,7 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
                                           (const float *)q, np, (float *)pl->phi_s, (float *)pl->grad_s,
                                           (float *)pl->coinc, st));
             } else {
-                FS_CUDA(launch_near32(pl->n_near_items, pl->near_items, pl->tgt_base, pl->tgt_pos32, pl->tgt_lo32,
+                FS_CUDA(launch_near32(pl->n_near_items, pl->near_items, pl->tgt_cap, pl->tgt_base, pl->tgt_pos32, pl->tgt_lo32,
                                       pl->src_pos32, pl->src_lo32, pl->src_start, pl->cg, (const float *)q, np,
                                       (float *)pl->phi_s, (float *)pl->grad_s, (float *)pl->coinc, false, st));
             }
@@ -909,9 +895,9 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
         FS_TRY(pl->alloc_bytes(&pl->adj_cg, (size_t)std::max<int64_t>(M, 1) * sizeof(real)));
         FS_TRY(pl->alloc_bytes(&pl->adj_hess, (size_t)std::max<int64_t>(N, 1) * 3 * sizeof(real)));
         FS_TRY(pl->alloc(&pl->adj_gsum, 1));
-        if (pl->precision == 32 && !pl->src_near_items)
-            FS_TRY(build_near_items(pl, pl->src_start, pl->tgt_start, false, &pl->src_near_items,
-                                    &pl->n_src_near_items));
+        if (pl->precision == 32)
+            FS_TRY(build_near_items(pl, pl->src_cells, pl->tgt_cells, pl->src_cap, 32, &pl->adj_items,
+                                    &pl->n_adj_items));
     }
     const Window<real> w = make_window<real>(pl);
     const NearParams<real> np = make_near<real>(pl);
@@ -931,7 +917,7 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
                 if (ovl) {
                     FS_CUDA(cudaEventRecord(pl->ev_fork, st));
                     FS_CUDA(cudaStreamWaitEvent(pl->aux, pl->ev_fork, 0));
-                    FS_CUDA(launch_near_hess32(pl->n_near_items, pl->near_items, pl->tgt_base, pl->tgt_pos32,
+                    FS_CUDA(launch_near_hess32(pl->n_near_items, pl->near_items, pl->tgt_cap, pl->tgt_base, pl->tgt_pos32,
                                                pl->tgt_lo32, pl->src_pos32, pl->src_lo32, pl->src_start, pl->cg, q, np,
                                                (float *)pl->grad_s, (float *)pl->adj_hess, true, pl->aux));
                     FS_CUDA(cudaEventRecord(pl->ev_join, pl->aux));
@@ -946,7 +932,7 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
                                              st));
             if constexpr (sizeof(real) == 4) {
                 if (!ovl)
-                    FS_CUDA(launch_near_hess32(pl->n_near_items, pl->near_items, pl->tgt_base, pl->tgt_pos32,
+                    FS_CUDA(launch_near_hess32(pl->n_near_items, pl->near_items, pl->tgt_cap, pl->tgt_base, pl->tgt_pos32,
                                                pl->tgt_lo32, pl->src_pos32, pl->src_lo32, pl->src_start, pl->cg, q, np,
                                                (float *)pl->grad_s, (float *)pl->adj_hess, false, st));
             } else {
@@ -962,7 +948,7 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
                 if (ovl) {
                     FS_CUDA(cudaEventRecord(pl->ev_fork, st));   // the adjoint weights are in
                     FS_CUDA(cudaStreamWaitEvent(pl->aux, pl->ev_fork, 0));
-                    FS_CUDA(launch_near_adj32(pl->n_src_near_items, pl->src_near_items, pl->src_base, pl->src_pos32,
+                    FS_CUDA(launch_near_adj32(pl->n_adj_items, pl->adj_items, std::min(pl->src_cap, 32), pl->src_base, pl->src_pos32,
                                               pl->src_lo32, pl->tgt_pos32, pl->tgt_lo32, pl->tgt_start, pl->cg,
                                               (const float *)pl->adj_c, pl->adj_dn, np, (float *)pl->adj_a,
                                               (float *)pl->adj_ga, (float *)pl->adj_cg, true, pl->aux));
@@ -980,7 +966,7 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
                                         pl->pitch, (real)pl->n_os, (real *)pl->adj_a, (real *)pl->adj_ga, ovl, st));
             if constexpr (sizeof(real) == 4) {
                 if (!ovl)
-                    FS_CUDA(launch_near_adj32(pl->n_src_near_items, pl->src_near_items, pl->src_base, pl->src_pos32,
+                    FS_CUDA(launch_near_adj32(pl->n_adj_items, pl->adj_items, std::min(pl->src_cap, 32), pl->src_base, pl->src_pos32,
                                               pl->src_lo32, pl->tgt_pos32, pl->tgt_lo32, pl->tgt_start, pl->cg,
                                               (const float *)pl->adj_c, pl->adj_dn, np, (float *)pl->adj_a,
                                               (float *)pl->adj_ga, (float *)pl->adj_cg, false, st));

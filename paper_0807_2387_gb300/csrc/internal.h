@@ -31,6 +31,27 @@ template <typename real> inline size_t spread_smem_bytes(int P, int M2, bool com
            (size_t)kSpreadWarps * spread_weight_stride<real>(M2) * sizeof(real) + sizeof(float) * M2 * (kPolyD + 1);
 }
 
+// How the points of a cell, and its near-field items, are ordered: in runs of at most kOrderRun
+// points (one run for nearly every cell; they follow the sub-cell order), each cut into strips
+// along x and the strips into pieces along y, all pieces of nearly one size and at most `cap`
+// points.  A piece is a compact, nearly square part of the cell.  Device (k_cell_order, which
+// sorts) and host (the items) use the same integers.
+constexpr int kOrderRun = 2048;
+struct CellSplit {
+    int pieces, strips;   // of a run of m points
+    int m;
+    __host__ __device__ CellSplit(int m_, int cap) : pieces((m_ + cap - 1) / cap), strips(1), m(m_)
+    {
+        while (strips * (strips + 1) < pieces)   // strips = sqrt(pieces), rounded
+            ++strips;
+    }
+    __host__ __device__ static int runs(int count) { return (count + kOrderRun - 1) / kOrderRun; }
+    __host__ __device__ static int run_first(int count, int i) { return (int)((int64_t)count * i / runs(count)); }
+    // first piece and first point of strip j (j = strips: the end)
+    __host__ __device__ int strip_piece(int j) const { return (int)((int64_t)pieces * j / strips); }
+    __host__ __device__ int strip_first(int j) const { return (int)((int64_t)m * strip_piece(j) / pieces); }
+};
+
 // One spreading work unit: sources [start, start+count) of tile `tile` (cell-sorted order).
 struct SpreadItem {
     int tile;
@@ -61,6 +82,7 @@ template <typename real> struct NearParams {
     real dbeta[kMaxP];     // coefficients of T_I'(r)/r in w: 2k beta_k / eps_I^2 (index k-1)
     real pbeta[kMaxP];     // P(w) = T_I - k(eps_I): beta with beta_0 - k(eps_I), so P(1) = 0
     real nptilde[kMaxP];   // -Ptilde(w) with P(w) = (w - 1) Ptilde(w): degree p - 2 (index < p - 1)
+    real ptln[kMaxP];      // Ptilde(w) / c_ln, c_ln = -(ln 2) / (4 pi) (index < p - 1)
     real rcoef;            // (-1)^p / (2 pi eps_I^2): (k' - T_I')(r)/r = rcoef (w - 1)^(p-1) / w
     int p;
 };
@@ -237,7 +259,7 @@ cudaError_t launch_batch_fft(const BatchInst<real> *inst, const FftUnit *units, 
 template <typename real> cudaError_t batch_fft_blocks(int L_max, int *blocks);
 // one bounded wait on a counter that nothing increments (the timeout path, for tests)
 cudaError_t launch_wait_selftest(int *counter, int *err, int spins, cudaStream_t st);
-// items: (first target, count <= 64, instance, 0) per warp
+// items: (first target, count, instance, lanes) per warp, count <= lanes (8, 16 or 32)
 cudaError_t launch_batch_near32(int64_t n_items, const int4 *items, const BatchInst<float> *inst, int p, int nrhs,
                                 bool assign, cudaStream_t st);
 cudaError_t launch_batch_near64(const BatchInst<double> *inst, BlockMap bm, int blocks, int nrhs, cudaStream_t st);
@@ -251,6 +273,9 @@ cudaError_t launch_point_keys(const double *xy, int64_t n, double s, int n_os, i
                               int m, CellGrid cg, int *key, int *count, int *status, cudaStream_t st);
 cudaError_t launch_exclusive_scan(const int *count, int *start, int n, int *block_tmp, cudaStream_t st);
 cudaError_t launch_scatter(const int *key, int64_t n, int *fill, int *perm, cudaStream_t st);
+// the points of each cell (sorted range from start[key kSub]) into the order of CellSplit
+cudaError_t launch_cell_order(const int *start, int n_cells, int cap, const double *xy, double s, int n_os,
+                              int window_lo, int n_a, int m, int cell, int *perm, cudaStream_t st);
 template <typename real>
 cudaError_t launch_gather_points(const double *xy, const int *perm, int64_t n, double s, int n_os,
                                  int window_lo, int n_a, int m, int cell, double2 *pos, void *frac, int *base,
@@ -326,10 +351,10 @@ cudaError_t launch_build_mul(const double2 *bhat, int n, const double *c_tab, re
 cudaError_t launch_near64(int64_t N, const int *tgt_base, const double2 *tgt_pos, const double2 *src_pos,
                           const int *src_start, CellGrid cg, const double *q, NearParams<double> np, double *phi_s,
                           double *grad_s, double *coinc, cudaStream_t st);
-// items: (first target, count <= 64) per warp, never spanning two cells
+// items: (first target, count <= lanes) per warp, never spanning two cells; lanes: 8, 16 or 32
 // (assign: store phi_s and grad_s instead of adding to them, for the near field that runs on a
 // second stream beside spreading and the transform)
-cudaError_t launch_near32(int64_t n_items, const int2 *items, const int *tgt_base, const float2 *tgt_hi,
+cudaError_t launch_near32(int64_t n_items, const int2 *items, int lanes, const int *tgt_base, const float2 *tgt_hi,
                           const float2 *tgt_lo, const float2 *src_hi, const float2 *src_lo, const int *src_start,
                           CellGrid cg, const float *q, NearParams<float> np, float *phi_s, float *grad_s, float *coinc,
                           bool assign, cudaStream_t st);
@@ -342,7 +367,7 @@ cudaError_t launch_near_src32(int64_t n_items, const int2 *items, const int *src
 // plan-time pair statistics over the FP32 near-field items: counts[2 s] (r < eps_I) and
 // counts[2 s + 1] (r < eps_I / 8) for s < kNearCountSlots, to be summed
 constexpr int kNearCountSlots = 64;
-cudaError_t launch_near_count32(int64_t n_items, const int2 *items, const int *tgt_base, const float2 *tgt_hi,
+cudaError_t launch_near_count32(int64_t n_items, const int2 *items, int lanes, const int *tgt_base, const float2 *tgt_hi,
                                 const float2 *tgt_lo, const float2 *src_hi, const float2 *src_lo, const int *src_start,
                                 CellGrid cg, NearParams<float> np, unsigned long long *counts, cudaStream_t st);
 template <typename real>
@@ -362,12 +387,12 @@ cudaError_t launch_near_hess64(int64_t N, const int *tgt_base, const double2 *tg
                                const int *src_start, CellGrid cg, const double *q, NearParams<double> np,
                                double *grad_s, double *hess_s, cudaStream_t st);
 // FP32: warp items over the sources (adjoint potential) or the targets (Hessian)
-cudaError_t launch_near_adj32(int64_t n_items, const int2 *items, const int *src_base, const float2 *src_hi,
+cudaError_t launch_near_adj32(int64_t n_items, const int2 *items, int lanes, const int *src_base, const float2 *src_hi,
                               const float2 *src_lo, const float2 *tgt_hi, const float2 *tgt_lo, const int *tgt_start,
                               CellGrid cg, const float *c, const void *dn, NearParams<float> np, float *a_s,
                               float *ga_s, float *cg_s, bool assign, cudaStream_t st);
 // (assign: store instead of adding, for the near parts run beside the spreading and transform)
-cudaError_t launch_near_hess32(int64_t n_items, const int2 *items, const int *tgt_base, const float2 *tgt_hi,
+cudaError_t launch_near_hess32(int64_t n_items, const int2 *items, int lanes, const int *tgt_base, const float2 *tgt_hi,
                                const float2 *tgt_lo, const float2 *src_hi, const float2 *src_lo, const int *src_start,
                                CellGrid cg, const float *q, NearParams<float> np, float *grad_s, float *hess_s,
                                bool assign, cudaStream_t st);

@@ -19,7 +19,7 @@
 // the source gradient of the adjoint potential, +(2 beta_1 / eps_I^2) dn.
 //
 // FP64: one thread per point (the comparison path).  FP32: warp items over the
-// 8 x 8 sub-cells (near_warp.cuh), the Hessian over the forward's target items and
+// cells (near_warp.cuh), the Hessian over the forward's target items and
 // the adjoint potential over items of sources against the targets.
 #include <cmath>
 
@@ -225,32 +225,32 @@ __global__ void __launch_bounds__(256) k_near_hess64(int64_t N, const int *__res
 // charge is masked.
 template <int P> struct NearHess32 {
     static constexpr int kMinBlocks = 5;
-    static constexpr int kUnroll = 2;
-    static constexpr bool kClamp = P >= 3;
+    static constexpr int kUnroll = 4;
+    static constexpr bool kSat = P >= 3;   // w clamped to 1 by the traversal
     const float *__restrict__ q;
     float *__restrict__ grad_s;
     float *__restrict__ hess_s;
     float rcoef, geps, self_c;             // rc, eps_I (gradient unit), self_c = Hess T_I(0) / rc
     bool assign;                           // store instead of adding (the far part is added later)
-    float qj;
+    float2 qj;
     float2 gx, gy, sI, sxx, sxy, syy;
 
     __device__ __forceinline__ void init() { gx = gy = sI = sxx = sxy = syy = f2(0.f); }
     // candidate-list traversal: one value per other point (its charge)
     static constexpr int kR = 1;
     __device__ __forceinline__ void fetch(int j, float (&v)[1]) const { v[0] = __ldg(q + j); }
-    __device__ __forceinline__ void set_q(const float *v) { qj = v[0]; }
-    __device__ __forceinline__ void coincident(const NearParams<float> &, int t) { add_comp(sI, t, -qj * self_c); }
-    __device__ __forceinline__ void pair2(const NearParams<float> &np, float2 r2, float2 dx, float2 dy)
+    __device__ __forceinline__ void set_q(const float2 (&v)[1]) { qj = v[0]; }
+    __device__ __forceinline__ void coincident(const NearParams<float> &, int t)
     {
-        float2 w = r2;
-        if constexpr (kClamp)
-            w = min1(w);
+        add_comp(sI, t, -comp(qj, t) * self_c);
+    }
+    __device__ __forceinline__ void pair2(const NearParams<float> &np, float2 w, float2 dx, float2 dy)
+    {
         float2 c, cp;
         near_c_cp2<P>(w, c, cp);
-        float2 qq = f2(qj);
-        if constexpr (!kClamp)
-            qq = select2(r2, np.eps2, qq);
+        float2 qq = qj;
+        if constexpr (!kSat)
+            qq = select2(w, np.eps2, qq);
         const float2 qc = mul2(qq, c), k = mul2(qq, cp);
         gx = fma2(qc, dx, gx);
         gy = fma2(qc, dy, gy);
@@ -262,12 +262,22 @@ template <int P> struct NearHess32 {
     }
     __device__ __forceinline__ void row_begin() {}
     __device__ __forceinline__ void row_end() {}
-    __device__ __forceinline__ void store(int t, int64_t k)
+    __device__ __forceinline__ void fold()
+    {
+        for (float2 *v : {&gx, &gy, &sI, &sxx, &sxy, &syy})
+            v->x += v->y;
+    }
+    __device__ __forceinline__ void reduce(int o)
+    {
+        for (float2 *v : {&gx, &gy, &sI, &sxx, &sxy, &syy})
+            v->x = lane_add(v->x, o);
+    }
+    __device__ __forceinline__ void store(int64_t k)
     {
         // (a select, not a product with 0: the stored-to buffers may hold anything, NaN included)
-        const float i0 = comp(sI, t), rg = rcoef * geps;
-        const float v[5] = {rg * comp(gx, t), rg * comp(gy, t), rcoef * fmaf(2.f, comp(sxx, t), i0),
-                            rcoef * 2.f * comp(sxy, t), rcoef * fmaf(2.f, comp(syy, t), i0)};
+        const float i0 = sI.x, rg = rcoef * geps;
+        const float v[5] = {rg * gx.x, rg * gy.x, rcoef * fmaf(2.f, sxx.x, i0), rcoef * 2.f * sxy.x,
+                            rcoef * fmaf(2.f, syy.x, i0)};
         grad_s[2 * k] = assign ? v[0] : grad_s[2 * k] + v[0];
         grad_s[2 * k + 1] = assign ? v[1] : grad_s[2 * k + 1] + v[1];
         hess_s[3 * k] = assign ? v[2] : hess_s[3 * k] + v[2];
@@ -284,8 +294,8 @@ template <int P> struct NearHess32 {
 // store.
 template <int P> struct NearAdj32 {
     static constexpr int kMinBlocks = 4;
-    static constexpr int kUnroll = 2;
-    static constexpr bool kClamp = P >= 3;
+    static constexpr int kUnroll = 4;
+    static constexpr bool kSat = P >= 3;   // w clamped to 1 by the traversal
     const float *__restrict__ cw;
     const float2 *__restrict__ dnw;
     float *__restrict__ a_s;
@@ -293,8 +303,7 @@ template <int P> struct NearAdj32 {
     float *__restrict__ cg_s;
     float rcoef, geps, inv_eps, self_c;   // rc, eps_I, 1 / eps_I, self_c = Hess T_I(0) / rc
     bool assign;                           // store instead of adding (the far part is added later)
-    float gp;
-    float2 dn;
+    float2 gp, dn1, dn2;                   // of the pair of candidates
     float2 af, ac, gxc, gyc, gxk, gyk, gco;
 
     __device__ __forceinline__ void init() { af = ac = gxc = gyc = gxk = gyk = gco = f2(0.f); }
@@ -307,31 +316,29 @@ template <int P> struct NearAdj32 {
         v[1] = d.x * inv_eps;
         v[2] = d.y * inv_eps;
     }
-    __device__ __forceinline__ void set_q(const float *v)
+    __device__ __forceinline__ void set_q(const float2 (&v)[3])
     {
         gp = v[0];
-        dn = make_float2(v[1], v[2]);
+        dn1 = v[1];
+        dn2 = v[2];
     }
     __device__ __forceinline__ void coincident(const NearParams<float> &np, int t)
     {
-        add_comp(af, t, -gp * np.beta[0]);
-        add_comp(gco, t, gp);
-        add_comp(gxc, t, self_c * dn.x);
-        add_comp(gyc, t, self_c * dn.y);
+        add_comp(af, t, -comp(gp, t) * np.beta[0]);
+        add_comp(gco, t, comp(gp, t));
+        add_comp(gxc, t, self_c * comp(dn1, t));
+        add_comp(gyc, t, self_c * comp(dn2, t));
     }
-    __device__ __forceinline__ void pair2(const NearParams<float> &np, float2 r2, float2 dx, float2 dy)
+    __device__ __forceinline__ void pair2(const NearParams<float> &np, float2 w, float2 dx, float2 dy)
     {
-        float2 w = r2;
-        if constexpr (kClamp)
-            w = min1(w);
         float2 c, cp;
         near_c_cp2<P>(w, c, cp);
         const float2 f = near_f2<P>(np, w);
-        float2 g = f2(gp), n1 = f2(dn.x), n2 = f2(dn.y);
-        if constexpr (!kClamp) {
-            g = select2(r2, np.eps2, g);
-            n1 = select2(r2, np.eps2, n1);
-            n2 = select2(r2, np.eps2, n2);
+        float2 g = gp, n1 = dn1, n2 = dn2;
+        if constexpr (!kSat) {
+            g = select2(w, np.eps2, g);
+            n1 = select2(w, np.eps2, n1);
+            n2 = select2(w, np.eps2, n2);
         }
         const float2 dD = fma2(n1, dx, mul2(n2, dy));
         af = fma2(g, f, af);
@@ -344,16 +351,26 @@ template <int P> struct NearAdj32 {
     }
     __device__ __forceinline__ void row_begin() {}
     __device__ __forceinline__ void row_end() {}
-    __device__ __forceinline__ void store(int t, int64_t k)
+    __device__ __forceinline__ void fold()
+    {
+        for (float2 *v : {&af, &ac, &gxc, &gyc, &gxk, &gyk, &gco})
+            v->x += v->y;
+    }
+    __device__ __forceinline__ void reduce(int o)
+    {
+        for (float2 *v : {&af, &ac, &gxc, &gyc, &gxk, &gyk, &gco})
+            v->x = lane_add(v->x, o);
+    }
+    __device__ __forceinline__ void store(int64_t k)
     {
         const float rg = rcoef * geps;
-        const float va = fmaf(-rg * geps, comp(ac, t), comp(af, t));
-        const float vx = rg * fmaf(-2.f, comp(gxk, t), comp(gxc, t));
-        const float vy = rg * fmaf(-2.f, comp(gyk, t), comp(gyc, t));
+        const float va = fmaf(-rg * geps, ac.x, af.x);
+        const float vx = rg * fmaf(-2.f, gxk.x, gxc.x);
+        const float vy = rg * fmaf(-2.f, gyk.x, gyc.x);
         a_s[k] = assign ? va : a_s[k] + va;
         ga_s[2 * k] = assign ? vx : ga_s[2 * k] + vx;
         ga_s[2 * k + 1] = assign ? vy : ga_s[2 * k + 1] + vy;
-        cg_s[k] = comp(gco, t);
+        cg_s[k] = gco.x;
     }
 };
 
@@ -455,7 +472,7 @@ cudaError_t launch_near_hess64(int64_t N, const int *tgt_base, const double2 *tg
     return cudaGetLastError();
 }
 
-cudaError_t launch_near_adj32(int64_t n_items, const int2 *items, const int *src_base, const float2 *src_hi,
+cudaError_t launch_near_adj32(int64_t n_items, const int2 *items, int lanes, const int *src_base, const float2 *src_hi,
                               const float2 *src_lo, const float2 *tgt_hi, const float2 *tgt_lo, const int *tgt_start,
                               CellGrid cg, const float *c, const void *dn, NearParams<float> np, float *a_s,
                               float *ga_s, float *cg_s, bool assign, cudaStream_t st)
@@ -473,11 +490,11 @@ cudaError_t launch_near_adj32(int64_t n_items, const int2 *items, const int *src
         op.geps = (float)std::sqrt((double)np.eps2);
         op.inv_eps = (float)(1.0 / std::sqrt((double)np.eps2));
         op.self_c = self_hessian(np) / np.rcoef;
-        return launch_near_list(n_items, items, sd, cg, np, op, st);
+        return launch_near_list(n_items, items, lanes, sd, cg, np, op, st);
     });
 }
 
-cudaError_t launch_near_hess32(int64_t n_items, const int2 *items, const int *tgt_base, const float2 *tgt_hi,
+cudaError_t launch_near_hess32(int64_t n_items, const int2 *items, int lanes, const int *tgt_base, const float2 *tgt_hi,
                                const float2 *tgt_lo, const float2 *src_hi, const float2 *src_lo, const int *src_start,
                                CellGrid cg, const float *q, NearParams<float> np, float *grad_s, float *hess_s,
                                bool assign, cudaStream_t st)
@@ -492,7 +509,7 @@ cudaError_t launch_near_hess32(int64_t n_items, const int2 *items, const int *tg
         op.rcoef = np.rcoef;
         op.geps = (float)std::sqrt((double)np.eps2);
         op.self_c = self_hessian(np) / np.rcoef;
-        return launch_near_list(n_items, items, sd, cg, np, op, st);
+        return launch_near_list(n_items, items, lanes, sd, cg, np, op, st);
     });
 }
 

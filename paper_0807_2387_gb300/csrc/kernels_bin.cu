@@ -4,7 +4,8 @@
 // in window coordinates u = n_os (x~ + 1/2) - window_lo, and counting-sorted by
 // a tile-major cell key (histogram -> exclusive scan -> scatter).  The
 // sorted order makes every near-field cell and every spreading tile a
-// contiguous range.  Within a cell the order follows the atomic scatter.
+// contiguous range.  Within a cell the points are then sorted into strips and pieces
+// (k_cell_order), so that any piece is compact.
 #include "internal.h"
 
 namespace fs {
@@ -139,6 +140,81 @@ __global__ void k_scatter(const int *__restrict__ key, int64_t n, int *__restric
         return;
     const int pos = atomicAdd(&fill[key[i]], 1);
     perm[pos] = (int)i;
+}
+
+// Ascending bitonic sort of n2 (a power of two) keys in shared memory by the whole block.
+__device__ __forceinline__ void sort_shared(unsigned long long *key, int n2)
+{
+    for (int k = 2; k <= n2; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int t = threadIdx.x; t < n2 / 2; t += blockDim.x) {
+                const int i = 2 * t - (t & (j - 1)), l = i + j;
+                const unsigned long long a = key[i], b = key[l];
+                if ((a > b) == ((i & k) == 0)) {
+                    key[i] = b;
+                    key[l] = a;
+                }
+            }
+            __syncthreads();
+        }
+}
+
+// Points of a cell into strips along x, each strip along y (CellSplit): one block per cell.  A
+// near-field item is a piece of a strip; against runs of the Morton sub-cell order its bounding
+// box is smaller, so fewer of the evaluated pairs lie beyond eps_I.  Runs once per plan.
+constexpr int kOrderThreads = 256;
+__global__ void __launch_bounds__(kOrderThreads) k_cell_order(const int *__restrict__ start, int cap,
+                                                              const double *__restrict__ xy, double s, int n_os,
+                                                              int window_lo, int n_a, int m, int cell,
+                                                              int *__restrict__ perm)
+{
+    __shared__ unsigned long long key[kOrderRun];
+    __shared__ unsigned qy[kOrderRun];
+    __shared__ int idx[kOrderRun];
+    const int a = start[blockIdx.x * kSub], count = start[(blockIdx.x + 1) * kSub] - a;
+    if (count <= cap)
+        return;
+    for (int r = 0; r < CellSplit::runs(count); ++r) {
+        const int first = a + CellSplit::run_first(count, r), n = a + CellSplit::run_first(count, r + 1) - first;
+        const CellSplit split(n, cap);
+        int n2 = 2;
+        while (n2 < n)
+            n2 <<= 1;
+        __syncthreads();   // the previous run's keys are read
+        for (int t = threadIdx.x; t < n2; t += blockDim.x) {
+            unsigned long long k = ~0ull;
+            if (t < n) {
+                const int i = perm[first + t];
+                unsigned q[2];
+#pragma unroll
+                for (int d = 0; d < 2; ++d) {
+                    int b;
+                    double f;
+                    grid_coord(xy[2 * (int64_t)i + d], s, n_os, window_lo, b, f);
+                    clamp_base(b, m, n_a);
+                    q[d] = (unsigned)((((double)(b % cell) + f) / cell) * 4194304.0);   // offset in the cell, 22 bits
+                }
+                idx[t] = i;
+                qy[t] = q[1];
+                k = ((unsigned long long)q[0] << 16) | (unsigned)t;
+            }
+            key[t] = k;
+        }
+        __syncthreads();
+        if (split.strips > 1)
+            sort_shared(key, n2);
+        for (int t = threadIdx.x; t < n; t += blockDim.x) {
+            int strip = 0;
+            while (t >= split.strip_first(strip + 1))
+                ++strip;
+            const unsigned slot = (unsigned)key[t] & 0xffffu;
+            key[t] = ((unsigned long long)strip << 48) | ((unsigned long long)qy[slot] << 16) | slot;
+        }
+        __syncthreads();
+        sort_shared(key, n2);
+        for (int t = threadIdx.x; t < n; t += blockDim.x)
+            perm[first + t] = idx[(unsigned)key[t] & 0xffffu];
+    }
 }
 
 // Sorted records: FP64 torus position, FP32 position relative to the point's cell corner
@@ -324,6 +400,15 @@ cudaError_t launch_scatter(const int *key, int64_t n, int *fill, int *perm, cuda
     if (n <= 0)
         return cudaSuccess;
     k_scatter<<<blocks_for(n, 256), 256, 0, st>>>(key, n, fill, perm);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cell_order(const int *start, int n_cells, int cap, const double *xy, double s, int n_os,
+                              int window_lo, int n_a, int m, int cell, int *perm, cudaStream_t st)
+{
+    if (n_cells <= 0)
+        return cudaSuccess;
+    k_cell_order<<<n_cells, kOrderThreads, 0, st>>>(start, cap, xy, s, n_os, window_lo, n_a, m, cell, perm);
     return cudaGetLastError();
 }
 

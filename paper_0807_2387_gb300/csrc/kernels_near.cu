@@ -11,11 +11,8 @@
 //
 // FP64 path: one thread per target, direct FP64 formulas (the comparison path).
 //
-// FP32 path: one warp per work item of at most 64 consecutive targets of one
-// cell (two per lane, so each source read serves two targets per lane), over the
-// source sub-cells near the item's bounding box (near_warp.cuh).  A dense
-// sub-cell gets warps of its own, so a warp's targets are spatially compact (and
-// a warp never spans two cells, whose bounding box could cross the whole domain).
+// FP32 path: one warp per work item, a compact piece of a cell of at most 32 targets (one per
+// lane), over the sources near the item's bounding box (near_warp.cuh).
 // The value and gradient use the cancellation-free forms of G - T_I and of its
 // radial derivative over r, c (w - 1)^(p-1) / w with w = r^2 / eps_I^2.
 //
@@ -118,24 +115,23 @@ __global__ void __launch_bounds__(256) k_batch_near64(const BatchInst<double> *_
 }
 
 // Forward correction at the targets for R right-hand sides at once (the pair geometry, the
-// log and the gradient coefficient are shared): phi += q f, grad += q c d, with the lane's
-// two targets as packed pairs and the factor rc eps_I of c applied once at the store (d
-// arrives in units of eps_I).  With one right-hand side the sums are split into partial sums
-// per list evaluation; with several the registers go to the extra accumulators instead.
+// log and the gradient coefficient are shared): phi += q f, grad += q c d for two candidates per
+// packed operation; the factor c_ln of f (near_g2) and rc eps_I of c are applied once at the
+// store (d arrives in units of eps_I).  With one right-hand side the sums are split into partial
+// sums per list evaluation; with several the registers go to the extra accumulators instead.
 // Right-hand side r reads q + r q_stride and writes at r n_stride.
 template <int P, int R, bool BATCH = false> struct NearFwd {
-    // four blocks per SM (up to 128 registers); the single right-hand-side kernel unrolls its
-    // candidate loop eightfold (2.77 -> 2.66 ms at 2^20 points against fourfold at five blocks
-    // per SM); the batched kernel holds the instance's constants in registers (the single-plan
-    // one reads them from the constant bank) and unrolls less
-    static constexpr int kMinBlocks = 4;
-    static constexpr int kUnroll = (R == 1 && !BATCH) ? 8 : (R >= 4 ? 1 : 2);
+    static constexpr int kMinBlocks = (R == 1 && !BATCH) ? 6 : 4;   // of four warps per SM: up to 80 and 128 registers
+    static constexpr int kUnroll = BATCH ? 4 : 2;
+    // |w - 1|^(p-1) / w, the gradient coefficient over rc up to the sign (-1)^(p-1) (applied at the
+    // store), as 2^((p-1) log2(1 - w) - log2 w) (log2 w is shared with the value; w = 1 gives 2^-inf):
+    // four MUFU operations and one FMA a pair of candidates, against two and the power's
+    // multiplications.  2.26 -> 2.19 ms at 2^20 points (p = 8) against alternating the two.  Several
+    // right-hand sides add FMA work that hides the difference (batched replay the same either way).
+    static constexpr bool kExp2 = P >= 5 && !BATCH;
     static constexpr bool kRows = R == 1;
-    // the gradient coefficient through exp2 / log2 (single right-hand side: 2.57 -> 2.52 ms at
-    // 2^20 points); the batched kernels, with more FMA work per pair and less unrolling, keep the
-    // power form, whose dependency chain is shorter (the exp2 form made the batched replay 2 %
-    // slower)
-    static constexpr bool kExp2 = P >= 2 && R == 1 && !BATCH;
+    static constexpr bool kSat = P >= 2;   // f(1) = 0 and (w - 1)^(p-1) = 0: clamping w masks a pair
+    static constexpr float kPhi = P >= 2 ? kLnCoef : 1.f;   // unit of the phi sums
     const float *__restrict__ q;
     float *__restrict__ phi_s;
     float *__restrict__ grad_s;
@@ -143,8 +139,9 @@ template <int P, int R, bool BATCH = false> struct NearFwd {
     int64_t q_stride, n_stride;
     float rcoef;   // rc eps_I: the pair differences arrive in units of eps_I
     bool assign;   // store phi_s / grad_s instead of adding (the far field is added later)
-    float qj[R];
-    float2 phi[R], gx[R], gy[R], qc[R];
+    float2 qj[R];
+    float2 phi[R], gx[R], gy[R];
+    float qc[R];
     float2 rphi[kRows ? R : 1], rgx[kRows ? R : 1], rgy[kRows ? R : 1];
 
     __device__ __forceinline__ float2 &acc_phi(int r) { return kRows ? rphi[0] : phi[r]; }
@@ -154,10 +151,12 @@ template <int P, int R, bool BATCH = false> struct NearFwd {
     __device__ __forceinline__ void init()
     {
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-            phi[r] = gx[r] = gy[r] = qc[r] = f2(0.f);
+        for (int r = 0; r < R; ++r) {
+            phi[r] = gx[r] = gy[r] = f2(0.f);
+            qc[r] = 0.f;
+        }
     }
-    // candidate-list traversal: the R charges of source j, and those of a listed candidate
+    // candidate-list traversal: the R charges of source j, and those of a pair of candidates
     static constexpr int kR = R;
     __device__ __forceinline__ void fetch(int j, float (&v)[R]) const
     {
@@ -165,7 +164,7 @@ template <int P, int R, bool BATCH = false> struct NearFwd {
         for (int r = 0; r < R; ++r)
             v[r] = __ldg(q + r * q_stride + j);
     }
-    __device__ __forceinline__ void set_q(const float *v)
+    __device__ __forceinline__ void set_q(const float2 (&v)[R])
     {
 #pragma unroll
         for (int r = 0; r < R; ++r)
@@ -175,71 +174,46 @@ template <int P, int R, bool BATCH = false> struct NearFwd {
     {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            add_comp(acc_phi(r), t, -qj[r] * np.beta[0]);   // G(0) := 0 removes the far field's T_I(0)
-            add_comp(qc[r], t, qj[r]);
+            const float qs = comp(qj[r], t);
+            add_comp(acc_phi(r), t, -qs * (np.beta[0] / kPhi));   // G(0) := 0 removes the far field's T_I(0)
+            qc[r] += qs;
         }
     }
-    __device__ __forceinline__ void pair2(const NearParams<float> &np, float2 r2, float2 dx, float2 dy)
+    __device__ __forceinline__ void pair2(const NearParams<float> &np, float2 w, float2 dx, float2 dy)
     {
-        float2 w = r2;                                    // the traversal works in units of eps_I
-        if constexpr (P >= 2)
-            w = min1(w);                                  // f(1) = 0 and (w - 1)^(p-1) = 0: masked
-        const float2 val = near_f2<P>(np, w);
-        float2 coef;
-        if constexpr (kExp2) {
-            // |w - 1|^(p-1) / w = 2^((p-1) log2(1 - w) - log2 w): two MUFU operations and one FMA
-            // instead of a reciprocal and five multiplications; log2 w is shared with val, and
-            // the sign (-1)^(p-1) is applied at the store.  w = 1 (masked) gives 2^-inf = 0.
-            const float2 lw = lg2_2(w);
-            const float2 om = add2(w, f2(-1.f));   // the value's w - 1: 1 - w = -om, no add of its own
-            const float2 lo = lg2_2(make_float2(-om.x, -om.y));
-            coef = ex2_2(fma2(f2((float)(P - 1)), lo, make_float2(-lw.x, -lw.y)));
+        float2 val, coef;
+        if constexpr (P >= 2) {
+            const float2 s = fma2(w, f2(-1.f), f2(1.f)), lw = lg2_2(w);
+            val = near_g2<P>(np, w, s, lw);
+            if constexpr (kExp2)
+                coef = ex2_2(fma2(f2((float)(P - 1)), lg2_2(s), make_float2(-lw.x, -lw.y)));   // s = 0: 2^-inf
+            else
+                coef = mul2(ipow2<P - 1>(s), rcp_2(w));
         } else {
+            val = near_f2<P>(np, w);
             coef = rcp_2(w);
-            if constexpr (P >= 2)
-                coef = mul2(ipow2<P - 1>(add2(w, f2(-1.f))), coef);
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                qj[r] = select2(w, np.eps2, qj[r]);
         }
-        if constexpr (R >= 3 && P >= 2) {
+        if constexpr (R >= 3) {
             // three or more right-hand sides: the pair's gradient vector once, then one FMA per
             // component and right-hand side (batched replay 8.01 -> 7.77 ms at three)
             const float2 cdx = mul2(coef, dx), cdy = mul2(coef, dy);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const float2 qq = f2(qj[r]);
-                acc_phi(r) = fma2(qq, val, acc_phi(r));
-                acc_gx(r) = fma2(qq, cdx, acc_gx(r));
-                acc_gy(r) = fma2(qq, cdy, acc_gy(r));
+                acc_phi(r) = fma2(qj[r], val, acc_phi(r));
+                acc_gx(r) = fma2(qj[r], cdx, acc_gx(r));
+                acc_gy(r) = fma2(qj[r], cdy, acc_gy(r));
             }
         } else {
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                float2 qq = f2(qj[r]);
-                if constexpr (P == 1)
-                    qq = select2(r2, np.eps2, qq);
-                acc_phi(r) = fma2(qq, val, acc_phi(r));
-                const float2 tq = mul2(qq, coef);
+                acc_phi(r) = fma2(qj[r], val, acc_phi(r));
+                const float2 tq = mul2(qj[r], coef);
                 acc_gx(r) = fma2(tq, dx, acc_gx(r));
                 acc_gy(r) = fma2(tq, dy, acc_gy(r));
             }
-        }
-    }
-    // every other far candidate takes the power form, (1 - w)^(p-1) / w (the exp2 form's sign):
-    // a reciprocal and five multiplications instead of two MUFU operations and one FMA, so that
-    // neither pipe runs alone at its limit (2.44 -> 2.41 ms at 2^20 points)
-    static constexpr bool kAlt = kExp2;
-    __device__ __forceinline__ void pair2_alt(const NearParams<float> &np, float2 r2, float2 dx, float2 dy)
-    {
-        float2 w = min1(r2);
-        const float2 val = near_f2<P>(np, w);
-        const float2 om = add2(w, f2(-1.f));
-        float2 coef = mul2(ipow2<P - 1>(make_float2(-om.x, -om.y)), rcp_2(w));
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            float2 qq = f2(qj[r]);
-            acc_phi(r) = fma2(qq, val, acc_phi(r));
-            const float2 tq = mul2(qq, coef);
-            acc_gx(r) = fma2(tq, dx, acc_gx(r));
-            acc_gy(r) = fma2(tq, dy, acc_gy(r));
         }
     }
     __device__ __forceinline__ void row_begin()
@@ -255,22 +229,36 @@ template <int P, int R, bool BATCH = false> struct NearFwd {
             gy[0] = add2(gy[0], rgy[0]);
         }
     }
-    __device__ __forceinline__ void store(int t, int64_t k)
+    __device__ __forceinline__ void fold()
     {
-        const float rc = (kExp2 && (P - 1) % 2 == 1) ? -rcoef : rcoef;   // the exp2 coef is |w - 1|^(p-1) / w
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            phi[r].x += phi[r].y;
+            gx[r].x += gx[r].y;
+            gy[r].x += gy[r].y;
+        }
+    }
+    __device__ __forceinline__ void reduce(int o)
+    {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            phi[r].x = lane_add(phi[r].x, o);
+            gx[r].x = lane_add(gx[r].x, o);
+            gy[r].x = lane_add(gy[r].x, o);
+            qc[r] = lane_add(qc[r], o);
+        }
+    }
+    __device__ __forceinline__ void store(int64_t k)
+    {
+        const float rc = (P >= 2 && (P - 1) % 2 == 1) ? -rcoef : rcoef;   // coef is |w - 1|^(p-1) / w
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int64_t kk = k + r * n_stride;
-            if (assign) {
-                phi_s[kk] = comp(phi[r], t);
-                grad_s[2 * kk] = rc * comp(gx[r], t);
-                grad_s[2 * kk + 1] = rc * comp(gy[r], t);
-            } else {
-                phi_s[kk] += comp(phi[r], t);
-                grad_s[2 * kk] += rc * comp(gx[r], t);
-                grad_s[2 * kk + 1] += rc * comp(gy[r], t);
-            }
-            coinc[kk] = comp(qc[r], t);
+            const float p = kPhi * phi[r].x, x = rc * gx[r].x, y = rc * gy[r].x;
+            phi_s[kk] = assign ? p : phi_s[kk] + p;
+            grad_s[2 * kk] = assign ? x : grad_s[2 * kk] + x;
+            grad_s[2 * kk + 1] = assign ? y : grad_s[2 * kk + 1] + y;
+            coinc[kk] = qc[r];
         }
     }
 };
@@ -282,38 +270,42 @@ static_assert(kNearCountSlots == 64, "counter slots");
 constexpr int kCountSlots = kNearCountSlots;
 struct NearCount {
     static constexpr int kMinBlocks = 6;
-    static constexpr int kUnroll = 2;
+    static constexpr int kUnroll = 1;
+    static constexpr bool kSat = false;
     unsigned long long *__restrict__ counts;   // 2 * kCountSlots
     unsigned n_near, n_close;
 
     __device__ __forceinline__ void init() { n_near = n_close = 0; }
     static constexpr int kR = 1;   // candidate-list traversal: no values per other point
     __device__ __forceinline__ void fetch(int, float (&v)[1]) const { v[0] = 0.f; }
-    __device__ __forceinline__ void set_q(const float *) {}
+    __device__ __forceinline__ void set_q(const float2 (&)[1]) {}
     __device__ __forceinline__ void coincident(const NearParams<float> &, int)
     {
         ++n_near;
         ++n_close;
     }
-    __device__ __forceinline__ void pair2(const NearParams<float> &np, float2 r2, float2, float2)
+    __device__ __forceinline__ void pair2(const NearParams<float> &np, float2 w, float2, float2)
     {
-        n_near += (r2.x < np.eps2 ? 1u : 0u) + (r2.y < np.eps2 ? 1u : 0u);
-        n_close += (r2.x < np.close2 ? 1u : 0u) + (r2.y < np.close2 ? 1u : 0u);
+        n_near += (w.x < np.eps2 ? 1u : 0u) + (w.y < np.eps2 ? 1u : 0u);
+        n_close += (w.x < np.close2 ? 1u : 0u) + (w.y < np.close2 ? 1u : 0u);
     }
     __device__ __forceinline__ void row_begin() {}
     __device__ __forceinline__ void row_end() {}
-    __device__ __forceinline__ void store(int t, int64_t)
+    __device__ __forceinline__ void fold() {}
+    __device__ __forceinline__ void reduce(int o)
     {
-        // both slots' counts are in the lane's totals (an idle slot never lands within eps_I)
-        if (t == 0) {
-            const int slot = threadIdx.x & (kCountSlots - 1);
-            atomicAdd(&counts[2 * slot], (unsigned long long)n_near);
-            atomicAdd(&counts[2 * slot + 1], (unsigned long long)n_close);
-        }
+        n_near += __shfl_xor_sync(0xffffffffu, n_near, o);
+        n_close += __shfl_xor_sync(0xffffffffu, n_close, o);
+    }
+    __device__ __forceinline__ void store(int64_t)
+    {
+        const int slot = (threadIdx.x + 7 * blockIdx.x) & (kCountSlots - 1);
+        atomicAdd(&counts[2 * slot], (unsigned long long)n_near);
+        atomicAdd(&counts[2 * slot + 1], (unsigned long long)n_close);
     }
 };
 
-// Batched FP32 near field: one warp per item (first target, count, instance); all R
+// Batched FP32 near field: one warp per item (first target, count, instance, lanes); all R
 // right-hand sides in one candidate-list traversal.
 template <int P, int R>
 __global__ void __launch_bounds__(32 * kNearWarps, NearFwd<P, R, true>::kMinBlocks * 4 / kNearWarps) k_batch_near32(int64_t n_items,
@@ -339,9 +331,8 @@ __global__ void __launch_bounds__(32 * kNearWarps, NearFwd<P, R, true>::kMinBloc
     op.n_stride = b.N;
     op.rcoef = np.rcoef * sqrtf(np.eps2);
     op.assign = assign;
-    __shared__ NearLists<R> L;
-    const int w = threadIdx.x >> 5;
-    near_traverse_list(make_int2(it.x, it.y), lane, sd, cg, np, op, L.xy[w], L.q[w], L.cxy[w], L.cl[w], L.cq[w]);
+    __shared__ __align__(16) NearList<R> L[kNearWarps];
+    near_traverse_list(make_int2(it.x, it.y), it.w, lane, sd, cg, np, op, L[threadIdx.x >> 5]);
 }
 
 template <typename real>
@@ -398,7 +389,7 @@ cudaError_t launch_near64(int64_t N, const int *tgt_base, const double2 *tgt_pos
     return cudaGetLastError();
 }
 
-cudaError_t launch_near32(int64_t n_items, const int2 *items, const int *tgt_base, const float2 *tgt_hi,
+cudaError_t launch_near32(int64_t n_items, const int2 *items, int lanes, const int *tgt_base, const float2 *tgt_hi,
                           const float2 *tgt_lo, const float2 *src_hi, const float2 *src_lo, const int *src_start,
                           CellGrid cg, const float *q, NearParams<float> np, float *phi_s, float *grad_s, float *coinc,
                           bool assign, cudaStream_t st)
@@ -414,7 +405,7 @@ cudaError_t launch_near32(int64_t n_items, const int2 *items, const int *tgt_bas
         op.n_stride = 0;
         op.rcoef = (float)((double)np.rcoef * std::sqrt((double)np.eps2));
         op.assign = assign;
-        return launch_near_list(n_items, items, sd, cg, np, op, st);
+        return launch_near_list(n_items, items, lanes, sd, cg, np, op, st);
     });
 }
 
@@ -451,14 +442,14 @@ template cudaError_t launch_unpermute<float>(int64_t, const float *, const float
 template cudaError_t launch_unpermute<double>(int64_t, const double *, const double *, const double *, const int *,
                                               double, const double *, double, void *, void *, int, cudaStream_t);
 
-cudaError_t launch_near_count32(int64_t n_items, const int2 *items, const int *tgt_base, const float2 *tgt_hi,
+cudaError_t launch_near_count32(int64_t n_items, const int2 *items, int lanes, const int *tgt_base, const float2 *tgt_hi,
                                 const float2 *tgt_lo, const float2 *src_hi, const float2 *src_lo, const int *src_start,
                                 CellGrid cg, NearParams<float> np, unsigned long long *counts, cudaStream_t st)
 {
     const NearSides sd{tgt_base, tgt_hi, tgt_lo, src_hi, src_lo, src_start};
     NearCount op{};
     op.counts = counts;
-    return launch_near_list(n_items, items, sd, cg, np, op, st);
+    return launch_near_list(n_items, items, lanes, sd, cg, np, op, st);
 }
 
 cudaError_t launch_batch_near32(int64_t n_items, const int4 *items, const BatchInst<float> *inst, int p, int nrhs,

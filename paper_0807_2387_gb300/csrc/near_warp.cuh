@@ -2,16 +2,15 @@
 // (phi and grad phi at the targets; one or several charge vectors), the Hessian of phi at
 // the targets, the adjoint potential at the sources and the plan's pair statistics.
 //
-// A work item is at most 64 consecutive "own" points of one cell (two per lane),
-// sorted by cell and, inside a cell, by 8 x 8 sub-cell in Morton order, so the item is
-// compact.  The warp forms the bounding box of its points, reads the "other" points of the
-// neighbour cells within eps_I of that box 32 at a time, keeps those within eps_I of the box
-// (ballot) and appends them to candidate lists in shared memory, which all 32 lanes then
-// evaluate with branch-free masked arithmetic against both of their points.  Positions are
-// FP32 offsets from the cell corner stored as hi + lo; candidates within eps_I / 8 of the box
-// go to a second list that carries their position in the item's frame as hi + lo as well, so
-// the pair difference keeps full FP32 relative accuracy for nearly coincident points, and
-// exactly coincident pairs are detected (G(0) := 0).
+// A work item is a piece of a cell: at most 8, 16 or 32 consecutive "own" points (one per lane),
+// compact because the cells are sorted into pieces (CellSplit).  The warp forms the bounding box of
+// its points, reads the "other" points of the neighbour cells within eps_I of that box 32 at a
+// time, keeps those within eps_I of the box (ballot) and appends them to candidate lists in shared
+// memory, which all lanes then evaluate with branch-free masked arithmetic.  Positions are FP32
+// offsets from the cell corner stored as hi + lo; candidates within eps_I / 8 of the box go to a
+// second list that carries their position in the item's frame as hi + lo as well, so the pair
+// difference keeps full FP32 relative accuracy for nearly coincident points, and exactly
+// coincident pairs are detected (G(0) := 0).
 //
 // With w = r^2 / eps_I^2 and f = G - T_I (T_I the inner polynomial of the
 // regularised kernel, p-fold contact with G at r = eps_I):
@@ -21,9 +20,8 @@
 // (the (p-1)-fold root at w = 1 keeps c free of cancellation near r = eps_I), so
 // grad f = c d and Hess f = c I + (2 c' / eps_I^2) d d^T for d = own - other.
 //
-// The two points of a lane meet the same other point, so their arithmetic is done as
-// packed pairs (Blackwell's two-wide FP32 add, multiply and fma: one instruction for
-// both).  Pairs beyond eps_I are masked without a select where the forms allow it:
+// An own point meets two candidates at a time, their arithmetic done as packed pairs
+// (Blackwell's two-wide FP32 add, multiply and fma: one instruction for both).  Pairs beyond eps_I are masked without a select where the forms allow it:
 // with w clamped to 1, P(w) = (w - 1) Ptilde(w) and (w - 1)^(p-1) vanish exactly, as
 // does log2(1).
 #pragma once
@@ -95,7 +93,7 @@ __device__ __forceinline__ float ex2_approx(float x)
     return y;
 }
 
-// ---- packed pairs of FP32 values (x: the lane's first point, y: its second)
+// ---- packed pairs of FP32 values (x: the first candidate, y: the second)
 
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -148,6 +146,19 @@ template <int P> __device__ __forceinline__ float2 near_f2(const NearParams<floa
     }
 }
 
+// f / c_ln with c_ln = -(ln 2) / (4 pi), applied by the caller at the store: since P(w) =
+// (w - 1) Ptilde(w), f / c_ln = log2 w + s Ptilde(w) / c_ln with s = 1 - w: one FMA after the
+// polynomial.  w <= 1 (clamped) and degree p >= 2.
+constexpr float kLnCoef = -0.69314718055994531f / (4.0f * 3.14159265358979324f);
+template <int P> __device__ __forceinline__ float2 near_g2(const NearParams<float> &np, float2 w, float2 s, float2 lw)
+{
+    float2 t = f2(np.ptln[P - 2]);
+#pragma unroll
+    for (int i = P - 3; i >= 0; --i)
+        t = fma2(t, w, f2(np.ptln[i]));
+    return fma2(s, t, lw);
+}
+
 // c / rc = (w - 1)^(p-1) / w and c' / rc = (w - 1)^(p-2) ((p - 2) w + 1) / w^2 (rc applied by the caller).
 template <int P> __device__ __forceinline__ void near_c_cp2(float2 w, float2 &c, float2 &cp)
 {
@@ -163,8 +174,7 @@ template <int P> __device__ __forceinline__ void near_c_cp2(float2 w, float2 &c,
     }
 }
 
-// The two point sets of a traversal: the item's own points (one per lane slot) and the
-// other side's points, visited by sub-cell.
+// The two point sets of a traversal: the items' own points and the other side's.
 struct NearSides {
     const int *own_base;
     const float2 *own_hi, *own_lo;
@@ -178,66 +188,80 @@ struct NearSides {
 // (a cell is one contiguous range, so the chunks are full, where sub-cells would hold only a
 // few points each), test each against the box (ballot) and append those within reach to the
 // warp's lists in shared memory: "far" candidates (beyond eps_I / 8 of the box: no pair can
-// need the refined difference) shifted into the item's cell frame and negated,
-// (-x, -x, -y, -y), with their Op::kR values (charges, or the adjoint's weights); "close"
-// candidates the same way as hi + lo pairs (the TwoSum of the cell step and -y_hi, with -y_lo
-// added to the low part), for the refined path.  A list is
-// evaluated when it fills and at the end: one shared broadcast load per candidate and no
-// per-candidate test or vote in the far loop.  Partial sums are kept per list evaluation
-// (op.row_begin / row_end).  An Op provides kMinBlocks, kUnroll, kR, init(), fetch(j, v)
-// (the kR values of other point j), set_q(v) (those of the current candidate),
-// coincident(np, t) (slot t = 0, 1 coincides with it), pair2(np, r2, dx, dy) (both slots
-// packed; dx, dy and r2 in units of eps_I, so w = r2, and np carries eps2 = inv_eps2 = 1 and
-// close2 = 1/64; pairs with r2 >= 1 must contribute nothing), row_begin(), row_end() and
-// store(t, k).
+// need the refined difference) shifted into the item's cell frame, negated and in units of eps_I,
+// with their Op::kR values (charges, or the adjoint's weights); "close" candidates the same way as
+// hi + lo (the TwoSum of the cell step and -y_hi, with -y_lo added to the low part), for the
+// refined path.  A list is one array per component (an append is one address, a read four
+// candidates per 16 bytes), padded with far-away entries of value 0 to a whole number of rounds
+// and evaluated when it fills and at the end: broadcast shared loads and no per-candidate test or
+// vote in the far loop.  Partial sums are kept per list evaluation (op.row_begin / row_end).
+//
+// An item holds at most `lanes` own points, one per lane; the 32 / lanes groups of the warp take
+// different candidates and their sums are added at the end (op.reduce).  Small items have small
+// boxes, so more of the evaluated pairs lie within eps_I, and there are more of them to fill the
+// GPU; large ones build fewer lists (near_item_lanes).
+//
+// What bounds it (2^20-point mixture, 32 lanes, 2.2e9 pairs within eps_I, 0.75 of the evaluated ones):
+// the issue slots; a pair of candidates is 26 instructions (34 FMA-pipe cycles and 40 of the MUFU
+// pipe for 64 pair slots), 1.2e9 of the 1.78e9 in all, the lists are most of the rest.  2.75 ms
+// with items of 64 targets (two per lane, runs of the Morton sub-cell order) -> 2.18 ms.  Tried and
+// not kept: bounding boxes of groups of 32 other points tested before the points (2.23 ms; at 45
+// points per cell 49 against 43 us); the lists' entries (first point, mask) kept with the plan
+// (2.09 ms, at 45 per cell 51 against 41 us, 40 bytes per target and twice the plan's time);
+// alternating the gradient's exp2 and power forms (2.26 ms).
+//
+// An Op provides kMinBlocks, kUnroll (fours of candidates), kR, kSat (w = min(r2, 1) is all it needs: the clamp rides on the last
+// FMA of r2), init(), fetch(j, v) (the kR values of other point j), set_q(v) (those of a pair of
+// candidates), coincident(np, t) (candidate t of the pair coincides with the own point),
+// pair2(np, w, dx, dy) (both candidates packed; dx, dy in units of eps_I, w = r^2, and np carries
+// eps2 = inv_eps2 = 1; pairs with w >= 1 must contribute nothing), row_begin(), row_end(), fold()
+// (the two packed halves of each sum together), reduce(o) (add the sums of the lane at xor distance
+// o) and store(k).
 constexpr int kListCap = 256;    // far candidates per warp
 constexpr int kCloseCap = 64;    // close candidates per warp
+constexpr float kPadPos = 1e9f;  // a padding entry's position: beyond eps_I of every point (idle lanes sit at 1e6 / eps_I)
 
-// Ops with kAlt = true alternate two forms of the pair arithmetic between consecutive far
-// candidates (pair2, pair2_alt) whose pipe mixes differ, so that the FMA and MUFU pipes share
-// the load; the others evaluate every candidate with pair2.
-template <class Op, class = void> struct AltForms : std::false_type {};
-template <class Op> struct AltForms<Op, std::void_t<decltype(Op::kAlt)>> : std::bool_constant<Op::kAlt> {};
+__device__ __forceinline__ float2 near_w2(bool sat, float2 dx, float2 dy)
+{
+    const float2 m = mul2(dx, dx);
+    if (sat)
+        return make_float2(__saturatef(fmaf(dy.x, dy.x, m.x)), __saturatef(fmaf(dy.y, dy.y, m.y)));
+    return fma2(dy, dy, m);
+}
 
+// Four values of each of the R arrays of stride `cap`, as two pairs.
+template <int R>
+__device__ __forceinline__ void near_list_q(const float *s_q, int cap, int e, float2 (&qa)[R], float2 (&qb)[R])
+{
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float4 q = *reinterpret_cast<const float4 *>(s_q + r * cap + 4 * e);
+        qa[r] = make_float2(q.x, q.y);
+        qb[r] = make_float2(q.z, q.w);
+    }
+}
+
+// n candidates (a multiple of 4 x groups); group g of `groups` takes every groups-th four of them.
 template <class Op>
-__device__ __forceinline__ void near_eval_far(const float4 *s_xy, const float *s_q, int n, float2 X, float2 Y,
-                                              const NearParams<float> &np, Op &op)
+__device__ __forceinline__ void near_eval_far(const float *s_x, const float *s_y, const float *s_q, int n, int g,
+                                              int groups, float2 X, float2 Y, const NearParams<float> &np, Op &op)
 {
     op.row_begin();
-    if constexpr (AltForms<Op>::value) {
-        int e = 0;
-#pragma unroll(Op::kUnroll / 2)
-        for (; e + 1 < n; e += 2) {
-            {
-                const float4 a = s_xy[e];
-                op.set_q(s_q + e * Op::kR);
-                const float2 dx = add2(X, make_float2(a.x, a.y));
-                const float2 dy = add2(Y, make_float2(a.z, a.w));
-                op.pair2(np, fma2(dy, dy, mul2(dx, dx)), dx, dy);
-            }
-            {
-                const float4 a = s_xy[e + 1];
-                op.set_q(s_q + (e + 1) * Op::kR);
-                const float2 dx = add2(X, make_float2(a.x, a.y));
-                const float2 dy = add2(Y, make_float2(a.z, a.w));
-                op.pair2_alt(np, fma2(dy, dy, mul2(dx, dx)), dx, dy);
-            }
-        }
-        if (e < n) {
-            const float4 a = s_xy[e];
-            op.set_q(s_q + e * Op::kR);
-            const float2 dx = add2(X, make_float2(a.x, a.y));
-            const float2 dy = add2(Y, make_float2(a.z, a.w));
-            op.pair2(np, fma2(dy, dy, mul2(dx, dx)), dx, dy);
-        }
-    } else {
+    const int quads = n >> 2;
 #pragma unroll(Op::kUnroll)
-        for (int e = 0; e < n; ++e) {
-            const float4 a = s_xy[e];
-            op.set_q(s_q + e * Op::kR);
-            const float2 dx = add2(X, make_float2(a.x, a.y));
-            const float2 dy = add2(Y, make_float2(a.z, a.w));
-            op.pair2(np, fma2(dy, dy, mul2(dx, dx)), dx, dy);
+    for (int e = g; e < quads; e += groups) {
+        const float4 x = *reinterpret_cast<const float4 *>(s_x + 4 * e), y = *reinterpret_cast<const float4 *>(s_y + 4 * e);
+        float2 qa[Op::kR], qb[Op::kR];
+        near_list_q<Op::kR>(s_q, kListCap, e, qa, qb);
+        {
+            const float2 dx = add2(X, make_float2(x.x, x.y)), dy = add2(Y, make_float2(y.x, y.y));
+            op.set_q(qa);
+            op.pair2(np, near_w2(Op::kSat, dx, dy), dx, dy);
+        }
+        {
+            const float2 dx = add2(X, make_float2(x.z, x.w)), dy = add2(Y, make_float2(y.z, y.w));
+            op.set_q(qb);
+            op.pair2(np, near_w2(Op::kSat, dx, dy), dx, dy);
         }
     }
     op.row_end();
@@ -251,76 +275,107 @@ __device__ __forceinline__ void near_eval_far(const float4 *s_xy, const float *s
 // (G(0) := 0); they are handled on a warp-uniform branch.  The exact difference is then scaled
 // by ie = 1 / eps_I, the unit of every difference handed to the Op.
 template <class Op>
-__device__ __forceinline__ void near_eval_close(const float4 *s_cxy, const float4 *s_cl, const float *s_cq, int n,
+__device__ __forceinline__ void near_eval_close(const float *s_x, const float *s_y, const float *s_lx,
+                                                const float *s_ly, const float *s_q, int n, int g, int groups,
                                                 float2 X, float2 Y, float2 XL, float2 YL, float ie,
                                                 const NearParams<float> &np, Op &op)
 {
     op.row_begin();
-    for (int e = 0; e < n; ++e) {
-        const float4 c = s_cxy[e];                // (n_hi.x, n_hi.x, n_hi.y, n_hi.y)
-        const float4 l = s_cl[e];                 // (n_lo.x, n_lo.x, n_lo.y, n_lo.y)
-        op.set_q(s_cq + e * Op::kR);
-        const float2 ex = add2(add2(X, make_float2(c.x, c.y)), add2(XL, make_float2(l.x, l.y)));
-        const float2 ey = add2(add2(Y, make_float2(c.z, c.w)), add2(YL, make_float2(l.z, l.w)));
-        const float2 dx = mul2(ex, f2(ie)), dy = mul2(ey, f2(ie));   // in units of eps_I
-        float2 r2 = fma2(dy, dy, mul2(dx, dx));
-        const bool z0 = ex.x == 0.f && ey.x == 0.f, z1 = ex.y == 0.f && ey.y == 0.f;
-        if (__any_sync(0xffffffffu, z0 || z1)) {
-            if (z0) {
-                op.coincident(np, 0);
-                r2.x = np.eps2;                   // masked out: w = 1
+    for (int e = g; e < n >> 2; e += groups) {
+        const float4 x = *reinterpret_cast<const float4 *>(s_x + 4 * e), y = *reinterpret_cast<const float4 *>(s_y + 4 * e);
+        const float4 lx = *reinterpret_cast<const float4 *>(s_lx + 4 * e), ly = *reinterpret_cast<const float4 *>(s_ly + 4 * e);
+        float2 q2[2][Op::kR];
+        near_list_q<Op::kR>(s_q, kCloseCap, e, q2[0], q2[1]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 hx = h ? make_float2(x.z, x.w) : make_float2(x.x, x.y);
+            const float2 hy = h ? make_float2(y.z, y.w) : make_float2(y.x, y.y);
+            const float2 ox = h ? make_float2(lx.z, lx.w) : make_float2(lx.x, lx.y);
+            const float2 oy = h ? make_float2(ly.z, ly.w) : make_float2(ly.x, ly.y);
+            op.set_q(q2[h]);
+            const float2 ex = add2(add2(X, hx), add2(XL, ox));
+            const float2 ey = add2(add2(Y, hy), add2(YL, oy));
+            const float2 dx = mul2(ex, f2(ie)), dy = mul2(ey, f2(ie));   // in units of eps_I
+            float2 w = near_w2(Op::kSat, dx, dy);
+            const bool z0 = ex.x == 0.f && ey.x == 0.f, z1 = ex.y == 0.f && ey.y == 0.f;
+            if (__any_sync(0xffffffffu, z0 || z1)) {
+                if (z0) {
+                    op.coincident(np, 0);
+                    w.x = 1.f;                        // masked out
+                }
+                if (z1) {
+                    op.coincident(np, 1);
+                    w.y = 1.f;
+                }
             }
-            if (z1) {
-                op.coincident(np, 1);
-                r2.y = np.eps2;
-            }
+            op.pair2(np, w, dx, dy);
         }
-        op.pair2(np, r2, dx, dy);
     }
     op.row_end();
 }
 
+// A warp's lists: x, y and the R values of kListCap far candidates; x, y, their low parts and the R
+// values of kCloseCap close ones.
+template <int R> struct NearList {
+    float x[kListCap], y[kListCap], q[kListCap * R];
+    float cx[kCloseCap], cy[kCloseCap], lx[kCloseCap], ly[kCloseCap], cq[kCloseCap * R];
+    __device__ __forceinline__ void put(int at, float px, float py, const float (&v)[R])
+    {
+        x[at] = px;
+        y[at] = py;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            q[r * kListCap + at] = v[r];
+    }
+    __device__ __forceinline__ void put_close(int at, float px, float py, float plx, float ply, const float (&v)[R])
+    {
+        cx[at] = px;
+        cy[at] = py;
+        lx[at] = plx;
+        ly[at] = ply;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            cq[r * kCloseCap + at] = v[r];
+    }
+    // pads n entries to a multiple of `unit` (at most 32); returns the padded count
+    __device__ __forceinline__ int pad(int n, int unit, int lane)
+    {
+        const float none[R] = {};
+        const int full = (n + unit - 1) & ~(unit - 1);
+        if (n + lane < full)
+            put(n + lane, kPadPos, kPadPos, none);
+        return full;
+    }
+    __device__ __forceinline__ int pad_close(int n, int unit, int lane)
+    {
+        const float none[R] = {};
+        const int full = (n + unit - 1) & ~(unit - 1);
+        if (n + lane < full)
+            put_close(n + lane, kPadPos, kPadPos, 0.f, 0.f, none);
+        return full;
+    }
+};
+
 template <class Op>
-__device__ __forceinline__ void near_traverse_list(int2 item, int lane, const NearSides &sd, const CellGrid &cg,
-                                                   const NearParams<float> &np, Op &op, float4 *s_xy, float *s_q,
-                                                   float4 *s_cxy, float4 *s_cl, float *s_cq)
+__device__ __forceinline__ void near_traverse_list(int2 item, int lanes, int lane, const NearSides &sd,
+                                                   const CellGrid &cg, const NearParams<float> &np, Op &op,
+                                                   NearList<Op::kR> &L)
 {
     constexpr int R = Op::kR;
     const float h = np.hcell, eps = sqrtf(np.eps2);
-    bool valid[2];
-    int64_t kt[2];
-    int cc1[2], cc2[2];
-    float2 xh[2], xl[2];
-    float tx0 = 3e38f, tx1 = -3e38f, ty0 = 3e38f, ty1 = -3e38f;
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        valid[t] = lane + 32 * t < item.y;
-        kt[t] = item.x + lane + 32 * t;
-        const int64_t kk = valid[t] ? kt[t] : item.x;
-        const int packed = sd.own_base[kk];
-        cc1[t] = base1(packed) / cg.cell;
-        cc2[t] = base2(packed) / cg.cell;
-        xh[t] = sd.own_hi[kk];
-        xl[t] = sd.own_lo[kk];
-        if (valid[t]) {
-            const float ax = (float)cc1[t] * h + xh[t].x, ay = (float)cc2[t] * h + xh[t].y;
-            tx0 = fminf(tx0, ax);
-            tx1 = fmaxf(tx1, ax);
-            ty0 = fminf(ty0, ay);
-            ty1 = fmaxf(ty1, ay);
-        }
-    }
-    tx0 = warp_min(tx0);
-    tx1 = warp_max(tx1);
-    ty0 = warp_min(ty0);
-    ty1 = warp_max(ty1);
-    const int c1 = cc1[0], c2 = cc2[0];
-#pragma unroll
-    for (int t = 0; t < 2; ++t)
-        if (!valid[t])
-            xh[t] = make_float2(1e6f, 1e6f);      // idle slots: every pair lands beyond eps_I
-    const float2 X = make_float2(xh[0].x, xh[1].x), Y = make_float2(xh[0].y, xh[1].y);
-    const float2 XL = make_float2(xl[0].x, xl[1].x), YL = make_float2(xl[0].y, xl[1].y);
+    const int groups = 32 / lanes, slot = lane & (lanes - 1), g = lane / lanes;
+    const bool valid = slot < item.y;
+    const int64_t k = item.x + (valid ? slot : 0);
+    const int packed = sd.own_base[k];
+    const int c1 = base1(packed) / cg.cell, c2 = base2(packed) / cg.cell;   // the item's cell
+    float2 xh = sd.own_hi[k];
+    const float2 xl = sd.own_lo[k];
+    // bounding box in the item's frame, offsets from its cell's corner (idle lanes hold the first point)
+    const float tx0 = warp_min(xh.x), tx1 = warp_max(xh.x);
+    const float ty0 = warp_min(xh.y), ty1 = warp_max(xh.y);
+    if (!valid)
+        xh = make_float2(1e6f, 1e6f);             // idle lanes: every pair lands beyond eps_I
+    const float2 X = f2(xh.x), Y = f2(xh.y), XL = f2(xl.x), YL = f2(xl.y);
     // the Op sees differences in units of eps_I, so w = r^2 needs no scaling per pair: the far
     // list holds sources in those units and the item's points are scaled once here
     const float ie = sqrtf(np.inv_eps2);
@@ -334,124 +389,136 @@ __device__ __forceinline__ void near_traverse_list(int2 item, int lane, const Ne
     const float reach2 = reach * reach;
     const float close_reach = sqrtf(np.close2) + margin;
     const float close_reach2 = close_reach * close_reach;
-    const int cx0 = max(0, (int)floorf((tx0 - reach) / h)), cx1 = min(cg.n_c - 1, (int)floorf((tx1 + reach) / h));
-    const int cy0 = max(0, (int)floorf((ty0 - reach) / h)), cy1 = min(cg.n_c - 1, (int)floorf((ty1 + reach) / h));
     const unsigned below = (1u << lane) - 1u;
     int nf = 0, nc = 0;
     op.init();
-    // whole neighbour cells (contiguous source ranges), read in full chunks of 32
-    for (int ex = cx0; ex <= cx1; ++ex) {
-        const float offx = (float)(c1 - ex) * h;
-        const float sx0 = (float)ex * h;
-        const float gapx = fmaxf(0.f, fmaxf(sx0 - tx1, tx0 - (sx0 + h)));
-        for (int ey = cy0; ey <= cy1; ++ey) {
-            const float offy = (float)(c2 - ey) * h;
-            const float sy0 = (float)ey * h;
-            const float gapy = fmaxf(0.f, fmaxf(sy0 - ty1, ty0 - (sy0 + h)));
-            if (gapx * gapx + gapy * gapy > reach2)
-                continue;                           // the whole cell is beyond reach (warp-uniform)
+    // the 3 x 3 cells around the item's (cells are at least eps_I wide), one per lane: those with
+    // points and within reach of the box
+    int c_j0 = 0, c_j1 = 0;
+    float c_ox = 0.f, c_oy = 0.f;                 // step from the cell's frame to the item's
+    if (lane < 9) {
+        const int ex = c1 - 1 + lane / 3, ey = c2 - 1 + lane % 3;
+        c_ox = (float)(c1 - ex) * h;
+        c_oy = (float)(c2 - ey) * h;
+        const float gapx = fmaxf(0.f, fmaxf(-c_ox - tx1, tx0 - (h - c_ox)));
+        const float gapy = fmaxf(0.f, fmaxf(-c_oy - ty1, ty0 - (h - c_oy)));
+        if (ex >= 0 && ex < cg.n_c && ey >= 0 && ey < cg.n_c && gapx * gapx + gapy * gapy <= reach2) {
             const int kbase = cg.key(ex, ey) * kSub;
-            const int j0 = sd.oth_start[kbase], j1 = sd.oth_start[kbase + kSub];
-            for (int jb = j0; jb < j1; jb += 32) {
-                const int j = jb + lane;
-                const bool in = j < j1;
-                float2 yh = make_float2(0.f, 0.f);
-                float qv[R];
+            c_j0 = sd.oth_start[kbase];
+            c_j1 = sd.oth_start[kbase + kSub];
+        }
+    }
+    unsigned cells = __ballot_sync(0xffffffffu, c_j0 < c_j1);
+    // their points in chunks of 32, each chunk's loads issued while the one before is listed
+    int jb = 0, j1 = 0;
+    float offx = 0.f, offy = 0.f;
+    auto next_cell = [&]() {
+        const int c = cells ? __ffs(cells) - 1 : 31;   // lane 31: an empty range
+        cells &= cells - 1;
+        jb = __shfl_sync(0xffffffffu, c_j0, c);
+        j1 = __shfl_sync(0xffffffffu, c_j1, c);
+        offx = __shfl_sync(0xffffffffu, c_ox, c);
+        offy = __shfl_sync(0xffffffffu, c_oy, c);
+    };
+    float2 ny = make_float2(0.f, 0.f);
+    float nq[R];
 #pragma unroll
-                for (int r = 0; r < R; ++r)
-                    qv[r] = 0.f;
-                if (in) {
-                    yh = __ldg(sd.oth_hi + j);
-                    op.fetch(j, qv);
-                }
-                const float ax = sx0 + yh.x, ay = sy0 + yh.y;
-                const float gx = fmaxf(0.f, fmaxf(ax - tx1, tx0 - ax));
-                const float gy = fmaxf(0.f, fmaxf(ay - ty1, ty0 - ay));
-                const float g2 = gx * gx + gy * gy;
-                const bool keep = in && g2 <= reach2;
-                const bool close = keep && g2 <= close_reach2;
-                const unsigned mf = __ballot_sync(0xffffffffu, keep && !close);
-                const unsigned mc = __ballot_sync(0xffffffffu, close);
-                if (keep && !close) {
-                    const int at = nf + __popc(mf & below);
-                    // -(source in the item's frame), in units of eps_I
-                    const float nx = (offx - yh.x) * ie, ny = (offy - yh.y) * ie;
-                    s_xy[at] = make_float4(nx, nx, ny, ny);
+    for (int r = 0; r < R; ++r)
+        nq[r] = 0.f;
+    auto load = [&]() {
+        if (jb + lane < j1) {
+            ny = __ldg(sd.oth_hi + jb + lane);
+            op.fetch(jb + lane, nq);
+        }
+    };
+    next_cell();
+    load();
+    while (jb < j1) {
+        const float2 yh = ny;
+        const int j = jb + lane;
+        const bool in = j < j1;
+        const float ox = offx, oy = offy;
+        float qv[R];
 #pragma unroll
-                    for (int r = 0; r < R; ++r)
-                        s_q[at * R + r] = qv[r];
-                }
-                if (close) {
-                    const int at = nc + __popc(mc & below);
-                    const float2 yl = __ldg(sd.oth_lo + j);
-                    // -(source in the item's frame) = off - y_hi - y_lo as hi + lo (TwoSum of off and -y_hi)
-                    const float hx = offx - yh.x, bx = hx - offx;
-                    const float lx = ((offx - (hx - bx)) + (-yh.x - bx)) - yl.x;
-                    const float hy = offy - yh.y, by = hy - offy;
-                    const float ly = ((offy - (hy - by)) + (-yh.y - by)) - yl.y;
-                    s_cxy[at] = make_float4(hx, hx, hy, hy);
-                    s_cl[at] = make_float4(lx, lx, ly, ly);
-#pragma unroll
-                    for (int r = 0; r < R; ++r)
-                        s_cq[at * R + r] = qv[r];
-                }
-                nf += __popc(mf);
-                nc += __popc(mc);
-                if (nf > kListCap - 32) {
-                    __syncwarp();
-                    near_eval_far(s_xy, s_q, nf, XS, YS, nps, op);
-                    nf = 0;
-                    __syncwarp();
-                }
-                if (nc > kCloseCap - 32) {
-                    __syncwarp();
-                    near_eval_close(s_cxy, s_cl, s_cq, nc, X, Y, XL, YL, ie, nps, op);
-                    nc = 0;
-                    __syncwarp();
-                }
+        for (int r = 0; r < R; ++r)
+            qv[r] = nq[r];
+        jb += 32;
+        if (jb >= j1)
+            next_cell();
+        load();
+        const float fx = ox - yh.x, fy = oy - yh.y;   // -(source in the item's frame)
+        const float gx = fmaxf(0.f, fmaxf(-fx - tx1, tx0 + fx));
+        const float gy = fmaxf(0.f, fmaxf(-fy - ty1, ty0 + fy));
+        const float g2 = gx * gx + gy * gy;
+        const bool keep = in && g2 <= reach2, close = in && g2 <= close_reach2;
+        const unsigned mc = __ballot_sync(0xffffffffu, close), mf = __ballot_sync(0xffffffffu, keep) & ~mc;
+        if (keep && !close)   // -(source in the item's frame), in units of eps_I
+            L.put(nf + __popc(mf & below), fx * ie, fy * ie, qv);
+        nf += __popc(mf);
+        if (nf > kListCap - 32) {
+            nf = L.pad(nf, 4 * groups, lane);
+            __syncwarp();
+            near_eval_far(L.x, L.y, L.q, nf, g, groups, XS, YS, nps, op);
+            nf = 0;
+            __syncwarp();
+        }
+        if (mc) {
+            if (close) {
+                const float2 yl = __ldg(sd.oth_lo + j);
+                // -(source in the item's frame) = off - y_hi - y_lo as hi + lo (TwoSum of off and -y_hi)
+                const float bx = fx - ox, by = fy - oy;
+                const float lx = ((ox - (fx - bx)) + (-yh.x - bx)) - yl.x;
+                const float ly = ((oy - (fy - by)) + (-yh.y - by)) - yl.y;
+                L.put_close(nc + __popc(mc & below), fx, fy, lx, ly, qv);
+            }
+            nc += __popc(mc);
+            if (nc > kCloseCap - 32) {
+                nc = L.pad_close(nc, 4 * groups, lane);
+                __syncwarp();
+                near_eval_close(L.cx, L.cy, L.lx, L.ly, L.cq, nc, g, groups, X, Y, XL, YL, ie, nps, op);
+                nc = 0;
+                __syncwarp();
             }
         }
     }
+    nf = L.pad(nf, 4 * groups, lane);
+    nc = L.pad_close(nc, 4 * groups, lane);
     __syncwarp();
-    near_eval_far(s_xy, s_q, nf, XS, YS, nps, op);
-    near_eval_close(s_cxy, s_cl, s_cq, nc, X, Y, XL, YL, ie, nps, op);
-#pragma unroll
-    for (int t = 0; t < 2; ++t)
-        if (valid[t])
-            op.store(t, kt[t]);
+    near_eval_far(L.x, L.y, L.q, nf, g, groups, XS, YS, nps, op);
+    near_eval_close(L.cx, L.cy, L.lx, L.ly, L.cq, nc, g, groups, X, Y, XL, YL, ie, nps, op);
+    op.fold();
+    for (int o = 16; o >= lanes; o >>= 1)
+        op.reduce(o);
+    if (valid && g == 0)
+        op.store(k);
 }
 
-// Warps per block of the candidate-list kernels (a warp per item), and their per-warp lists
-// (R charges per candidate).  An Op's kMinBlocks counts blocks of four warps.
-constexpr int kNearWarps = 4;
-template <int R> struct NearLists {
-    float4 xy[kNearWarps][kListCap];
-    float q[kNearWarps][kListCap * R];
-    float4 cxy[kNearWarps][kCloseCap];
-    float4 cl[kNearWarps][kCloseCap];
-    float cq[kNearWarps][kCloseCap * R];
-};
+__device__ __forceinline__ float lane_add(float v, int o) { return v + __shfl_xor_sync(0xffffffffu, v, o); }
 
+// Warps per block of the candidate-list kernels (a warp per item).  An Op's kMinBlocks counts
+// blocks of four warps.
+constexpr int kNearWarps = 4;
 template <class Op>
 __global__ void __launch_bounds__(32 * kNearWarps, Op::kMinBlocks * 4 / kNearWarps) k_near_list(int64_t n_items, const int2 *__restrict__ items,
-                                                                   NearSides sd, CellGrid cg, NearParams<float> np,
-                                                                   Op op)
+                                                                   int lanes, NearSides sd, CellGrid cg,
+                                                                   NearParams<float> np, Op op)
 {
-    __shared__ NearLists<Op::kR> L;
+    __shared__ __align__(16) NearList<Op::kR> L[kNearWarps];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (warp >= n_items)
         return;                                   // whole warp past the end; no block-wide barrier follows
-    near_traverse_list(items[warp], lane, sd, cg, np, op, L.xy[w], L.q[w], L.cxy[w], L.cl[w], L.cq[w]);
+    near_traverse_list(items[warp], lanes, lane, sd, cg, np, op, L[w]);
 }
 
-template <class Op> cudaError_t launch_near_list(int64_t n_items, const int2 *items, const NearSides &sd, CellGrid cg,
-                                                 const NearParams<float> &np, const Op &op, cudaStream_t st)
+template <class Op> cudaError_t launch_near_list(int64_t n_items, const int2 *items, int lanes, const NearSides &sd,
+                                                 CellGrid cg, const NearParams<float> &np, const Op &op,
+                                                 cudaStream_t st)
 {
     if (n_items <= 0)
         return cudaSuccess;
     const unsigned blocks = (unsigned)((n_items + kNearWarps - 1) / kNearWarps);
-    k_near_list<Op><<<blocks, 32 * kNearWarps, 0, st>>>(n_items, items, sd, cg, np, op);
+    k_near_list<Op><<<blocks, 32 * kNearWarps, 0, st>>>(n_items, items, lanes, sd, cg, np, op);
     return cudaGetLastError();
 }
 

@@ -17,6 +17,14 @@ namespace fs {
 fs_status fail(fs_status st, const std::string &msg);
 
 constexpr int kStages = 8;
+
+// A cell's run of near-field items: `count` items of one size from item `first` on, and the
+// estimated pair work of each.
+struct NearCell {
+    int64_t work;
+    int first, count;
+};
+constexpr int kSrcMajorItem = 64;   // sources per item of the source-major near field
 constexpr int kSpreadChunk = 512;   // sources per spreading work item
 // 2D plans whose occupied spreading tiles hold fewer sources than this on average spread with
 // global atomics (the plan's choice in plan_init).  Zero: on GB300 the tiles won at every
@@ -69,6 +77,8 @@ struct fs_plan {
     float2 *src_pos32 = nullptr, *tgt_pos32 = nullptr;
     float2 *src_lo32 = nullptr, *tgt_lo32 = nullptr;
     int *src_start = nullptr, *tgt_start = nullptr;
+    std::vector<int> src_cells, tgt_cells;   // the cells' first points (host)
+    int src_cap = 0, tgt_cap = 0;            // points per piece of a cell: 8, 16, 32 (64: source-major)
     fs::SpreadItem *items = nullptr;
     int n_items = 0;
     fs::SpreadItem *tgt_items = nullptr;  // adjoint: spreading at the targets
@@ -77,12 +87,14 @@ struct fs_plan {
     void *adj_c = nullptr, *adj_dn = nullptr, *adj_df = nullptr;
     void *adj_a = nullptr, *adj_ga = nullptr, *adj_cg = nullptr, *adj_hess = nullptr;
     double *adj_gsum = nullptr;
-    int2 *near_items = nullptr;       // FP32 near field: (first target, count <= 64) per warp
+    int2 *near_items = nullptr;       // FP32 near field: (first target, count <= tgt_cap) per warp
     int64_t n_near_items = 0;
     std::vector<int2> near_items_h;   // host copies (merged into batch work lists)
-    std::vector<int64_t> near_work_h; // estimated pair work per near item
+    std::vector<fs::NearCell> near_cells_h;
     std::vector<fs::SpreadItem> items_h;
-    int2 *src_near_items = nullptr;   // FP32 adjoint and source-major near field: (first source, count <= 64)
+    int2 *adj_items = nullptr;        // FP32 adjoint: (first source, count <= min(src_cap, 32))
+    int64_t n_adj_items = 0;
+    int2 *src_near_items = nullptr;   // source-major near field: (first source, count <= 64)
     int64_t n_src_near_items = 0;
     bool src_major = false;           // FP32 forward near field over source items (many more sources than targets)
     void *mul = nullptr, *tw = nullptr;
@@ -216,6 +228,9 @@ template <typename real> inline NearParams<real> make_near(const fs_plan *pl)
             t[k] = a[k + 1] + (k + 1 <= pl->p - 2 ? t[k + 1] : 0.0);
         for (int k = 0; k + 1 < pl->p; ++k)
             np.nptilde[k] = (real)(-t[k]);
+        const double c_ln = -std::log(2.0) / (4.0 * kPi);
+        for (int k = 0; k + 1 < pl->p; ++k)
+            np.ptln[k] = (real)(t[k] / c_ln);
     }
     // R(w) = c (w-1)^(p-1) with R(0) = -(1/2pi) gives c = (-1)^p / (2pi), independent of beta
     np.rcoef = (real)(((pl->p % 2 == 0) ? 1.0 : -1.0) / (2.0 * kPi * pl->eps_I * pl->eps_I));

@@ -1,0 +1,42 @@
+"""The FP32 near field's items: cells sorted into pieces, 8, 16 or 32 points to a warp (GPU).
+
+The FP64 path, which loops over the points of the cells, is the reference.  Tolerance: 2e-5, the bar of
+the FP32-vs-FP64 gates of small cases (FP32 rounding of the pair sums and of the grid, ~1e-6 here).
+"""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def rel(a, b):
+    a, b = a.double().cpu().numpy(), b.double().cpu().numpy()
+    return max(np.linalg.norm(a - b) / np.linalg.norm(b), np.max(np.abs(a - b)) / np.max(np.abs(b)))
+
+
+@pytest.mark.parametrize("n_src,n_tgt", [(1, 1), (7, 9), (24, 26), (33, 31), (65, 63), (99, 101), (129, 513), (2048, 2049),
+                                         (4500, 40)])
+def test_one_crowded_cell(n_src, n_tgt):
+    """All points but a rim in one near-field cell: edges of an item (8, 16, 32), of the strips, of a
+    sorted run (2048) and of the candidate lists; forward, gradients and Hessian."""
+    import paper_0807_2387_gb300 as fs
+    rng = np.random.default_rng(n_src + 7 * n_tgt)
+    rim = 0.24 * np.stack([np.cos(np.arange(5)), np.sin(np.arange(5))], 1)
+    src = np.concatenate([rng.uniform(0.002, 0.030, (n_src, 2)), rim])
+    tgt = np.concatenate([rng.uniform(0.002, 0.030, (n_tgt, 2)), -rim])
+    dev = torch.device("cuda", 0)
+    s, t = torch.tensor(src, device=dev), torch.tensor(tgt, device=dev)
+    q = torch.tensor(rng.standard_normal(len(src)), device=dev)
+    gp, gh = torch.tensor(rng.standard_normal(len(tgt)), device=dev), torch.tensor(rng.standard_normal((len(tgt), 2)), device=dev)
+    got = {}
+    for precision in (64, 32):
+        plan = fs.FastSum(s, t, 32, 2.0, 5, 4 / 32, precision=precision)
+        plan.set_charges(q)
+        phi, H = plan.field(dtype=torch.float64)
+        got[precision] = (phi, H, *plan.adjoint(gp, gh, True, True, True, dtype=torch.float64))
+        plan.sync()
+    for name, a, b in zip(("phi", "H", "dq", "dsrc", "dtgt"), got[32], got[64]):
+        assert rel(a, b) <= 2e-5, (name, rel(a, b))
