@@ -320,6 +320,8 @@ template <typename real> fs_status batch_build(fs_batch *b, const fs_instance *i
         d.s = pl->s;
         d.shift = std::log(pl->s) / (2.0 * kPi);
         d.np = make_near<real>(pl);
+        if constexpr (sizeof(real) == 8)
+            d.np64 = near64_params(d.np);
     }
     FS_TRY(b->alloc((unsigned char **)&b->inst, sizeof(BatchInst<real>) * K));
     FS_CUDA(cudaMemcpy(b->inst, h.data(), sizeof(BatchInst<real>) * K, cudaMemcpyHostToDevice));
@@ -435,7 +437,8 @@ template <typename real> fs_status batch_enqueue(fs_batch *b, int q_f64, int out
         FS_CUDA(launch_batch_interp_out<real>(inst, b->io, tgt_map, b->tgt_blocks, R, b->m, w, p0->wpoly, out_f64, st));
     } else {
         FS_CUDA(launch_batch_interp<real>(inst, tgt_map, b->tgt_blocks, R, b->m, w, p0->wpoly, st));
-        FS_CUDA(launch_batch_near64((const BatchInst<double> *)b->inst, tgt_map, b->tgt_blocks, R, st));
+        FS_CUDA(launch_batch_near64((const BatchInst<double> *)b->inst, tgt_map, b->tgt_blocks, R, b->p,
+                                    b->plans[0]->near64_tables, st));
         FS_CUDA(launch_batch_unpermute<real>(inst, b->io, tgt_map, b->tgt_blocks, R, out_f64, st));
     }
     return FS_OK;

@@ -193,13 +193,10 @@ fs_status bin_points(fs_plan *pl, const double *xy, int64_t n, int **perm, int *
     FS_TRY(pl->alloc(base, n));
     FS_TRY(pl->alloc_bytes(frac, (size_t)std::max<int64_t>(n, 1) * 2 * sizeof(real)));
     FS_TRY(pl->alloc(pos, n));
-    if (pl->precision == 32) {
-        FS_TRY(pl->alloc(pos32, n));
+    FS_TRY(pl->alloc(pos32, n));   // FP64 plans: for the near field's test of reach
+    *lo32 = nullptr;
+    if (pl->precision == 32)
         FS_TRY(pl->alloc(lo32, n));
-    } else {
-        *pos32 = nullptr;
-        *lo32 = nullptr;
-    }
     FS_TRY(pl->alloc(start, (size_t)pl->n_keys + 1));
     int *key = nullptr, *count = nullptr, *fill = nullptr, *tmp = nullptr;
     FS_TRY(pl->alloc(&key, n));
@@ -551,6 +548,18 @@ fs_status plan_init(fs_plan *pl, const double *src, int64_t M, const double *tgt
                                     &pl->n_src_near_items));
     }
 
+    if (pl->precision == 64) {
+        std::vector<double> t(kNear64Table);
+        for (int i = 0; i < kLogTab; ++i) {
+            t[2 * i] = 1.0 / (1.0 + i / 128.0);
+            t[2 * i + 1] = -std::log(t[2 * i]);
+        }
+        for (int k = 0; k < kLogExp; ++k)
+            t[2 * kLogTab + k] = -(k * std::log(2.0));
+        FS_TRY(pl->alloc(&pl->near64_tables, t.size()));
+        FS_CUDA(cudaMemcpy(pl->near64_tables, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice));
+    }
+
     // coefficient table and FFT twiddles
     FS_TRY(coefficients<real>(pl));
     FS_TRY(twiddles<real>(pl, L, &pl->tw));
@@ -798,8 +807,7 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
                                       (float *)pl->phi_s, (float *)pl->grad_s, (float *)pl->coinc, false, st));
             }
         } else
-            FS_CUDA(launch_near64(pl->N, pl->tgt_base, pl->tgt_pos, pl->src_pos, pl->src_start, pl->cg,
-                                  (const double *)q, np, (double *)pl->phi_s, (double *)pl->grad_s,
+            FS_CUDA(launch_near64(pl->N, near64_sides(pl, true), pl->cg, (const double *)q, np, (double *)pl->phi_s, (double *)pl->grad_s,
                                   (double *)pl->coinc, st));
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[6], st));
@@ -936,7 +944,7 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
                                                pl->tgt_lo32, pl->src_pos32, pl->src_lo32, pl->src_start, pl->cg, q, np,
                                                (float *)pl->grad_s, (float *)pl->adj_hess, false, st));
             } else {
-                FS_CUDA(launch_near_hess64(N, pl->tgt_base, pl->tgt_pos, pl->src_pos, pl->src_start, pl->cg, q, np,
+                FS_CUDA(launch_near_hess64(N, near64_sides(pl, true), pl->cg, q, np,
                                            (double *)pl->grad_s, (double *)pl->adj_hess, st));
             }
         }
@@ -971,7 +979,7 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
                                               (const float *)pl->adj_c, pl->adj_dn, np, (float *)pl->adj_a,
                                               (float *)pl->adj_ga, (float *)pl->adj_cg, false, st));
             } else
-                FS_CUDA(launch_near_adj64(M, pl->src_base, pl->src_pos, pl->tgt_pos, pl->tgt_start, pl->cg,
+                FS_CUDA(launch_near_adj64(M, near64_sides(pl, false), pl->cg,
                                           (const double *)pl->adj_c, pl->adj_dn, np, (double *)pl->adj_a,
                                           (double *)pl->adj_ga, (double *)pl->adj_cg, st));
             void *o_dq = dq ? (unsigned char *)dq + (size_t)r * M * osz : nullptr;

@@ -87,6 +87,29 @@ template <typename real> struct NearParams {
     int p;
 };
 
+// FP64 near field (near64.cuh): its constants, the two point sets (cell-relative FP32 positions for
+// the test of reach), and its tables: kLogTab pairs (c_i, -log c_i) of the reciprocals c_i = 1 / (1 +
+// i / 128) of the mantissa, then kLogExp multiples -k ln 2.
+struct Near64Params {
+    double eps2, inv_eps2, beta0, hess0;
+    float h, reach2;               // cell width; squared reach of the FP32 test (torus units)
+    double f[kMaxP], c[kMaxP], cp[kMaxP];   // 4 pi Ptilde (p - 1 terms), 4 pi P' (p - 1), 4 pi P'' (p - 2)
+    int p;
+};
+
+struct Near64Sides {
+    const int *own_base;
+    const double2 *own_pos;
+    const float2 *own_hi;
+    const double2 *oth_pos;
+    const float2 *oth_hi;
+    const int *oth_start;
+    const double *tables;
+};
+
+constexpr int kLogTab = 129, kLogExp = 128, kNear64Table = 2 * kLogTab + kLogExp;
+Near64Params near64_params(const NearParams<double> &np);
+
 // ---- 3D kernel 1/(4 pi r) (kernels3d.cu; transform and coefficients in kernels_fft.cu)
 
 // Near-field cells of the 3D path: n_c^3 cubes of `cell` grid lines, cell key
@@ -210,6 +233,7 @@ template <typename real> struct BatchInst {
     int64_t grid_stride, spec_stride;
     double s, shift;
     NearParams<real> np;
+    Near64Params np64;                               // FP64 batches
 };
 
 // Caller buffers of one instance for one batched evaluation (device pointers).
@@ -262,7 +286,8 @@ cudaError_t launch_wait_selftest(int *counter, int *err, int spins, cudaStream_t
 // items: (first target, count, instance, lanes) per warp, count <= lanes (8, 16 or 32)
 cudaError_t launch_batch_near32(int64_t n_items, const int4 *items, const BatchInst<float> *inst, int p, int nrhs,
                                 bool assign, cudaStream_t st);
-cudaError_t launch_batch_near64(const BatchInst<double> *inst, BlockMap bm, int blocks, int nrhs, cudaStream_t st);
+cudaError_t launch_batch_near64(const BatchInst<double> *inst, BlockMap bm, int blocks, int nrhs, int p,
+                                const double *tables, cudaStream_t st);
 template <typename real>
 cudaError_t launch_batch_unpermute(const BatchInst<real> *inst, const BatchIO *io, BlockMap bm, int blocks, int nrhs,
                                    int out_is_f64, cudaStream_t st);
@@ -348,9 +373,8 @@ template <typename real>
 cudaError_t launch_build_mul(const double2 *bhat, int n, const double *c_tab, real *mul, cudaStream_t st);
 
 // ---- near field and output (kernels_near.cu)
-cudaError_t launch_near64(int64_t N, const int *tgt_base, const double2 *tgt_pos, const double2 *src_pos,
-                          const int *src_start, CellGrid cg, const double *q, NearParams<double> np, double *phi_s,
-                          double *grad_s, double *coinc, cudaStream_t st);
+cudaError_t launch_near64(int64_t N, const Near64Sides &sd, CellGrid cg, const double *q, const NearParams<double> &np,
+                          double *phi_s, double *grad_s, double *coinc, cudaStream_t st);
 // items: (first target, count <= lanes) per warp, never spanning two cells; lanes: 8, 16 or 32
 // (assign: store phi_s and grad_s instead of adding to them, for the near field that runs on a
 // second stream beside spreading and the transform)
@@ -379,13 +403,11 @@ cudaError_t launch_unpermute(int64_t N, const real *phi_s, const real *grad_s, c
 template <typename real>
 cudaError_t launch_gather_adj(int64_t N, const int *perm, const void *gphi, const void *gH, int in_f64, double s,
                               double n_os, real *c, void *dn, void *df, double *gsum, cudaStream_t st);
-// FP64: one thread per point over the 3 x 3 cells
-cudaError_t launch_near_adj64(int64_t M, const int *src_base, const double2 *src_pos, const double2 *tgt_pos,
-                              const int *tgt_start, CellGrid cg, const double *c, const void *dn,
-                              NearParams<double> np, double *a_s, double *ga_s, double *cg_s, cudaStream_t st);
-cudaError_t launch_near_hess64(int64_t N, const int *tgt_base, const double2 *tgt_pos, const double2 *src_pos,
-                               const int *src_start, CellGrid cg, const double *q, NearParams<double> np,
-                               double *grad_s, double *hess_s, cudaStream_t st);
+// FP64: one warp per point over the 3 x 3 cells
+cudaError_t launch_near_adj64(int64_t M, const Near64Sides &sd, CellGrid cg, const double *c, const void *dn,
+                              const NearParams<double> &np, double *a_s, double *ga_s, double *cg_s, cudaStream_t st);
+cudaError_t launch_near_hess64(int64_t N, const Near64Sides &sd, CellGrid cg, const double *q,
+                               const NearParams<double> &np, double *grad_s, double *hess_s, cudaStream_t st);
 // FP32: warp items over the sources (adjoint potential) or the targets (Hessian)
 cudaError_t launch_near_adj32(int64_t n_items, const int2 *items, int lanes, const int *src_base, const float2 *src_hi,
                               const float2 *src_lo, const float2 *tgt_hi, const float2 *tgt_lo, const int *tgt_start,

@@ -24,32 +24,13 @@
 #include <cmath>
 
 #include "internal.h"
-#include "near_warp.cuh"
+#include "near64.cuh"
 
 namespace fs {
 
 namespace {
 
 template <typename real> using real2_t = typename Cplx<real>::type;
-
-// f = G - T_I, c(w) = (G' - T_I')(r) / r and c'(w) = dc/dw at w = r^2 / eps_I^2 (FP64 sum forms).
-__device__ __forceinline__ void near_fcd64(const NearParams<double> &np, double r2, double &f, double &c, double &cp)
-{
-    const double w = r2 * np.inv_eps2;
-    const int p = np.p;
-    double t = np.beta[p - 1];
-    for (int i = p - 2; i >= 0; --i)
-        t = t * w + np.beta[i];
-    f = -1.0 / (4.0 * kPi) * log(r2) - t;
-    double tp = 0.0, tpp = 0.0;
-    for (int k = p - 1; k >= 1; --k)
-        tp = tp * w + (double)(2 * k) * np.beta[k];
-    for (int k = p - 1; k >= 2; --k)
-        tpp = tpp * w + (double)(2 * k * (k - 1)) * np.beta[k];
-    const double inv2pi = 1.0 / (2.0 * kPi);
-    c = (-inv2pi / w - tp) * np.inv_eps2;
-    cp = (inv2pi / (w * w) - tpp) * np.inv_eps2;
-}
 
 // Hess T_I(0) = hess0 I.
 template <typename real> __host__ __device__ __forceinline__ real self_hessian(const NearParams<real> &np)
@@ -100,121 +81,91 @@ __global__ void k_gather_adj(int64_t N, const int *__restrict__ perm, const void
 }
 
 // Near part of the adjoint potential at the sources (sorted source order): value, gradient
-// with respect to the source position, and the coincident gphi.  FP64.
-__global__ void __launch_bounds__(256) k_near_adj64(int64_t M, const int *__restrict__ src_base,
-                                                    const double2 *__restrict__ src_pos,
-                                                    const double2 *__restrict__ tgt_pos,
-                                                    const int *__restrict__ tgt_start, CellGrid cg,
-                                                    const double *__restrict__ c, const double2 *__restrict__ dn,
-                                                    NearParams<double> np, double *__restrict__ a_s,
-                                                    double *__restrict__ ga_s, double *__restrict__ cg_s)
-{
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (j >= M)
-        return;
-    const double2 Y = src_pos[j];
-    const int packed = src_base[j];
-    const int c1 = base1(packed) / cg.cell, c2 = base2(packed) / cg.cell;
-    const double two_over_eps2 = 2.0 * np.inv_eps2;
-    const double hess0 = self_hessian(np);
-    double A = 0, gx = 0, gy = 0, gco = 0;
-    for (int d1 = -1; d1 <= 1; ++d1) {
-        const int e1 = c1 + d1;
-        if (e1 < 0 || e1 >= cg.n_c)
-            continue;
-        for (int d2 = -1; d2 <= 1; ++d2) {
-            const int e2 = c2 + d2;
-            if (e2 < 0 || e2 >= cg.n_c)
-                continue;
-            const int key = cg.key(e1, e2);
-            const int end = tgt_start[(key + 1) * kSub];
-            for (int i = tgt_start[key * kSub]; i < end; ++i) {
-                const double2 X = tgt_pos[i];
-                const double Dx = X.x - Y.x, Dy = X.y - Y.y;
-                const double rr2 = Dx * Dx + Dy * Dy;
-                if (!(rr2 < np.eps2))
-                    continue;
-                const double gp = c[i];
-                const double2 dd = dn[i];
-                if (rr2 == 0.0) {
-                    A -= gp * np.beta[0];
-                    gco += gp;
-                    gx += hess0 * dd.x;
-                    gy += hess0 * dd.y;
-                    continue;
-                }
-                double f, cc, cp;
-                near_fcd64(np, rr2, f, cc, cp);
-                const double dD = dd.x * Dx + dd.y * Dy;
-                A += gp * f + dD * cc;
-                const double k2 = two_over_eps2 * cp * dD;
-                gx -= gp * cc * Dx + cc * dd.x + k2 * Dx;
-                gy -= gp * cc * Dy + cc * dd.y + k2 * Dy;
-            }
-        }
+// with respect to the source position, and the coincident gphi.  FP64; own = source, other =
+// target, d = y - x = -D: A += gphi f - (dn . d) c, grad_y A += c (gphi d - dn) - (2 c' / eps_I^2)
+// (dn . d) d.
+template <int P> struct Near64Adj {
+    static constexpr int kV = 4;
+    const double *__restrict__ c_w;
+    const double2 *__restrict__ dn;
+    double *__restrict__ a_s;
+    double *__restrict__ ga_s;
+    double *__restrict__ cg_s;
+    double v[4];
+
+    __device__ __forceinline__ void init() { v[0] = v[1] = v[2] = v[3] = 0.0; }
+    __device__ __forceinline__ void coincident(const Near64Params &np, int i)
+    {
+        const double gp = c_w[i];
+        const double2 dd = dn[i];
+        v[0] -= gp * np.beta0;
+        v[3] += gp;
+        v[1] += np.hess0 * dd.x;
+        v[2] += np.hess0 * dd.y;
     }
-    a_s[j] += A;
-    ga_s[2 * j] += gx;
-    ga_s[2 * j + 1] += gy;
-    cg_s[j] = gco;
-}
+    __device__ __forceinline__ void pair(const Near64Params &np, const Near64Tables &tab, int i, bool in, double w, double dx,
+                                         double dy)
+    {
+        const double gp = in ? c_w[i] : 0.0;
+        double2 dd = dn[i];
+        dd.x = in ? dd.x : 0.0;
+        dd.y = in ? dd.y : 0.0;
+        const double y = near64_rcp(w), ce = np.inv_eps2 / (2.0 * kPi);
+        const double f = near64_f<P>(np, tab, w, 1.0 - w) * (1.0 / (4.0 * kPi));
+        const double c = -ce * near64_c<P>(np, w, y), cp = ce * near64_cp<P>(np, w, y);
+        const double nd = fma(dd.x, dx, dd.y * dy);
+        v[0] = fma(gp, f, fma(-nd, c, v[0]));
+        const double k = 2.0 * np.inv_eps2 * cp * nd;
+        v[1] += c * fma(gp, dx, -dd.x) - k * dx;
+        v[2] += c * fma(gp, dy, -dd.y) - k * dy;
+    }
+    __device__ __forceinline__ void store(const Near64Params &np, int64_t j, int i, double r) const
+    {
+        if (i == 0)
+            a_s[j] += r;
+        else if (i == 3)
+            cg_s[j] = r;
+        else
+            ga_s[2 * j + i - 1] += r;
+    }
+};
 
 // Near part of grad phi and Hess phi at the targets (sorted target order), torus units.  FP64.
-__global__ void __launch_bounds__(256) k_near_hess64(int64_t N, const int *__restrict__ tgt_base,
-                                                     const double2 *__restrict__ tgt_pos,
-                                                     const double2 *__restrict__ src_pos,
-                                                     const int *__restrict__ src_start, CellGrid cg,
-                                                     const double *__restrict__ q, NearParams<double> np,
-                                                     double *__restrict__ grad_s, double *__restrict__ hess_s)
-{
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= N)
-        return;
-    const double2 X = tgt_pos[k];
-    const int packed = tgt_base[k];
-    const int c1 = base1(packed) / cg.cell, c2 = base2(packed) / cg.cell;
-    const double two_over_eps2 = 2.0 * np.inv_eps2;
-    const double hess0 = self_hessian(np);
-    double gx = 0, gy = 0, hxx = 0, hxy = 0, hyy = 0;
-    for (int d1 = -1; d1 <= 1; ++d1) {
-        const int e1 = c1 + d1;
-        if (e1 < 0 || e1 >= cg.n_c)
-            continue;
-        for (int d2 = -1; d2 <= 1; ++d2) {
-            const int e2 = c2 + d2;
-            if (e2 < 0 || e2 >= cg.n_c)
-                continue;
-            const int key = cg.key(e1, e2);
-            const int end = src_start[(key + 1) * kSub];
-            for (int j = src_start[key * kSub]; j < end; ++j) {
-                const double2 Y = src_pos[j];
-                const double Dx = X.x - Y.x, Dy = X.y - Y.y;
-                const double rr2 = Dx * Dx + Dy * Dy;
-                if (!(rr2 < np.eps2))
-                    continue;
-                const double qj = q[j];
-                if (rr2 == 0.0) {
-                    hxx -= qj * hess0;
-                    hyy -= qj * hess0;
-                    continue;
-                }
-                double f, cc, cp;
-                near_fcd64(np, rr2, f, cc, cp);
-                gx += qj * cc * Dx;
-                gy += qj * cc * Dy;
-                const double k2 = qj * two_over_eps2 * cp;
-                hxx += qj * cc + k2 * Dx * Dx;
-                hxy += k2 * Dx * Dy;
-                hyy += qj * cc + k2 * Dy * Dy;
-            }
-        }
+template <int P> struct Near64Hess {
+    static constexpr int kV = 5;
+    const double *__restrict__ q;
+    double *__restrict__ grad_s;
+    double *__restrict__ hess_s;
+    double v[5];
+
+    __device__ __forceinline__ void init() { v[0] = v[1] = v[2] = v[3] = v[4] = 0.0; }
+    __device__ __forceinline__ void coincident(const Near64Params &np, int j)
+    {
+        const double h = q[j] * np.hess0;
+        v[2] -= h;
+        v[4] -= h;
     }
-    grad_s[2 * k] += gx;
-    grad_s[2 * k + 1] += gy;
-    hess_s[3 * k] += hxx;
-    hess_s[3 * k + 1] += hxy;
-    hess_s[3 * k + 2] += hyy;
-}
+    __device__ __forceinline__ void pair(const Near64Params &np, const Near64Tables &tab, int j, bool in, double w, double dx,
+                                         double dy)
+    {
+        const double y = near64_rcp(w), ce = np.inv_eps2 / (2.0 * kPi);
+        const double t = in ? q[j] * ce : 0.0;
+        const double qc = -t * near64_c<P>(np, w, y), k = 2.0 * np.inv_eps2 * t * near64_cp<P>(np, w, y);
+        v[0] = fma(qc, dx, v[0]);
+        v[1] = fma(qc, dy, v[1]);
+        const double kx = k * dx, ky = k * dy;
+        v[2] += fma(kx, dx, qc);
+        v[3] = fma(kx, dy, v[3]);
+        v[4] += fma(ky, dy, qc);
+    }
+    __device__ __forceinline__ void store(const Near64Params &np, int64_t k, int i, double r) const
+    {
+        if (i < 2)
+            grad_s[2 * k + i] += r;
+        else
+            hess_s[3 * k + i - 2] += r;
+    }
+};
 
 // Hessian at the targets (FP32 warp items, own = targets, other = sources, d = x - y):
 // grad += q c d, Hess += q (c I + (2 c' / eps_I^2) d d^T), with c = rc c^ and c' = rc c'^;
@@ -450,26 +401,30 @@ cudaError_t launch_gather_adj(int64_t N, const int *perm, const void *gphi, cons
     return cudaGetLastError();
 }
 
-cudaError_t launch_near_adj64(int64_t M, const int *src_base, const double2 *src_pos, const double2 *tgt_pos,
-                              const int *tgt_start, CellGrid cg, const double *c, const void *dn,
-                              NearParams<double> np, double *a_s, double *ga_s, double *cg_s, cudaStream_t st)
+cudaError_t launch_near_adj64(int64_t M, const Near64Sides &sd, CellGrid cg, const double *c, const void *dn,
+                              const NearParams<double> &np, double *a_s, double *ga_s, double *cg_s, cudaStream_t st)
 {
-    if (M <= 0)
-        return cudaSuccess;
-    k_near_adj64<<<nblocks(M, 256), 256, 0, st>>>(M, src_base, src_pos, tgt_pos, tgt_start, cg, c,
-                                                  (const double2 *)dn, np, a_s, ga_s, cg_s);
-    return cudaGetLastError();
+    return with_degree(np.p, [&](auto pc) {
+        Near64Adj<decltype(pc)::value> op{};
+        op.c_w = c;
+        op.dn = (const double2 *)dn;
+        op.a_s = a_s;
+        op.ga_s = ga_s;
+        op.cg_s = cg_s;
+        return launch_near64_points(M, sd, cg, near64_params(np), op, st);
+    });
 }
 
-cudaError_t launch_near_hess64(int64_t N, const int *tgt_base, const double2 *tgt_pos, const double2 *src_pos,
-                               const int *src_start, CellGrid cg, const double *q, NearParams<double> np,
-                               double *grad_s, double *hess_s, cudaStream_t st)
+cudaError_t launch_near_hess64(int64_t N, const Near64Sides &sd, CellGrid cg, const double *q,
+                               const NearParams<double> &np, double *grad_s, double *hess_s, cudaStream_t st)
 {
-    if (N <= 0)
-        return cudaSuccess;
-    k_near_hess64<<<nblocks(N, 256), 256, 0, st>>>(N, tgt_base, tgt_pos, src_pos, src_start, cg, q, np, grad_s,
-                                                   hess_s);
-    return cudaGetLastError();
+    return with_degree(np.p, [&](auto pc) {
+        Near64Hess<decltype(pc)::value> op{};
+        op.q = q;
+        op.grad_s = grad_s;
+        op.hess_s = hess_s;
+        return launch_near64_points(N, sd, cg, near64_params(np), op, st);
+    });
 }
 
 cudaError_t launch_near_adj32(int64_t n_items, const int2 *items, int lanes, const int *src_base, const float2 *src_hi,

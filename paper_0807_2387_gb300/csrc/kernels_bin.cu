@@ -251,7 +251,8 @@ __global__ void k_gather_points(const double *__restrict__ xy, const int *__rest
         const double o1 = xt - c1, o2 = yt - c2;
         const float h1 = (float)o1, h2 = (float)o2;
         pos32[k] = make_float2(h1, h2);
-        pos32_lo[k] = make_float2((float)(o1 - (double)h1), (float)(o2 - (double)h2));
+        if (pos32_lo)
+            pos32_lo[k] = make_float2((float)(o1 - (double)h1), (float)(o2 - (double)h2));
     }
 }
 

@@ -9,7 +9,7 @@
 // Cells are at least eps_I wide, so a target's partners lie in the 3 x 3 cells
 // around its own.
 //
-// FP64 path: one thread per target, direct FP64 formulas (the comparison path).
+// FP64 path: one warp per target (near64.cuh).
 //
 // FP32 path: one warp per work item, a compact piece of a cell of at most 32 targets (one per
 // lane), over the sources near the item's bounding box (near_warp.cuh).
@@ -23,95 +23,75 @@
 
 #include "internal.h"
 #include "output.cuh"
-#include "near_warp.cuh"
+#include "near64.cuh"
 
 namespace fs {
 
 namespace {
 
-__device__ __forceinline__ void near64_target(int64_t k, const int *__restrict__ tgt_base,
-                                              const double2 *__restrict__ tgt_pos, const double2 *__restrict__ src_pos,
-                                              const int *__restrict__ src_start, const CellGrid &cg,
-                                              const double *__restrict__ q, const NearParams<double> &np,
-                                              double *__restrict__ phi_s, double *__restrict__ grad_s,
-                                              double *__restrict__ coinc)
-{
-    const double2 X = tgt_pos[k];
-    const int packed = tgt_base[k];
-    const int c1 = base1(packed) / cg.cell, c2 = base2(packed) / cg.cell;
-    const double inv4pi = 1.0 / (4.0 * kPi);
-    const double inv2pi = 1.0 / (2.0 * kPi);
-    double phi = 0, gx = 0, gy = 0, qc = 0;
-    for (int d1 = -1; d1 <= 1; ++d1) {
-        const int e1 = c1 + d1;
-        if (e1 < 0 || e1 >= cg.n_c)
-            continue;
-        for (int d2 = -1; d2 <= 1; ++d2) {
-            const int e2 = c2 + d2;
-            if (e2 < 0 || e2 >= cg.n_c)
-                continue;
-            const int key = cg.key(e1, e2);
-            const int end = src_start[(key + 1) * kSub];
-            for (int j = src_start[key * kSub]; j < end; ++j) {
-                const double2 Y = src_pos[j];
-                const double dx = X.x - Y.x, dy = X.y - Y.y;
-                const double r2 = dx * dx + dy * dy;
-                if (!(r2 < np.eps2))
-                    continue;
-                const double qj = q[j];
-                if (r2 == 0.0) {
-                    phi -= qj * np.beta[0];
-                    qc += qj;
-                    continue;
-                }
-                const double u2 = r2 * np.inv_eps2;
-                double t = np.beta[np.p - 1];
-                for (int i = np.p - 2; i >= 0; --i)
-                    t = t * u2 + np.beta[i];
-                double tp = 0.0;
-                if (np.p > 1) {
-                    tp = np.dbeta[np.p - 2];
-                    for (int i = np.p - 3; i >= 0; --i)
-                        tp = tp * u2 + np.dbeta[i];
-                }
-                const double val = -inv4pi * log(r2) - t;
-                const double coef = -inv2pi / r2 - tp;
-                phi += qj * val;
-                gx += qj * coef * dx;
-                gy += qj * coef * dy;
-            }
-        }
+// phi += q f, grad += q c d, and the coincident charge (4 pi f and -2 pi eps_I^2 c are summed).
+template <int P> struct Near64Fwd {
+    static constexpr int kV = 4;
+    const double *__restrict__ q;
+    double *__restrict__ phi_s;
+    double *__restrict__ grad_s;
+    double *__restrict__ coinc;
+    double v[4];
+
+    __device__ __forceinline__ void init() { v[0] = v[1] = v[2] = v[3] = 0.0; }
+    __device__ __forceinline__ void coincident(const Near64Params &np, int j)
+    {
+        const double qj = q[j];
+        v[0] -= qj * (4.0 * kPi * np.beta0);
+        v[3] += qj;
     }
-    phi_s[k] += phi;
-    grad_s[2 * k] += gx;
-    grad_s[2 * k + 1] += gy;
-    coinc[k] = qc;
-}
+    __device__ __forceinline__ void pair(const Near64Params &np, const Near64Tables &tab, int j, bool in, double w, double dx,
+                                         double dy)
+    {
+        const double qj = in ? q[j] : 0.0;
+        v[0] = fma(qj, near64_f<P>(np, tab, w, 1.0 - w), v[0]);
+        const double t = qj * near64_c<P>(np, w, near64_rcp(w));
+        v[1] = fma(t, dx, v[1]);
+        v[2] = fma(t, dy, v[2]);
+    }
+    __device__ __forceinline__ void store(const Near64Params &np, int64_t k, int i, double r) const
+    {
+        if (i == 0)
+            phi_s[k] += r * (1.0 / (4.0 * kPi));
+        else if (i == 3)
+            coinc[k] = r;
+        else
+            grad_s[2 * k + i - 1] -= r * (np.inv_eps2 / (2.0 * kPi));
+    }
+};
 
-__global__ void __launch_bounds__(256) k_near64(int64_t N, const int *__restrict__ tgt_base,
-                                                const double2 *__restrict__ tgt_pos,
-                                                const double2 *__restrict__ src_pos, const int *__restrict__ src_start,
-                                                CellGrid cg, const double *__restrict__ q, NearParams<double> np,
-                                                double *__restrict__ phi_s, double *__restrict__ grad_s,
-                                                double *__restrict__ coinc)
+// Batched FP64 near field: block -> (instance, block of its targets), blockIdx.y = right-hand side;
+// the block's warps take its targets in turn.
+template <int P>
+__global__ void __launch_bounds__(32 * kNear64Warps) k_batch_near64(const BatchInst<double> *__restrict__ inst,
+                                                                    BlockMap bm, const double *__restrict__ tables,
+                                                                    int per_block)
 {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k < N)
-        near64_target(k, tgt_base, tgt_pos, src_pos, src_start, cg, q, np, phi_s, grad_s, coinc);
-}
-
-// Batched FP64 near field: block -> (instance, block of its targets), blockIdx.y = right-hand side.
-__global__ void __launch_bounds__(256) k_batch_near64(const BatchInst<double> *__restrict__ inst, BlockMap bm)
-{
-    const int i = bm.inst[blockIdx.x];
+    __shared__ Near64Tables tab;
+    __shared__ int queue[kNear64Warps][64];
+    __shared__ Near64Params np;
+    tab.load(tables);
+    const int i = bm.inst[blockIdx.x], r = blockIdx.y;
     const BatchInst<double> &b = inst[i];
-    const int64_t k = (int64_t)(blockIdx.x - bm.first[i]) * blockDim.x + threadIdx.x;
-    const int64_t N = b.N;
-    if (k >= N)
-        return;
-    const int r = blockIdx.y;
-    near64_target(k, b.tgt_base, b.tgt_pos, b.src_pos, b.src_start, b.cg, b.q + (int64_t)r * b.M, b.np,
-                  b.phi_s + (int64_t)r * N, b.grad_s + 2 * (int64_t)r * N, b.coinc + (int64_t)r * N);
+    for (int t = threadIdx.x; t < (int)(sizeof(np) / sizeof(int)); t += blockDim.x)
+        reinterpret_cast<int *>(&np)[t] = reinterpret_cast<const int *>(&b.np64)[t];
+    __syncthreads();
+    const Near64Sides sd{b.tgt_base, b.tgt_pos, b.tgt_hi, b.src_pos, b.src_hi, b.src_start, tables};
+    const CellGrid cg = b.cg;
+    const int64_t N = b.N, first = (int64_t)(blockIdx.x - bm.first[i]) * per_block;
+    Near64Fwd<P> op{};
+    op.q = b.q + (int64_t)r * b.M;
+    op.phi_s = b.phi_s + (int64_t)r * N;
+    op.grad_s = b.grad_s + 2 * (int64_t)r * N;
+    op.coinc = b.coinc + (int64_t)r * N;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int64_t k = first + w; k < first + per_block && k < N; k += kNear64Warps)
+        near64_point(k, lane, sd, cg, np, tab, op, queue[w]);
 }
 
 // Forward correction at the targets for R right-hand sides at once (the pair geometry, the
@@ -378,15 +358,40 @@ __global__ void k_batch_unpermute(const BatchInst<real> *__restrict__ inst, cons
 
 }  // namespace
 
-cudaError_t launch_near64(int64_t N, const int *tgt_base, const double2 *tgt_pos, const double2 *src_pos,
-                          const int *src_start, CellGrid cg, const double *q, NearParams<double> np, double *phi_s,
-                          double *grad_s, double *coinc, cudaStream_t st)
+Near64Params near64_params(const NearParams<double> &np)
 {
-    if (N <= 0)
-        return cudaSuccess;
-    k_near64<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(N, tgt_base, tgt_pos, src_pos, src_start, cg, q, np, phi_s,
-                                                           grad_s, coinc);
-    return cudaGetLastError();
+    Near64Params o{};
+    o.eps2 = np.eps2;
+    o.inv_eps2 = np.inv_eps2;
+    o.beta0 = np.beta[0];
+    o.hess0 = np.p > 1 ? 2.0 * np.beta[1] * np.inv_eps2 : 0.0;
+    o.h = (float)np.hcell;
+    const float reach = sqrtf((float)np.eps2) * (1.f + 1e-4f) + 1e-5f;
+    o.reach2 = reach * reach;
+    o.p = np.p;
+    const double four_pi = 4.0 * kPi;
+    for (int k = 0; k + 1 < np.p; ++k)
+        o.f[k] = -four_pi * np.nptilde[k];
+    if (np.p == 1)
+        o.f[0] = -four_pi * np.pbeta[0];      // p = 1: P is a constant
+    for (int k = 1; k < np.p; ++k)
+        o.c[k - 1] = four_pi * k * np.beta[k];
+    for (int k = 2; k < np.p; ++k)
+        o.cp[k - 2] = four_pi * k * (k - 1) * np.beta[k];
+    return o;
+}
+
+cudaError_t launch_near64(int64_t N, const Near64Sides &sd, CellGrid cg, const double *q, const NearParams<double> &np,
+                          double *phi_s, double *grad_s, double *coinc, cudaStream_t st)
+{
+    return with_degree(np.p, [&](auto pc) {
+        Near64Fwd<decltype(pc)::value> op{};
+        op.q = q;
+        op.phi_s = phi_s;
+        op.grad_s = grad_s;
+        op.coinc = coinc;
+        return launch_near64_points(N, sd, cg, near64_params(np), op, st);
+    });
 }
 
 cudaError_t launch_near32(int64_t n_items, const int2 *items, int lanes, const int *tgt_base, const float2 *tgt_hi,
@@ -472,12 +477,16 @@ cudaError_t launch_batch_near32(int64_t n_items, const int4 *items, const BatchI
     });
 }
 
-cudaError_t launch_batch_near64(const BatchInst<double> *inst, BlockMap bm, int blocks, int nrhs, cudaStream_t st)
+cudaError_t launch_batch_near64(const BatchInst<double> *inst, BlockMap bm, int blocks, int nrhs, int p,
+                                const double *tables, cudaStream_t st)
 {
     if (blocks <= 0 || nrhs <= 0)
         return cudaSuccess;
-    k_batch_near64<<<dim3((unsigned)blocks, (unsigned)nrhs), 256, 0, st>>>(inst, bm);
-    return cudaGetLastError();
+    return with_degree(p, [&](auto pc) {
+        k_batch_near64<decltype(pc)::value><<<dim3((unsigned)blocks, (unsigned)nrhs), 32 * kNear64Warps, 0, st>>>(
+            inst, bm, tables, 256);
+        return cudaGetLastError();
+    });
 }
 
 template <typename real>

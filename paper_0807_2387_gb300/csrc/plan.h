@@ -75,6 +75,7 @@ struct fs_plan {
     void *src_frac = nullptr, *tgt_frac = nullptr;
     double2 *src_pos = nullptr, *tgt_pos = nullptr;
     float2 *src_pos32 = nullptr, *tgt_pos32 = nullptr;
+    double *near64_tables = nullptr;      // FP64 plans (Near64Sides)
     float2 *src_lo32 = nullptr, *tgt_lo32 = nullptr;
     int *src_start = nullptr, *tgt_start = nullptr;
     std::vector<int> src_cells, tgt_cells;   // the cells' first points (host)
@@ -235,6 +236,13 @@ template <typename real> inline NearParams<real> make_near(const fs_plan *pl)
     // R(w) = c (w-1)^(p-1) with R(0) = -(1/2pi) gives c = (-1)^p / (2pi), independent of beta
     np.rcoef = (real)(((pl->p % 2 == 0) ? 1.0 : -1.0) / (2.0 * kPi * pl->eps_I * pl->eps_I));
     return np;
+}
+
+inline Near64Sides near64_sides(const fs_plan *pl, bool own_targets)
+{
+    if (own_targets)
+        return {pl->tgt_base, pl->tgt_pos, pl->tgt_pos32, pl->src_pos, pl->src_pos32, pl->src_start, pl->near64_tables};
+    return {pl->src_base, pl->src_pos, pl->src_pos32, pl->tgt_pos, pl->tgt_pos32, pl->tgt_start, pl->near64_tables};
 }
 
 }  // namespace fs

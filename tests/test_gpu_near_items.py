@@ -40,3 +40,23 @@ def test_one_crowded_cell(n_src, n_tgt):
         plan.sync()
     for name, a, b in zip(("phi", "H", "dq", "dsrc", "dtgt"), got[32], got[64]):
         assert rel(a, b) <= 2e-5, (name, rel(a, b))
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 7, 8])
+def test_fp64_pair_functions_by_degree(p):
+    """The FP64 near field's log, reciprocal and polynomials at every form of the degree, over pairs from
+    coincident to eps_I apart: 1e-12 of the oracle, the bar of the FP64 gates."""
+    import paper_0807_2387_gb300 as fs
+    from oracle import fastsum as F
+    from oracle import kernel as K
+    rng = np.random.default_rng(90 + p)
+    src = rng.uniform(-0.17, 0.17, (333, 2))
+    near = src[:200] + 10.0 ** rng.uniform(-9, -1.2, (200, 1)) * rng.standard_normal((200, 2))
+    tgt = np.clip(np.concatenate([near, src[200:260], rng.uniform(-0.17, 0.17, (41, 2))]), -0.17, 0.17)
+    q = rng.standard_normal(len(src))
+    dev = torch.device("cuda", 0)
+    plan = fs.FastSum(torch.tensor(src, device=dev), torch.tensor(tgt, device=dev), 64, 2.0, 5, 5 / 64, precision=64, p=p)
+    phi, H = plan.set_charges(torch.tensor(q, device=dev)).field()
+    phi_o, H_o = F.fast_sum(src, tgt, q, K.make_params(64, 2.0, 5, 5 / 64, p), "nfft")
+    for name, a, b in (("phi", phi, phi_o), ("H", H, H_o)):
+        assert rel(a, torch.tensor(b)) <= 1e-12, (name, rel(a, torch.tensor(b)))
