@@ -417,7 +417,6 @@ template <typename real> fs_status batch_enqueue(fs_batch *b, int q_f64, int out
     const int K = b->count, R = b->nrhs;
     const auto *inst = (const BatchInst<real> *)b->inst;
     const fs_plan *p0 = b->plans[0];
-    const Window<real> w = make_window<real>(p0);
     const BlockMap src_map{b->src_inst, b->src_first}, tgt_map{b->tgt_inst, b->tgt_first};
     FS_CUDA(cudaMemsetAsync(b->q_sum, 0, sizeof(double) * K * R, st));
     FS_CUDA(cudaMemsetAsync(b->grids, 0, b->grid_bytes, st));
@@ -429,14 +428,14 @@ template <typename real> fs_status batch_enqueue(fs_batch *b, int q_f64, int out
         FS_CUDA(launch_batch_near32(b->n_near_items, b->near_items, (const BatchInst<float> *)b->inst, b->p, R, true,
                                     st));
     }
-    FS_CUDA(launch_batch_spread<real>(b->spread_items, b->n_spread_items, R, inst, b->m, b->max_tile, w, p0->wpoly,
+    FS_CUDA(launch_batch_spread<real>(b->spread_items, b->n_spread_items, R, inst, b->m, b->max_tile, win_poly<real>(p0),
                                       b->kahan, st));
     FS_CUDA(launch_batch_fft<real>(inst, b->fft_units, b->n_fft_units, K, R, b->L_max, b->fft_blocks, b->counters,
                                    b->err, kWaitSpins, st));
     if constexpr (sizeof(real) == 4) {
-        FS_CUDA(launch_batch_interp_out<real>(inst, b->io, tgt_map, b->tgt_blocks, R, b->m, w, p0->wpoly, out_f64, st));
+        FS_CUDA(launch_batch_interp_out<real>(inst, b->io, tgt_map, b->tgt_blocks, R, b->m, win_poly<real>(p0), out_f64, st));
     } else {
-        FS_CUDA(launch_batch_interp<real>(inst, tgt_map, b->tgt_blocks, R, b->m, w, p0->wpoly, st));
+        FS_CUDA(launch_batch_interp<real>(inst, tgt_map, b->tgt_blocks, R, b->m, win_poly<real>(p0), st));
         FS_CUDA(launch_batch_near64((const BatchInst<double> *)b->inst, tgt_map, b->tgt_blocks, R, b->p,
                                     b->plans[0]->near64_tables, st));
         FS_CUDA(launch_batch_unpermute<real>(inst, b->io, tgt_map, b->tgt_blocks, R, out_f64, st));

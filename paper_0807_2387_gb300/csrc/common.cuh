@@ -169,28 +169,43 @@ __device__ __forceinline__ void kb_value_slope_curv(const Window<real> &w, real 
     dd = -w.b * w.b * e * (F - w.b * w.b * x * x * kb_curv_factor<real>(z));
 }
 
-template <int DEG> __device__ __forceinline__ float poly_eval(const float *c, float t)
+// FP64 window: the same polynomials of degree kPolyD64 for the taps a < m (the window is even, so tap
+// 2m-1-a at t is tap a at -t).  The tail of the Chebyshev series is below 1e-17 of a tap's largest
+// value for m <= 8 (degree 17 to 21 by m and oversampling), so they are as exact as the closed
+// form, whose exp, expm1 and square root cost over 100 FP64 instructions a tap against 21.  The
+// closed support edge (frac = 0, the last tap) is 0, as in the closed form.
+constexpr int kPolyD64 = 21;
+struct WindowPoly64 {
+    double c[kMaxM][kPolyD64 + 1];
+    double d[kMaxM][kPolyD64];
+    double e[kMaxM][kPolyD64 - 1];
+};
+template <typename real> struct WinPolyOf { using type = WindowPoly; static constexpr int D = kPolyD; };
+template <> struct WinPolyOf<double> { using type = WindowPoly64; static constexpr int D = kPolyD64; };
+template <typename real> using WinPoly = typename WinPolyOf<real>::type;
+
+template <int DEG, typename real> __device__ __forceinline__ real poly_eval(const real *c, real t)
 {
-    float acc = c[DEG];
+    real acc = c[DEG];
 #pragma unroll
     for (int i = DEG - 1; i >= 0; --i)
-        acc = fmaf(acc, t, c[i]);
+        acc = fma(acc, t, c[i]);
     return acc;
 }
 
 // Even and odd parts of sum_i c[i] t^i as polynomials in s = t^2: e = sum_j c[2j] s^j,
 // o = sum_j c[2j+1] s^j, so that the polynomial at +-t is e +- t o.
-template <int DEG> __device__ __forceinline__ void poly_even_odd(const float *c, float s, float &e, float &o)
+template <int DEG, typename real> __device__ __forceinline__ void poly_even_odd(const real *c, real s, real &e, real &o)
 {
     constexpr int NE = DEG / 2, NO = (DEG - 1) / 2;   // highest even / odd half-index
     e = c[2 * NE];
 #pragma unroll
     for (int j = NE - 1; j >= 0; --j)
-        e = fmaf(e, s, c[2 * j]);
+        e = fma(e, s, c[2 * j]);
     o = c[2 * NO + 1];
 #pragma unroll
     for (int j = NO - 1; j >= 0; --j)
-        o = fmaf(o, s, c[2 * j + 1]);
+        o = fma(o, s, c[2 * j + 1]);
 }
 
 // Spreading tiles in shared memory: a warp's tile holds `rows` x `rows` grid lines at a row

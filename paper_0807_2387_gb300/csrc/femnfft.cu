@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -118,11 +119,68 @@ bool near_coefficients(double eps, int p, double *beta)
 
 namespace {
 
+// psi(x) in extended precision, without cancellation in the exponent (kb_value).
+long double window_value(long double b, int m, long double x)
+{
+    const long double t = ((long double)m - x) * ((long double)m + x);
+    if (t <= 0)
+        return 0;
+    const long double tau = sqrtl(t), z = b * tau;
+    return (long double)m * b * expl(-b * x * x / (tau + m)) * -expm1l(-2 * z) / (z * -expm1l(-2 * b * m));
+}
+
 // Per-tap polynomial form of the normalised window for the FP32 kernels: for tap a the
 // function frac -> psi(frac + m - 1 - a) on [0, 1) is interpolated at kPolyD + 1 Chebyshev
 // points in FP64 and rewritten in monomials of t = frac - 1/2; the slope polynomial is its
 // exact derivative.
 }  // namespace
+
+// As build_window_poly, of degree kPolyD64 for the taps a < m, in extended precision throughout.
+void fs::build_window_poly64(double sigma, int m, WindowPoly64 *wp)
+{
+    static std::mutex mu;
+    static std::map<std::pair<double, int>, WindowPoly64> known;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = known.find({sigma, m});
+    if (it != known.end()) {
+        *wp = it->second;
+        return;
+    }
+    constexpr int K = kPolyD64 + 1;
+    const long double pi = 3.14159265358979323846264338327950288L;
+    const double b = kPi * (2.0 - 1.0 / sigma);   // the deconvolution's b
+    long double cs[4 * K], T[K][K] = {};   // cos(pi j / (2 K)); monomial coefficients of T_n(u)
+    for (int j = 0; j < 4 * K; ++j)
+        cs[j] = cosl(pi * j / (2 * K));
+    T[0][0] = T[1][1] = 1;
+    for (int n = 2; n < K; ++n)
+        for (int i = 0; i < K; ++i)
+            T[n][i] = (i > 0 ? 2 * T[n - 1][i - 1] : 0) - T[n - 2][i];
+    std::memset(wp, 0, sizeof(*wp));
+    for (int a = 0; a < m; ++a) {
+        long double f[K], mono[K] = {};
+        for (int k = 0; k < K; ++k)
+            f[k] = window_value(b, m, 0.5L + 0.5L * cs[2 * k + 1] + (m - 1 - a));
+        for (int n = 0; n < K; ++n) {
+            long double acc = 0;
+            for (int k = 0; k < K; ++k)
+                acc += f[k] * cs[n * (2 * k + 1) % (4 * K)];
+            acc *= (n == 0 ? 1.0L : 2.0L) / K;
+            for (int i = 0; i <= n; ++i)
+                mono[i] += acc * T[n][i];
+        }
+        long double scale = 1;   // u = 2t: coefficient of t^i is 2^i times that of u^i
+        for (int i = 0; i < K; ++i, scale *= 2) {
+            wp->c[a][i] = (double)(mono[i] * scale);
+            if (i > 0)
+                wp->d[a][i - 1] = (double)(mono[i] * scale * i);
+            if (i > 1)
+                wp->e[a][i - 2] = (double)(mono[i] * scale * i * (i - 1));
+        }
+    }
+    if (known.size() < 64)
+        known[{sigma, m}] = *wp;
+}
 
 void fs::build_window_poly(double sigma, int m, WindowPoly *wp)
 {
@@ -483,7 +541,10 @@ fs_status plan_init(fs_plan *pl, const double *src, int64_t M, const double *tgt
         pl->kp.k_half = std::log(2.0) * inv2pi;
     }
 
-    build_window_poly(pl->sigma, pl->m, &pl->wpoly);
+    if (sizeof(real) == 8)
+        build_window_poly64(pl->sigma, pl->m, &pl->wpoly64);
+    else
+        build_window_poly(pl->sigma, pl->m, &pl->wpoly);
 
     // binning
     // FEM plans (several quadrature points around every node): a cell holds few targets, so a
@@ -701,18 +762,18 @@ template <typename real> fs_status set_charges_t(fs_plan *pl, const void *q, fs_
 
 // Step (c): the grid is zeroed and the charges spread into it, through shared-memory tiles or
 // (sparse plans, FS_FLAG_SPREAD_DIRECT) with global atomics and a compensation plane.
-template <typename real> fs_status spread_forward(fs_plan *pl, const real *q, const Window<real> &w, cudaStream_t st)
+template <typename real> fs_status spread_forward(fs_plan *pl, const real *q, cudaStream_t st)
 {
     const size_t grid_bytes = (size_t)pl->n_a * pl->pitch * sizeof(real);
     FS_CUDA(cudaMemsetAsync(pl->grid, 0, grid_bytes, st));
     if (!pl->spread_direct) {
-        FS_CUDA(launch_spread<real>(pl->items, pl->n_items, pl->cg, pl->m, pl->src_base, pl->src_frac, q, w, pl->wpoly,
+        FS_CUDA(launch_spread<real>(pl->items, pl->n_items, pl->cg, pl->m, pl->src_base, pl->src_frac, q, win_poly<real>(pl),
                                     (real *)pl->grid, pl->pitch, pl->n_a, pl->kahan, st));
         return FS_OK;
     }
     if (pl->grid_comp)
         FS_CUDA(cudaMemsetAsync(pl->grid_comp, 0, grid_bytes, st));
-    FS_CUDA(launch_spread_direct<real>(pl->M, pl->m, pl->src_base, pl->src_frac, q, w, pl->wpoly, (real *)pl->grid,
+    FS_CUDA(launch_spread_direct<real>(pl->M, pl->m, pl->src_base, pl->src_frac, q, make_window<real>(pl), win_poly<real>(pl), (real *)pl->grid,
                                        (real *)pl->grid_comp, pl->pitch, pl->n_a, pl->kahan, st));
     return FS_OK;
 }
@@ -720,7 +781,6 @@ template <typename real> fs_status spread_forward(fs_plan *pl, const real *q, co
 template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dtype dtype)
 {
     cudaStream_t st = pl->stream;
-    const Window<real> w = make_window<real>(pl);
     const NearParams<real> np = make_near<real>(pl);
     using C = typename Cplx<real>::type;
     const double shift = std::log(pl->s) / (2.0 * kPi);
@@ -732,7 +792,7 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
             FS_CUDA(cudaEventRecord(pl->ev[0], st));
         if (pl->overlap)
             FS_CUDA(cudaEventRecord(pl->ev_fork, st));   // the charges are in
-        FS_TRY(spread_forward<real>(pl, q, w, st));
+        FS_TRY(spread_forward<real>(pl, q, st));
         if (pl->overlap) {
             // the near field (stored, not added) on the second stream, submitted after the
             // spreading so that the spreading's blocks are scheduled first
@@ -778,7 +838,7 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
                 FS_CUDA(cudaEventRecord(pl->ev_j, st));
             // steps (f) and (h) in one pass: the far field added to the near field's sums and
             // written to the caller's buffers (the output stage's time is in the interpolation's)
-            FS_CUDA(launch_interp_out<real>(pl->N, pl->m, pl->tgt_base, pl->tgt_frac, w, pl->wpoly,
+            FS_CUDA(launch_interp_out<real>(pl->N, pl->m, pl->tgt_base, pl->tgt_frac, win_poly<real>(pl),
                                             (const real *)pl->grid, pl->pitch, (real)pl->n_os,
                                             (const real *)pl->phi_s, (const real *)pl->grad_s,
                                             (const real *)pl->coinc, pl->tgt_perm, shift, pl->q_sum + r, pl->s, po, ho,
@@ -790,7 +850,7 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
             }
             continue;
         }
-        FS_CUDA(launch_interp<real>(pl->N, pl->m, pl->tgt_base, pl->tgt_frac, w, pl->wpoly, (const real *)pl->grid, pl->pitch,
+        FS_CUDA(launch_interp<real>(pl->N, pl->m, pl->tgt_base, pl->tgt_frac, win_poly<real>(pl), (const real *)pl->grid, pl->pitch,
                                     (real)pl->n_os, (real *)pl->phi_s, (real *)pl->grad_s, false, st));
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[5], st));
@@ -907,7 +967,6 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
             FS_TRY(build_near_items(pl, pl->src_cells, pl->tgt_cells, pl->src_cap, 32, &pl->adj_items,
                                     &pl->n_adj_items));
     }
-    const Window<real> w = make_window<real>(pl);
     const NearParams<real> np = make_near<real>(pl);
     const double shift = std::log(pl->s) / (2.0 * kPi);
     const size_t isz = in_dtype == FS_F64 ? 8 : 4, osz = out_dtype == FS_F64 ? 8 : 4;
@@ -931,11 +990,11 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
                     FS_CUDA(cudaEventRecord(pl->ev_join, pl->aux));
                 }
             }
-            FS_TRY(spread_forward<real>(pl, q, w, st));
+            FS_TRY(spread_forward<real>(pl, q, st));
             FS_TRY(spectral_pipeline<real>(pl));
             if (ovl)
                 FS_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
-            FS_CUDA(launch_interp_hess<real>(N, pl->m, pl->tgt_base, pl->tgt_frac, w, pl->wpoly, (const real *)pl->grid,
+            FS_CUDA(launch_interp_hess<real>(N, pl->m, pl->tgt_base, pl->tgt_frac, win_poly<real>(pl), (const real *)pl->grid,
                                              pl->pitch, (real)pl->n_os, (real *)pl->grad_s, (real *)pl->adj_hess, ovl,
                                              st));
             if constexpr (sizeof(real) == 4) {
@@ -965,12 +1024,12 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
             }
             FS_CUDA(cudaMemsetAsync(pl->grid, 0, grid_bytes, st));
             FS_CUDA(launch_spread_dip<real>(pl->tgt_items, pl->n_tgt_items, pl->cg, pl->m, pl->tgt_base, pl->tgt_frac,
-                                            (const real *)pl->adj_c, pl->adj_df, w, pl->wpoly, (real *)pl->grid,
+                                            (const real *)pl->adj_c, pl->adj_df, win_poly<real>(pl), (real *)pl->grid,
                                             pl->pitch, pl->n_a, pl->kahan, st));
             FS_TRY(spectral_pipeline<real>(pl));
             if (ovl)
                 FS_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
-            FS_CUDA(launch_interp<real>(M, pl->m, pl->src_base, pl->src_frac, w, pl->wpoly, (const real *)pl->grid,
+            FS_CUDA(launch_interp<real>(M, pl->m, pl->src_base, pl->src_frac, win_poly<real>(pl), (const real *)pl->grid,
                                         pl->pitch, (real)pl->n_os, (real *)pl->adj_a, (real *)pl->adj_ga, ovl, st));
             if constexpr (sizeof(real) == 4) {
                 if (!ovl)

@@ -265,16 +265,16 @@ cudaError_t launch_batch_gather_charges(const BatchInst<real> *inst, const Batch
                                         int nrhs, int q_is_f64, cudaStream_t st);
 template <typename real>
 cudaError_t launch_batch_spread(const SpreadItem *items, int n_items, int nrhs, const BatchInst<real> *inst, int m,
-                                int max_tile, Window<real> w, const WindowPoly &wp, bool kahan, cudaStream_t st);
+                                int max_tile, const WinPoly<real> &wp, bool kahan, cudaStream_t st);
 template <typename real>
 cudaError_t prepare_batch_spread(int m, int max_tile, bool kahan);
 template <typename real>
 cudaError_t launch_batch_interp(const BatchInst<real> *inst, BlockMap bm, int blocks, int nrhs, int m,
-                                Window<real> w, const WindowPoly &wp, cudaStream_t st);
+                                const WinPoly<real> &wp, cudaStream_t st);
 // FP32 batches: interpolation and output in one pass, after the near field stored its sums
 template <typename real>
 cudaError_t launch_batch_interp_out(const BatchInst<real> *inst, const BatchIO *io, BlockMap bm, int blocks, int nrhs,
-                                    int m, Window<real> w, const WindowPoly &wp, int out_is_f64, cudaStream_t st);
+                                    int m, const WinPoly<real> &wp, int out_is_f64, cudaStream_t st);
 // counters: 2 * n_inst * nrhs ints (rows done, columns done) plus the queue head, zeroed
 // before each launch; err: set to 1 when a wait ran out of spins
 template <typename real>
@@ -315,37 +315,34 @@ cudaError_t launch_near_count(const double2 *tgt_pos, const int *tgt_base, int64
 // ---- spreading / interpolation (kernels_spread.cu)
 template <typename real>
 cudaError_t launch_spread(const SpreadItem *items, int n_items, CellGrid cg, int m, const int *base,
-                          const void *frac, const real *q, Window<real> w, const WindowPoly &wp, real *grid,
+                          const void *frac, const real *q, const WinPoly<real> &wp, real *grid,
                           int pitch, int n_a, bool kahan, cudaStream_t st);
 // direct spreading (global atomics, no tiles); comp: compensation plane of the grid's size
 // (FP32 with compensation; folded into the grid at the end), may be null otherwise
 template <typename real>
 cudaError_t launch_spread_direct(int64_t M, int m, const int *base, const void *frac, const real *q, Window<real> w,
-                                 const WindowPoly &wp, real *grid, real *comp, int pitch, int n_a, bool kahan,
+                                 const WinPoly<real> &wp, real *grid, real *comp, int pitch, int n_a, bool kahan,
                                  cudaStream_t st);
 template <typename real>
 // acc: add to phi_s / grad_s (the near field already stored there) instead of writing them
-cudaError_t launch_interp(int64_t N, int m, const int *base, const void *frac, Window<real> w,
-                          const WindowPoly &wp, const real *grid, int pitch, real n_os, real *phi_s, real *grad_s,
+cudaError_t launch_interp(int64_t N, int m, const int *base, const void *frac, const WinPoly<real> &wp, const real *grid, int pitch, real n_os, real *phi_s, real *grad_s,
                           bool acc, cudaStream_t st);
 
 // Interpolation and output in one pass (plans whose near field stored phi_s / grad_s / coinc
 // first): the caller's phi and H at perm[k], as launch_interp with acc followed by launch_unpermute.
 template <typename real>
-cudaError_t launch_interp_out(int64_t N, int m, const int *base, const void *frac, Window<real> w,
-                              const WindowPoly &wp, const real *grid, int pitch, real n_os, const real *phi_s,
+cudaError_t launch_interp_out(int64_t N, int m, const int *base, const void *frac, const WinPoly<real> &wp, const real *grid, int pitch, real n_os, const real *phi_s,
                               const real *grad_s, const real *coinc, const int *perm, double shift,
                               const double *q_sum, double s, void *phi_out, void *H_out, int out_is_f64,
                               cudaStream_t st);
 
 template <typename real>
 cudaError_t launch_spread_dip(const SpreadItem *items, int n_items, CellGrid cg, int m, const int *base,
-                              const void *frac, const real *cq, const void *dq, Window<real> w, const WindowPoly &wp,
+                              const void *frac, const real *cq, const void *dq, const WinPoly<real> &wp,
                               real *grid, int pitch, int n_a, bool kahan, cudaStream_t st);
 template <typename real>
 // (acc: add to grad_s / hess_s, where the near part was stored first)
-cudaError_t launch_interp_hess(int64_t N, int m, const int *base, const void *frac, Window<real> w,
-                               const WindowPoly &wp, const real *grid, int pitch, real n_os, real *grad_s,
+cudaError_t launch_interp_hess(int64_t N, int m, const int *base, const void *frac, const WinPoly<real> &wp, const real *grid, int pitch, real n_os, real *grad_s,
                                real *hess_s, bool acc, cudaStream_t st);
 
 // ---- FFT and spectral multiply (kernels_fft.cu)

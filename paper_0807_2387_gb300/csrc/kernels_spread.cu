@@ -62,7 +62,7 @@ __device__ __forceinline__ float2 sub2f(float2 a, float2 b)   // a - b, one roun
 template <typename real, int M2, bool KAHAN, int TGC = 0>
 __device__ __forceinline__ void spread_item(const SpreadItem &it, const CellGrid &cg, const int *__restrict__ base,
                                             const real2_t<real> *__restrict__ frac, const real *__restrict__ q,
-                                            const Window<real> &w, const WindowPoly &wp, real *__restrict__ grid,
+                                            const WinPoly<real> &wp, real *__restrict__ grid,
                                             int pitch, int n_a)
 {
     constexpr int m = M2 / 2;
@@ -72,7 +72,8 @@ __device__ __forceinline__ void spread_item(const SpreadItem &it, const CellGrid
     constexpr int RPAD = (RPL + VW - 1) / VW * VW;            // a group's row weights, vector-aligned
     constexpr int WSTRIDE = spread_weight_stride<real>(M2);
     constexpr int PLANES = KAHAN ? 2 : 1;
-    constexpr bool kPoly = sizeof(real) == 4;
+    constexpr bool kF32 = sizeof(real) == 4;
+    constexpr int D = WinPolyOf<real>::D;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int kQ = TGC > 0 ? spread_group_pitch(TGC + M2 - 1, M2) : 0;
     const int TG = TGC > 0 ? TGC : cg.T * cg.cell;
@@ -84,7 +85,7 @@ __device__ __forceinline__ void spread_item(const SpreadItem &it, const CellGrid
     unsigned char *after_tiles = smem_raw + spread_tiles_bytes<real>(P, Q, PLANES);
     real *wb = reinterpret_cast<real *>(after_tiles) + warp * WSTRIDE;
     float *poly = reinterpret_cast<float *>(after_tiles + (size_t)kSpreadWarps * WSTRIDE * sizeof(real));
-    if (kPoly) {
+    if constexpr (kF32) {
         for (int i = threadIdx.x; i < M2 * (kPolyD + 1); i += blockDim.x)
             poly[i] = wp.c[i / (kPolyD + 1)][i % (kPolyD + 1)];
     }
@@ -98,12 +99,16 @@ __device__ __forceinline__ void spread_item(const SpreadItem &it, const CellGrid
     const bool first = lane < M2;
     const int jw = first ? lane : lane - M2;
     const int wslot = first ? (jw / RPL) * RPAD + (jw % RPL) : G * RPAD + jw;
-    float pc[kPolyD + 1];   // the lane's window polynomial (FP32 path), in registers for the item
+    real pc[D + 1];   // the lane's window polynomial, in registers for the item (FP64: tap min(jw, 2m-1-jw) at +-t)
     {
-        const float *prow = poly + (lane < 2 * M2 ? jw : 0) * (kPolyD + 1);
+        const int row = lane < 2 * M2 ? jw : 0;
 #pragma unroll
-        for (int k = 0; k <= kPolyD; ++k)
-            pc[k] = kPoly ? prow[k] : 0.f;
+        for (int k = 0; k <= D; ++k) {
+            if constexpr (kF32)
+                pc[k] = poly[row * (kPolyD + 1) + k];
+            else
+                pc[k] = wp.c[row < m ? row : M2 - 1 - row][k];
+        }
     }
     // tap lanes: lane (g, b) owns column b and rows g RPL .. g RPL + RPL - 1 of every source
     const bool tap_lane = lane < G * M2;
@@ -133,10 +138,13 @@ __device__ __forceinline__ void spread_item(const SpreadItem &it, const CellGrid
         if (lane < 2 * M2) {
             const real fr = first ? f.x : f.y;
             real wv;
-            if constexpr (kPoly)
-                wv = poly_eval<kPolyD>(pc, (float)fr - 0.5f);
-            else
-                wv = kb_value<real>(w, fr, m - 1 - jw);
+            if constexpr (kF32) {
+                wv = poly_eval<D>(pc, fr - real(0.5));
+            } else {
+                wv = poly_eval<D>(pc, jw < m ? fr - 0.5 : 0.5 - fr);
+                if (jw == M2 - 1 && fr == 0.0)
+                    wv = 0.0;
+            }
             wb[wslot] = first ? wv : wv * qj;
         }
         __syncwarp();
@@ -180,7 +188,7 @@ __device__ __forceinline__ void spread_item(const SpreadItem &it, const CellGrid
             } else {
 #pragma unroll
                 for (int i = 0; i < RPL; ++i) {
-                    const real sm = old[i] + v[i];
+                    const real sm = kF32 ? old[i] + v[i] : fma(w1[i], w2, old[i]);
                     cell[i * Q] = sm;
                     if (KAHAN) {
                         const real bb = sm - old[i];
@@ -219,7 +227,7 @@ __device__ __forceinline__ void spread_item(const SpreadItem &it, const CellGrid
 template <typename real, int M2, bool KAHAN>
 __global__ void __launch_bounds__(256) k_spread_direct(int64_t M, const int *__restrict__ base,
                                                        const real2_t<real> *__restrict__ frac,
-                                                       const real *__restrict__ q, Window<real> w, WindowPoly wp,
+                                                       const real *__restrict__ q, Window<real> w, WinPoly<real> wp,
                                                        real *__restrict__ grid, real *__restrict__ comp, int pitch)
 {
     constexpr int m = M2 / 2;
@@ -233,7 +241,7 @@ __global__ void __launch_bounds__(256) k_spread_direct(int64_t M, const int *__r
     float pc[kPolyD + 1];
 #pragma unroll
     for (int k = 0; k <= kPolyD; ++k)
-        pc[k] = (kPoly && lane < 2 * M2) ? wp.c[jw][k] : 0.f;
+        pc[k] = (kPoly && lane < 2 * M2) ? (float)wp.c[kPoly ? jw : 0][k] : 0.f;
     const bool tap_lane = lane < G * M2;
     const int g = lane / M2, b = lane - (lane / M2) * M2;
     for (int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; j < M; j += warps) {
@@ -244,7 +252,7 @@ __global__ void __launch_bounds__(256) k_spread_direct(int64_t M, const int *__r
         if (lane < 2 * M2) {
             const real fr = first ? f.x : f.y;
             if constexpr (kPoly)
-                wv = poly_eval<kPolyD>(pc, (float)fr - 0.5f);
+                wv = poly_eval<kPolyD, float>(pc, (float)fr - 0.5f);
             else
                 wv = kb_value<real>(w, fr, m - 1 - jw);
             if (!first)
@@ -287,24 +295,24 @@ template <typename real, int M2, bool KAHAN, int TGC>
 __global__ void __launch_bounds__(kSpreadWarps * 32) k_spread(const SpreadItem *__restrict__ items, CellGrid cg,
                                                               const int *__restrict__ base,
                                                               const real2_t<real> *__restrict__ frac,
-                                                              const real *__restrict__ q, Window<real> w, WindowPoly wp,
+                                                              const real *__restrict__ q, WinPoly<real> wp,
                                                               real *__restrict__ grid, int pitch, int n_a)
 {
-    spread_item<real, M2, KAHAN, TGC>(items[blockIdx.x], cg, base, frac, q, w, wp, grid, pitch, n_a);
+    spread_item<real, M2, KAHAN, TGC>(items[blockIdx.x], cg, base, frac, q, wp, grid, pitch, n_a);
 }
 
 // Batched spreading: items carry their instance in `pad`; blockIdx.y = right-hand side.
 template <typename real, int M2, bool KAHAN>
 __global__ void __launch_bounds__(kSpreadWarps * 32) k_batch_spread(const SpreadItem *__restrict__ items,
                                                                     const BatchInst<real> *__restrict__ inst,
-                                                                    Window<real> w, WindowPoly wp)
+                                                                    WinPoly<real> wp)
 {
     const SpreadItem it = items[blockIdx.x];
     const BatchInst<real> &b = inst[it.pad];
     const int r = blockIdx.y;
     auto go = [&](auto tg) {
         spread_item<real, M2, KAHAN, decltype(tg)::value>(it, b.cg, b.src_base, (const real2_t<real> *)b.src_frac,
-                                                          b.q + (int64_t)r * b.M, w, wp,
+                                                          b.q + (int64_t)r * b.M, wp,
                                                           b.grid + (int64_t)r * b.grid_stride, b.pitch, b.n_a);
     };
     // FP32 compensated batches: the tile edges the autotuner picks for the batched instance
@@ -359,12 +367,11 @@ __device__ __forceinline__ void interp_row(const real *__restrict__ rowp, const 
 // the gradient).
 template <typename real, int M2>
 __device__ __forceinline__ void interp_sums(int64_t k, const int *__restrict__ base,
-                                            const real2_t<real> *__restrict__ frac, const Window<real> &w,
-                                            const WindowPoly &wp, const real *__restrict__ grid, int pitch, real &phi,
-                                            real &g1, real &g2)
+                                            const real2_t<real> *__restrict__ frac, const WinPoly<real> &wp,
+                                            const real *__restrict__ grid, int pitch, real &phi, real &g1, real &g2)
 {
-    constexpr int m = M2 / 2;
-    constexpr bool kRef = sizeof(real) == 4 && m >= 5;
+    constexpr int m = M2 / 2, D = WinPolyOf<real>::D;
+    constexpr bool kRef = sizeof(real) == 4 && m >= 5, kEdge = sizeof(real) == 8;
     const int packed = base[k];
     const real2_t<real> f = frac[k];
     const int row0 = base1(packed) - m + 1;
@@ -372,48 +379,38 @@ __device__ __forceinline__ void interp_sums(int64_t k, const int *__restrict__ b
     real rs_ref = 0;
     phi = g1 = g2 = 0;
     real w2[M2], d2[M2];
-    if constexpr (sizeof(real) == 4) {
-        // FP32: per-tap window polynomials in t = frac - 1/2 (coefficients are warp-uniform kernel
-        // parameters).  The window is even, so tap M2-1-a at t is tap a at -t: each pair takes
-        // the even and odd parts of tap a's polynomials in t^2 once (value p(+-t) = E +- t O,
-        // slope of the mirrored tap -p'(-t) = t O' - E'), about half the FMAs of 2 evaluations.
-        // The column weights are held for all rows; the row weights of each symmetric pair of
-        // rows are evaluated just before those two rows (middle pair first, so that row m - 1,
-        // the reference, comes first), which keeps 2 M2 fewer values live across the loop.
-        const float t1 = (float)f.x - 0.5f, t2 = (float)f.y - 0.5f;
-        const float s1 = t1 * t1, s2 = t2 * t2;
+    // Per-tap window polynomials in t = frac - 1/2 (coefficients are warp-uniform kernel
+    // parameters).  The window is even, so tap M2-1-a at t is tap a at -t: each pair takes
+    // the even and odd parts of tap a's polynomials in t^2 once (value p(+-t) = E +- t O,
+    // slope of the mirrored tap -p'(-t) = t O' - E'), about half the FMAs of 2 evaluations.
+    // The column weights are held for all rows; the row weights of each symmetric pair of
+    // rows are evaluated just before those two rows (middle pair first, so that row m - 1,
+    // the reference, comes first), which keeps 2 M2 fewer values live across the loop.
+    const real t1 = f.x - real(0.5), t2 = f.y - real(0.5);
+    const real s1 = t1 * t1, s2 = t2 * t2;
 #pragma unroll
-        for (int a = 0; a < m; ++a) {
-            float e, o;
-            poly_even_odd<kPolyD>(wp.c[a], s2, e, o);
-            w2[a] = fmaf(t2, o, e);
-            w2[M2 - 1 - a] = fmaf(-t2, o, e);
-            poly_even_odd<kPolyD - 1>(wp.d[a], s2, e, o);
-            d2[a] = fmaf(t2, o, e);
-            d2[M2 - 1 - a] = fmaf(t2, o, -e);
-        }
+    for (int a = 0; a < m; ++a) {
+        real e, o;
+        poly_even_odd<D>(wp.c[a], s2, e, o);
+        w2[a] = fma(t2, o, e);
+        w2[M2 - 1 - a] = fma(-t2, o, e);
+        poly_even_odd<D - 1>(wp.d[a], s2, e, o);
+        d2[a] = fma(t2, o, e);
+        d2[M2 - 1 - a] = fma(t2, o, -e);
+    }
+    if (kEdge && f.y == real(0))
+        w2[M2 - 1] = d2[M2 - 1] = real(0);
 #pragma unroll
-        for (int q = 0; q < m; ++q) {
-            const int a = m - 1 - q, a2 = M2 - 1 - a;
-            float e, o, de, dd;
-            poly_even_odd<kPolyD>(wp.c[a], s1, e, o);
-            poly_even_odd<kPolyD - 1>(wp.d[a], s1, de, dd);
-            interp_row<real, M2, kRef>(grid + (int64_t)(row0 + a) * pitch + col0, w2, d2, fmaf(t1, o, e),
-                                       fmaf(t1, dd, de), q == 0, rs_ref, phi, g1, g2);
-            interp_row<real, M2, kRef>(grid + (int64_t)(row0 + a2) * pitch + col0, w2, d2, fmaf(-t1, o, e),
-                                       fmaf(t1, dd, -de), false, rs_ref, phi, g1, g2);
-        }
-    } else {
-        real w1[M2], d1[M2];
-#pragma unroll
-        for (int a = 0; a < M2; ++a) {
-            kb_value_slope<real>(w, f.x, m - 1 - a, w1[a], d1[a]);
-            kb_value_slope<real>(w, f.y, m - 1 - a, w2[a], d2[a]);
-        }
-#pragma unroll
-        for (int a = 0; a < M2; ++a)
-            interp_row<real, M2, kRef>(grid + (int64_t)(row0 + a) * pitch + col0, w2, d2, w1[a], d1[a], false,
-                                       rs_ref, phi, g1, g2);
+    for (int q = 0; q < m; ++q) {
+        const int a = m - 1 - q, a2 = M2 - 1 - a;
+        real e, o, de, dd;
+        poly_even_odd<D>(wp.c[a], s1, e, o);
+        poly_even_odd<D - 1>(wp.d[a], s1, de, dd);
+        const bool edge = kEdge && a == 0 && f.x == real(0);
+        interp_row<real, M2, kRef>(grid + (int64_t)(row0 + a) * pitch + col0, w2, d2, fma(t1, o, e), fma(t1, dd, de),
+                                   q == 0, rs_ref, phi, g1, g2);
+        interp_row<real, M2, kRef>(grid + (int64_t)(row0 + a2) * pitch + col0, w2, d2, edge ? real(0) : fma(-t1, o, e),
+                                   edge ? real(0) : fma(t1, dd, -de), false, rs_ref, phi, g1, g2);
     }
 }
 
@@ -467,13 +464,13 @@ __device__ __forceinline__ void interp_sums_rhs(int64_t k, const int *__restrict
 
 template <typename real, int M2>
 __device__ __forceinline__ void interp_point(int64_t k, const int *__restrict__ base,
-                                             const real2_t<real> *__restrict__ frac, const Window<real> &w,
-                                             const WindowPoly &wp, const real *__restrict__ grid, int pitch, real n_os,
+                                             const real2_t<real> *__restrict__ frac,
+                                             const WinPoly<real> &wp, const real *__restrict__ grid, int pitch, real n_os,
                                              real *__restrict__ phi_s, real *__restrict__ grad_s,
                                              bool acc = false)
 {
     real phi, g1, g2;
-    interp_sums<real, M2>(k, base, frac, w, wp, grid, pitch, phi, g1, g2);
+    interp_sums<real, M2>(k, base, frac, wp, grid, pitch, phi, g1, g2);
     // acc: the near field was stored first (overlapped with spreading and the transform)
     phi_s[k] = acc ? phi_s[k] + phi : phi;
     grad_s[2 * k] = acc ? grad_s[2 * k] + n_os * g1 : n_os * g1;
@@ -482,13 +479,13 @@ __device__ __forceinline__ void interp_point(int64_t k, const int *__restrict__ 
 
 template <typename real, int M2>
 __global__ void __launch_bounds__(256) k_interp(int64_t N, const int *__restrict__ base,
-                                                const real2_t<real> *__restrict__ frac, Window<real> w, WindowPoly wp,
+                                                const real2_t<real> *__restrict__ frac, WinPoly<real> wp,
                                                 const real *__restrict__ grid, int pitch, real n_os,
                                                 real *__restrict__ phi_s, real *__restrict__ grad_s, bool acc)
 {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k < N)
-        interp_point<real, M2>(k, base, frac, w, wp, grid, pitch, n_os, phi_s, grad_s, acc);
+        interp_point<real, M2>(k, base, frac, wp, grid, pitch, n_os, phi_s, grad_s, acc);
 }
 
 // Interpolation and output in one pass, for plans whose near field was stored first: the far
@@ -497,8 +494,8 @@ __global__ void __launch_bounds__(256) k_interp(int64_t N, const int *__restrict
 // written back and read again.
 template <typename real, int M2>
 __global__ void __launch_bounds__(256, 3) k_interp_out(int64_t N, const int *__restrict__ base,
-                                                    const real2_t<real> *__restrict__ frac, Window<real> w,
-                                                    WindowPoly wp, const real *__restrict__ grid, int pitch, real n_os,
+                                                    const real2_t<real> *__restrict__ frac,
+                                                    WinPoly<real> wp, const real *__restrict__ grid, int pitch, real n_os,
                                                     const real *__restrict__ phi_s, const real *__restrict__ grad_s,
                                                     const real *__restrict__ coinc, const int *__restrict__ perm,
                                                     double shift, const double *__restrict__ q_sum, double s,
@@ -508,7 +505,7 @@ __global__ void __launch_bounds__(256, 3) k_interp_out(int64_t N, const int *__r
     if (k >= N)
         return;
     real phi, g1, g2;
-    interp_sums<real, M2>(k, base, frac, w, wp, grid, pitch, phi, g1, g2);
+    interp_sums<real, M2>(k, base, frac, wp, grid, pitch, phi, g1, g2);
     const real pt = phi_s[k] + phi;
     const real gx = grad_s[2 * k] + n_os * g1;
     const real gy = grad_s[2 * k + 1] + n_os * g2;
@@ -518,7 +515,7 @@ __global__ void __launch_bounds__(256, 3) k_interp_out(int64_t N, const int *__r
 // Batched interpolation: block -> (instance, block of its targets), blockIdx.y = right-hand side.
 template <typename real, int M2>
 __global__ void __launch_bounds__(256) k_batch_interp(const BatchInst<real> *__restrict__ inst, BlockMap bm,
-                                                      Window<real> w, WindowPoly wp)
+                                                      WinPoly<real> wp)
 {
     const int i = bm.inst[blockIdx.x];
     const BatchInst<real> &b = inst[i];
@@ -527,7 +524,7 @@ __global__ void __launch_bounds__(256) k_batch_interp(const BatchInst<real> *__r
     if (k >= N)
         return;
     const int r = blockIdx.y;
-    interp_point<real, M2>(k, b.tgt_base, (const real2_t<real> *)b.tgt_frac, w, wp,
+    interp_point<real, M2>(k, b.tgt_base, (const real2_t<real> *)b.tgt_frac, wp,
                            b.grid + (int64_t)r * b.grid_stride, b.pitch, (real)b.L, b.phi_s + (int64_t)r * N,
                            b.grad_s + 2 * (int64_t)r * N);
 }
@@ -537,8 +534,8 @@ __global__ void __launch_bounds__(256) k_batch_interp(const BatchInst<real> *__r
 // caller's (nrhs, N) and (nrhs, N, 2) buffers of each instance.
 template <typename real, int M2>
 __global__ void __launch_bounds__(256, 3) k_batch_interp_out(const BatchInst<real> *__restrict__ inst,
-                                                          const BatchIO *__restrict__ io, BlockMap bm, Window<real> w,
-                                                          WindowPoly wp, int out_is_f64)
+                                                          const BatchIO *__restrict__ io, BlockMap bm,
+                                                          WinPoly<real> wp, int out_is_f64)
 {
     const int i = bm.inst[blockIdx.x];
     const BatchInst<real> &b = inst[i];
@@ -548,7 +545,7 @@ __global__ void __launch_bounds__(256, 3) k_batch_interp_out(const BatchInst<rea
         return;
     const int r = blockIdx.y;
     real phi, g1, g2;
-    interp_sums<real, M2>(k, b.tgt_base, (const real2_t<real> *)b.tgt_frac, w, wp, b.grid + (int64_t)r * b.grid_stride,
+    interp_sums<real, M2>(k, b.tgt_base, (const real2_t<real> *)b.tgt_frac, wp, b.grid + (int64_t)r * b.grid_stride,
                           b.pitch, phi, g1, g2);
     const real n_os = (real)b.L;
     const real *ps = b.phi_s + (int64_t)r * N, *gs = b.grad_s + 2 * (int64_t)r * N;
@@ -595,15 +592,16 @@ __global__ void __launch_bounds__(kSpreadWarps * 32) k_spread_dip(const SpreadIt
                                                                   const int *__restrict__ base,
                                                                   const real2_t<real> *__restrict__ frac,
                                                                   const real *__restrict__ cq,
-                                                                  const real2_t<real> *__restrict__ dq, Window<real> w,
-                                                                  WindowPoly wp, real *__restrict__ grid, int pitch,
+                                                                  const real2_t<real> *__restrict__ dq,
+                                                                  WinPoly<real> wp, real *__restrict__ grid, int pitch,
                                                                   int n_a)
 {
     constexpr int m = M2 / 2;
     constexpr int TAPS = M2 * M2;
     constexpr int PER = (TAPS + 31) / 32;
     constexpr int PLANES = KAHAN ? 2 : 1;
-    constexpr bool kPoly = sizeof(real) == 4;
+    constexpr bool kF32 = sizeof(real) == 4;
+    constexpr int D = WinPolyOf<real>::D;
     extern __shared__ unsigned char smem_raw[];
     const int TG = cg.T * cg.cell;
     const int P = TG + M2 - 1;
@@ -612,7 +610,7 @@ __global__ void __launch_bounds__(kSpreadWarps * 32) k_spread_dip(const SpreadIt
     const int PP = P * Q;                             // one plane of a warp tile
     real *acc = reinterpret_cast<real *>(smem_raw) + (size_t)warp * PP * PLANES;
     float *poly = reinterpret_cast<float *>(reinterpret_cast<real *>(smem_raw) + (size_t)kSpreadWarps * PP * PLANES);
-    if (kPoly) {
+    if constexpr (kF32) {
         for (int i = threadIdx.x; i < M2 * (kPolyD + 1); i += blockDim.x)
             poly[i] = wp.c[i / (kPolyD + 1)][i % (kPolyD + 1)];
         for (int i = threadIdx.x; i < M2 * kPolyD; i += blockDim.x)
@@ -629,16 +627,26 @@ __global__ void __launch_bounds__(kSpreadWarps * 32) k_spread_dip(const SpreadIt
     spread_lane_taps<M2, PER>(lane, Q, ta, tb, toff, valid);
     const bool first = lane < M2;
     const int jw = first ? lane : lane - M2;
-    float pc[kPolyD + 1], pd[kPolyD];   // the lane's value and slope polynomials, in registers
+    real pc[D + 1], pd[D];   // the lane's value and slope polynomials, in registers (FP64: of the tap or its mirror)
     {
-        const float *prow = poly + (lane < 2 * M2 ? jw : 0) * (kPolyD + 1);
-        const float *drow = poly + M2 * (kPolyD + 1) + (lane < 2 * M2 ? jw : 0) * kPolyD;
+        const int row = lane < 2 * M2 ? jw : 0;
+        if constexpr (kF32) {
+            const float *prow = poly + row * (kPolyD + 1), *drow = poly + M2 * (kPolyD + 1) + row * kPolyD;
 #pragma unroll
-        for (int k = 0; k <= kPolyD; ++k)
-            pc[k] = kPoly ? prow[k] : 0.f;
+            for (int k = 0; k <= kPolyD; ++k)
+                pc[k] = prow[k];
 #pragma unroll
-        for (int k = 0; k < kPolyD; ++k)
-            pd[k] = kPoly ? drow[k] : 0.f;
+            for (int k = 0; k < kPolyD; ++k)
+                pd[k] = drow[k];
+        } else {
+            const int a = row < m ? row : M2 - 1 - row;
+#pragma unroll
+            for (int k = 0; k <= D; ++k)
+                pc[k] = wp.c[a][k];
+#pragma unroll
+            for (int k = 0; k < D; ++k)
+                pd[k] = wp.d[a][k];
+        }
     }
     for (int j = it.start + warp; j < it.start + it.count; j += kSpreadWarps) {
         const int packed = base[j];
@@ -648,11 +656,14 @@ __global__ void __launch_bounds__(kSpreadWarps * 32) k_spread_dip(const SpreadIt
         real wv = real(0), wd = real(0);
         if (lane < 2 * M2) {
             const real fr = first ? f.x : f.y;
-            if constexpr (kPoly) {
-                wv = poly_eval<kPolyD>(pc, (float)fr - 0.5f);
-                wd = poly_eval<kPolyD - 1>(pd, (float)fr - 0.5f);
-            } else {
-                kb_value_slope<real>(w, fr, m - 1 - jw, wv, wd);
+            const real t = kF32 || jw < m ? fr - real(0.5) : real(0.5) - fr;
+            wv = poly_eval<D>(pc, t);
+            wd = poly_eval<D - 1>(pd, t);
+            if constexpr (!kF32) {
+                if (jw >= m)
+                    wd = -wd;
+                if (jw == M2 - 1 && fr == 0.0)
+                    wv = wd = 0.0;
             }
         }
         real *corner = acc + (base1(packed) - m + 1 - o1) * Q + (base2(packed) - m + 1 - o2);
@@ -707,37 +718,49 @@ __global__ void __launch_bounds__(kSpreadWarps * 32) k_spread_dip(const SpreadIt
 // FP32 with m >= 5 forms the derivative sums against a reference tap (see k_interp).
 template <typename real, int M2>
 __global__ void __launch_bounds__(256) k_interp_hess(int64_t N, const int *__restrict__ base,
-                                                     const real2_t<real> *__restrict__ frac, Window<real> w,
-                                                     WindowPoly wp, const real *__restrict__ grid, int pitch,
+                                                     const real2_t<real> *__restrict__ frac,
+                                                     WinPoly<real> wp, const real *__restrict__ grid, int pitch,
                                                      real n_os, real *__restrict__ grad_s, real *__restrict__ hess_s,
                                                      bool acc)
 {
     constexpr int m = M2 / 2;
     constexpr bool kRef = sizeof(real) == 4 && m >= 5;
+    constexpr int D = WinPolyOf<real>::D;
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= N)
         return;
     const int packed = base[k];
     const real2_t<real> f = frac[k];
     real w1[M2], d1[M2], e1[M2], w2[M2], d2[M2], e2[M2];
-    if constexpr (sizeof(real) == 4) {
-        const float t1 = (float)f.x - 0.5f, t2 = (float)f.y - 0.5f;
+    // each symmetric pair of taps from the even and odd parts of one's polynomials (interp_sums); the
+    // curvature of the mirrored tap is p''(-t)
+    const real t1 = f.x - real(0.5), t2 = f.y - real(0.5), s1 = t1 * t1, s2 = t2 * t2;
 #pragma unroll
-        for (int a = 0; a < M2; ++a) {
-            w1[a] = poly_eval<kPolyD>(wp.c[a], t1);
-            d1[a] = poly_eval<kPolyD - 1>(wp.d[a], t1);
-            e1[a] = poly_eval<kPolyD - 2>(wp.e[a], t1);
-            w2[a] = poly_eval<kPolyD>(wp.c[a], t2);
-            d2[a] = poly_eval<kPolyD - 1>(wp.d[a], t2);
-            e2[a] = poly_eval<kPolyD - 2>(wp.e[a], t2);
-        }
-    } else {
-#pragma unroll
-        for (int a = 0; a < M2; ++a) {
-            kb_value_slope_curv<real>(w, f.x, m - 1 - a, w1[a], d1[a], e1[a]);
-            kb_value_slope_curv<real>(w, f.y, m - 1 - a, w2[a], d2[a], e2[a]);
-        }
+    for (int a = 0; a < m; ++a) {
+        real e, o;
+        poly_even_odd<D>(wp.c[a], s1, e, o);
+        w1[a] = fma(t1, o, e);
+        w1[M2 - 1 - a] = fma(-t1, o, e);
+        poly_even_odd<D - 1>(wp.d[a], s1, e, o);
+        d1[a] = fma(t1, o, e);
+        d1[M2 - 1 - a] = fma(t1, o, -e);
+        poly_even_odd<D - 2>(wp.e[a], s1, e, o);
+        e1[a] = fma(t1, o, e);
+        e1[M2 - 1 - a] = fma(-t1, o, e);
+        poly_even_odd<D>(wp.c[a], s2, e, o);
+        w2[a] = fma(t2, o, e);
+        w2[M2 - 1 - a] = fma(-t2, o, e);
+        poly_even_odd<D - 1>(wp.d[a], s2, e, o);
+        d2[a] = fma(t2, o, e);
+        d2[M2 - 1 - a] = fma(t2, o, -e);
+        poly_even_odd<D - 2>(wp.e[a], s2, e, o);
+        e2[a] = fma(t2, o, e);
+        e2[M2 - 1 - a] = fma(-t2, o, e);
     }
+    if (sizeof(real) == 8 && f.x == real(0))
+        w1[M2 - 1] = d1[M2 - 1] = e1[M2 - 1] = real(0);
+    if (sizeof(real) == 8 && f.y == real(0))
+        w2[M2 - 1] = d2[M2 - 1] = e2[M2 - 1] = real(0);
     const int row0 = base1(packed) - m + 1;
     const int col0 = base2(packed) - m + 1;
     real rs[M2], rd[M2];
@@ -782,7 +805,7 @@ __global__ void __launch_bounds__(256) k_interp_hess(int64_t N, const int *__res
 
 template <typename real, int M2>
 cudaError_t spread_m(const SpreadItem *items, int n_items, CellGrid cg, const int *base, const void *frac,
-                     const real *q, Window<real> w, const WindowPoly &wp, real *grid, int pitch, int n_a, bool kahan,
+                     const real *q, const WinPoly<real> &wp, real *grid, int pitch, int n_a, bool kahan,
                      cudaStream_t st)
 {
     const int TG = cg.T * cg.cell;
@@ -793,7 +816,7 @@ cudaError_t spread_m(const SpreadItem *items, int n_items, CellGrid cg, const in
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess)
             return e;
-        kern<<<n_items, kSpreadWarps * 32, smem, st>>>(items, cg, base, fr, q, w, wp, grid, pitch, n_a);
+        kern<<<n_items, kSpreadWarps * 32, smem, st>>>(items, cg, base, fr, q, wp, grid, pitch, n_a);
         return cudaGetLastError();
     };
     // the tile edges of the 2D plans' two tile rules (16 and 24 grid lines) compiled as constants
@@ -805,18 +828,18 @@ cudaError_t spread_m(const SpreadItem *items, int n_items, CellGrid cg, const in
 }
 
 template <typename real, int M2>
-cudaError_t interp_m(int64_t N, const int *base, const void *frac, Window<real> w, const WindowPoly &wp,
+cudaError_t interp_m(int64_t N, const int *base, const void *frac, const WinPoly<real> &wp,
                      const real *grid, int pitch, real n_os, real *phi_s, real *grad_s, bool acc, cudaStream_t st)
 {
     const unsigned blocks = (unsigned)((N + 255) / 256);
-    k_interp<real, M2><<<blocks, 256, 0, st>>>(N, base, (const real2_t<real> *)frac, w, wp, grid, pitch, n_os, phi_s,
+    k_interp<real, M2><<<blocks, 256, 0, st>>>(N, base, (const real2_t<real> *)frac, wp, grid, pitch, n_os, phi_s,
                                                 grad_s, acc);
     return cudaGetLastError();
 }
 
 template <typename real, int M2>
 cudaError_t spread_dip_m(const SpreadItem *items, int n_items, CellGrid cg, const int *base, const void *frac,
-                         const real *cq, const void *dq, Window<real> w, const WindowPoly &wp, real *grid, int pitch,
+                         const real *cq, const void *dq, const WinPoly<real> &wp, real *grid, int pitch,
                          int n_a, bool kahan, cudaStream_t st)
 {
     const int TG = cg.T * cg.cell;
@@ -830,24 +853,24 @@ cudaError_t spread_dip_m(const SpreadItem *items, int n_items, CellGrid cg, cons
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess)
             return e;
-        kern<<<n_items, kSpreadWarps * 32, smem, st>>>(items, cg, base, fr, cq, dd, w, wp, grid, pitch, n_a);
+        kern<<<n_items, kSpreadWarps * 32, smem, st>>>(items, cg, base, fr, cq, dd, wp, grid, pitch, n_a);
     } else {
         auto kern = k_spread_dip<real, M2, false>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess)
             return e;
-        kern<<<n_items, kSpreadWarps * 32, smem, st>>>(items, cg, base, fr, cq, dd, w, wp, grid, pitch, n_a);
+        kern<<<n_items, kSpreadWarps * 32, smem, st>>>(items, cg, base, fr, cq, dd, wp, grid, pitch, n_a);
     }
     return cudaGetLastError();
 }
 
 template <typename real, int M2>
-cudaError_t interp_hess_m(int64_t N, const int *base, const void *frac, Window<real> w, const WindowPoly &wp,
+cudaError_t interp_hess_m(int64_t N, const int *base, const void *frac, const WinPoly<real> &wp,
                           const real *grid, int pitch, real n_os, real *grad_s, real *hess_s, bool acc,
                           cudaStream_t st)
 {
     const unsigned blocks = (unsigned)((N + 255) / 256);
-    k_interp_hess<real, M2><<<blocks, 256, 0, st>>>(N, base, (const real2_t<real> *)frac, w, wp, grid, pitch, n_os,
+    k_interp_hess<real, M2><<<blocks, 256, 0, st>>>(N, base, (const real2_t<real> *)frac, wp, grid, pitch, n_os,
                                                      grad_s, hess_s, acc);
     return cudaGetLastError();
 }
@@ -856,7 +879,7 @@ cudaError_t interp_hess_m(int64_t N, const int *base, const void *frac, Window<r
 
 template <typename real>
 cudaError_t launch_spread_dip(const SpreadItem *items, int n_items, CellGrid cg, int m, const int *base,
-                              const void *frac, const real *cq, const void *dq, Window<real> w, const WindowPoly &wp,
+                              const void *frac, const real *cq, const void *dq, const WinPoly<real> &wp,
                               real *grid, int pitch, int n_a, bool kahan, cudaStream_t st)
 {
     if (n_items <= 0)
@@ -865,7 +888,7 @@ cudaError_t launch_spread_dip(const SpreadItem *items, int n_items, CellGrid cg,
     switch (m) {
 #define FS_DIP_CASE(MM)                                                                                          \
     case MM:                                                                                                     \
-        return spread_dip_m<real, 2 * MM>(items, n_items, cg, base, frac, cq, dq, w, wp, grid, pitch, n_a, comp, st);
+        return spread_dip_m<real, 2 * MM>(items, n_items, cg, base, frac, cq, dq, wp, grid, pitch, n_a, comp, st);
         FS_DIP_CASE(2)
         FS_DIP_CASE(3)
         FS_DIP_CASE(4)
@@ -879,8 +902,7 @@ cudaError_t launch_spread_dip(const SpreadItem *items, int n_items, CellGrid cg,
 }
 
 template <typename real>
-cudaError_t launch_interp_hess(int64_t N, int m, const int *base, const void *frac, Window<real> w,
-                               const WindowPoly &wp, const real *grid, int pitch, real n_os, real *grad_s,
+cudaError_t launch_interp_hess(int64_t N, int m, const int *base, const void *frac, const WinPoly<real> &wp, const real *grid, int pitch, real n_os, real *grad_s,
                                real *hess_s, bool acc, cudaStream_t st)
 {
     if (N <= 0)
@@ -888,7 +910,7 @@ cudaError_t launch_interp_hess(int64_t N, int m, const int *base, const void *fr
     switch (m) {
 #define FS_HESS_CASE(MM)                                                                                         \
     case MM:                                                                                                     \
-        return interp_hess_m<real, 2 * MM>(N, base, frac, w, wp, grid, pitch, n_os, grad_s, hess_s, acc, st);
+        return interp_hess_m<real, 2 * MM>(N, base, frac, wp, grid, pitch, n_os, grad_s, hess_s, acc, st);
         FS_HESS_CASE(2)
         FS_HESS_CASE(3)
         FS_HESS_CASE(4)
@@ -902,16 +924,14 @@ cudaError_t launch_interp_hess(int64_t N, int m, const int *base, const void *fr
 }
 
 template cudaError_t launch_spread_dip<float>(const SpreadItem *, int, CellGrid, int, const int *, const void *,
-                                              const float *, const void *, Window<float>, const WindowPoly &, float *,
+                                              const float *, const void *, const WindowPoly &, float *,
                                               int, int, bool, cudaStream_t);
 template cudaError_t launch_spread_dip<double>(const SpreadItem *, int, CellGrid, int, const int *, const void *,
-                                               const double *, const void *, Window<double>, const WindowPoly &,
+                                               const double *, const void *, const WindowPoly64 &,
                                                double *, int, int, bool, cudaStream_t);
-template cudaError_t launch_interp_hess<float>(int64_t, int, const int *, const void *, Window<float>,
-                                               const WindowPoly &, const float *, int, float, float *, float *, bool,
+template cudaError_t launch_interp_hess<float>(int64_t, int, const int *, const void *, const WindowPoly &, const float *, int, float, float *, float *, bool,
                                                cudaStream_t);
-template cudaError_t launch_interp_hess<double>(int64_t, int, const int *, const void *, Window<double>,
-                                                const WindowPoly &, const double *, int, double, double *, double *,
+template cudaError_t launch_interp_hess<double>(int64_t, int, const int *, const void *, const WindowPoly64 &, const double *, int, double, double *, double *,
                                                 bool, cudaStream_t);
 
 // Calls f(std::integral_constant<int, 2m>) for the window half-width m in 2..8.
@@ -931,52 +951,52 @@ template <class F> cudaError_t with_width_spread(int m, F &&f)
 
 template <typename real>
 cudaError_t launch_spread(const SpreadItem *items, int n_items, CellGrid cg, int m, const int *base, const void *frac,
-                          const real *q, Window<real> w, const WindowPoly &wp, real *grid, int pitch, int n_a,
+                          const real *q, const WinPoly<real> &wp, real *grid, int pitch, int n_a,
                           bool kahan, cudaStream_t st)
 {
     if (n_items <= 0)
         return cudaSuccess;
     const bool comp = kahan && sizeof(real) == 4;
     switch (m) {
-    case 2: return spread_m<real, 4>(items, n_items, cg, base, frac, q, w, wp, grid, pitch, n_a, comp, st);
-    case 3: return spread_m<real, 6>(items, n_items, cg, base, frac, q, w, wp, grid, pitch, n_a, comp, st);
-    case 4: return spread_m<real, 8>(items, n_items, cg, base, frac, q, w, wp, grid, pitch, n_a, comp, st);
-    case 5: return spread_m<real, 10>(items, n_items, cg, base, frac, q, w, wp, grid, pitch, n_a, comp, st);
-    case 6: return spread_m<real, 12>(items, n_items, cg, base, frac, q, w, wp, grid, pitch, n_a, comp, st);
-    case 7: return spread_m<real, 14>(items, n_items, cg, base, frac, q, w, wp, grid, pitch, n_a, comp, st);
-    case 8: return spread_m<real, 16>(items, n_items, cg, base, frac, q, w, wp, grid, pitch, n_a, comp, st);
+    case 2: return spread_m<real, 4>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
+    case 3: return spread_m<real, 6>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
+    case 4: return spread_m<real, 8>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
+    case 5: return spread_m<real, 10>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
+    case 6: return spread_m<real, 12>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
+    case 7: return spread_m<real, 14>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
+    case 8: return spread_m<real, 16>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
     default: return cudaErrorInvalidValue;
     }
 }
 
 template <typename real>
-cudaError_t launch_interp(int64_t N, int m, const int *base, const void *frac, Window<real> w, const WindowPoly &wp,
+cudaError_t launch_interp(int64_t N, int m, const int *base, const void *frac, const WinPoly<real> &wp,
                           const real *grid, int pitch, real n_os, real *phi_s, real *grad_s, bool acc,
                           cudaStream_t st)
 {
     if (N <= 0)
         return cudaSuccess;
     switch (m) {
-    case 2: return interp_m<real, 4>(N, base, frac, w, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
-    case 3: return interp_m<real, 6>(N, base, frac, w, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
-    case 4: return interp_m<real, 8>(N, base, frac, w, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
-    case 5: return interp_m<real, 10>(N, base, frac, w, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
-    case 6: return interp_m<real, 12>(N, base, frac, w, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
-    case 7: return interp_m<real, 14>(N, base, frac, w, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
-    case 8: return interp_m<real, 16>(N, base, frac, w, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
+    case 2: return interp_m<real, 4>(N, base, frac, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
+    case 3: return interp_m<real, 6>(N, base, frac, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
+    case 4: return interp_m<real, 8>(N, base, frac, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
+    case 5: return interp_m<real, 10>(N, base, frac, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
+    case 6: return interp_m<real, 12>(N, base, frac, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
+    case 7: return interp_m<real, 14>(N, base, frac, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
+    case 8: return interp_m<real, 16>(N, base, frac, wp, grid, pitch, n_os, phi_s, grad_s, acc, st);
     default: return cudaErrorInvalidValue;
     }
 }
 
 template cudaError_t launch_spread<float>(const SpreadItem *, int, CellGrid, int, const int *, const void *,
-                                          const float *, Window<float>, const WindowPoly &, float *, int, int, bool,
+                                          const float *, const WindowPoly &, float *, int, int, bool,
                                           cudaStream_t);
 template cudaError_t launch_spread<double>(const SpreadItem *, int, CellGrid, int, const int *, const void *,
-                                           const double *, Window<double>, const WindowPoly &, double *, int, int,
+                                           const double *, const WindowPoly64 &, double *, int, int,
                                            bool, cudaStream_t);
 template <typename real>
 cudaError_t launch_spread_direct(int64_t M, int m, const int *base, const void *frac, const real *q, Window<real> w,
-                                 const WindowPoly &wp, real *grid, real *comp, int pitch, int n_a, bool kahan,
+                                 const WinPoly<real> &wp, real *grid, real *comp, int pitch, int n_a, bool kahan,
                                  cudaStream_t st)
 {
     if (M <= 0)
@@ -1009,13 +1029,12 @@ cudaError_t launch_spread_direct(int64_t M, int m, const int *base, const void *
 template cudaError_t launch_spread_direct<float>(int64_t, int, const int *, const void *, const float *, Window<float>,
                                                  const WindowPoly &, float *, float *, int, int, bool, cudaStream_t);
 template cudaError_t launch_spread_direct<double>(int64_t, int, const int *, const void *, const double *,
-                                                  Window<double>, const WindowPoly &, double *, double *, int, int,
+                                                  Window<double>, const WindowPoly64 &, double *, double *, int, int,
                                                   bool, cudaStream_t);
 
-template cudaError_t launch_interp<float>(int64_t, int, const int *, const void *, Window<float>, const WindowPoly &,
+template cudaError_t launch_interp<float>(int64_t, int, const int *, const void *, const WindowPoly &,
                                           const float *, int, float, float *, float *, bool, cudaStream_t);
-template cudaError_t launch_interp<double>(int64_t, int, const int *, const void *, Window<double>,
-                                           const WindowPoly &, const double *, int, double, double *, double *, bool,
+template cudaError_t launch_interp<double>(int64_t, int, const int *, const void *, const WindowPoly64 &, const double *, int, double, double *, double *, bool,
                                            cudaStream_t);
 
 namespace {
@@ -1049,7 +1068,7 @@ template <typename real> size_t batch_spread_smem(int M2, int max_tile, bool com
 }  // namespace
 
 template <typename real>
-cudaError_t launch_interp_out(int64_t N, int m, const int *base, const void *frac, Window<real> w, const WindowPoly &wp,
+cudaError_t launch_interp_out(int64_t N, int m, const int *base, const void *frac, const WinPoly<real> &wp,
                               const real *grid, int pitch, real n_os, const real *phi_s, const real *grad_s,
                               const real *coinc, const int *perm, double shift, const double *q_sum, double s,
                               void *phi_out, void *H_out, int out_is_f64, cudaStream_t st)
@@ -1059,17 +1078,15 @@ cudaError_t launch_interp_out(int64_t N, int m, const int *base, const void *fra
     return with_width(m, [&](auto mc) {
         constexpr int M2 = decltype(mc)::value;
         k_interp_out<real, M2><<<(unsigned)((N + 255) / 256), 256, 0, st>>>(
-            N, base, (const real2_t<real> *)frac, w, wp, grid, pitch, n_os, phi_s, grad_s, coinc, perm, shift, q_sum, s,
+            N, base, (const real2_t<real> *)frac, wp, grid, pitch, n_os, phi_s, grad_s, coinc, perm, shift, q_sum, s,
             phi_out, H_out, out_is_f64);
         return cudaGetLastError();
     });
 }
-template cudaError_t launch_interp_out<float>(int64_t, int, const int *, const void *, Window<float>,
-                                              const WindowPoly &, const float *, int, float, const float *,
+template cudaError_t launch_interp_out<float>(int64_t, int, const int *, const void *, const WindowPoly &, const float *, int, float, const float *,
                                               const float *, const float *, const int *, double, const double *,
                                               double, void *, void *, int, cudaStream_t);
-template cudaError_t launch_interp_out<double>(int64_t, int, const int *, const void *, Window<double>,
-                                               const WindowPoly &, const double *, int, double, const double *,
+template cudaError_t launch_interp_out<double>(int64_t, int, const int *, const void *, const WindowPoly64 &, const double *, int, double, const double *,
                                                const double *, const double *, const int *, double, const double *,
                                                double, void *, void *, int, cudaStream_t);
 
@@ -1089,7 +1106,7 @@ template <typename real> cudaError_t prepare_batch_spread(int m, int max_tile, b
 
 template <typename real>
 cudaError_t launch_batch_spread(const SpreadItem *items, int n_items, int nrhs, const BatchInst<real> *inst, int m,
-                                int max_tile, Window<real> w, const WindowPoly &wp, bool kahan, cudaStream_t st)
+                                int max_tile, const WinPoly<real> &wp, bool kahan, cudaStream_t st)
 {
     if (n_items <= 0 || nrhs <= 0)
         return cudaSuccess;
@@ -1099,29 +1116,29 @@ cudaError_t launch_batch_spread(const SpreadItem *items, int n_items, int nrhs, 
         const size_t smem = batch_spread_smem<real>(M2, max_tile, comp);
         const dim3 grid((unsigned)n_items, (unsigned)nrhs);
         if (comp)
-            k_batch_spread<real, M2, true><<<grid, kSpreadWarps * 32, smem, st>>>(items, inst, w, wp);
+            k_batch_spread<real, M2, true><<<grid, kSpreadWarps * 32, smem, st>>>(items, inst, wp);
         else
-            k_batch_spread<real, M2, false><<<grid, kSpreadWarps * 32, smem, st>>>(items, inst, w, wp);
+            k_batch_spread<real, M2, false><<<grid, kSpreadWarps * 32, smem, st>>>(items, inst, wp);
         return cudaGetLastError();
     });
 }
 
 template <typename real>
 cudaError_t launch_batch_interp(const BatchInst<real> *inst, BlockMap bm, int blocks, int nrhs, int m,
-                                Window<real> w, const WindowPoly &wp, cudaStream_t st)
+                                const WinPoly<real> &wp, cudaStream_t st)
 {
     if (blocks <= 0 || nrhs <= 0)
         return cudaSuccess;
     return with_width(m, [&](auto mc) {
         constexpr int M2 = decltype(mc)::value;
-        k_batch_interp<real, M2><<<dim3((unsigned)blocks, (unsigned)nrhs), 256, 0, st>>>(inst, bm, w, wp);
+        k_batch_interp<real, M2><<<dim3((unsigned)blocks, (unsigned)nrhs), 256, 0, st>>>(inst, bm, wp);
         return cudaGetLastError();
     });
 }
 
 template <typename real>
 cudaError_t launch_batch_interp_out(const BatchInst<real> *inst, const BatchIO *io, BlockMap bm, int blocks, int nrhs,
-                                    int m, Window<real> w, const WindowPoly &wp, int out_is_f64, cudaStream_t st)
+                                    int m, const WinPoly<real> &wp, int out_is_f64, cudaStream_t st)
 {
     if (blocks <= 0 || nrhs <= 0)
         return cudaSuccess;
@@ -1139,7 +1156,7 @@ cudaError_t launch_batch_interp_out(const BatchInst<real> *inst, const BatchIO *
             default: break;
             }
         }
-        k_batch_interp_out<real, M2><<<dim3((unsigned)blocks, (unsigned)nrhs), 256, 0, st>>>(inst, io, bm, w, wp,
+        k_batch_interp_out<real, M2><<<dim3((unsigned)blocks, (unsigned)nrhs), 256, 0, st>>>(inst, io, bm, wp,
                                                                                            out_is_f64);
         return cudaGetLastError();
     });
@@ -1148,11 +1165,11 @@ cudaError_t launch_batch_interp_out(const BatchInst<real> *inst, const BatchIO *
 #define FS_INST(real)                                                                                          \
     template cudaError_t prepare_batch_spread<real>(int, int, bool);                                           \
     template cudaError_t launch_batch_spread<real>(const SpreadItem *, int, int, const BatchInst<real> *, int, \
-                                                   int, Window<real>, const WindowPoly &, bool, cudaStream_t); \
+                                                   int, const WinPoly<real> &, bool, cudaStream_t); \
     template cudaError_t launch_batch_interp<real>(const BatchInst<real> *, BlockMap, int, int, int,           \
-                                                   Window<real>, const WindowPoly &, cudaStream_t);           \
+                                                   const WinPoly<real> &, cudaStream_t);           \
     template cudaError_t launch_batch_interp_out<real>(const BatchInst<real> *, const BatchIO *, BlockMap, int, \
-                                                       int, int, Window<real>, const WindowPoly &, int,        \
+                                                       int, int, const WinPoly<real> &, int,        \
                                                        cudaStream_t);
 FS_INST(float)
 FS_INST(double)

@@ -64,7 +64,8 @@ struct fs_plan {
     bool kahan = true;
     fs::KernelParams kp{};
     double beta[fs::kMaxP] = {0};
-    fs::WindowPoly wpoly{};               // FP32 window polynomials (per tap)
+    fs::WindowPoly wpoly{};               // window polynomials (per tap) of FP32 plans
+    fs::WindowPoly64 wpoly64{};           // and of FP64 plans
     // device memory
     std::vector<void *> allocs;
     int64_t bytes = 0;
@@ -177,12 +178,22 @@ double bessel_i0(double x);
 // Per-tap polynomial form of the normalised Kaiser-Bessel window (FP32 kernels) for
 // oversampling sigma and half-width m.
 void build_window_poly(double sigma, int m, WindowPoly *wp);
+// The FP64 kernels' (kept per (sigma, m) for the process: a few of at most 4 KB).
+void build_window_poly64(double sigma, int m, WindowPoly64 *wp);
 
 // Validates the parameters and builds the plan (binning, tables, items) on its stream.
 fs_status plan_create_common(const double *src, int64_t M, const double *tgt, int64_t N, int n_grid,
                              double sigma_os, int m, double eps_I, const fs_opts *opts, fs_plan *pl);
 // Waits for the plan's stream and frees everything it owns.
 void plan_destroy(fs_plan *pl);
+
+template <typename real> inline const WinPoly<real> &win_poly(const fs_plan *pl)
+{
+    if constexpr (sizeof(real) == 8)
+        return pl->wpoly64;
+    else
+        return pl->wpoly;
+}
 
 template <typename real> inline Window<real> make_window(double sigma, int m_window)
 {
