@@ -165,6 +165,18 @@ constexpr int kSpread3TileMinPerCell = 300;
 size_t spread3_tile_smem(int cell, int m);
 cudaError_t launch_spread3_tile(const int2 *items, int n_items, int m, int cell, const int *base, const float *frac,
                                 const float *q, const WindowPoly &wp, float *grid, int n_a, cudaStream_t st);
+// FP32 spreading through one shared tile per block with the sources of a cell in the order of their
+// base grid lines (order: run order -> cell order; base, frac: in run order); m = 4 and cells of at
+// most 9 lines, else spread3_runs_smem is 0.  Items: at most kSpread3RunMax sources of one cell.
+constexpr int kSpread3RunMax = 256;
+size_t spread3_runs_smem(int cell, int m);
+cudaError_t launch_spread3_keys(int64_t M, const int *base, CellGrid3 cg, int *key, int *count,
+                                 cudaStream_t st);
+cudaError_t launch_spread3_gather(int64_t M, const int *order, const int *base, const float *frac, int *run_base,
+                                  float *run_frac, cudaStream_t st);
+cudaError_t launch_spread3_runs(const int2 *items, int n_items, int m, int cell, const int *base, const float *frac,
+                                const int *order, const float *q, const WindowPoly &wp, float *grid, int n_a,
+                                cudaStream_t st);
 // acc: add to phi_s / grad_s (the near field stored there first) instead of writing them
 template <typename real>
 cudaError_t launch_interp3(int64_t N, int m, const int *base, const real *frac, Window<real> w, const WindowPoly &wp,

@@ -6,9 +6,10 @@
 //   spreading    g_k = sum_j q_j psi(k1 - u_j1) psi(k2 - u_j2) psi(k3 - u_j3) over the
 //                (2m)^3 grid lines around each source; one warp per source, lanes 0..6m-1
 //                hold the window values of the three coordinates and every lane owns
-//                (2m)^3 / 32 taps.  FP32: warp-private shared tiles of the source cell with a
-//                TwoSum compensation plane, flushed once per item (k_spread3_tile); FP64 (or
-//                tiles too large for shared memory): global atomics (k_spread3);
+//                (2m)^3 / 32 taps.  FP32: shared tiles of the source cell with a TwoSum
+//                compensation plane, flushed once per item (m = 4: k_spread3_runs, a tile per
+//                block; other widths: k_spread3_tile, a tile per warp); FP64 (or tiles too large
+//                for shared memory, or few sources): global atomics (k_spread3);
 //   interpolation phi and grad phi from the same taps, the window and its slope;
 //   near field   q (1/(4 pi r) - T_I(r)) and its gradient for 0 < r < eps_I over the 27
 //                cells around, -q T_I(0) for coincident points.  FP32: warp items over the
@@ -297,6 +298,153 @@ __global__ void __launch_bounds__(kSpread3Warps * 32) k_spread3_tile(const int2 
         if (v != 0.f && gx >= 0 && gx < n_a && gy >= 0 && gy < n_a && gz >= 0 && gz < n_a)
             atomicAdd(grid + ((int64_t)gz * n_a + gy) * n_a + gx, v);
     }
+}
+
+// FP32 spreading at 2m = 8 through one shared tile per block, sources of a cell in the order of their
+// base grid lines (k_spread3_order).  Warp w of the block's four adds, for every source of the item,
+// the taps on the tile planes z = w (mod 4): two of the source's eight, a plane belongs to one warp,
+// and a lane holds one x and two y of both planes, four taps.  So the tile is shared without atomics
+// (21.6 KB for 6-line cells, ten blocks per SM) where a tile per warp left three blocks of four.
+// Consecutive sources with the same base lines (4.5 of them at 970 per 6^3-line cell) have the same
+// taps and are summed in registers, value and TwoSum error, before the tile is read and written.
+// The weights of 128 sources at a time are evaluated a source per thread, coefficients from the
+// constant bank, into shared memory.  Rows are 16 floats, pairs of rows rotated by 8, so that the 8
+// x and 4 y of a warp's access fall on 32 banks.
+// It is bound by the shared-memory pipe and the issue slots (about 140 instructions a source over the
+// four warps, against some 300 and 64 conflicting shared accesses).  Measured: 1.59M quadrature
+// points of the 384,000-tetrahedron cube 1330 -> 421 us; 2^18 points of a ball (41 per cell) 206 us
+// with global atomics, 162 us here.
+constexpr int kSpread3RunThreads = 128;
+constexpr int kSpread3WeightPitch = 25;   // 24 weights a source, odd
+template <int kM2 = 8>
+__global__ void __launch_bounds__(kSpread3RunThreads) k_spread3_runs(const int2 *__restrict__ items,
+                                                                     const int *__restrict__ base,
+                                                                     const float *__restrict__ frac,
+                                                                     const int *__restrict__ order,
+                                                                     const float *__restrict__ q, WindowPoly wp,
+                                                                     int cell, float *__restrict__ grid, int n_a)
+{
+    constexpr int m = kM2 / 2;
+    static_assert(kM2 == 8, "two planes, two rows and one column of taps a lane");
+    extern __shared__ __align__(16) float sm[];
+    const int P = cell + kM2 - 1, plane = P * P * 16;   // words of the value tile; the compensation tile follows
+    float *acc = sm, *wt = sm + 2 * plane;
+    int *bs = reinterpret_cast<int *>(wt + kSpread3RunThreads * kSpread3WeightPitch);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int2 it = items[blockIdx.x];
+    for (int i = threadIdx.x; i < plane / 2; i += kSpread3RunThreads)
+        reinterpret_cast<float4 *>(acc)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int pk0 = base[it.x];
+    const int ox = (b3x(pk0) / cell) * cell - (m - 1), oy = (b3y(pk0) / cell) * cell - (m - 1),
+              oz = (b3z(pk0) / cell) * cell - (m - 1);
+    int run = -1, z0 = 0, at[4] = {0, 0, 0, 0};
+    float2 s0 = f2(0.f), s1 = s0, c0 = s0, c1 = s0;   // planes z0, z0 + 4: rows y, y + 4
+    auto flush = [&]() {
+        const float v[4] = {s0.x, s0.y, s1.x, s1.y}, c[4] = {c0.x, c0.y, c1.x, c1.y};
+        float old[4], cmp[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            old[k] = acc[at[k]];
+            cmp[k] = acc[plane + at[k]];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float t = old[k] + v[k], bb = t - old[k];
+            acc[at[k]] = t;
+            acc[plane + at[k]] = cmp[k] + (((old[k] - (t - bb)) + (v[k] - bb)) + c[k]);
+        }
+        __syncwarp();   // the next run's cells may be other lanes' of this one
+    };
+    for (int first = 0; first < it.y; first += kSpread3RunThreads) {
+        const int n = min(kSpread3RunThreads, it.y - first);
+        __syncthreads();   // the last weights are read (and the tile is zeroed)
+        if (threadIdx.x < n) {
+            const int j = it.x + first + threadIdx.x;
+            float *o = wt + threadIdx.x * kSpread3WeightPitch;
+            const float qj = q[order[j]];
+            bs[threadIdx.x] = base[j];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const float t = frac[3 * (int64_t)j + d] - 0.5f, s = t * t;
+#pragma unroll
+                for (int a = 0; a < m; ++a) {
+                    float e, od;
+                    poly_even_odd<kPolyD>(wp.c[a], s, e, od);
+                    o[8 * d + a] = fmaf(t, od, e) * (d == 0 ? qj : 1.f);
+                    o[8 * d + kM2 - 1 - a] = fmaf(-t, od, e) * (d == 0 ? qj : 1.f);
+                }
+            }
+        }
+        __syncthreads();
+        for (int i = 0; i < n; ++i) {
+            const int pk = bs[i];
+            if (pk != run) {
+                if (run >= 0)
+                    flush();
+                run = pk;
+                const int lz = b3z(pk) - m + 1 - oz, y = b3y(pk) - m + 1 - oy + (lane >> 3),
+                          x = b3x(pk) - m + 1 - ox + (lane & 7);
+                z0 = (warp - lz) & 3;
+                const int r = (lz + z0) * P + y;   // tile row of plane z0 and row y
+                at[0] = r * 16 + ((x + 8 * ((y >> 1) & 1)) & 15);
+                at[1] = at[0] + 4 * 16;
+                at[2] = at[0] + 4 * P * 16;
+                at[3] = at[1] + 4 * P * 16;
+                s0 = s1 = c0 = c1 = f2(0.f);
+            }
+            const float *o = wt + i * kSpread3WeightPitch;
+            const float wx = o[lane & 7];
+            const float2 wxy = make_float2(wx * o[8 + (lane >> 3)], wx * o[12 + (lane >> 3)]);
+            const float2 v0 = mul2(wxy, f2(o[16 + z0])), v1 = mul2(wxy, f2(o[20 + z0]));
+            const float2 t0 = add2(s0, v0), t1 = add2(s1, v1);
+            const float2 b0 = add2(t0, make_float2(-s0.x, -s0.y)), b1 = add2(t1, make_float2(-s1.x, -s1.y));
+            const float2 e0 = add2(add2(s0, fma2(b0, f2(1.f), make_float2(-t0.x, -t0.y))),
+                                   add2(v0, make_float2(-b0.x, -b0.y)));
+            const float2 e1 = add2(add2(s1, fma2(b1, f2(1.f), make_float2(-t1.x, -t1.y))),
+                                   add2(v1, make_float2(-b1.x, -b1.y)));
+            c0 = add2(c0, e0);
+            c1 = add2(c1, e1);
+            s0 = t0;
+            s1 = t1;
+        }
+    }
+    if (run >= 0)
+        flush();
+    __syncthreads();
+    for (int i = threadIdx.x; i < plane; i += kSpread3RunThreads) {
+        const int x = i & 15, r = i >> 4, y = r % P, z = r / P;
+        const float v = acc[i] + acc[plane + i];
+        const int gx = ox + ((x - 8 * ((y >> 1) & 1)) & 15), gy = oy + y, gz = oz + z;
+        if (v != 0.f && gx >= 0 && gx < n_a && gy >= 0 && gy < n_a && gz >= 0 && gz < n_a)
+            atomicAdd(grid + ((int64_t)gz * n_a + gy) * n_a + gx, v);
+    }
+}
+
+// Sort keys of the run order: cell key x cell^3 + base grid lines inside the cell.
+__global__ void k_spread3_keys(const int *__restrict__ base, int64_t M, CellGrid3 cg, int *__restrict__ key,
+                               int *__restrict__ count)
+{
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (j >= M)
+        return;
+    const int pk = base[j], c = cg.cell;
+    const int x = b3x(pk), y = b3y(pk), z = b3z(pk);
+    const int k = cg.key(x / c, y / c, z / c) * (c * c * c) + ((z % c) * c + y % c) * c + x % c;
+    key[j] = k;
+    atomicAdd(&count[k], 1);
+}
+
+__global__ void k_spread3_order(const int *__restrict__ order, int64_t M, const int *__restrict__ base,
+                                const float *__restrict__ frac, int *__restrict__ run_base,
+                                float *__restrict__ run_frac)
+{
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k >= M)
+        return;
+    const int64_t j = order[k];
+    run_base[k] = base[j];
+    for (int d = 0; d < 3; ++d)
+        run_frac[3 * k + d] = frac[3 * j + d];
 }
 
 // phi~ and grad~ phi~ at the targets from the filtered grid (thread per target).
@@ -957,6 +1105,48 @@ size_t spread3_tile_smem(int cell, int m)
     const size_t P = (size_t)cell + 2 * m - 1;
     const size_t bytes = (size_t)kSpread3Warps * 2 * P * P * P * sizeof(float);
     return bytes <= 112 * 1024 ? bytes : 0;
+}
+
+size_t spread3_runs_smem(int cell, int m)
+{
+    const int P = cell + 2 * m - 1;
+    if (m != 4 || P > 16)
+        return 0;
+    return sizeof(float) * (2 * (size_t)P * P * 16 + kSpread3RunThreads * (kSpread3WeightPitch + 1));
+}
+
+cudaError_t launch_spread3_keys(int64_t M, const int *base, CellGrid3 cg, int *key, int *count, cudaStream_t st)
+{
+    if (M <= 0)
+        return cudaSuccess;
+    k_spread3_keys<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(base, M, cg, key, count);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_spread3_gather(int64_t M, const int *order, const int *base, const float *frac, int *run_base,
+                                  float *run_frac, cudaStream_t st)
+{
+    if (M <= 0)
+        return cudaSuccess;
+    k_spread3_order<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(order, M, base, frac, run_base, run_frac);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_spread3_runs(const int2 *items, int n_items, int m, int cell, const int *base, const float *frac,
+                                const int *order, const float *q, const WindowPoly &wp, float *grid, int n_a,
+                                cudaStream_t st)
+{
+    if (n_items <= 0)
+        return cudaSuccess;
+    const size_t smem = spread3_runs_smem(cell, m);
+    if (smem == 0)
+        return cudaErrorInvalidValue;
+    const cudaError_t e = cudaFuncSetAttribute(k_spread3_runs<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess)
+        return e;
+    k_spread3_runs<8><<<(unsigned)n_items, kSpread3RunThreads, smem, st>>>(items, base, frac, order, q, wp, cell, grid,
+                                                                         n_a);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_spread3_tile(const int2 *items, int n_items, int m, int cell, const int *base, const float *frac,

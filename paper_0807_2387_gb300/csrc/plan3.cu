@@ -46,6 +46,9 @@ struct fs3_plan {
     bool spread_tiles = false;
     int2 *spread_items = nullptr;
     int n_spread_items = 0;
+    // the sources in run order (launch_spread3_runs), where that kernel serves the plan
+    int *run_order = nullptr, *run_base = nullptr;
+    float *run_frac = nullptr;
     // source-major near field (many more sources than targets): items over the sources
     bool src_major = false;
     int2 *src_items = nullptr;
@@ -154,6 +157,11 @@ template <typename real> fs_status twiddles3(fs3_plan *pl, int L, void **out)
 }
 
 fs_status near_setup3(fs3_plan *pl);
+
+// Plans spread in run order (launch_spread3_runs) when the occupied cells are many enough to fill the
+// GPU with a block each and hold enough sources to pay for a tile's zeroing and flush.
+constexpr int64_t kScanMost = 4096 * 4096;   // launch_exclusive_scan's range
+constexpr int64_t kSpread3RunMinCells = 304, kSpread3RunMinPerCell = 8;
 
 template <typename real> NearParams<real> make_near3(const fs3_plan *pl)
 {
@@ -372,14 +380,41 @@ fs_status near_setup3(fs3_plan *pl)
         int64_t occupied = 0;
         for (int c = 0; c < n_cells; ++c)
             occupied += sstart[(size_t)(c + 1) * S3] > sstart[(size_t)c * S3];
-        pl->spread_tiles = pl->M >= (int64_t)kSpread3TileMinPerCell * occupied;
+        const int c3 = pl->cg.cell * pl->cg.cell * pl->cg.cell;
+        const bool runs = spread3_runs_smem(pl->cg.cell, pl->m) > 0 && (int64_t)n_cells * c3 <= kScanMost;
+        pl->spread_tiles = pl->M >= (int64_t)kSpread3TileMinPerCell * occupied ||
+                           (runs && occupied >= kSpread3RunMinCells && pl->M >= kSpread3RunMinPerCell * occupied);
+        if (pl->spread_tiles && runs) {
+            const int n_lines = n_cells * c3;
+            int *key = nullptr, *count = nullptr, *first = nullptr, *tmp = nullptr;
+            FS_TRY(pl->alloc(&pl->run_order, pl->M));
+            FS_TRY(pl->alloc(&pl->run_base, pl->M));
+            FS_TRY(pl->alloc(&pl->run_frac, 3 * (size_t)pl->M));
+            FS_TRY(pl->alloc(&key, pl->M));
+            FS_TRY(pl->alloc(&count, n_lines));
+            FS_TRY(pl->alloc(&first, (size_t)n_lines + 1));
+            FS_TRY(pl->alloc(&tmp, (size_t)n_lines / 4096 + 2));
+            FS_CUDA(cudaMemsetAsync(count, 0, sizeof(int) * (size_t)n_lines, st));
+            FS_CUDA(launch_spread3_keys(pl->M, pl->src_base, pl->cg, key, count, st));
+            FS_CUDA(launch_exclusive_scan(count, first, n_lines, tmp, st));
+            FS_CUDA(launch_scatter(key, pl->M, first, pl->run_order, st));
+            FS_CUDA(launch_spread3_gather(pl->M, pl->run_order, pl->src_base, (const float *)pl->src_frac, pl->run_base,
+                                          pl->run_frac, st));
+            FS_CUDA(cudaStreamSynchronize(st));
+            for (int *p : {key, count, first, tmp})
+                pl->release(p);
+        }
     }
     if (pl->spread_tiles) {
+        const int most = pl->run_order ? kSpread3RunMax : kSpread3ItemMax;
         std::vector<int2> sitems;
         for (int c = 0; c < n_cells; ++c) {
-            const int a = sstart[(size_t)c * S3], b = sstart[(size_t)(c + 1) * S3];
-            for (int lo = a; lo < b; lo += kSpread3ItemMax)
-                sitems.push_back(make_int2(lo, std::min(kSpread3ItemMax, b - lo)));
+            const int a = sstart[(size_t)c * S3], count = sstart[(size_t)(c + 1) * S3] - a;
+            const int pieces = (count + most - 1) / most;
+            for (int k = 0; k < pieces; ++k) {
+                const int lo = (int)((int64_t)count * k / pieces), hi = (int)((int64_t)count * (k + 1) / pieces);
+                sitems.push_back(make_int2(a + lo, hi - lo));
+            }
         }
         pl->n_spread_items = (int)sitems.size();
         FS_TRY(pl->alloc(&pl->spread_items, sitems.size()));
@@ -546,7 +581,11 @@ template <typename real> fs_status eval3_t(fs3_plan *pl, void *phi, void *H, fs_
         if (overlap)
             FS_CUDA(cudaEventRecord(pl->ev_fork, st));   // the charges are in
         FS_CUDA(cudaMemsetAsync(pl->grid, 0, cube * sizeof(real), st));
-        if (sizeof(real) == 4 && pl->spread_tiles)
+        if (sizeof(real) == 4 && pl->run_order)
+            FS_CUDA(launch_spread3_runs(pl->spread_items, pl->n_spread_items, pl->m, pl->cg.cell, pl->run_base,
+                                        pl->run_frac, pl->run_order, (const float *)q, pl->wpoly, (float *)pl->grid,
+                                        pl->n_a, st));
+        else if (sizeof(real) == 4 && pl->spread_tiles)
             FS_CUDA(launch_spread3_tile(pl->spread_items, pl->n_spread_items, pl->m, pl->cg.cell, pl->src_base,
                                         (const float *)pl->src_frac, (const float *)q, pl->wpoly, (float *)pl->grid,
                                         pl->n_a, st));

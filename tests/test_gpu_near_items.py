@@ -60,3 +60,26 @@ def test_fp64_pair_functions_by_degree(p):
     phi_o, H_o = F.fast_sum(src, tgt, q, K.make_params(64, 2.0, 5, 5 / 64, p), "nfft")
     for name, a, b in (("phi", phi, phi_o), ("H", H, H_o)):
         assert rel(a, torch.tensor(b)) <= 1e-12, (name, rel(a, torch.tensor(b)))
+
+
+@pytest.mark.parametrize("ns,n,lines", [(18000, 64, 2), (15000, 64, 3), (120000, 64, 2), (120000, 64, 4.4)])
+def test_3d_run_spreading(ns, n, lines):
+    """3D spreading with the sources of a cell in runs of equal base lines: few and many to a run, items of
+    one and several pieces, cells of 4, 6 and 9 lines (the widest tile), against FP64 within the FP32
+    bar of the 3D gates."""
+    import paper_0807_2387_gb300 as fs
+    rng = np.random.default_rng(ns)
+    v = rng.standard_normal((ns, 3))
+    src = 0.25 * v / np.linalg.norm(v, axis=1)[:, None] * rng.random((ns, 1)) ** (1 / 3)
+    src[: ns // 4] = src[0] + rng.uniform(-0.004, 0.004, (ns // 4, 3)) if np.linalg.norm(src[0]) < 0.24 else src[: ns // 4]
+    dev = torch.device("cuda", 0)
+    s, t = torch.tensor(src, device=dev), torch.tensor(src[::3] * 0.97 + 1e-3, device=dev)
+    q = torch.tensor(rng.standard_normal(ns), device=dev)
+    got = {}
+    for precision in (64, 32):
+        plan = fs.FastSum3(s, t, n, 2.0, 4, lines / n, precision=precision, p=3)
+        got[precision] = plan.set_charges(q).field(dtype=torch.float64)
+        plan.sync()
+    assert plan.info["spread_items"] > 0
+    assert rel(got[32][0], got[64][0]) <= 5e-6, rel(got[32][0], got[64][0])
+    assert rel(got[32][1], got[64][1]) <= 5e-6, rel(got[32][1], got[64][1])
