@@ -372,7 +372,7 @@ fs_status near_setup3(fs3_plan *pl)
     // spreading items: the sources of each cell in pieces of at most kSpread3ItemMax, where
     // the tiles fit in shared memory and the occupied cells are dense enough to pay for them
     std::vector<int> sstart;
-    if (spread3_tile_smem(pl->cg.cell, pl->m) > 0 && pl->M > 0) {
+    if ((spread3_tile_smem(pl->cg.cell, pl->m) > 0 || spread3_runs_smem(pl->cg.cell, pl->m) > 0) && pl->M > 0) {
         sstart.resize((size_t)pl->cg.n_keys() + 1);
         FS_CUDA(cudaMemcpyAsync(sstart.data(), pl->src_start, sizeof(int) * sstart.size(), cudaMemcpyDeviceToHost,
                                 st));
@@ -382,7 +382,8 @@ fs_status near_setup3(fs3_plan *pl)
             occupied += sstart[(size_t)(c + 1) * S3] > sstart[(size_t)c * S3];
         const int c3 = pl->cg.cell * pl->cg.cell * pl->cg.cell;
         const bool runs = spread3_runs_smem(pl->cg.cell, pl->m) > 0 && (int64_t)n_cells * c3 <= kScanMost;
-        pl->spread_tiles = pl->M >= (int64_t)kSpread3TileMinPerCell * occupied ||
+        pl->spread_tiles = ((runs || spread3_tile_smem(pl->cg.cell, pl->m) > 0) &&
+                            pl->M >= (int64_t)kSpread3TileMinPerCell * occupied) ||
                            (runs && occupied >= kSpread3RunMinCells && pl->M >= kSpread3RunMinPerCell * occupied);
         if (pl->spread_tiles && runs) {
             const int n_lines = n_cells * c3;
