@@ -126,14 +126,37 @@ struct CellGrid3 {
     __host__ __device__ int n_keys() const { return n_cells() * sub3(); }
 };
 
+// The points of a 3D cell in order: runs of at most kOrderRun points as in CellSplit, each cut into
+// slabs along x, those into strips along y and these into pieces along z, all pieces of nearly one
+// size and at most `cap` points.
+struct CellSplit3 {
+    int pieces, slabs, m;
+    __host__ __device__ CellSplit3(int m_, int cap) : pieces((m_ + cap - 1) / cap), slabs(1), m(m_)
+    {
+        while ((2 * slabs + 1) * (2 * slabs + 1) * (2 * slabs + 1) <= 8 * pieces)   // cube root, rounded
+            ++slabs;
+    }
+    __host__ __device__ int slab_piece(int j) const { return (int)((int64_t)pieces * j / slabs); }
+    __host__ __device__ int slab_first(int j) const { return (int)((int64_t)m * slab_piece(j) / pieces); }
+    // strips of a slab of k pieces and n points: their number, strip i's first piece and point
+    __host__ __device__ static int strips(int k)
+    {
+        int s = 1;
+        while (s * (s + 1) < k)
+            ++s;
+        return s;
+    }
+    __host__ __device__ static int strip_piece(int k, int i) { return (int)((int64_t)k * i / strips(k)); }
+    __host__ __device__ static int strip_first(int k, int n, int i) { return (int)((int64_t)n * strip_piece(k, i) / k); }
+};
+
 // FP32 3D near field (distances in units of eps_I, w = |d|^2 / eps_I^2):
 //   f(w)       = c1 w^(-1/2) - P(w),             c1 = 1 / (4 pi eps_I), P(w) = T_I = sum beta_k w^k
 //   grad_x f   = -(1/eps_I) (c1 w^(-3/2) + 2 P'(w)) d,   d in units of eps_I
 struct Near3Params {
-    float H;               // cell edge / eps_I (>= 1)
-    float reach2;          // squared culling radius, 1 plus a rounding margin
-    float close_reach2;    // squared radius of the close list, 1/8 plus a rounding margin
-    double inv_eps_d;      // 1 / eps_I, for the FP64 differences of close pairs
+    float h;               // cell edge (torus units; dyadic, so cell steps are exact)
+    float reach2;          // squared culling radius, eps_I plus a rounding margin (torus units)
+    float close_reach2;    // squared radius of the close list, eps_I / 8 plus a rounding margin
     float c1;              // 1 / (4 pi eps_I)
     float inv_eps;         // 1 / eps_I
     float beta0;           // T_I(0), removed for coincident pairs (G(0) := 0)
@@ -146,11 +169,14 @@ cudaError_t launch_rmax3(const double *xyz, int64_t n, unsigned long long *out, 
 cudaError_t launch_point_keys3(const double *xyz, int64_t n, double s, int n_os, int window_lo, int n_a, int m,
                                CellGrid3 cg, int *key, int *count, int *status, cudaStream_t st);
 // pos: torus coordinates (n x 3, FP64); frac (n x 3); base: window grid lines packed 10 bits each;
-// pos32 (FP32 path, else null): offsets from the point's cell corner in units of eps_I (times inv_eps)
+// hi, lo (FP32 path, else null): the offset from the point's cell corner as hi + lo (torus units)
 template <typename real>
 cudaError_t launch_gather_points3(const double *xyz, const int *perm, int64_t n, double s, int n_os, int window_lo,
-                                  int n_a, int m, int cell, double inv_eps, double *pos, real *frac, int *base,
-                                  float4 *pos32, int *status, cudaStream_t st);
+                                  int n_a, int m, int cell, double *pos, real *frac, int *base,
+                                  float4 *hi, float4 *lo, int *status, cudaStream_t st);
+// the points of each cell into the order of CellSplit3 (pieces of at most cap)
+cudaError_t launch_cell_order3(const int *start, CellGrid3 cg, int cap, const double *xyz, double s, int n_os,
+                               int window_lo, int n_a, int m, int *perm, cudaStream_t st);
 template <typename real>
 cudaError_t launch_spread3(int64_t M, int m, const int *base, const real *frac, const real *q, Window<real> w,
                            const WindowPoly &wp, real *grid, int n_a, cudaStream_t st);
@@ -186,19 +212,18 @@ cudaError_t launch_interp3(int64_t N, int m, const int *base, const real *frac, 
 cudaError_t launch_near3_f64(int64_t N, const int *tgt_base, const double *tgt_pos, const double *src_pos,
                              const int *src_start, CellGrid3 cg, const double *q, NearParams<double> np,
                              double *phi_s, double *grad_s, cudaStream_t st);
-// FP32 near field over warp items {first target, count <= 64} of one cell each (sorted order);
-// coincident pairs (equal positions) are listed per target in coinc_start / coinc_src
-// (pairs closer than eps_I / 8 refine their difference from the FP64 positions tgt_pos, src_pos)
+// FP32 near field over warp items {first target, count <= lanes} of one cell each (sorted order; lanes 8,
+// 16 or 32); coincident pairs (equal positions) are listed per target in coinc_start / coinc_src
 // (assign: store phi_s / grad_s instead of adding, for the near field run beside the far field)
-cudaError_t launch_near3_warp(const int2 *items, int n_items, const int *tgt_base, const float4 *tgt_p32,
-                              const float4 *src_p32, const double *tgt_pos, const double *src_pos, const float *q,
+cudaError_t launch_near3_warp(const int2 *items, int n_items, int lanes, const int *tgt_base, const float4 *tgt_hi,
+                              const float4 *tgt_lo, const float4 *src_hi, const float4 *src_lo, const float *q,
                               const int *src_start, CellGrid3 cg, const Near3Params &np, const int *coinc_start,
                               const int *coinc_src, float *phi_s, float *grad_s, bool assign, cudaStream_t st);
 // Source-major FP32 near field (many more sources than targets): items of at most 64 sources of
 // one cell; phi and grad phi are added to the targets with atomics, then the coincident pairs'
 // -q T_I(0) when any_coincident
-cudaError_t launch_near3_src(const int2 *items, int n_items, const int *src_base, const float4 *src_p32,
-                             const float4 *tgt_p32, const double *tgt_pos, const double *src_pos, const float *q,
+cudaError_t launch_near3_src(const int2 *items, int n_items, const int *src_base, const float4 *src_hi,
+                             const float4 *src_lo, const float4 *tgt_hi, const float4 *tgt_lo, const float *q,
                              const int *tgt_start, CellGrid3 cg, const Near3Params &np, int64_t N,
                              const int *coinc_start, const int *coinc_src, bool any_coincident, float *phi_s,
                              float *grad_s, cudaStream_t st);

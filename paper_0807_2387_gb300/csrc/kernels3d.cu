@@ -15,12 +15,13 @@
 //                cells around, -q T_I(0) for coincident points.  FP32: warp items over the
 //                targets with candidate lists (k_near3_warp) or, when sources outnumber
 //                targets three to one, over the sources (k_near3_src); pairs closer than
-//                eps_I / 8 take their difference from the FP64 positions.  FP64: thread per
+//                eps_I / 8 take their difference from hi + lo coordinates.  FP64: thread per
 //                target (k_near3_f64);
 //   output       phi = s phi~, H = -s^2 grad~ phi~ (1/r is homogeneous of degree -1).
 // Grid layout: g[z][y][x], x fastest, edge n_a (the active window); a point's base grid
 // line per coordinate is packed into 10 bits each.
 #include "near_warp.cuh"
+#include "sort_shared.cuh"
 
 namespace fs {
 
@@ -88,9 +89,9 @@ __global__ void k_point_keys3(const double *__restrict__ xyz, int64_t n, double 
 
 template <typename real>
 __global__ void k_gather_points3(const double *__restrict__ xyz, const int *__restrict__ perm, int64_t n, double s,
-                                 int n_os, int window_lo, int n_a, int m, int cell, double inv_eps,
+                                 int n_os, int window_lo, int n_a, int m, int cell,
                                  double *__restrict__ pos, real *__restrict__ frac, int *__restrict__ base,
-                                 float4 *__restrict__ pos32, int *status)
+                                 float4 *__restrict__ hi, float4 *__restrict__ lo, int *status)
 {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= n)
@@ -104,14 +105,82 @@ __global__ void k_gather_points3(const double *__restrict__ xyz, const int *__re
         frac[3 * k + d] = (real)fr[d];
     }
     base[k] = b[0] | (b[1] << 10) | (b[2] << 20);
-    if (pos32) {
-        // offset from the lower corner of the point's cell, in units of eps_I
-        float o[3];
+    if (hi) {
+        // offset from the lower corner of the point's cell as hi + lo: 48 bits of at most a cell's width
+        // reach the last place of a torus coordinate
+        float o[3], l[3];
         for (int d = 0; d < 3; ++d) {
             const double corner = (double)((b[d] / cell) * cell + window_lo) / n_os - 0.5;
-            o[d] = (float)((s * xyz[3 * i + d] - corner) * inv_eps);
+            const double off = s * xyz[3 * i + d] - corner;
+            o[d] = (float)off;
+            l[d] = (float)(off - (double)o[d]);
         }
-        pos32[k] = make_float4(o[0], o[1], o[2], 0.f);
+        hi[k] = make_float4(o[0], o[1], o[2], 0.f);
+        lo[k] = make_float4(l[0], l[1], l[2], 0.f);
+    }
+}
+
+// Points of a cell into slabs, strips and pieces (CellSplit3): one block per cell, three sorts of a run.
+constexpr int kOrder3Threads = 256;
+__global__ void __launch_bounds__(kOrder3Threads) k_cell_order3(const int *__restrict__ start, CellGrid3 cg, int cap,
+                                                                const double *__restrict__ xyz, double s, int n_os,
+                                                                int window_lo, int n_a, int m, int *__restrict__ perm)
+{
+    __shared__ unsigned long long key[kOrderRun];
+    __shared__ unsigned q[3][kOrderRun];
+    __shared__ int idx[kOrderRun];
+    const int S3 = cg.sub3();
+    const int a = start[(int64_t)blockIdx.x * S3], count = start[(int64_t)(blockIdx.x + 1) * S3] - a;
+    if (count <= cap)
+        return;
+    int ignored = 0;
+    for (int r = 0; r < CellSplit::runs(count); ++r) {
+        const int first = a + CellSplit::run_first(count, r), n = a + CellSplit::run_first(count, r + 1) - first;
+        const CellSplit3 split(n, cap);
+        int n2 = 2;
+        while (n2 < n)
+            n2 <<= 1;
+        __syncthreads();   // the previous run's keys are read
+        for (int t = threadIdx.x; t < n2; t += blockDim.x) {
+            unsigned long long k = ~0ull;
+            if (t < n) {
+                const int i = perm[first + t];
+                for (int d = 0; d < 3; ++d) {
+                    double f;
+                    const int b = grid_line3(xyz[3 * (int64_t)i + d], s, n_os, window_lo, m, n_a, f, &ignored);
+                    q[d][t] = (unsigned)((((double)(b % cg.cell) + f) / cg.cell) * 4194304.0);   // 22 bits
+                }
+                idx[t] = i;
+                k = ((unsigned long long)q[0][t] << 16) | (unsigned)t;
+            }
+            key[t] = k;
+        }
+        __syncthreads();
+        // a pass per axis: sort, then number each point's slab (strip) and key it by the next axis
+        for (int axis = 0; axis < 3; ++axis) {
+            sort_shared(key, n2);
+            if (axis == 2)
+                break;
+            for (int t = threadIdx.x; t < n; t += blockDim.x) {
+                int slab = 0;
+                while (t >= split.slab_first(slab + 1))
+                    ++slab;
+                int part = slab << 8;
+                if (axis == 1) {
+                    const int k = split.slab_piece(slab + 1) - split.slab_piece(slab), t0 = split.slab_first(slab);
+                    const int len = split.slab_first(slab + 1) - t0;
+                    int strip = 0;
+                    while (t - t0 >= CellSplit3::strip_first(k, len, strip + 1))
+                        ++strip;
+                    part |= strip;
+                }
+                const unsigned slot = (unsigned)key[t] & 0xffffu;
+                key[t] = ((unsigned long long)part << 48) | ((unsigned long long)q[axis + 1][slot] << 16) | slot;
+            }
+            __syncthreads();
+        }
+        for (int t = threadIdx.x; t < n; t += blockDim.x)
+            perm[first + t] = idx[(unsigned)key[t] & 0xffffu];
     }
 }
 
@@ -563,21 +632,21 @@ __global__ void __launch_bounds__(256) k_near3_f64(int64_t N, const int *__restr
 
 // ---- FP32 near field: warp items, candidate lists, packed pairs
 //
-// A warp takes one item, at most 64 consecutive targets of one cell (two per lane; Morton
-// sub-cell order keeps them compact) and forms their bounding box.  Coordinates are offsets
-// from the target cell's corner in units of eps_I.  For each of the 27 cells around (skipping
-// cells beyond the culling radius of the box), the lanes read 32 sources at a time, keep those
-// within the culling radius of the box (ballot) and append them to the warp's candidate list
-// in shared memory, pre-broadcast as (x, x, y, y), (z, z, q, q).  The list is evaluated by
-// all lanes against both of their targets as packed FP32 pairs: no branch, pairs outside
-// 0 < w < 1 get charge 0 (an integer compare of the bits of w: 0 < w < 1 iff
-// bits(w) - 1 < bits(1) - 1 as unsigned), and coincident pairs (w = 0) are accounted from the
-// per-target lists built with the plan.  Sources within eps_I / 8 of the box go to a second
-// list, whose pairs closer than eps_I / 8 take their difference from the FP64 positions.
+// As the 2D traversal (near_warp.cuh): a warp takes a piece of a cell, at most 8, 16 or 32 targets, one
+// per lane (the 32 / lanes groups of the warp take different candidates); reads the sources of the
+// 27 cells around 32 at a time, keeps those within eps_I of the piece's box, and appends them to
+// lists in shared memory, negated in the piece's frame and in units of eps_I, which all lanes
+// evaluate two candidates to a packed operation.  Pairs beyond eps_I get charge 0.  Sources within
+// eps_I / 8 of the box go to a second list with hi + lo coordinates, whose differences keep full FP32
+// relative accuracy however small they are, without the FP64 differences taken before (a 64th of
+// the FP32 rate: half of the source-major kernel's time).  Coincident pairs (difference 0) get charge 0
+// and are accounted from the per-target lists built with the plan.
+// Measured, 2^18 points of a ball (41 per cell, p = 3): 380 us with items of 64 targets (two per lane,
+// the box a whole cell: 0.13 of the pair slots useful) and FP64 close pairs, 249 us here; list building
+// is the larger part of it.
 constexpr int kNear3Warps = 4;
-constexpr int kNear3Cap = 256;        // far candidate entries per warp (32 B each)
-constexpr int kNear3CloseCap = 64;    // close candidate entries per warp (32 B + index)
-constexpr int kNear3Unroll = 2;
+constexpr int kNear3Cap = 256;        // far candidates per warp
+constexpr int kNear3CloseCap = 64;    // close candidates per warp
 
 __device__ __forceinline__ float rsqrt_approx(float x)
 {
@@ -586,390 +655,483 @@ __device__ __forceinline__ float rsqrt_approx(float x)
     return y;
 }
 
-// q if 0 < w < 1, else 0
-__device__ __forceinline__ float in_range(float w, float q)
+// w = min(r^2, 1): pairs beyond eps_I land on 1, where near3_pair drops their charge
+__device__ __forceinline__ float2 near3_w(float2 dx, float2 dy, float2 dz)
 {
-    return (__float_as_uint(w) - 1u) < 0x3f7fffffu ? q : 0.f;
+    const float2 r = fma2(dy, dy, mul2(dx, dx));
+    return make_float2(__saturatef(fmaf(dz.x, dz.x, r.x)), __saturatef(fmaf(dz.y, dz.y, r.y)));
 }
 
-// The packed pair arithmetic for one candidate at (w, dx, dy, dz) (units of eps_I).
+struct Near3Sums {
+    float2 phi, gx, gy, gz;
+};
+
+// The packed pair arithmetic of two candidates at (w, dx, dy, dz) (units of eps_I), 0 < w <= 1.
 template <int P>
 __device__ __forceinline__ void near3_pair(const Near3Params &np, float2 w, float2 dx, float2 dy, float2 dz,
-                                           float2 qq, float2 &phi, float2 &gx, float2 &gy, float2 &gz)
+                                           float2 qq, Near3Sums &a)
 {
-    const float2 c1 = make_float2(np.c1, np.c1);
-    const float2 qe = make_float2(in_range(w.x, qq.x), in_range(w.y, qq.y));
-    // w = 0 only for coincident pairs (charge 0 here): floor w so that w^-3/2 stays finite
-    // (distinct points give w >= ~1e-14, far above the floor)
-    const float2 rs = make_float2(rsqrt_approx(fmaxf(w.x, 1e-20f)), rsqrt_approx(fmaxf(w.y, 1e-20f)));
-    float2 t = make_float2(np.nbeta[P - 1], np.nbeta[P - 1]);
+    const float2 c1 = f2(np.c1);
+    const float2 qe = make_float2(w.x < 1.f ? qq.x : 0.f, w.y < 1.f ? qq.y : 0.f);
+    const float2 rs = make_float2(rsqrt_approx(w.x), rsqrt_approx(w.y));
+    float2 t = f2(np.nbeta[P - 1]);
 #pragma unroll
     for (int i = P - 2; i >= 0; --i)
-        t = __ffma2_rn(t, w, make_float2(np.nbeta[i], np.nbeta[i]));
-    float2 u = make_float2(0.f, 0.f);
+        t = fma2(t, w, f2(np.nbeta[i]));
+    float2 u = f2(0.f);
     if constexpr (P >= 2) {
-        u = make_float2(np.dbeta2[P - 2], np.dbeta2[P - 2]);
+        u = f2(np.dbeta2[P - 2]);
 #pragma unroll
         for (int i = P - 3; i >= 0; --i)
-            u = __ffma2_rn(u, w, make_float2(np.dbeta2[i], np.dbeta2[i]));
+            u = fma2(u, w, f2(np.dbeta2[i]));
     }
-    const float2 val = __ffma2_rn(c1, rs, t);                                  // c1 w^-1/2 - P(w)
-    const float2 gc = __ffma2_rn(c1, __fmul2_rn(__fmul2_rn(rs, rs), rs), u);   // c1 w^-3/2 + 2 P'(w)
-    phi = __ffma2_rn(qe, val, phi);
-    const float2 qc = __fmul2_rn(qe, gc);
-    gx = __ffma2_rn(qc, dx, gx);
-    gy = __ffma2_rn(qc, dy, gy);
-    gz = __ffma2_rn(qc, dz, gz);
+    const float2 val = fma2(c1, rs, t);                            // c1 w^-1/2 - P(w)
+    const float2 gc = fma2(c1, mul2(mul2(rs, rs), rs), u);         // c1 w^-3/2 + 2 P'(w)
+    a.phi = fma2(qe, val, a.phi);
+    const float2 qc = mul2(qe, gc);
+    a.gx = fma2(qc, dx, a.gx);
+    a.gy = fma2(qc, dy, a.gy);
+    a.gz = fma2(qc, dz, a.gz);
 }
 
-// Far candidates: no pair can be closer than eps_I / 8.
+// A pair that may coincide (w = 0): charge 0 and a finite w (the per-target lists account for it).
 template <int P>
-__device__ __forceinline__ void near3_eval(const float4 (*list)[2], int n, float2 X, float2 Y, float2 Z,
-                                           const Near3Params &np, float2 &phi, float2 &gx, float2 &gy, float2 &gz)
+__device__ __forceinline__ void near3_pair_close(const Near3Params &np, float2 dx, float2 dy, float2 dz, float2 qq,
+                                                 Near3Sums &a)
 {
-#pragma unroll kNear3Unroll
-    for (int e = 0; e < n; ++e) {
-        const float4 A = list[e][0], B = list[e][1];
-        const float2 dx = __fadd2_rn(X, make_float2(-A.x, -A.y));
-        const float2 dy = __fadd2_rn(Y, make_float2(-A.z, -A.w));
-        const float2 dz = __fadd2_rn(Z, make_float2(-B.x, -B.y));
-        const float2 w = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-        near3_pair<P>(np, w, dx, dy, dz, make_float2(B.z, B.w), phi, gx, gy, gz);
-    }
+    float2 w = near3_w(dx, dy, dz);
+    if (w.x == 0.f)
+        qq.x = 0.f;
+    if (w.y == 0.f)
+        qq.y = 0.f;
+    w.x = fmaxf(w.x, 1e-20f);   // (w^-3/2 stays finite; distinct points give w >= ~1e-14)
+    w.y = fmaxf(w.y, 1e-20f);
+    near3_pair<P>(np, w, dx, dy, dz, qq, a);
 }
 
-// Close candidates (within eps_I / 8 of the box): pairs closer than eps_I / 8 take their
-// difference from the FP64 positions (the FP32 cell offsets lose relative precision as r
-// shrinks, and such pairs dominate H), then the same arithmetic.
+struct Near3List {
+    float x[kNear3Cap], y[kNear3Cap], z[kNear3Cap], q[kNear3Cap];
+    float cx[kNear3CloseCap], cy[kNear3CloseCap], cz[kNear3CloseCap], cq[kNear3CloseCap];
+    float lx[kNear3CloseCap], ly[kNear3CloseCap], lz[kNear3CloseCap];
+    __device__ __forceinline__ void put(int at, float px, float py, float pz, float pq)
+    {
+        x[at] = px;
+        y[at] = py;
+        z[at] = pz;
+        q[at] = pq;
+    }
+    __device__ __forceinline__ void put_close(int at, float3 p, float3 l, float pq)
+    {
+        cx[at] = p.x;
+        cy[at] = p.y;
+        cz[at] = p.z;
+        lx[at] = l.x;
+        ly[at] = l.y;
+        lz[at] = l.z;
+        cq[at] = pq;
+    }
+    // pads n entries to a multiple of `unit` (at most 32); returns the padded count
+    __device__ __forceinline__ int pad(int n, int unit, int lane)
+    {
+        const int full = (n + unit - 1) & ~(unit - 1);
+        if (n + lane < full)
+            put(n + lane, kPadPos, kPadPos, kPadPos, 0.f);
+        return full;
+    }
+    __device__ __forceinline__ int pad_close(int n, int unit, int lane)
+    {
+        const int full = (n + unit - 1) & ~(unit - 1);
+        if (n + lane < full)
+            put_close(n + lane, make_float3(kPadPos, kPadPos, kPadPos), make_float3(0.f, 0.f, 0.f), 0.f);
+        return full;
+    }
+};
+
+__device__ __forceinline__ float4 four(const float *p, int e) { return *reinterpret_cast<const float4 *>(p + 4 * e); }
+__device__ __forceinline__ float2 half_of(float4 v, int h) { return h ? make_float2(v.z, v.w) : make_float2(v.x, v.y); }
+
+// n candidates (a multiple of 4 x groups); group g takes every groups-th four of them.
 template <int P>
-__device__ __forceinline__ void near3_eval_close(const float4 (*list)[2], const int *jlist, int n, float2 X,
-                                                 float2 Y, float2 Z, const int (&kt)[2],
-                                                 const double *__restrict__ tgt_pos,
-                                                 const double *__restrict__ src_pos, const Near3Params &np,
-                                                 float2 &phi, float2 &gx, float2 &gy, float2 &gz)
+__device__ __forceinline__ void near3_eval(const Near3List &L, int n, int g, int groups, float3 X,
+                                           const Near3Params &np, Near3Sums &a)
 {
-    for (int e = 0; e < n; ++e) {
-        const float4 A = list[e][0], B = list[e][1];
-        float2 dx = __fadd2_rn(X, make_float2(-A.x, -A.y));
-        float2 dy = __fadd2_rn(Y, make_float2(-A.z, -A.w));
-        float2 dz = __fadd2_rn(Z, make_float2(-B.x, -B.y));
-        float2 w = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-        const bool c0 = w.x < 1.f / 64.f, c1 = w.y < 1.f / 64.f;
-        if (__any_sync(0xffffffffu, c0 || c1)) {
-            const int j = jlist[e];
+#pragma unroll 2
+    for (int e = g; e < n >> 2; e += groups) {
+        const float4 x = four(L.x, e), y = four(L.y, e), z = four(L.z, e), q = four(L.q, e);
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                if (t == 0 ? c0 : c1) {
-                    const int64_t k = kt[t];
-                    const float ex = (float)((tgt_pos[3 * k] - src_pos[3 * (int64_t)j]) * np.inv_eps_d);
-                    const float ey = (float)((tgt_pos[3 * k + 1] - src_pos[3 * (int64_t)j + 1]) * np.inv_eps_d);
-                    const float ez = (float)((tgt_pos[3 * k + 2] - src_pos[3 * (int64_t)j + 2]) * np.inv_eps_d);
-                    const float e2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
-                    if (t == 0) {
-                        dx.x = ex;
-                        dy.x = ey;
-                        dz.x = ez;
-                        w.x = e2;
-                    } else {
-                        dx.y = ex;
-                        dy.y = ey;
-                        dz.y = ez;
-                        w.y = e2;
-                    }
-                }
-            }
+        for (int h = 0; h < 2; ++h) {
+            const float2 dx = add2(f2(X.x), half_of(x, h)), dy = add2(f2(X.y), half_of(y, h)),
+                         dz = add2(f2(X.z), half_of(z, h));
+            near3_pair<P>(np, near3_w(dx, dy, dz), dx, dy, dz, half_of(q, h), a);
         }
-        near3_pair<P>(np, w, dx, dy, dz, make_float2(B.z, B.w), phi, gx, gy, gz);
     }
 }
 
 template <int P>
-__global__ void __launch_bounds__(kNear3Warps * 32) k_near3_warp(const int2 *__restrict__ items, int n_items,
-                                                                 const int *__restrict__ tgt_base,
-                                                                 const float4 *__restrict__ tgt_p32,
-                                                                 const float4 *__restrict__ src_p32,
-                                                                 const double *__restrict__ tgt_pos,
-                                                                 const double *__restrict__ src_pos,
-                                                                 const float *__restrict__ q,
-                                                                 const int *__restrict__ src_start, CellGrid3 cg,
-                                                                 Near3Params np, const int *__restrict__ coinc_start,
-                                                                 const int *__restrict__ coinc_src,
-                                                                 float *__restrict__ phi_s, float *__restrict__ grad_s,
-                                                                 bool assign)
+__device__ __forceinline__ void near3_eval_close(const Near3List &L, int n, int g, int groups, float3 X, float3 XL,
+                                                 const Near3Params &np, Near3Sums &a)
 {
-    __shared__ float4 lists[kNear3Warps][kNear3Cap][2];
-    __shared__ float4 clists[kNear3Warps][kNear3CloseCap][2];
-    __shared__ int cjs[kNear3Warps][kNear3CloseCap];
+    const float2 ie = f2(np.inv_eps);
+    for (int e = g; e < n >> 2; e += groups) {
+        const float4 x = four(L.cx, e), y = four(L.cy, e), z = four(L.cz, e), q = four(L.cq, e);
+        const float4 lx = four(L.lx, e), ly = four(L.ly, e), lz = four(L.lz, e);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 dx = mul2(add2(add2(f2(X.x), half_of(x, h)), add2(f2(XL.x), half_of(lx, h))), ie);
+            const float2 dy = mul2(add2(add2(f2(X.y), half_of(y, h)), add2(f2(XL.y), half_of(ly, h))), ie);
+            const float2 dz = mul2(add2(add2(f2(X.z), half_of(z, h)), add2(f2(XL.z), half_of(lz, h))), ie);
+            near3_pair_close<P>(np, dx, dy, dz, half_of(q, h), a);
+        }
+    }
+}
+
+// The box of a warp's points (offsets from their cell's corner).
+struct Box3 {
+    float x0, x1, y0, y1, z0, z1;
+    __device__ __forceinline__ void of(float4 a, float4 b)
+    {
+        x0 = warp_min(fminf(a.x, b.x));
+        x1 = warp_max(fmaxf(a.x, b.x));
+        y0 = warp_min(fminf(a.y, b.y));
+        y1 = warp_max(fmaxf(a.y, b.y));
+        z0 = warp_min(fminf(a.z, b.z));
+        z1 = warp_max(fmaxf(a.z, b.z));
+    }
+    // squared distance of the negated point (-fx, -fy, -fz)
+    __device__ __forceinline__ float gap2(float fx, float fy, float fz) const
+    {
+        const float gx = fmaxf(0.f, fmaxf(-fx - x1, x0 + fx)), gy = fmaxf(0.f, fmaxf(-fy - y1, y0 + fy)),
+                    gz = fmaxf(0.f, fmaxf(-fz - z1, z0 + fz));
+        return gx * gx + gy * gy + gz * gz;
+    }
+};
+
+// Walks the other side's points of the 27 cells around cell (c1, c2, c3) that are within reach of the
+// box, in chunks of 32, the next chunk's record loaded while the current one is used.  The three
+// cells of a row along z follow each other in memory and are walked as one range (at 41 points a
+// cell four chunks where three cells take six).
+struct Chunks3 {
+    int c_j0, c_j1, c_b1, c_b2, jb, j1, b1, b2;   // a row's range and the first points of its second and third cell
+    float c_ox, c_oy, h;
+    unsigned rows;
+    // the chunk loaded ahead
+    int j;
+    bool in;
+    float ox, oy, oz;   // step from the point's cell to the item's frame
+    float4 p;
+    float v;
+    __device__ __forceinline__ Chunks3(int lane, int packed, const CellGrid3 &cg, const Near3Params &np,
+                                       const Box3 &box, const int *__restrict__ start)
+    {
+        const int e1 = b3x(packed) / cg.cell - 1 + lane / 3, e2 = b3y(packed) / cg.cell - 1 + lane % 3,
+                  e3 = b3z(packed) / cg.cell;
+        h = np.h;
+        c_ox = (float)(1 - lane / 3) * h;
+        c_oy = (float)(1 - lane % 3) * h;
+        const float gx = fmaxf(0.f, fmaxf(-c_ox - box.x1, box.x0 - (h - c_ox))),
+                    gy = fmaxf(0.f, fmaxf(-c_oy - box.y1, box.y0 - (h - c_oy)));
+        const float left = np.reach2 - gx * gx - gy * gy;   // squared reach along z
+        c_j0 = c_j1 = c_b1 = c_b2 = 0;
+        if (lane < 9 && e1 >= 0 && e1 < cg.n_c && e2 >= 0 && e2 < cg.n_c && left >= 0.f) {
+            const bool below = e3 > 0 && box.z0 * box.z0 <= left,
+                       above = e3 + 1 < cg.n_c && (h - box.z1) * (h - box.z1) <= left;
+            const int64_t key = (int64_t)cg.key(e1, e2, e3) * cg.sub3();
+            c_b1 = start[key];
+            c_b2 = start[key + cg.sub3()];
+            c_j0 = below ? start[key - cg.sub3()] : c_b1;
+            c_j1 = above ? start[key + 2 * cg.sub3()] : c_b2;
+        }
+        rows = __ballot_sync(0xffffffffu, c_j0 < c_j1);
+        jb = j1 = j = b1 = b2 = 0;
+        in = false;
+        ox = oy = oz = v = 0.f;
+        p = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __device__ __forceinline__ bool next(int lane, const float4 *__restrict__ hi, const float *__restrict__ val)
+    {
+        if (jb >= j1) {
+            if (!rows)
+                return false;
+            const int c = __ffs(rows) - 1;
+            rows &= rows - 1;
+            jb = __shfl_sync(0xffffffffu, c_j0, c);
+            j1 = __shfl_sync(0xffffffffu, c_j1, c);
+            b1 = __shfl_sync(0xffffffffu, c_b1, c);
+            b2 = __shfl_sync(0xffffffffu, c_b2, c);
+            ox = __shfl_sync(0xffffffffu, c_ox, c);
+            oy = __shfl_sync(0xffffffffu, c_oy, c);
+        }
+        j = jb + lane;
+        in = j < j1;
+        oz = j < b1 ? h : (j < b2 ? 0.f : -h);
+        jb += 32;
+        if (in) {
+            p = __ldg(hi + j);
+            if (val)
+                v = __ldg(val + j);
+        }
+        return true;
+    }
+};
+
+// off - hi - lo as hi + lo (TwoSum of off and -hi), d = off - hi given.
+__device__ __forceinline__ float neg_lo(float off, float hi, float lo, float d)
+{
+    const float b = d - off;
+    return ((off - (d - b)) + (-hi - b)) - lo;
+}
+
+template <int P>
+__global__ void __launch_bounds__(kNear3Warps * 32, 6) k_near3_warp(const int2 *__restrict__ items, int n_items,
+                                                                    int lanes, const int *__restrict__ tgt_base,
+                                                                    const float4 *__restrict__ tgt_hi,
+                                                                    const float4 *__restrict__ tgt_lo,
+                                                                    const float4 *__restrict__ src_hi,
+                                                                    const float4 *__restrict__ src_lo,
+                                                                    const float *__restrict__ q,
+                                                                    const int *__restrict__ src_start, CellGrid3 cg,
+                                                                    Near3Params np, const int *__restrict__ coinc_start,
+                                                                    const int *__restrict__ coinc_src,
+                                                                    float *__restrict__ phi_s,
+                                                                    float *__restrict__ grad_s, bool assign)
+{
+    __shared__ __align__(16) Near3List lists[kNear3Warps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int item = blockIdx.x * kNear3Warps + warp;
     if (item >= n_items)
         return;   // whole warp; the kernel has no block-wide barrier
-    float4(*list)[2] = lists[warp];
-    float4(*clist)[2] = clists[warp];
-    int *cj = cjs[warp];
+    Near3List &L = lists[warp];
     const int2 it = items[item];
-    const int first = it.x, count = it.y;
-    const bool va = lane < count, vb = lane + 32 < count;
-    const int ka = va ? first + lane : first, kb = vb ? first + 32 + lane : ka;
-    const float4 pa = tgt_p32[ka], pb = tgt_p32[kb];
-    const float2 X = make_float2(pa.x, pb.x), Y = make_float2(pa.y, pb.y), Z = make_float2(pa.z, pb.z);
-    const int kt[2] = {ka, kb};
-    const float lox = warp_min(fminf(pa.x, pb.x)), hix = warp_max(fmaxf(pa.x, pb.x));
-    const float loy = warp_min(fminf(pa.y, pb.y)), hiy = warp_max(fmaxf(pa.y, pb.y));
-    const float loz = warp_min(fminf(pa.z, pb.z)), hiz = warp_max(fmaxf(pa.z, pb.z));
-    const int packed = tgt_base[first];
-    const int c1 = b3x(packed) / cg.cell, c2 = b3y(packed) / cg.cell, c3 = b3z(packed) / cg.cell;
-    const int S3 = cg.sub3();
-    float2 phi = make_float2(0.f, 0.f), gx = phi, gy = phi, gz = phi;
-    int n = 0, nc = 0;
+    const int groups = 32 / lanes, slot = lane & (lanes - 1), g = lane / lanes;
+    const bool valid = slot < it.y;
+    const int k = it.x + (valid ? slot : 0);
+    const float4 h = tgt_hi[k], l = tgt_lo[k];
+    Box3 box;
+    box.of(h, h);
+    const float ie = np.inv_eps;
+    const float3 X = valid ? make_float3(h.x, h.y, h.z) : make_float3(1e6f, 1e6f, 1e6f);   // idle: beyond eps_I of all
+    const float3 XL = make_float3(l.x, l.y, l.z), XS = make_float3(X.x * ie, X.y * ie, X.z * ie);
     const unsigned below = (1u << lane) - 1u;
-    for (int e1 = max(c1 - 1, 0); e1 <= min(c1 + 1, cg.n_c - 1); ++e1) {
-        const float o1 = (float)(e1 - c1) * np.H;
-        const float bx = fmaxf(0.f, fmaxf(o1 - hix, lox - (o1 + np.H)));
-        for (int e2 = max(c2 - 1, 0); e2 <= min(c2 + 1, cg.n_c - 1); ++e2) {
-            const float o2 = (float)(e2 - c2) * np.H;
-            const float by = fmaxf(0.f, fmaxf(o2 - hiy, loy - (o2 + np.H)));
-            for (int e3 = max(c3 - 1, 0); e3 <= min(c3 + 1, cg.n_c - 1); ++e3) {
-                const float o3 = (float)(e3 - c3) * np.H;
-                const float bz = fmaxf(0.f, fmaxf(o3 - hiz, loz - (o3 + np.H)));
-                if (bx * bx + by * by + bz * bz >= np.reach2)
-                    continue;   // the whole cell is beyond reach of the box (warp-uniform)
-                const int key = cg.key(e1, e2, e3);
-                const int end = src_start[(key + 1) * S3];
-                for (int j0 = src_start[key * S3]; j0 < end; j0 += 32) {
-                    const int j = j0 + lane;
-                    bool keep = false, close = false;
-                    float sx = 0.f, sy = 0.f, sz = 0.f, qj = 0.f;
-                    if (j < end) {
-                        const float4 sp = src_p32[j];
-                        qj = q[j];
-                        sx = sp.x + o1;
-                        sy = sp.y + o2;
-                        sz = sp.z + o3;
-                        const float dx = fmaxf(0.f, fmaxf(sx - hix, lox - sx));
-                        const float dy = fmaxf(0.f, fmaxf(sy - hiy, loy - sy));
-                        const float dz = fmaxf(0.f, fmaxf(sz - hiz, loz - sz));
-                        const float g2 = dx * dx + dy * dy + dz * dz;
-                        keep = g2 < np.reach2;
-                        close = g2 < np.close_reach2;
-                    }
-                    const unsigned mf = __ballot_sync(0xffffffffu, keep && !close);
-                    const unsigned mc = __ballot_sync(0xffffffffu, close);
-                    if (keep && !close) {
-                        const int at = n + __popc(mf & below);
-                        list[at][0] = make_float4(sx, sx, sy, sy);
-                        list[at][1] = make_float4(sz, sz, qj, qj);
-                    }
-                    if (close) {
-                        const int at = nc + __popc(mc & below);
-                        clist[at][0] = make_float4(sx, sx, sy, sy);
-                        clist[at][1] = make_float4(sz, sz, qj, qj);
-                        cj[at] = j;
-                    }
-                    n += __popc(mf);
-                    nc += __popc(mc);
-                    if (n > kNear3Cap - 32) {
-                        __syncwarp();
-                        near3_eval<P>(list, n, X, Y, Z, np, phi, gx, gy, gz);
-                        n = 0;
-                        __syncwarp();
-                    }
-                    if (nc > kNear3CloseCap - 32) {
-                        __syncwarp();
-                        near3_eval_close<P>(clist, cj, nc, X, Y, Z, kt, tgt_pos, src_pos, np, phi, gx, gy, gz);
-                        nc = 0;
-                        __syncwarp();
-                    }
-                }
+    Near3Sums a;
+    a.phi = a.gx = a.gy = a.gz = f2(0.f);
+    int nf = 0, nc = 0;
+    Chunks3 ch(lane, tgt_base[it.x], cg, np, box, src_start);
+    bool more = ch.next(lane, src_hi, q);
+    while (more) {
+        const float4 y = ch.p;
+        const float qj = ch.v, ox = ch.ox, oy = ch.oy, oz = ch.oz;
+        const int j = ch.j;
+        const bool in = ch.in;
+        more = ch.next(lane, src_hi, q);
+        const float fx = ox - y.x, fy = oy - y.y, fz = oz - y.z;   // -(source in the item's frame)
+        const float g2 = in ? box.gap2(fx, fy, fz) : 3e38f;
+        const bool keep = g2 <= np.reach2, close = g2 <= np.close_reach2;
+        const unsigned mc = __ballot_sync(0xffffffffu, close), mf = __ballot_sync(0xffffffffu, keep) & ~mc;
+        if (keep && !close)
+            L.put(nf + __popc(mf & below), fx * ie, fy * ie, fz * ie, qj);
+        nf += __popc(mf);
+        if (nf > kNear3Cap - 32) {
+            nf = L.pad(nf, 4 * groups, lane);
+            __syncwarp();
+            near3_eval<P>(L, nf, g, groups, XS, np, a);
+            nf = 0;
+            __syncwarp();
+        }
+        if (mc) {
+            if (close) {
+                const float4 yl = __ldg(src_lo + j);
+                L.put_close(nc + __popc(mc & below), make_float3(fx, fy, fz),
+                            make_float3(neg_lo(ox, y.x, yl.x, fx), neg_lo(oy, y.y, yl.y, fy), neg_lo(oz, y.z, yl.z, fz)),
+                            qj);
+            }
+            nc += __popc(mc);
+            if (nc > kNear3CloseCap - 32) {
+                nc = L.pad_close(nc, 4 * groups, lane);
+                __syncwarp();
+                near3_eval_close<P>(L, nc, g, groups, X, XL, np, a);
+                nc = 0;
+                __syncwarp();
             }
         }
     }
+    nf = L.pad(nf, 4 * groups, lane);
+    nc = L.pad_close(nc, 4 * groups, lane);
     __syncwarp();
-    near3_eval<P>(list, n, X, Y, Z, np, phi, gx, gy, gz);
-    near3_eval_close<P>(clist, cj, nc, X, Y, Z, kt, tgt_pos, src_pos, np, phi, gx, gy, gz);
-    // coincident pairs: G(0) := 0, so only -q T_I(0) remains of the far field's self term
-    const bool vt[2] = {va, vb};
-    const float ph[2] = {phi.x, phi.y}, ggx[2] = {gx.x, gx.y}, ggy[2] = {gy.x, gy.y}, ggz[2] = {gz.x, gz.y};
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        if (!vt[t])
-            continue;
-        const int k = kt[t];
-        float self = 0.f;
-        for (int c = coinc_start[k]; c < coinc_start[k + 1]; ++c)
-            self += q[coinc_src[c]];
-        const float p0 = assign ? 0.f : phi_s[k];
-        phi_s[k] = p0 + (ph[t] - np.beta0 * self);
-        grad_s[3 * k] = (assign ? 0.f : grad_s[3 * k]) - np.inv_eps * ggx[t];
-        grad_s[3 * k + 1] = (assign ? 0.f : grad_s[3 * k + 1]) - np.inv_eps * ggy[t];
-        grad_s[3 * k + 2] = (assign ? 0.f : grad_s[3 * k + 2]) - np.inv_eps * ggz[t];
+    near3_eval<P>(L, nf, g, groups, XS, np, a);
+    near3_eval_close<P>(L, nc, g, groups, X, XL, np, a);
+    float ph = a.phi.x + a.phi.y, gx = a.gx.x + a.gx.y, gy = a.gy.x + a.gy.y, gz = a.gz.x + a.gz.y;
+    for (int o = 16; o >= lanes; o >>= 1) {
+        ph = lane_add(ph, o);
+        gx = lane_add(gx, o);
+        gy = lane_add(gy, o);
+        gz = lane_add(gz, o);
     }
+    if (!valid || g != 0)
+        return;
+    // coincident pairs: G(0) := 0, so only -q T_I(0) remains of the far field's self term
+    float self = 0.f;
+    for (int c = coinc_start[k]; c < coinc_start[k + 1]; ++c)
+        self += q[coinc_src[c]];
+    const int64_t k3 = 3 * (int64_t)k;
+    phi_s[k] = (assign ? 0.f : phi_s[k]) + (ph - np.beta0 * self);
+    grad_s[k3] = (assign ? 0.f : grad_s[k3]) - np.inv_eps * gx;
+    grad_s[k3 + 1] = (assign ? 0.f : grad_s[k3 + 1]) - np.inv_eps * gy;
+    grad_s[k3 + 2] = (assign ? 0.f : grad_s[k3 + 2]) - np.inv_eps * gz;
 }
 
 // ---- FP32 near field, source-major (plans with many more sources than targets: FEM meshes,
 // where every node meets the quadrature points of several elements)
 //
-// Target items hold only the few targets of a cell, so their box is the whole cell and most
-// candidates lie beyond eps_I of most targets.  Here a warp takes an item of at most 64 sources
-// of one cell (compact: Morton sub-cell order) and keeps them in shared memory as packed pairs;
-// it reads the targets of the 27 cells around 32 at a time, keeps those within eps_I of the
-// sources' box (ballot) in a list (those within eps_I / 8 of the box in a second one), and
-// each lane then takes one listed target and sums the item's sources on it, two per packed
-// operation, adding phi and grad phi to the target with atomics.  Pairs closer than eps_I / 8
-// take their difference from the FP64 positions, as in k_near3_warp; coincident pairs are
-// removed by k_coincident3_apply.
-constexpr int kSrcListCap = 128;
+// Target items would hold the few targets of a cell, their boxes large.  Here a warp takes a piece
+// of at most 64 sources of one cell and keeps them in shared memory as packed pairs; it reads the
+// targets of the 27 cells around 32 at a time, keeps those within eps_I of the sources' box (ballot)
+// in a list (those within eps_I / 8 of the box in a second one, hi + lo), and each lane then takes one
+// listed target and sums the item's sources on it, two per packed operation, adding phi and grad
+// phi to the target with atomics.  Coincident pairs are removed by k_coincident3_apply.
+// Measured, 1.59M quadrature points and 68,921 nodes of the 384,000-tetrahedron cube (p = 3): 1144 us
+// with runs of the Morton order and FP64 differences of the close pairs, 497 us here.
+constexpr int kSrcListCap = 128, kSrcCloseCap = 64;
 
-template <int P, bool CLOSE>
-__device__ __forceinline__ void near3_src_eval(const float4 (*spairs)[2], const float4 *tlist, int n, int first,
-                                               int count, float dummy, const double *__restrict__ tgt_pos,
-                                               const double *__restrict__ src_pos, const Near3Params &np,
+struct Near3Sources {
+    float4 xy[32], zq[32];            // (xa, xb, ya, yb), (za, zb, qa, qb), units of eps_I
+    float4 hxy[32], lxy[32];          // hi and lo parts (torus units) for the close list
+    float2 hz[32], lz[32];
+    float4 far[kSrcListCap];          // listed targets: x, y, z (units of eps_I), index
+    float4 chi[kSrcCloseCap], clo[kSrcCloseCap];   // hi (torus units) and index, lo
+};
+
+__device__ __forceinline__ void near3_src_add(const Near3Sums &a, int k, const Near3Params &np,
+                                              float *__restrict__ phi_s, float *__restrict__ grad_s)
+{
+    atomicAdd(phi_s + k, a.phi.x + a.phi.y);
+    atomicAdd(grad_s + 3 * (int64_t)k, -np.inv_eps * (a.gx.x + a.gx.y));
+    atomicAdd(grad_s + 3 * (int64_t)k + 1, -np.inv_eps * (a.gy.x + a.gy.y));
+    atomicAdd(grad_s + 3 * (int64_t)k + 2, -np.inv_eps * (a.gz.x + a.gz.y));
+}
+
+template <int P>
+__device__ __forceinline__ void near3_src_eval(const Near3Sources &S, int n, int pairs, const Near3Params &np,
                                                float *__restrict__ phi_s, float *__restrict__ grad_s, int lane)
 {
     for (int base = 0; base < n; base += 32) {
-        const int e = base + lane;
-        const bool valid = e < n;
-        const float4 T = valid ? tlist[e] : make_float4(dummy, dummy, dummy, 0.f);
-        const int k = __float_as_int(T.w);
-        const float2 X = make_float2(T.x, T.x), Y = make_float2(T.y, T.y), Z = make_float2(T.z, T.z);
-        float2 phi = make_float2(0.f, 0.f), gx = phi, gy = phi, gz = phi;
+        const bool valid = base + lane < n;
+        const float4 T = valid ? S.far[base + lane] : make_float4(kPadPos, kPadPos, kPadPos, 0.f);
+        Near3Sums a;
+        a.phi = a.gx = a.gy = a.gz = f2(0.f);
+#pragma unroll 4
+        for (int i = 0; i < pairs; ++i) {
+            const float4 A = S.xy[i], B = S.zq[i];
+            const float2 dx = add2(f2(T.x), make_float2(-A.x, -A.y)), dy = add2(f2(T.y), make_float2(-A.z, -A.w)),
+                         dz = add2(f2(T.z), make_float2(-B.x, -B.y));
+            near3_pair<P>(np, near3_w(dx, dy, dz), dx, dy, dz, make_float2(B.z, B.w), a);
+        }
+        if (valid)
+            near3_src_add(a, __float_as_int(T.w), np, phi_s, grad_s);
+    }
+}
+
+template <int P>
+__device__ __forceinline__ void near3_src_eval_close(const Near3Sources &S, int n, int pairs, const Near3Params &np,
+                                                     float *__restrict__ phi_s, float *__restrict__ grad_s, int lane)
+{
+    const float2 ie = f2(np.inv_eps);
+    for (int base = 0; base < n; base += 32) {
+        const bool valid = base + lane < n;
+        const float4 T = valid ? S.chi[base + lane] : make_float4(kPadPos, kPadPos, kPadPos, 0.f);
+        const float4 TL = valid ? S.clo[base + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+        Near3Sums a;
+        a.phi = a.gx = a.gy = a.gz = f2(0.f);
 #pragma unroll 2
-        for (int i = 0; i < 32; ++i) {
-            const float4 A = spairs[i][0], B = spairs[i][1];   // (xa, xb, ya, yb), (za, zb, qa, qb)
-            float2 dx = __fadd2_rn(X, make_float2(-A.x, -A.y));
-            float2 dy = __fadd2_rn(Y, make_float2(-A.z, -A.w));
-            float2 dz = __fadd2_rn(Z, make_float2(-B.x, -B.y));
-            float2 w = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-            if constexpr (CLOSE) {
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    // (idle source slots, i + 32 t >= count, carry charge 0 and are not refined)
-                    if (valid && i + 32 * t < count && (t == 0 ? w.x : w.y) < 1.f / 64.f) {
-                        const int64_t j = first + i + 32 * t;
-                        const float ex = (float)((tgt_pos[3 * (int64_t)k] - src_pos[3 * j]) * np.inv_eps_d);
-                        const float ey = (float)((tgt_pos[3 * (int64_t)k + 1] - src_pos[3 * j + 1]) * np.inv_eps_d);
-                        const float ez = (float)((tgt_pos[3 * (int64_t)k + 2] - src_pos[3 * j + 2]) * np.inv_eps_d);
-                        const float e2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
-                        if (t == 0) {
-                            dx.x = ex;
-                            dy.x = ey;
-                            dz.x = ez;
-                            w.x = e2;
-                        } else {
-                            dx.y = ex;
-                            dy.y = ey;
-                            dz.y = ez;
-                            w.y = e2;
-                        }
-                    }
-                }
-            }
-            near3_pair<P>(np, w, dx, dy, dz, make_float2(B.z, B.w), phi, gx, gy, gz);
+        for (int i = 0; i < pairs; ++i) {
+            const float4 A = S.hxy[i], AL = S.lxy[i], B = S.zq[i];
+            const float2 Z = S.hz[i], ZL = S.lz[i];
+            const float2 dx = mul2(add2(add2(f2(T.x), make_float2(-A.x, -A.y)), add2(f2(TL.x), make_float2(-AL.x, -AL.y))), ie);
+            const float2 dy = mul2(add2(add2(f2(T.y), make_float2(-A.z, -A.w)), add2(f2(TL.y), make_float2(-AL.z, -AL.w))), ie);
+            const float2 dz = mul2(add2(add2(f2(T.z), make_float2(-Z.x, -Z.y)), add2(f2(TL.z), make_float2(-ZL.x, -ZL.y))), ie);
+            near3_pair_close<P>(np, dx, dy, dz, make_float2(B.z, B.w), a);
         }
-        if (valid) {
-            atomicAdd(phi_s + k, phi.x + phi.y);
-            atomicAdd(grad_s + 3 * (int64_t)k, -np.inv_eps * (gx.x + gx.y));
-            atomicAdd(grad_s + 3 * (int64_t)k + 1, -np.inv_eps * (gy.x + gy.y));
-            atomicAdd(grad_s + 3 * (int64_t)k + 2, -np.inv_eps * (gz.x + gz.y));
-        }
+        if (valid)
+            near3_src_add(a, __float_as_int(T.w), np, phi_s, grad_s);
     }
 }
 
 template <int P>
 __global__ void __launch_bounds__(kNear3Warps * 32) k_near3_src(const int2 *__restrict__ items, int n_items,
                                                                 const int *__restrict__ src_base,
-                                                                const float4 *__restrict__ src_p32,
-                                                                const float4 *__restrict__ tgt_p32,
-                                                                const double *__restrict__ tgt_pos,
-                                                                const double *__restrict__ src_pos,
+                                                                const float4 *__restrict__ src_hi,
+                                                                const float4 *__restrict__ src_lo,
+                                                                const float4 *__restrict__ tgt_hi,
+                                                                const float4 *__restrict__ tgt_lo,
                                                                 const float *__restrict__ q,
                                                                 const int *__restrict__ tgt_start, CellGrid3 cg,
                                                                 Near3Params np, float *__restrict__ phi_s,
                                                                 float *__restrict__ grad_s)
 {
-    __shared__ float4 spairs_all[kNear3Warps][32][2];
-    __shared__ float4 flist_all[kNear3Warps][kSrcListCap];
-    __shared__ float4 clist_all[kNear3Warps][kSrcListCap];
+    __shared__ Near3Sources all[kNear3Warps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int item = blockIdx.x * kNear3Warps + warp;
     if (item >= n_items)
         return;   // whole warp; the kernel has no block-wide barrier
-    float4(*spairs)[2] = spairs_all[warp];
-    float4 *flist = flist_all[warp], *clist = clist_all[warp];
+    Near3Sources &S = all[warp];
     const int2 it = items[item];
-    const int first = it.x, count = it.y;
-    const bool va = lane < count, vb = lane + 32 < count;
-    const float4 pa = src_p32[va ? first + lane : first], pb = src_p32[vb ? first + 32 + lane : first];
-    spairs[lane][0] = make_float4(pa.x, pb.x, pa.y, pb.y);
-    spairs[lane][1] = make_float4(pa.z, pb.z, va ? q[first + lane] : 0.f, vb ? q[first + 32 + lane] : 0.f);
-    const float lox = warp_min(fminf(pa.x, pb.x)), hix = warp_max(fmaxf(pa.x, pb.x));
-    const float loy = warp_min(fminf(pa.y, pb.y)), hiy = warp_max(fmaxf(pa.y, pb.y));
-    const float loz = warp_min(fminf(pa.z, pb.z)), hiz = warp_max(fmaxf(pa.z, pb.z));
-    const float dummy = fminf(lox, fminf(loy, loz)) - 3.f;   // idle lanes: every pair beyond eps_I
+    // pair i: sources i and i + pairs; an idle second one copies the first source with charge 0
+    const int pairs = (it.y + 1) / 2;
+    const int ja = it.x + (lane < pairs ? lane : 0);
+    const bool vb = lane < pairs && lane + pairs < it.y;
+    const int jb = vb ? ja + pairs : it.x;
+    const float4 ha = src_hi[ja], hb = src_hi[jb], la = src_lo[ja], lb = src_lo[jb];
+    const float ie = np.inv_eps;
+    S.xy[lane] = make_float4(ha.x * ie, hb.x * ie, ha.y * ie, hb.y * ie);
+    S.zq[lane] = make_float4(ha.z * ie, hb.z * ie, q[ja], vb ? q[jb] : 0.f);
+    S.hxy[lane] = make_float4(ha.x, hb.x, ha.y, hb.y);
+    S.lxy[lane] = make_float4(la.x, lb.x, la.y, lb.y);
+    S.hz[lane] = make_float2(ha.z, hb.z);
+    S.lz[lane] = make_float2(la.z, lb.z);
+    Box3 box;
+    box.of(ha, hb);
     __syncwarp();
-    const int packed = src_base[first];
-    const int c1 = b3x(packed) / cg.cell, c2 = b3y(packed) / cg.cell, c3 = b3z(packed) / cg.cell;
-    const int S3 = cg.sub3();
     const unsigned below = (1u << lane) - 1u;
     int nf = 0, nc = 0;
-    for (int e1 = max(c1 - 1, 0); e1 <= min(c1 + 1, cg.n_c - 1); ++e1) {
-        const float o1 = (float)(e1 - c1) * np.H;
-        const float bx = fmaxf(0.f, fmaxf(o1 - hix, lox - (o1 + np.H)));
-        for (int e2 = max(c2 - 1, 0); e2 <= min(c2 + 1, cg.n_c - 1); ++e2) {
-            const float o2 = (float)(e2 - c2) * np.H;
-            const float by = fmaxf(0.f, fmaxf(o2 - hiy, loy - (o2 + np.H)));
-            for (int e3 = max(c3 - 1, 0); e3 <= min(c3 + 1, cg.n_c - 1); ++e3) {
-                const float o3 = (float)(e3 - c3) * np.H;
-                const float bz = fmaxf(0.f, fmaxf(o3 - hiz, loz - (o3 + np.H)));
-                if (bx * bx + by * by + bz * bz >= np.reach2)
-                    continue;
-                const int key = cg.key(e1, e2, e3);
-                const int end = tgt_start[(key + 1) * S3];
-                for (int j0 = tgt_start[key * S3]; j0 < end; j0 += 32) {
-                    const int j = j0 + lane;
-                    bool keep = false, close = false;
-                    float tx = 0.f, ty = 0.f, tz = 0.f;
-                    if (j < end) {
-                        const float4 tp = tgt_p32[j];
-                        tx = tp.x + o1;
-                        ty = tp.y + o2;
-                        tz = tp.z + o3;
-                        const float dx = fmaxf(0.f, fmaxf(tx - hix, lox - tx));
-                        const float dy = fmaxf(0.f, fmaxf(ty - hiy, loy - ty));
-                        const float dz = fmaxf(0.f, fmaxf(tz - hiz, loz - tz));
-                        const float g2 = dx * dx + dy * dy + dz * dz;
-                        keep = g2 < np.reach2;
-                        close = g2 < np.close_reach2;
-                    }
-                    const unsigned mf = __ballot_sync(0xffffffffu, keep && !close);
-                    const unsigned mc = __ballot_sync(0xffffffffu, close);
-                    if (keep && !close)
-                        flist[nf + __popc(mf & below)] = make_float4(tx, ty, tz, __int_as_float(j));
-                    if (close)
-                        clist[nc + __popc(mc & below)] = make_float4(tx, ty, tz, __int_as_float(j));
-                    nf += __popc(mf);
-                    nc += __popc(mc);
-                    if (nf > kSrcListCap - 32) {
-                        __syncwarp();
-                        near3_src_eval<P, false>(spairs, flist, nf, first, count, dummy, tgt_pos, src_pos, np, phi_s, grad_s,
-                                                 lane);
-                        nf = 0;
-                        __syncwarp();
-                    }
-                    if (nc > kSrcListCap - 32) {
-                        __syncwarp();
-                        near3_src_eval<P, true>(spairs, clist, nc, first, count, dummy, tgt_pos, src_pos, np, phi_s, grad_s,
-                                                lane);
-                        nc = 0;
-                        __syncwarp();
-                    }
-                }
+    Chunks3 ch(lane, src_base[it.x], cg, np, box, tgt_start);
+    bool more = ch.next(lane, tgt_hi, nullptr);
+    while (more) {
+        const float4 y = ch.p;
+        const float ox = ch.ox, oy = ch.oy, oz = ch.oz;
+        const int j = ch.j;
+        const bool in = ch.in;
+        more = ch.next(lane, tgt_hi, nullptr);
+        const float fx = ox - y.x, fy = oy - y.y, fz = oz - y.z;   // -(target in the item's frame)
+        const float g2 = in ? box.gap2(fx, fy, fz) : 3e38f;
+        const bool keep = g2 <= np.reach2, close = g2 <= np.close_reach2;
+        const unsigned mc = __ballot_sync(0xffffffffu, close), mf = __ballot_sync(0xffffffffu, keep) & ~mc;
+        if (keep && !close)
+            S.far[nf + __popc(mf & below)] = make_float4(-fx * ie, -fy * ie, -fz * ie, __int_as_float(j));
+        nf += __popc(mf);
+        if (nf > kSrcListCap - 32) {
+            __syncwarp();
+            near3_src_eval<P>(S, nf, pairs, np, phi_s, grad_s, lane);
+            nf = 0;
+            __syncwarp();
+        }
+        if (mc) {
+            if (close) {
+                const int at = nc + __popc(mc & below);
+                const float4 yl = __ldg(tgt_lo + j);
+                S.chi[at] = make_float4(-fx, -fy, -fz, __int_as_float(j));
+                S.clo[at] = make_float4(-neg_lo(ox, y.x, yl.x, fx), -neg_lo(oy, y.y, yl.y, fy), -neg_lo(oz, y.z, yl.z, fz), 0.f);
+            }
+            nc += __popc(mc);
+            if (nc > kSrcCloseCap - 32) {
+                __syncwarp();
+                near3_src_eval_close<P>(S, nc, pairs, np, phi_s, grad_s, lane);
+                nc = 0;
+                __syncwarp();
             }
         }
     }
     __syncwarp();
-    near3_src_eval<P, false>(spairs, flist, nf, first, count, dummy, tgt_pos, src_pos, np, phi_s, grad_s, lane);
-    near3_src_eval<P, true>(spairs, clist, nc, first, count, dummy, tgt_pos, src_pos, np, phi_s, grad_s, lane);
+    near3_src_eval<P>(S, nf, pairs, np, phi_s, grad_s, lane);
+    near3_src_eval_close<P>(S, nc, pairs, np, phi_s, grad_s, lane);
 }
 
 // Coincident pairs for the source-major kernel: phi -= T_I(0) (sum of the coincident charges).
@@ -1073,13 +1235,13 @@ cudaError_t launch_point_keys3(const double *xyz, int64_t n, double s, int n_os,
 
 template <typename real>
 cudaError_t launch_gather_points3(const double *xyz, const int *perm, int64_t n, double s, int n_os, int window_lo,
-                                  int n_a, int m, int cell, double inv_eps, double *pos, real *frac, int *base,
-                                  float4 *pos32, int *status, cudaStream_t st)
+                                  int n_a, int m, int cell, double *pos, real *frac, int *base,
+                                  float4 *hi, float4 *lo, int *status, cudaStream_t st)
 {
     if (n <= 0)
         return cudaSuccess;
-    k_gather_points3<real><<<nblk(n, 256), 256, 0, st>>>(xyz, perm, n, s, n_os, window_lo, n_a, m, cell, inv_eps, pos,
-                                                        frac, base, pos32, status);
+    k_gather_points3<real><<<nblk(n, 256), 256, 0, st>>>(xyz, perm, n, s, n_os, window_lo, n_a, m, cell, pos, frac,
+                                                         base, hi, lo, status);
     return cudaGetLastError();
 }
 
@@ -1192,8 +1354,17 @@ cudaError_t launch_near3_f64(int64_t N, const int *tgt_base, const double *tgt_p
     return cudaGetLastError();
 }
 
-cudaError_t launch_near3_warp(const int2 *items, int n_items, const int *tgt_base, const float4 *tgt_p32,
-                              const float4 *src_p32, const double *tgt_pos, const double *src_pos, const float *q,
+cudaError_t launch_cell_order3(const int *start, CellGrid3 cg, int cap, const double *xyz, double s, int n_os,
+                               int window_lo, int n_a, int m, int *perm, cudaStream_t st)
+{
+    if (cg.n_cells() <= 0)
+        return cudaSuccess;
+    k_cell_order3<<<(unsigned)cg.n_cells(), kOrder3Threads, 0, st>>>(start, cg, cap, xyz, s, n_os, window_lo, n_a, m, perm);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_near3_warp(const int2 *items, int n_items, int lanes, const int *tgt_base, const float4 *tgt_hi,
+                              const float4 *tgt_lo, const float4 *src_hi, const float4 *src_lo, const float *q,
                               const int *src_start, CellGrid3 cg, const Near3Params &np, const int *coinc_start,
                               const int *coinc_src, float *phi_s, float *grad_s, bool assign, cudaStream_t st)
 {
@@ -1202,25 +1373,25 @@ cudaError_t launch_near3_warp(const int2 *items, int n_items, const int *tgt_bas
     const unsigned blocks = (unsigned)((n_items + kNear3Warps - 1) / kNear3Warps);
     return with_degree(np.p, [&](auto pc) {
         constexpr int P = decltype(pc)::value;
-        k_near3_warp<P><<<blocks, kNear3Warps * 32, 0, st>>>(items, n_items, tgt_base, tgt_p32, src_p32, tgt_pos,
-                                                              src_pos, q, src_start, cg, np, coinc_start, coinc_src,
-                                                              phi_s, grad_s, assign);
+        k_near3_warp<P><<<blocks, kNear3Warps * 32, 0, st>>>(items, n_items, lanes, tgt_base, tgt_hi, tgt_lo, src_hi,
+                                                             src_lo, q, src_start, cg, np, coinc_start, coinc_src,
+                                                             phi_s, grad_s, assign);
         return cudaGetLastError();
     });
 }
 
-cudaError_t launch_near3_src(const int2 *items, int n_items, const int *src_base, const float4 *src_p32,
-                             const float4 *tgt_p32, const double *tgt_pos, const double *src_pos, const float *q,
+cudaError_t launch_near3_src(const int2 *items, int n_items, const int *src_base, const float4 *src_hi,
+                             const float4 *src_lo, const float4 *tgt_hi, const float4 *tgt_lo, const float *q,
                              const int *tgt_start, CellGrid3 cg, const Near3Params &np, int64_t N,
                              const int *coinc_start, const int *coinc_src, bool any_coincident, float *phi_s,
                              float *grad_s, cudaStream_t st)
 {
     if (n_items > 0) {
         const unsigned blocks = (unsigned)((n_items + kNear3Warps - 1) / kNear3Warps);
-        cudaError_t e = with_degree(np.p, [&](auto pc) {
+        const cudaError_t e = with_degree(np.p, [&](auto pc) {
             constexpr int P = decltype(pc)::value;
-            k_near3_src<P><<<blocks, kNear3Warps * 32, 0, st>>>(items, n_items, src_base, src_p32, tgt_p32, tgt_pos,
-                                                                 src_pos, q, tgt_start, cg, np, phi_s, grad_s);
+            k_near3_src<P><<<blocks, kNear3Warps * 32, 0, st>>>(items, n_items, src_base, src_hi, src_lo, tgt_hi, tgt_lo,
+                                                                q, tgt_start, cg, np, phi_s, grad_s);
             return cudaGetLastError();
         });
         if (e != cudaSuccess)
@@ -1256,7 +1427,7 @@ cudaError_t launch_unpermute3(int64_t N, const real *phi_s, const real *grad_s, 
 
 #define FS_INST3(real)                                                                                            \
     template cudaError_t launch_gather_points3<real>(const double *, const int *, int64_t, double, int, int, int, \
-                                                     int, int, double, double *, real *, int *, float4 *, int *,  \
+                                                     int, int, double *, real *, int *, float4 *, float4 *, int *,  \
                                                      cudaStream_t);                                               \
     template cudaError_t launch_spread3<real>(int64_t, int, const int *, const real *, const real *, Window<real>, \
                                               const WindowPoly &, real *, int, cudaStream_t);                     \

@@ -7,6 +7,7 @@
 // contiguous range.  Within a cell the points are then sorted into strips and pieces
 // (k_cell_order), so that any piece is compact.
 #include "internal.h"
+#include "sort_shared.cuh"
 
 namespace fs {
 
@@ -140,23 +141,6 @@ __global__ void k_scatter(const int *__restrict__ key, int64_t n, int *__restric
         return;
     const int pos = atomicAdd(&fill[key[i]], 1);
     perm[pos] = (int)i;
-}
-
-// Ascending bitonic sort of n2 (a power of two) keys in shared memory by the whole block.
-__device__ __forceinline__ void sort_shared(unsigned long long *key, int n2)
-{
-    for (int k = 2; k <= n2; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int t = threadIdx.x; t < n2 / 2; t += blockDim.x) {
-                const int i = 2 * t - (t & (j - 1)), l = i + j;
-                const unsigned long long a = key[i], b = key[l];
-                if ((a > b) == ((i & k) == 0)) {
-                    key[i] = b;
-                    key[l] = a;
-                }
-            }
-            __syncthreads();
-        }
 }
 
 // Points of a cell into strips along x, each strip along y (CellSplit): one block per cell.  A

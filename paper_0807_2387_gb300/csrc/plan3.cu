@@ -31,7 +31,9 @@ struct fs3_plan {
     int *src_start = nullptr, *tgt_start = nullptr;
     void *src_frac = nullptr, *tgt_frac = nullptr;
     double *src_pos = nullptr, *tgt_pos = nullptr;
-    float4 *src_p32 = nullptr, *tgt_p32 = nullptr;
+    float4 *src_hi = nullptr, *tgt_hi = nullptr, *src_lo = nullptr, *tgt_lo = nullptr;   // FP32: offsets in the cell
+    std::vector<int> src_cells, tgt_cells;   // FP32: the cells' first points
+    int src_cap = 0, tgt_cap = 0;            // points per piece of a cell (CellSplit3)
     void *mul = nullptr, *tw = nullptr;
     void *grid = nullptr, *spec1 = nullptr, *spec2 = nullptr;
     void *phi_s = nullptr, *grad_s = nullptr;
@@ -176,9 +178,16 @@ template <typename real> NearParams<real> make_near3(const fs3_plan *pl)
     return np;
 }
 
+// Targets per near-field warp item, from their mean number per cell as one of them sees it: a whole
+// sparse cell, so that the groups of the warp share its candidates; from 20 on the full warp, since
+// every item lists the candidates of 27 cells (the ball of 2^18 points at 41 per cell, its step with
+// 8 / 16 / 32: 706 / 629 / 617 us).
+int near3_item_lanes(double per_cell) { return per_cell < 8.0 ? 8 : (per_cell < 20.0 ? 16 : 32); }
+constexpr int kSrcMajorItem3 = 64;   // sources per item of the source-major near field
+
 template <typename real>
 fs_status bin3(fs3_plan *pl, const double *xyz, int64_t n, int **perm, int **base, void **frac, double **pos,
-               float4 **p32, int **start)
+               float4 **hi, float4 **lo, int **start, int *cap, std::vector<int> *cells)
 {
     cudaStream_t st = pl->stream;
     const int n_keys = pl->cg.n_keys();
@@ -188,9 +197,11 @@ fs_status bin3(fs3_plan *pl, const double *xyz, int64_t n, int **perm, int **bas
     FS_TRY(pl->alloc(&fr, 3 * (size_t)std::max<int64_t>(n, 1)));
     *frac = fr;
     FS_TRY(pl->alloc(pos, 3 * (size_t)std::max<int64_t>(n, 1)));
-    *p32 = nullptr;
-    if (pl->precision == 32)
-        FS_TRY(pl->alloc(p32, n));
+    *hi = *lo = nullptr;
+    if (pl->precision == 32) {
+        FS_TRY(pl->alloc(hi, n));
+        FS_TRY(pl->alloc(lo, n));
+    }
     FS_TRY(pl->alloc(start, (size_t)n_keys + 1));
     int *key = nullptr, *count = nullptr, *fill = nullptr, *tmp = nullptr;
     FS_TRY(pl->alloc(&key, n));
@@ -204,8 +215,24 @@ fs_status bin3(fs3_plan *pl, const double *xyz, int64_t n, int **perm, int **bas
     FS_CUDA(launch_exclusive_scan(count, *start, n_keys, tmp, st));
     FS_CUDA(cudaMemcpyAsync(fill, *start, sizeof(int) * ((size_t)n_keys + 1), cudaMemcpyDeviceToDevice, st));
     FS_CUDA(launch_scatter(key, n, fill, *perm, st));
+    if (pl->precision == 32) {
+        const int n_cells = pl->cg.n_cells(), S3 = pl->cg.sub3();
+        std::vector<int> all((size_t)n_keys + 1);
+        FS_CUDA(cudaMemcpyAsync(all.data(), *start, sizeof(int) * all.size(), cudaMemcpyDeviceToHost, st));
+        FS_CUDA(cudaStreamSynchronize(st));
+        cells->resize((size_t)n_cells + 1);
+        double sq = 0.0;
+        for (int c = 0; c <= n_cells; ++c) {
+            (*cells)[c] = all[(size_t)c * S3];
+            const double k = c > 0 ? (*cells)[c] - (*cells)[c - 1] : 0;
+            sq += k * k;
+        }
+        if (*cap == 0)
+            *cap = near3_item_lanes(n > 0 ? sq / (double)n : 0.0);
+        FS_CUDA(launch_cell_order3(*start, pl->cg, *cap, xyz, pl->s, pl->n_os, pl->window_lo, pl->n_a, pl->m, *perm, st));
+    }
     FS_CUDA(launch_gather_points3<real>(xyz, *perm, n, pl->s, pl->n_os, pl->window_lo, pl->n_a, pl->m, pl->cg.cell,
-                                        1.0 / pl->eps_I, *pos, fr, *base, *p32, pl->status, st));
+                                        *pos, fr, *base, *hi, *lo, pl->status, st));
     FS_CUDA(cudaStreamSynchronize(st));
     pl->release(key);
     pl->release(count);
@@ -258,10 +285,14 @@ fs_status plan3_init(fs3_plan *pl, const double *src, int64_t M, const double *t
         return fail(FS_EINVAL, "too many near-field cells (eps_I too small for this grid)");
     FS_TRY(pl->alloc(&pl->status, 1));
     FS_CUDA(cudaMemset(pl->status, 0, sizeof(int)));
-    FS_TRY(bin3<real>(pl, src, M, &pl->src_perm, &pl->src_base, &pl->src_frac, &pl->src_pos, &pl->src_p32,
-                      &pl->src_start));
-    FS_TRY(bin3<real>(pl, tgt, N, &pl->tgt_perm, &pl->tgt_base, &pl->tgt_frac, &pl->tgt_pos, &pl->tgt_p32,
-                      &pl->tgt_start));
+    // targets much sparser than sources (FEM meshes): near-field items over the sources instead,
+    // whose boxes stay small where a cell's few targets would span the whole cell
+    pl->src_major = N > 0 && M >= 3 * N;
+    pl->src_cap = pl->src_major ? kSrcMajorItem3 : 32;
+    FS_TRY(bin3<real>(pl, src, M, &pl->src_perm, &pl->src_base, &pl->src_frac, &pl->src_pos, &pl->src_hi, &pl->src_lo,
+                      &pl->src_start, &pl->src_cap, &pl->src_cells));
+    FS_TRY(bin3<real>(pl, tgt, N, &pl->tgt_perm, &pl->tgt_base, &pl->tgt_frac, &pl->tgt_pos, &pl->tgt_hi, &pl->tgt_lo,
+                      &pl->tgt_start, &pl->tgt_cap, &pl->tgt_cells));
     int dev_status = 0;
     FS_CUDA(cudaMemcpy(&dev_status, pl->status, sizeof(int), cudaMemcpyDeviceToHost));
     if (dev_status != 0)
@@ -345,41 +376,45 @@ fs_status near_setup3(fs3_plan *pl)
     cudaStream_t st = pl->stream;
     if (pl->N > ((int64_t)1 << 24))
         return fail(FS_EINVAL, "FP32 3D plans take at most 2^24 targets");
-    const int n_cells = pl->cg.n_cells(), S3 = pl->cg.sub3();
-    // the sorted points of each cell, split evenly into pieces of at most 64
-    auto make_items = [&](const int *dev_start, int2 **out, int *n_out) -> fs_status {
-        std::vector<int> start((size_t)pl->cg.n_keys() + 1);
-        FS_CUDA(cudaMemcpyAsync(start.data(), dev_start, sizeof(int) * start.size(), cudaMemcpyDeviceToHost, st));
-        FS_CUDA(cudaStreamSynchronize(st));
+    const int n_cells = pl->cg.n_cells();
+    // the pieces that the points of each cell are sorted into
+    auto make_items = [&](const std::vector<int> &cells, int cap, int2 **out, int *n_out) -> fs_status {
         std::vector<int2> items;
         for (int c = 0; c < n_cells; ++c) {
-            const int a = start[(size_t)c * S3], b = start[(size_t)(c + 1) * S3];
-            const int cnt = b - a;
-            if (cnt <= 0)
-                continue;
-            const int pieces = (cnt + 63) / 64;
-            for (int k = 0; k < pieces; ++k) {
-                const int lo = a + (int)((int64_t)cnt * k / pieces), hi = a + (int)((int64_t)cnt * (k + 1) / pieces);
-                items.push_back(make_int2(lo, hi - lo));
+            const int a = cells[c], count = cells[c + 1] - a;
+            for (int r = 0; r < CellSplit::runs(count); ++r) {
+                const int run = CellSplit::run_first(count, r);
+                const CellSplit3 split(CellSplit::run_first(count, r + 1) - run, cap);
+                for (int j = 0; j < split.slabs; ++j) {
+                    const int k = split.slab_piece(j + 1) - split.slab_piece(j), at = split.slab_first(j),
+                              n = split.slab_first(j + 1) - at;
+                    for (int i = 0; i < CellSplit3::strips(k); ++i) {
+                        const int parts = CellSplit3::strip_piece(k, i + 1) - CellSplit3::strip_piece(k, i),
+                                  lo = CellSplit3::strip_first(k, n, i),
+                                  len = CellSplit3::strip_first(k, n, i + 1) - lo;
+                        for (int t = 0; t < parts; ++t) {
+                            const int p0 = (int)((int64_t)len * t / parts), p1 = (int)((int64_t)len * (t + 1) / parts);
+                            items.push_back(make_int2(a + run + at + lo + p0, p1 - p0));
+                        }
+                    }
+                }
             }
         }
         *n_out = (int)items.size();
         FS_TRY(pl->alloc(out, items.size()));
-        if (!items.empty())
+        if (!items.empty()) {
             FS_CUDA(cudaMemcpyAsync(*out, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice, st));
+            FS_CUDA(cudaStreamSynchronize(st));   // the host array is read
+        }
         return FS_OK;
     };
     // spreading items: the sources of each cell in pieces of at most kSpread3ItemMax, where
     // the tiles fit in shared memory and the occupied cells are dense enough to pay for them
-    std::vector<int> sstart;
+    const std::vector<int> &cells = pl->src_cells;
     if ((spread3_tile_smem(pl->cg.cell, pl->m) > 0 || spread3_runs_smem(pl->cg.cell, pl->m) > 0) && pl->M > 0) {
-        sstart.resize((size_t)pl->cg.n_keys() + 1);
-        FS_CUDA(cudaMemcpyAsync(sstart.data(), pl->src_start, sizeof(int) * sstart.size(), cudaMemcpyDeviceToHost,
-                                st));
-        FS_CUDA(cudaStreamSynchronize(st));
         int64_t occupied = 0;
         for (int c = 0; c < n_cells; ++c)
-            occupied += sstart[(size_t)(c + 1) * S3] > sstart[(size_t)c * S3];
+            occupied += cells[c + 1] > cells[c];
         const int c3 = pl->cg.cell * pl->cg.cell * pl->cg.cell;
         const bool runs = spread3_runs_smem(pl->cg.cell, pl->m) > 0 && (int64_t)n_cells * c3 <= kScanMost;
         pl->spread_tiles = ((runs || spread3_tile_smem(pl->cg.cell, pl->m) > 0) &&
@@ -410,7 +445,7 @@ fs_status near_setup3(fs3_plan *pl)
         const int most = pl->run_order ? kSpread3RunMax : kSpread3ItemMax;
         std::vector<int2> sitems;
         for (int c = 0; c < n_cells; ++c) {
-            const int a = sstart[(size_t)c * S3], count = sstart[(size_t)(c + 1) * S3] - a;
+            const int a = cells[c], count = cells[c + 1] - a;
             const int pieces = (count + most - 1) / most;
             for (int k = 0; k < pieces; ++k) {
                 const int lo = (int)((int64_t)count * k / pieces), hi = (int)((int64_t)count * (k + 1) / pieces);
@@ -423,18 +458,15 @@ fs_status near_setup3(fs3_plan *pl)
             FS_CUDA(cudaMemcpyAsync(pl->spread_items, sitems.data(), sizeof(int2) * sitems.size(),
                                     cudaMemcpyHostToDevice, st));
     }
-    // targets much sparser than sources (FEM meshes): near-field items over the sources
-    // instead, whose boxes stay small where a cell's few targets would span the whole cell
-    pl->src_major = pl->N > 0 && pl->M >= 3 * pl->N;
     if (pl->N > 0) {
         FS_CUDA(cudaStreamCreateWithFlags(&pl->aux, cudaStreamNonBlocking));
         FS_CUDA(cudaEventCreateWithFlags(&pl->ev_fork, cudaEventDisableTiming));
         FS_CUDA(cudaEventCreateWithFlags(&pl->ev_join, cudaEventDisableTiming));
     }
     if (pl->src_major)
-        FS_TRY(make_items(pl->src_start, &pl->src_items, &pl->n_src_items));
+        FS_TRY(make_items(pl->src_cells, pl->src_cap, &pl->src_items, &pl->n_src_items));
     else
-        FS_TRY(make_items(pl->tgt_start, &pl->near_items, &pl->n_near_items));
+        FS_TRY(make_items(pl->tgt_cells, pl->tgt_cap, &pl->near_items, &pl->n_near_items));
     // coincident sources: count, scan, fill
     const int64_t N = pl->N;
     int *count = nullptr, *tmp = nullptr;
@@ -465,10 +497,9 @@ Near3Params make_near3_f32(const fs3_plan *pl)
     Near3Params np{};
     const double eps = pl->eps_I;
     np.p = pl->p;
-    np.H = (float)((double)pl->cg.cell / pl->n_os / eps);
-    np.reach2 = (float)((1.0 + 2e-4) * (1.0 + 2e-4));
-    np.close_reach2 = (float)((0.125 + 2e-4) * (0.125 + 2e-4));
-    np.inv_eps_d = 1.0 / eps;
+    np.h = (float)((double)pl->cg.cell / pl->n_os);
+    np.reach2 = (float)((1.0 + 2e-4) * (1.0 + 2e-4) * eps * eps);
+    np.close_reach2 = (float)((0.125 + 2e-4) * (0.125 + 2e-4) * eps * eps);
     np.c1 = (float)(1.0 / (4.0 * kPi * eps));
     np.inv_eps = (float)(1.0 / eps);
     np.beta0 = (float)pl->kp.beta[0];
@@ -600,13 +631,13 @@ template <typename real> fs_status eval3_t(fs3_plan *pl, void *phi, void *H, fs_
                 if (pl->src_major) {
                     FS_CUDA(cudaMemsetAsync(pl->phi_s, 0, sizeof(float) * (size_t)pl->N, sa));
                     FS_CUDA(cudaMemsetAsync(pl->grad_s, 0, sizeof(float) * 3 * (size_t)pl->N, sa));
-                    FS_CUDA(launch_near3_src(pl->src_items, pl->n_src_items, pl->src_base, pl->src_p32, pl->tgt_p32,
-                                             pl->tgt_pos, pl->src_pos, (const float *)q, pl->tgt_start, pl->cg, np32,
+                    FS_CUDA(launch_near3_src(pl->src_items, pl->n_src_items, pl->src_base, pl->src_hi, pl->src_lo,
+                                             pl->tgt_hi, pl->tgt_lo, (const float *)q, pl->tgt_start, pl->cg, np32,
                                              pl->N, pl->coinc_start, pl->coinc_src, pl->n_coinc > 0,
                                              (float *)pl->phi_s, (float *)pl->grad_s, sa));
                 } else {
-                    FS_CUDA(launch_near3_warp(pl->near_items, pl->n_near_items, pl->tgt_base, pl->tgt_p32,
-                                              pl->src_p32, pl->tgt_pos, pl->src_pos, (const float *)q, pl->src_start,
+                    FS_CUDA(launch_near3_warp(pl->near_items, pl->n_near_items, pl->tgt_cap, pl->tgt_base, pl->tgt_hi,
+                                              pl->tgt_lo, pl->src_hi, pl->src_lo, (const float *)q, pl->src_start,
                                               pl->cg, np32, pl->coinc_start, pl->coinc_src, (float *)pl->phi_s,
                                               (float *)pl->grad_s, true, sa));
                 }
