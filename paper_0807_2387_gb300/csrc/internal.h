@@ -208,6 +208,10 @@ template <typename real>
 cudaError_t launch_interp3(int64_t N, int m, const int *base, const real *frac, Window<real> w, const WindowPoly &wp,
                            const real *grid, int n_a, real n_os, real *phi_s, real *grad_s, bool acc,
                            cudaStream_t st);
+// Interpolation and output in one pass for FP32 plans of m = 4 whose near field stored phi_s and grad_s
+cudaError_t launch_interp3_out(int64_t N, int m, const int *base, const float *frac, const WindowPoly &wp,
+                               const float *grid, int n_a, float n_os, const float *phi_s, const float *grad_s,
+                               const int *perm, double s, void *phi_out, void *H_out, int out_f64, cudaStream_t st);
 // FP64 near field, thread per target over the 27 cells around its own
 cudaError_t launch_near3_f64(int64_t N, const int *tgt_base, const double *tgt_pos, const double *src_pos,
                              const int *src_start, CellGrid3 cg, const double *q, NearParams<double> np,

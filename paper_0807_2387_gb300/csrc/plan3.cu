@@ -648,14 +648,22 @@ template <typename real> fs_status eval3_t(fs3_plan *pl, void *phi, void *H, fs_
                                   (const real *)pl->mul, (const C *)pl->tw, st));
         if (overlap)
             FS_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
+        void *po = phi ? (unsigned char *)phi + (size_t)r * pl->N * osz : nullptr;
+        void *ho = H ? (unsigned char *)H + (size_t)r * pl->N * 3 * osz : nullptr;
+        if constexpr (sizeof(real) == 4) {
+            if (overlap && pl->m == 4) {
+                FS_CUDA(launch_interp3_out(pl->N, pl->m, pl->tgt_base, (const float *)pl->tgt_frac, pl->wpoly,
+                                           (const float *)pl->grid, pl->n_a, (float)pl->n_os, (const float *)pl->phi_s,
+                                           (const float *)pl->grad_s, pl->tgt_perm, pl->s, po, ho, dtype == FS_F64, st));
+                continue;
+            }
+        }
         FS_CUDA(launch_interp3<real>(pl->N, pl->m, pl->tgt_base, (const real *)pl->tgt_frac, w, pl->wpoly,
                                      (const real *)pl->grid, pl->n_a, (real)pl->n_os, (real *)pl->phi_s,
                                      (real *)pl->grad_s, overlap, st));
         if constexpr (sizeof(real) == 8)
             FS_CUDA(launch_near3_f64(pl->N, pl->tgt_base, pl->tgt_pos, pl->src_pos, pl->src_start, pl->cg,
                                      (const double *)q, np, (double *)pl->phi_s, (double *)pl->grad_s, st));
-        void *po = phi ? (unsigned char *)phi + (size_t)r * pl->N * osz : nullptr;
-        void *ho = H ? (unsigned char *)H + (size_t)r * pl->N * 3 * osz : nullptr;
         FS_CUDA(launch_unpermute3<real>(pl->N, (const real *)pl->phi_s, (const real *)pl->grad_s, pl->tgt_perm, pl->s,
                                         po, ho, dtype == FS_F64, st));
     }
