@@ -730,6 +730,31 @@ void plan_destroy(fs_plan *pl)
 
 namespace {
 
+// Room for min(nrhs, kRhsGroup) charge vectors in the grid, the spectrum and the sums, where they are
+// evaluated together.  Without memory for it the plan goes on one vector at a time.
+template <typename real> fs_status reserve_rhs(fs_plan *pl, int nrhs)
+{
+    const int want = std::min(nrhs, kRhsGroup);
+    if (want <= pl->rhs_cap || pl->events || pl->spread_direct || (sizeof(real) == 4 && !pl->overlap))
+        return FS_OK;
+    const size_t grid_bytes = (size_t)pl->n_a * pl->pitch * sizeof(real);
+    const size_t spec_bytes = (size_t)(pl->n / 2 + 1) * pl->ld * 2 * sizeof(real);
+    auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
+    const size_t spec_at = up(grid_bytes * want), sums_at = spec_at + up(spec_bytes * want);
+    // one allocation; the single-vector buffers stay until the plan is destroyed (freeing them here
+    // would wait for the device)
+    unsigned char *p = nullptr;
+    if (pl->alloc(&p, sums_at + (size_t)pl->sums_n * 4 * want * sizeof(real)) != FS_OK)
+        return FS_OK;
+    pl->grid = p;
+    pl->spec = p + spec_at;
+    pl->phi_s = p + sums_at;
+    pl->grad_s = (unsigned char *)pl->phi_s + (size_t)pl->sums_n * want * sizeof(real);
+    pl->coinc = (unsigned char *)pl->phi_s + (size_t)pl->sums_n * 3 * want * sizeof(real);
+    pl->rhs_cap = want;
+    return FS_OK;
+}
+
 // Sorted-charge storage for nrhs vectors (kept when large enough).
 template <typename real> fs_status reserve_charges(fs_plan *pl, int nrhs)
 {
@@ -741,6 +766,7 @@ template <typename real> fs_status reserve_charges(fs_plan *pl, int nrhs)
         FS_TRY(pl->alloc_bytes(&pl->q_sorted, (size_t)std::max<int64_t>(pl->M, 1) * nrhs * sizeof(real)));
         FS_TRY(pl->alloc(&pl->q_sum, nrhs));
         pl->nrhs_cap = nrhs;
+        FS_TRY(reserve_rhs<real>(pl, nrhs));
     }
     return FS_OK;
 }
@@ -761,77 +787,101 @@ template <typename real> fs_status set_charges_t(fs_plan *pl, const void *q, fs_
 }
 
 // Step (c): the grid is zeroed and the charges spread into it, through shared-memory tiles or
-// (sparse plans, FS_FLAG_SPREAD_DIRECT) with global atomics and a compensation plane.
-template <typename real> fs_status spread_forward(fs_plan *pl, const real *q, cudaStream_t st)
+// (sparse plans, FS_FLAG_SPREAD_DIRECT: one vector) with global atomics and a compensation plane.
+template <typename real> fs_status spread_forward(fs_plan *pl, const real *q, int nrhs, cudaStream_t st)
 {
-    const size_t grid_bytes = (size_t)pl->n_a * pl->pitch * sizeof(real);
-    FS_CUDA(cudaMemsetAsync(pl->grid, 0, grid_bytes, st));
+    const int64_t grid_n = (int64_t)pl->n_a * pl->pitch;
+    FS_CUDA(cudaMemsetAsync(pl->grid, 0, (size_t)grid_n * nrhs * sizeof(real), st));
     if (!pl->spread_direct) {
-        FS_CUDA(launch_spread<real>(pl->items, pl->n_items, pl->cg, pl->m, pl->src_base, pl->src_frac, q, win_poly<real>(pl),
-                                    (real *)pl->grid, pl->pitch, pl->n_a, pl->kahan, st));
+        FS_CUDA(launch_spread<real>(pl->items, pl->n_items, pl->cg, pl->m, pl->src_base, pl->src_frac, q,
+                                    win_poly<real>(pl), (real *)pl->grid, pl->pitch, pl->n_a, pl->kahan, nrhs, pl->M,
+                                    grid_n, st));
         return FS_OK;
     }
     if (pl->grid_comp)
-        FS_CUDA(cudaMemsetAsync(pl->grid_comp, 0, grid_bytes, st));
-    FS_CUDA(launch_spread_direct<real>(pl->M, pl->m, pl->src_base, pl->src_frac, q, make_window<real>(pl), win_poly<real>(pl), (real *)pl->grid,
-                                       (real *)pl->grid_comp, pl->pitch, pl->n_a, pl->kahan, st));
+        FS_CUDA(cudaMemsetAsync(pl->grid_comp, 0, (size_t)grid_n * sizeof(real), st));
+    FS_CUDA(launch_spread_direct<real>(pl->M, pl->m, pl->src_base, pl->src_frac, q, make_window<real>(pl),
+                                       win_poly<real>(pl), (real *)pl->grid, (real *)pl->grid_comp, pl->pitch, pl->n_a,
+                                       pl->kahan, st));
     return FS_OK;
 }
 
+// The FP32 near field of `nrhs` charge vectors stored in phi_s, grad_s and coinc (plans with a second
+// stream), or added to one vector's.
+fs_status near_forward32(fs_plan *pl, const float *q, int nrhs, bool assign, cudaStream_t st)
+{
+    const NearParams<float> np = make_near<float>(pl);
+    float *phi = (float *)pl->phi_s, *grad = (float *)pl->grad_s, *coinc = (float *)pl->coinc;
+    const int64_t n = pl->sums_n;
+    if (pl->src_major) {
+        // source items add with atomics: zero the sums first (one block)
+        if (assign)
+            FS_CUDA(cudaMemsetAsync(phi, 0, sizeof(float) * 4 * (size_t)n * pl->rhs_cap, st));
+        else
+            FS_CUDA(cudaMemsetAsync(coinc, 0, sizeof(float) * (size_t)n, st));
+        for (int r = 0; r < nrhs; ++r)
+            FS_CUDA(launch_near_src32(pl->n_src_near_items, pl->src_near_items, pl->src_base, pl->src_pos32,
+                                      pl->src_lo32, pl->tgt_pos32, pl->tgt_lo32, pl->tgt_start, pl->cg, q + r * pl->M, np,
+                                      phi + r * n, grad + 2 * r * n, coinc + r * n, st));
+    } else if (nrhs == 1) {
+        FS_CUDA(launch_near32(pl->n_near_items, pl->near_items, pl->tgt_cap, pl->tgt_base, pl->tgt_pos32,
+                              pl->tgt_lo32, pl->src_pos32, pl->src_lo32, pl->src_start, pl->cg, q, np, phi, grad, coinc,
+                              assign, st));
+    } else {
+        FS_CUDA(launch_near32_rhs(pl->n_near_items, pl->near_items, pl->tgt_cap, pl->tgt_base, pl->tgt_pos32,
+                                  pl->tgt_lo32, pl->src_pos32, pl->src_lo32, pl->src_start, pl->cg, q, np, phi, grad,
+                                  coinc, nrhs, pl->M, n, st));
+    }
+    return FS_OK;
+}
+
+// Up to rhs_cap charge vectors go through each stage together: one launch per stage, and one traversal
+// of the near field's pairs (three vectors, 100,003 sources, 65,537 targets: 257 -> 152 us).
 template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dtype dtype)
 {
     cudaStream_t st = pl->stream;
-    const NearParams<real> np = make_near<real>(pl);
     using C = typename Cplx<real>::type;
     const double shift = std::log(pl->s) / (2.0 * kPi);
     const size_t osz = dtype == FS_F64 ? 8 : 4;
-    for (int r = 0; r < pl->nrhs; ++r) {
-        const bool rec = pl->events && r == pl->nrhs - 1;
-        const real *q = (const real *)pl->q_sorted + (int64_t)r * pl->M;
+    const int64_t grid_n = (int64_t)pl->n_a * pl->pitch, spec_n = (int64_t)(pl->n / 2 + 1) * pl->ld;
+    for (int r0 = 0; r0 < pl->nrhs; r0 += pl->rhs_cap) {
+        const int R = std::min(pl->rhs_cap, pl->nrhs - r0);
+        const bool rec = pl->events && r0 + R == pl->nrhs;
+        const real *q = (const real *)pl->q_sorted + (int64_t)r0 * pl->M;
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[0], st));
         if (pl->overlap)
             FS_CUDA(cudaEventRecord(pl->ev_fork, st));   // the charges are in
-        FS_TRY(spread_forward<real>(pl, q, st));
-        if (pl->overlap) {
-            // the near field (stored, not added) on the second stream, submitted after the
-            // spreading so that the spreading's blocks are scheduled first
-            FS_CUDA(cudaStreamWaitEvent(pl->aux, pl->ev_fork, 0));
-            if (rec)
-                FS_CUDA(cudaEventRecord(pl->ev_n0, pl->aux));
-            if (pl->src_major) {
-                // source items add with atomics: zero the near-field sums first (one block)
-                FS_CUDA(cudaMemsetAsync(pl->phi_s, 0, sizeof(float) * 4 * (size_t)pl->sums_n, pl->aux));
-                FS_CUDA(launch_near_src32(pl->n_src_near_items, pl->src_near_items, pl->src_base, pl->src_pos32,
-                                          pl->src_lo32, pl->tgt_pos32, pl->tgt_lo32, pl->tgt_start, pl->cg,
-                                          (const float *)q, make_near<float>(pl), (float *)pl->phi_s,
-                                          (float *)pl->grad_s, (float *)pl->coinc, pl->aux));
-            } else {
-                FS_CUDA(launch_near32(pl->n_near_items, pl->near_items, pl->tgt_cap, pl->tgt_base, pl->tgt_pos32, pl->tgt_lo32,
-                                      pl->src_pos32, pl->src_lo32, pl->src_start, pl->cg, (const float *)q,
-                                      make_near<float>(pl), (float *)pl->phi_s, (float *)pl->grad_s,
-                                      (float *)pl->coinc, true, pl->aux));
+        FS_TRY(spread_forward<real>(pl, q, R, st));
+        if constexpr (sizeof(real) == 4) {
+            if (pl->overlap) {
+                // the near field (stored, not added) on the second stream, submitted after the
+                // spreading so that the spreading's blocks are scheduled first
+                FS_CUDA(cudaStreamWaitEvent(pl->aux, pl->ev_fork, 0));
+                if (rec)
+                    FS_CUDA(cudaEventRecord(pl->ev_n0, pl->aux));
+                FS_TRY(near_forward32(pl, q, R, true, pl->aux));
+                if (rec)
+                    FS_CUDA(cudaEventRecord(pl->ev_n1, pl->aux));
+                FS_CUDA(cudaEventRecord(pl->ev_join, pl->aux));
             }
-            if (rec)
-                FS_CUDA(cudaEventRecord(pl->ev_n1, pl->aux));
-            FS_CUDA(cudaEventRecord(pl->ev_join, pl->aux));
         }
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[1], st));
         FS_CUDA(launch_fft_rows_fwd<real>((const real *)pl->grid, pl->pitch, pl->n_a, pl->n_os, pl->n / 2,
-                                          (C *)pl->spec, pl->ld, (const C *)pl->tw, st));
+                                          (C *)pl->spec, pl->ld, (const C *)pl->tw, R, grid_n, spec_n, st));
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[2], st));
         FS_CUDA(launch_fft_cols<real>((C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n, (const real *)pl->mul,
-                                      (const C *)pl->tw, st));
+                                      (const C *)pl->tw, R, spec_n, st));
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[3], st));
         FS_CUDA(launch_fft_rows_inv<real>((const C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n / 2,
-                                          (real *)pl->grid, pl->pitch, (const C *)pl->tw, st));
+                                          (real *)pl->grid, pl->pitch, (const C *)pl->tw, R, grid_n, spec_n, st));
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[4], st));
-        void *po = phi ? (unsigned char *)phi + (size_t)r * pl->N * osz : nullptr;
-        void *ho = H ? (unsigned char *)H + (size_t)r * pl->N * 2 * osz : nullptr;
+        auto out_phi = [&](int r) { return phi ? (unsigned char *)phi + (size_t)(r0 + r) * pl->N * osz : nullptr; };
+        auto out_h = [&](int r) { return H ? (unsigned char *)H + (size_t)(r0 + r) * pl->N * 2 * osz : nullptr; };
         if (pl->overlap) {
             FS_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
             if (rec)
@@ -841,8 +891,8 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
             FS_CUDA(launch_interp_out<real>(pl->N, pl->m, pl->tgt_base, pl->tgt_frac, win_poly<real>(pl),
                                             (const real *)pl->grid, pl->pitch, (real)pl->n_os,
                                             (const real *)pl->phi_s, (const real *)pl->grad_s,
-                                            (const real *)pl->coinc, pl->tgt_perm, shift, pl->q_sum + r, pl->s, po, ho,
-                                            dtype == FS_F64, st));
+                                            (const real *)pl->coinc, pl->tgt_perm, shift, pl->q_sum + r0, pl->s,
+                                            out_phi(0), out_h(0), dtype == FS_F64, R, grid_n, pl->sums_n, st));
             if (rec) {
                 FS_CUDA(cudaEventRecord(pl->ev[5], st));
                 FS_CUDA(cudaEventRecord(pl->ev[6], st));
@@ -850,30 +900,24 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
             }
             continue;
         }
-        FS_CUDA(launch_interp<real>(pl->N, pl->m, pl->tgt_base, pl->tgt_frac, win_poly<real>(pl), (const real *)pl->grid, pl->pitch,
-                                    (real)pl->n_os, (real *)pl->phi_s, (real *)pl->grad_s, false, st));
-        if (rec)
-            FS_CUDA(cudaEventRecord(pl->ev[5], st));
-        if constexpr (sizeof(real) == 4) {
-            if (pl->src_major) {
-                FS_CUDA(cudaMemsetAsync(pl->coinc, 0, sizeof(float) * (size_t)std::max<int64_t>(pl->N, 1), st));
-                FS_CUDA(launch_near_src32(pl->n_src_near_items, pl->src_near_items, pl->src_base, pl->src_pos32,
-                                          pl->src_lo32, pl->tgt_pos32, pl->tgt_lo32, pl->tgt_start, pl->cg,
-                                          (const float *)q, np, (float *)pl->phi_s, (float *)pl->grad_s,
-                                          (float *)pl->coinc, st));
-            } else {
-                FS_CUDA(launch_near32(pl->n_near_items, pl->near_items, pl->tgt_cap, pl->tgt_base, pl->tgt_pos32, pl->tgt_lo32,
-                                      pl->src_pos32, pl->src_lo32, pl->src_start, pl->cg, (const float *)q, np,
-                                      (float *)pl->phi_s, (float *)pl->grad_s, (float *)pl->coinc, false, st));
-            }
-        } else
-            FS_CUDA(launch_near64(pl->N, near64_sides(pl, true), pl->cg, (const double *)q, np, (double *)pl->phi_s, (double *)pl->grad_s,
-                                  (double *)pl->coinc, st));
-        if (rec)
-            FS_CUDA(cudaEventRecord(pl->ev[6], st));
-        FS_CUDA(launch_unpermute<real>(pl->N, (const real *)pl->phi_s, (const real *)pl->grad_s,
-                                       (const real *)pl->coinc, pl->tgt_perm, shift, pl->q_sum + r, pl->s, po, ho,
-                                       dtype == FS_F64, st));
+        for (int r = 0; r < R; ++r) {
+            FS_CUDA(launch_interp<real>(pl->N, pl->m, pl->tgt_base, pl->tgt_frac, win_poly<real>(pl),
+                                        (const real *)pl->grid + r * grid_n, pl->pitch, (real)pl->n_os,
+                                        (real *)pl->phi_s, (real *)pl->grad_s, false, st));
+            if (rec)
+                FS_CUDA(cudaEventRecord(pl->ev[5], st));
+            if constexpr (sizeof(real) == 4)
+                FS_TRY(near_forward32(pl, q + r * pl->M, 1, false, st));
+            else
+                FS_CUDA(launch_near64(pl->N, near64_sides(pl, true), pl->cg, (const double *)q + r * pl->M,
+                                      make_near<real>(pl), (double *)pl->phi_s, (double *)pl->grad_s,
+                                      (double *)pl->coinc, st));
+            if (rec)
+                FS_CUDA(cudaEventRecord(pl->ev[6], st));
+            FS_CUDA(launch_unpermute<real>(pl->N, (const real *)pl->phi_s, (const real *)pl->grad_s,
+                                           (const real *)pl->coinc, pl->tgt_perm, shift, pl->q_sum + r0 + r, pl->s,
+                                           out_phi(r), out_h(r), dtype == FS_F64, st));
+        }
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[7], st));
     }
@@ -940,11 +984,11 @@ template <typename real> fs_status spectral_pipeline(fs_plan *pl)
     using C = typename Cplx<real>::type;
     cudaStream_t st = pl->stream;
     FS_CUDA(launch_fft_rows_fwd<real>((const real *)pl->grid, pl->pitch, pl->n_a, pl->n_os, pl->n / 2, (C *)pl->spec,
-                                      pl->ld, (const C *)pl->tw, st));
+                                      pl->ld, (const C *)pl->tw, 1, 0, 0, st));
     FS_CUDA(launch_fft_cols<real>((C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n, (const real *)pl->mul,
-                                  (const C *)pl->tw, st));
+                                  (const C *)pl->tw, 1, 0, st));
     FS_CUDA(launch_fft_rows_inv<real>((const C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n / 2, (real *)pl->grid,
-                                      pl->pitch, (const C *)pl->tw, st));
+                                      pl->pitch, (const C *)pl->tw, 1, 0, 0, st));
     return FS_OK;
 }
 
@@ -990,7 +1034,7 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
                     FS_CUDA(cudaEventRecord(pl->ev_join, pl->aux));
                 }
             }
-            FS_TRY(spread_forward<real>(pl, q, st));
+            FS_TRY(spread_forward<real>(pl, q, 1, st));
             FS_TRY(spectral_pipeline<real>(pl));
             if (ovl)
                 FS_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));

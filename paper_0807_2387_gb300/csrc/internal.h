@@ -357,7 +357,7 @@ cudaError_t launch_near_count(const double2 *tgt_pos, const int *tgt_base, int64
 template <typename real>
 cudaError_t launch_spread(const SpreadItem *items, int n_items, CellGrid cg, int m, const int *base,
                           const void *frac, const real *q, const WinPoly<real> &wp, real *grid,
-                          int pitch, int n_a, bool kahan, cudaStream_t st);
+                          int pitch, int n_a, bool kahan, int nrhs, int64_t q_stride, int64_t grid_stride, cudaStream_t st);
 // direct spreading (global atomics, no tiles); comp: compensation plane of the grid's size
 // (FP32 with compensation; folded into the grid at the end), may be null otherwise
 template <typename real>
@@ -375,7 +375,7 @@ template <typename real>
 cudaError_t launch_interp_out(int64_t N, int m, const int *base, const void *frac, const WinPoly<real> &wp, const real *grid, int pitch, real n_os, const real *phi_s,
                               const real *grad_s, const real *coinc, const int *perm, double shift,
                               const double *q_sum, double s, void *phi_out, void *H_out, int out_is_f64,
-                              cudaStream_t st);
+                              int nrhs, int64_t grid_stride, int64_t n_stride, cudaStream_t st);
 
 template <typename real>
 cudaError_t launch_spread_dip(const SpreadItem *items, int n_items, CellGrid cg, int m, const int *base,
@@ -386,7 +386,8 @@ template <typename real>
 cudaError_t launch_interp_hess(int64_t N, int m, const int *base, const void *frac, const WinPoly<real> &wp, const real *grid, int pitch, real n_os, real *grad_s,
                                real *hess_s, bool acc, cudaStream_t st);
 
-// ---- FFT and spectral multiply (kernels_fft.cu)
+// ---- FFT and spectral multiply (kernels_fft.cu); nrhs charge vectors in one launch, grids and spectra
+// at their strides
 // Radix of the Stockham pass that follows the first L / rest points: 8 while 8 divides the
 // rest, then one pass of 4 or 2.
 __host__ __device__ constexpr int fft_pass_radix(int rest) { return rest % 8 == 0 ? 8 : (rest == 4 ? 4 : 2); }
@@ -397,13 +398,15 @@ template <typename real> void fft_twiddle_table(int L, real *re_im);
 template <typename real>
 cudaError_t launch_fft_rows_fwd(const real *grid, int pitch, int n_a, int L, int n_half,
                                 typename Cplx<real>::type *spec, int ld, const typename Cplx<real>::type *tw,
-                                cudaStream_t st);
+                                int nrhs, int64_t grid_stride, int64_t spec_stride, cudaStream_t st);
 template <typename real>
 cudaError_t launch_fft_cols(typename Cplx<real>::type *spec, int ld, int n_a, int L, int n,
-                            const real *mul, const typename Cplx<real>::type *tw, cudaStream_t st);
+                            const real *mul, const typename Cplx<real>::type *tw, int nrhs, int64_t spec_stride,
+                            cudaStream_t st);
 template <typename real>
 cudaError_t launch_fft_rows_inv(const typename Cplx<real>::type *spec, int ld, int n_a, int L, int n_half,
-                                real *grid, int pitch, const typename Cplx<real>::type *tw, cudaStream_t st);
+                                real *grid, int pitch, const typename Cplx<real>::type *tw, int nrhs, int64_t grid_stride,
+                                int64_t spec_stride, cudaStream_t st);
 cudaError_t launch_kernel_samples(double2 *samp, int n, KernelParams kp, cudaStream_t st);
 cudaError_t launch_fft_lines_c64(double2 *data, int lines, int L, const double2 *tw, cudaStream_t st);
 cudaError_t launch_transpose_c64(const double2 *in, double2 *out, int n, cudaStream_t st);
@@ -420,6 +423,12 @@ cudaError_t launch_near32(int64_t n_items, const int2 *items, int lanes, const i
                           const float2 *tgt_lo, const float2 *src_hi, const float2 *src_lo, const int *src_start,
                           CellGrid cg, const float *q, NearParams<float> np, float *phi_s, float *grad_s, float *coinc,
                           bool assign, cudaStream_t st);
+// two to four charge vectors at once, storing their sums: vector r reads q + r q_stride and writes phi_s and
+// coinc at r n_stride, grad_s at 2 r n_stride (kernels_near_rhs.cu)
+cudaError_t launch_near32_rhs(int64_t n_items, const int2 *items, int lanes, const int *tgt_base, const float2 *tgt_hi,
+                              const float2 *tgt_lo, const float2 *src_hi, const float2 *src_lo, const int *src_start,
+                              CellGrid cg, const float *q, NearParams<float> np, float *phi_s, float *grad_s,
+                              float *coinc, int nrhs, int64_t q_stride, int64_t n_stride, cudaStream_t st);
 // source-major variant for plans with many more sources than targets: items (first source,
 // count <= 64) per warp; phi_s, grad_s and coinc (zeroed by the caller) receive atomic adds
 cudaError_t launch_near_src32(int64_t n_items, const int2 *items, const int *src_base, const float2 *src_hi,

@@ -655,39 +655,45 @@ __host__ __device__ constexpr int fft_threads(int L) { return L / 4 > 256 ? 256 
 
 // The three 2D kernels.  LC > 0 fixes the line length at compile time (one instance per
 // length the plans use, 256 .. 4096 points), LC = 0 takes it at run time.
+// blockIdx.y: the charge vector (grids and spectra at their strides).
 template <typename real, int LC>
 __global__ void __launch_bounds__(256) k_fft_rows_fwd(const real *__restrict__ grid, int pitch, int n_a, int L,
                                                       int n_half, cplx<real> *__restrict__ spec, int ld,
-                                                      const cplx<real> *__restrict__ tw)
+                                                      const cplx<real> *__restrict__ tw, int64_t grid_stride,
+                                                      int64_t spec_stride)
 {
     constexpr int NT = LC ? fft_threads(LC) : 0;
     extern __shared__ unsigned char smem_raw[];
     cplx<real> *a = reinterpret_cast<cplx<real> *>(smem_raw);
     cplx<real> *s_tw = stage_twiddles<real, LC, NT>(a + 2 * L, tw, L);   // published by the unit's first barrier
-    rows_fwd_unit<real, LC, NT>(blockIdx.x, grid, pitch, n_a, L, n_half, spec, ld, s_tw, a, a + L);
+    rows_fwd_unit<real, LC, NT>(blockIdx.x, grid + blockIdx.y * grid_stride, pitch, n_a, L, n_half,
+                                spec + blockIdx.y * spec_stride, ld, s_tw, a, a + L);
 }
 
 template <typename real, int LC>
 __global__ void __launch_bounds__(256) k_fft_cols(cplx<real> *__restrict__ spec, int ld, int n_a, int L, int n,
-                                                  const real *__restrict__ mul, const cplx<real> *__restrict__ tw)
+                                                  const real *__restrict__ mul, const cplx<real> *__restrict__ tw,
+                                                  int64_t spec_stride)
 {
     constexpr int NT = LC ? fft_threads(LC) : 0;
     extern __shared__ unsigned char smem_raw[];
     cplx<real> *a = reinterpret_cast<cplx<real> *>(smem_raw);
     cplx<real> *s_tw = stage_twiddles<real, LC, NT>(a + 2 * L, tw, L);
-    cols_unit<real, false, LC, NT>(blockIdx.x, spec, ld, n_a, L, n, mul, s_tw, a, a + L);
+    cols_unit<real, false, LC, NT>(blockIdx.x, spec + blockIdx.y * spec_stride, ld, n_a, L, n, mul, s_tw, a, a + L);
 }
 
 template <typename real, int LC>
 __global__ void __launch_bounds__(256) k_fft_rows_inv(const cplx<real> *__restrict__ spec, int ld, int n_a, int L,
                                                       int n_half, real *__restrict__ grid, int pitch,
-                                                      const cplx<real> *__restrict__ tw)
+                                                      const cplx<real> *__restrict__ tw, int64_t grid_stride,
+                                                      int64_t spec_stride)
 {
     constexpr int NT = LC ? fft_threads(LC) : 0;
     extern __shared__ unsigned char smem_raw[];
     cplx<real> *a = reinterpret_cast<cplx<real> *>(smem_raw);
     cplx<real> *s_tw = stage_twiddles<real, LC, NT>(a + 2 * L, tw, L);
-    rows_inv_unit<real, false, LC, NT>(blockIdx.x, spec, ld, n_a, L, n_half, grid, pitch, s_tw, a, a + L);
+    rows_inv_unit<real, false, LC, NT>(blockIdx.x, spec + blockIdx.y * spec_stride, ld, n_a, L, n_half,
+                                       grid + blockIdx.y * grid_stride, pitch, s_tw, a, a + L);
 }
 
 // Thread 0 waits until *ctr >= target; the wait ends early (failed) when the error word is
@@ -1099,7 +1105,7 @@ template <typename F> cudaError_t with_line_length(int L, F &&f)
 
 template <typename real>
 cudaError_t launch_fft_rows_fwd(const real *grid, int pitch, int n_a, int L, int n_half, cplx<real> *spec, int ld,
-                                const cplx<real> *tw, cudaStream_t st)
+                                const cplx<real> *tw, int nrhs, int64_t grid_stride, int64_t spec_stride, cudaStream_t st)
 {
     const size_t smem = 3 * (size_t)L * sizeof(cplx<real>);   // two line buffers and the twiddles
     return with_line_length(L, [&](auto lc) {
@@ -1107,15 +1113,15 @@ cudaError_t launch_fft_rows_fwd(const real *grid, int pitch, int n_a, int L, int
         cudaError_t e = set_smem(k_fft_rows_fwd<real, LC>, smem);
         if (e != cudaSuccess)
             return e;
-        k_fft_rows_fwd<real, LC><<<(n_a + 1) / 2, fft_threads(L), smem, st>>>(grid, pitch, n_a, L, n_half, spec, ld,
-                                                                              tw);
+        k_fft_rows_fwd<real, LC><<<dim3((n_a + 1) / 2, nrhs), fft_threads(L), smem, st>>>(grid, pitch, n_a, L, n_half, spec,
+                                                                                            ld, tw, grid_stride, spec_stride);
         return cudaGetLastError();
     });
 }
 
 template <typename real>
 cudaError_t launch_fft_cols(cplx<real> *spec, int ld, int n_a, int L, int n, const real *mul, const cplx<real> *tw,
-                            cudaStream_t st)
+                            int nrhs, int64_t spec_stride, cudaStream_t st)
 {
     const size_t smem = 3 * (size_t)L * sizeof(cplx<real>);   // two line buffers and the twiddles
     return with_line_length(L, [&](auto lc) {
@@ -1123,14 +1129,15 @@ cudaError_t launch_fft_cols(cplx<real> *spec, int ld, int n_a, int L, int n, con
         cudaError_t e = set_smem(k_fft_cols<real, LC>, smem);
         if (e != cudaSuccess)
             return e;
-        k_fft_cols<real, LC><<<n / 2 + 1, fft_threads(L), smem, st>>>(spec, ld, n_a, L, n, mul, tw);
+        k_fft_cols<real, LC><<<dim3(n / 2 + 1, nrhs), fft_threads(L), smem, st>>>(spec, ld, n_a, L, n, mul, tw, spec_stride);
         return cudaGetLastError();
     });
 }
 
 template <typename real>
 cudaError_t launch_fft_rows_inv(const cplx<real> *spec, int ld, int n_a, int L, int n_half, real *grid, int pitch,
-                                const cplx<real> *tw, cudaStream_t st)
+                                const cplx<real> *tw, int nrhs, int64_t grid_stride, int64_t spec_stride,
+                                cudaStream_t st)
 {
     const size_t smem = 3 * (size_t)L * sizeof(cplx<real>);   // two line buffers and the twiddles
     return with_line_length(L, [&](auto lc) {
@@ -1138,8 +1145,8 @@ cudaError_t launch_fft_rows_inv(const cplx<real> *spec, int ld, int n_a, int L, 
         cudaError_t e = set_smem(k_fft_rows_inv<real, LC>, smem);
         if (e != cudaSuccess)
             return e;
-        k_fft_rows_inv<real, LC><<<(n_a + 1) / 2, fft_threads(L), smem, st>>>(spec, ld, n_a, L, n_half, grid, pitch,
-                                                                              tw);
+        k_fft_rows_inv<real, LC><<<dim3((n_a + 1) / 2, nrhs), fft_threads(L), smem, st>>>(spec, ld, n_a, L, n_half, grid,
+                                                                                            pitch, tw, grid_stride, spec_stride);
         return cudaGetLastError();
     });
 }
@@ -1279,17 +1286,18 @@ template <typename real> void fft_twiddle_table(int L, real *re_im)
 template void fft_twiddle_table<float>(int, float *);
 template void fft_twiddle_table<double>(int, double *);
 
-template cudaError_t launch_fft_rows_fwd<float>(const float *, int, int, int, int, float2 *, int, const float2 *,
-                                                cudaStream_t);
-template cudaError_t launch_fft_rows_fwd<double>(const double *, int, int, int, int, double2 *, int, const double2 *,
-                                                 cudaStream_t);
-template cudaError_t launch_fft_cols<float>(float2 *, int, int, int, int, const float *, const float2 *, cudaStream_t);
-template cudaError_t launch_fft_cols<double>(double2 *, int, int, int, int, const double *, const double2 *,
-                                             cudaStream_t);
-template cudaError_t launch_fft_rows_inv<float>(const float2 *, int, int, int, int, float *, int, const float2 *,
-                                                cudaStream_t);
-template cudaError_t launch_fft_rows_inv<double>(const double2 *, int, int, int, int, double *, int, const double2 *,
-                                                 cudaStream_t);
+template cudaError_t launch_fft_rows_fwd<float>(const float *, int, int, int, int, float2 *, int, const float2 *, int,
+                                                int64_t, int64_t, cudaStream_t);
+template cudaError_t launch_fft_rows_fwd<double>(const double *, int, int, int, int, double2 *, int, const double2 *, int,
+                                                int64_t, int64_t, cudaStream_t);
+template cudaError_t launch_fft_cols<float>(float2 *, int, int, int, int, const float *, const float2 *, int, int64_t,
+                                            cudaStream_t);
+template cudaError_t launch_fft_cols<double>(double2 *, int, int, int, int, const double *, const double2 *, int, int64_t,
+                                            cudaStream_t);
+template cudaError_t launch_fft_rows_inv<float>(const float2 *, int, int, int, int, float *, int, const float2 *, int,
+                                                int64_t, int64_t, cudaStream_t);
+template cudaError_t launch_fft_rows_inv<double>(const double2 *, int, int, int, int, double *, int, const double2 *, int,
+                                                int64_t, int64_t, cudaStream_t);
 template cudaError_t launch_build_mul<float>(const double2 *, int, const double *, float *, cudaStream_t);
 template cudaError_t launch_build_mul<double>(const double2 *, int, const double *, double *, cudaStream_t);
 

@@ -24,6 +24,7 @@
 #include "internal.h"
 #include "output.cuh"
 #include "near64.cuh"
+#include "near_fwd.cuh"
 
 namespace fs {
 
@@ -93,155 +94,6 @@ __global__ void __launch_bounds__(32 * kNear64Warps) k_batch_near64(const BatchI
     for (int64_t k = first + w; k < first + per_block && k < N; k += kNear64Warps)
         near64_point(k, lane, sd, cg, np, tab, op, queue[w]);
 }
-
-// Forward correction at the targets for R right-hand sides at once (the pair geometry, the
-// log and the gradient coefficient are shared): phi += q f, grad += q c d for two candidates per
-// packed operation; the factor c_ln of f (near_g2) and rc eps_I of c are applied once at the
-// store (d arrives in units of eps_I).  With one right-hand side the sums are split into partial
-// sums per list evaluation; with several the registers go to the extra accumulators instead.
-// Right-hand side r reads q + r q_stride and writes at r n_stride.
-template <int P, int R, bool BATCH = false> struct NearFwd {
-    static constexpr int kMinBlocks = (R == 1 && !BATCH) ? 6 : 4;   // of four warps per SM: up to 80 and 128 registers
-    static constexpr int kUnroll = BATCH ? 4 : 2;
-    // |w - 1|^(p-1) / w, the gradient coefficient over rc up to the sign (-1)^(p-1) (applied at the
-    // store), as 2^((p-1) log2(1 - w) - log2 w) (log2 w is shared with the value; w = 1 gives 2^-inf):
-    // four MUFU operations and one FMA a pair of candidates, against two and the power's
-    // multiplications.  2.26 -> 2.19 ms at 2^20 points (p = 8) against alternating the two.  Several
-    // right-hand sides add FMA work that hides the difference (batched replay the same either way).
-    static constexpr bool kExp2 = P >= 5 && !BATCH;
-    static constexpr bool kRows = R == 1;
-    static constexpr bool kSat = P >= 2;   // f(1) = 0 and (w - 1)^(p-1) = 0: clamping w masks a pair
-    static constexpr float kPhi = P >= 2 ? kLnCoef : 1.f;   // unit of the phi sums
-    const float *__restrict__ q;
-    float *__restrict__ phi_s;
-    float *__restrict__ grad_s;
-    float *__restrict__ coinc;
-    int64_t q_stride, n_stride;
-    float rcoef;   // rc eps_I: the pair differences arrive in units of eps_I
-    bool assign;   // store phi_s / grad_s instead of adding (the far field is added later)
-    float2 qj[R];
-    float2 phi[R], gx[R], gy[R];
-    float qc[R];
-    float2 rphi[kRows ? R : 1], rgx[kRows ? R : 1], rgy[kRows ? R : 1];
-
-    __device__ __forceinline__ float2 &acc_phi(int r) { return kRows ? rphi[0] : phi[r]; }
-    __device__ __forceinline__ float2 &acc_gx(int r) { return kRows ? rgx[0] : gx[r]; }
-    __device__ __forceinline__ float2 &acc_gy(int r) { return kRows ? rgy[0] : gy[r]; }
-
-    __device__ __forceinline__ void init()
-    {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            phi[r] = gx[r] = gy[r] = f2(0.f);
-            qc[r] = 0.f;
-        }
-    }
-    // candidate-list traversal: the R charges of source j, and those of a pair of candidates
-    static constexpr int kR = R;
-    __device__ __forceinline__ void fetch(int j, float (&v)[R]) const
-    {
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            v[r] = __ldg(q + r * q_stride + j);
-    }
-    __device__ __forceinline__ void set_q(const float2 (&v)[R])
-    {
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            qj[r] = v[r];
-    }
-    __device__ __forceinline__ void coincident(const NearParams<float> &np, int t)
-    {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float qs = comp(qj[r], t);
-            add_comp(acc_phi(r), t, -qs * (np.beta[0] / kPhi));   // G(0) := 0 removes the far field's T_I(0)
-            qc[r] += qs;
-        }
-    }
-    __device__ __forceinline__ void pair2(const NearParams<float> &np, float2 w, float2 dx, float2 dy)
-    {
-        float2 val, coef;
-        if constexpr (P >= 2) {
-            const float2 s = fma2(w, f2(-1.f), f2(1.f)), lw = lg2_2(w);
-            val = near_g2<P>(np, w, s, lw);
-            if constexpr (kExp2)
-                coef = ex2_2(fma2(f2((float)(P - 1)), lg2_2(s), make_float2(-lw.x, -lw.y)));   // s = 0: 2^-inf
-            else
-                coef = mul2(ipow2<P - 1>(s), rcp_2(w));
-        } else {
-            val = near_f2<P>(np, w);
-            coef = rcp_2(w);
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                qj[r] = select2(w, np.eps2, qj[r]);
-        }
-        if constexpr (R >= 3) {
-            // three or more right-hand sides: the pair's gradient vector once, then one FMA per
-            // component and right-hand side (batched replay 8.01 -> 7.77 ms at three)
-            const float2 cdx = mul2(coef, dx), cdy = mul2(coef, dy);
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                acc_phi(r) = fma2(qj[r], val, acc_phi(r));
-                acc_gx(r) = fma2(qj[r], cdx, acc_gx(r));
-                acc_gy(r) = fma2(qj[r], cdy, acc_gy(r));
-            }
-        } else {
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                acc_phi(r) = fma2(qj[r], val, acc_phi(r));
-                const float2 tq = mul2(qj[r], coef);
-                acc_gx(r) = fma2(tq, dx, acc_gx(r));
-                acc_gy(r) = fma2(tq, dy, acc_gy(r));
-            }
-        }
-    }
-    __device__ __forceinline__ void row_begin()
-    {
-        if constexpr (kRows)
-            rphi[0] = rgx[0] = rgy[0] = f2(0.f);
-    }
-    __device__ __forceinline__ void row_end()
-    {
-        if constexpr (kRows) {
-            phi[0] = add2(phi[0], rphi[0]);
-            gx[0] = add2(gx[0], rgx[0]);
-            gy[0] = add2(gy[0], rgy[0]);
-        }
-    }
-    __device__ __forceinline__ void fold()
-    {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            phi[r].x += phi[r].y;
-            gx[r].x += gx[r].y;
-            gy[r].x += gy[r].y;
-        }
-    }
-    __device__ __forceinline__ void reduce(int o)
-    {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            phi[r].x = lane_add(phi[r].x, o);
-            gx[r].x = lane_add(gx[r].x, o);
-            gy[r].x = lane_add(gy[r].x, o);
-            qc[r] = lane_add(qc[r], o);
-        }
-    }
-    __device__ __forceinline__ void store(int64_t k)
-    {
-        const float rc = (P >= 2 && (P - 1) % 2 == 1) ? -rcoef : rcoef;   // coef is |w - 1|^(p-1) / w
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int64_t kk = k + r * n_stride;
-            const float p = kPhi * phi[r].x, x = rc * gx[r].x, y = rc * gy[r].x;
-            phi_s[kk] = assign ? p : phi_s[kk] + p;
-            grad_s[2 * kk] = assign ? x : grad_s[2 * kk] + x;
-            grad_s[2 * kk + 1] = assign ? y : grad_s[2 * kk + 1] + y;
-            coinc[kk] = qc[r];
-        }
-    }
-};
 
 // Plan-time statistics: pairs with r < eps_I and with r < eps_I / 8 (coincident pairs
 // included), counted by the same traversal and the same FP32 differences as the field

@@ -291,14 +291,17 @@ __global__ void __launch_bounds__(256) k_fold_comp(int64_t n, real *__restrict__
         grid[k] += comp[k];
 }
 
+// blockIdx.y: the charge vector.
 template <typename real, int M2, bool KAHAN, int TGC>
 __global__ void __launch_bounds__(kSpreadWarps * 32) k_spread(const SpreadItem *__restrict__ items, CellGrid cg,
                                                               const int *__restrict__ base,
                                                               const real2_t<real> *__restrict__ frac,
                                                               const real *__restrict__ q, WinPoly<real> wp,
-                                                              real *__restrict__ grid, int pitch, int n_a)
+                                                              real *__restrict__ grid, int pitch, int n_a,
+                                                              int64_t q_stride, int64_t grid_stride)
 {
-    spread_item<real, M2, KAHAN, TGC>(items[blockIdx.x], cg, base, frac, q, wp, grid, pitch, n_a);
+    spread_item<real, M2, KAHAN, TGC>(items[blockIdx.x], cg, base, frac, q + blockIdx.y * q_stride, wp,
+                                      grid + blockIdx.y * grid_stride, pitch, n_a);
 }
 
 // Batched spreading: items carry their instance in `pad`; blockIdx.y = right-hand side.
@@ -499,17 +502,22 @@ __global__ void __launch_bounds__(256, 3) k_interp_out(int64_t N, const int *__r
                                                     const real *__restrict__ phi_s, const real *__restrict__ grad_s,
                                                     const real *__restrict__ coinc, const int *__restrict__ perm,
                                                     double shift, const double *__restrict__ q_sum, double s,
-                                                    void *__restrict__ phi_out, void *__restrict__ H_out, int out_is_f64)
+                                                    void *__restrict__ phi_out, void *__restrict__ H_out, int out_is_f64,
+                                                    int64_t grid_stride, int64_t n_stride)
 {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= N)
         return;
+    const int r = blockIdx.y;   // the charge vector
     real phi, g1, g2;
-    interp_sums<real, M2>(k, base, frac, wp, grid, pitch, phi, g1, g2);
-    const real pt = phi_s[k] + phi;
-    const real gx = grad_s[2 * k] + n_os * g1;
-    const real gy = grad_s[2 * k + 1] + n_os * g2;
-    output_point<real>(k, pt, gx, gy, coinc[k], perm, shift, q_sum[0], s, phi_out, H_out, out_is_f64);
+    interp_sums<real, M2>(k, base, frac, wp, grid + r * grid_stride, pitch, phi, g1, g2);
+    const int64_t kk = k + r * n_stride;
+    const real pt = phi_s[kk] + phi;
+    const real gx = grad_s[2 * kk] + n_os * g1;
+    const real gy = grad_s[2 * kk + 1] + n_os * g2;
+    const int64_t o = r * N * (out_is_f64 ? 8 : 4);
+    output_point<real>(k, pt, gx, gy, coinc[kk], perm, shift, q_sum[r], s, phi_out ? (char *)phi_out + o : nullptr,
+                       H_out ? (char *)H_out + 2 * o : nullptr, out_is_f64);
 }
 
 // Batched interpolation: block -> (instance, block of its targets), blockIdx.y = right-hand side.
@@ -806,7 +814,7 @@ __global__ void __launch_bounds__(256) k_interp_hess(int64_t N, const int *__res
 template <typename real, int M2>
 cudaError_t spread_m(const SpreadItem *items, int n_items, CellGrid cg, const int *base, const void *frac,
                      const real *q, const WinPoly<real> &wp, real *grid, int pitch, int n_a, bool kahan,
-                     cudaStream_t st)
+                     int nrhs, int64_t q_stride, int64_t grid_stride, cudaStream_t st)
 {
     const int TG = cg.T * cg.cell;
     const int P = TG + M2 - 1;
@@ -816,7 +824,8 @@ cudaError_t spread_m(const SpreadItem *items, int n_items, CellGrid cg, const in
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess)
             return e;
-        kern<<<n_items, kSpreadWarps * 32, smem, st>>>(items, cg, base, fr, q, wp, grid, pitch, n_a);
+        kern<<<dim3((unsigned)n_items, (unsigned)nrhs), kSpreadWarps * 32, smem, st>>>(items, cg, base, fr, q, wp, grid,
+                                                                                     pitch, n_a, q_stride, grid_stride);
         return cudaGetLastError();
     };
     // the tile edges of the 2D plans' two tile rules (16 and 24 grid lines) compiled as constants
@@ -952,19 +961,26 @@ template <class F> cudaError_t with_width_spread(int m, F &&f)
 template <typename real>
 cudaError_t launch_spread(const SpreadItem *items, int n_items, CellGrid cg, int m, const int *base, const void *frac,
                           const real *q, const WinPoly<real> &wp, real *grid, int pitch, int n_a,
-                          bool kahan, cudaStream_t st)
+                          bool kahan, int nrhs, int64_t q_stride, int64_t grid_stride, cudaStream_t st)
 {
     if (n_items <= 0)
         return cudaSuccess;
     const bool comp = kahan && sizeof(real) == 4;
     switch (m) {
-    case 2: return spread_m<real, 4>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
-    case 3: return spread_m<real, 6>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
-    case 4: return spread_m<real, 8>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
-    case 5: return spread_m<real, 10>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
-    case 6: return spread_m<real, 12>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
-    case 7: return spread_m<real, 14>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
-    case 8: return spread_m<real, 16>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, st);
+    case 2: return spread_m<real, 4>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, nrhs, q_stride,
+                                          grid_stride, st);
+    case 3: return spread_m<real, 6>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, nrhs, q_stride,
+                                          grid_stride, st);
+    case 4: return spread_m<real, 8>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, nrhs, q_stride,
+                                          grid_stride, st);
+    case 5: return spread_m<real, 10>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, nrhs, q_stride,
+                                          grid_stride, st);
+    case 6: return spread_m<real, 12>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, nrhs, q_stride,
+                                          grid_stride, st);
+    case 7: return spread_m<real, 14>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, nrhs, q_stride,
+                                          grid_stride, st);
+    case 8: return spread_m<real, 16>(items, n_items, cg, base, frac, q, wp, grid, pitch, n_a, comp, nrhs, q_stride,
+                                          grid_stride, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -989,11 +1005,12 @@ cudaError_t launch_interp(int64_t N, int m, const int *base, const void *frac, c
 }
 
 template cudaError_t launch_spread<float>(const SpreadItem *, int, CellGrid, int, const int *, const void *,
-                                          const float *, const WindowPoly &, float *, int, int, bool,
-                                          cudaStream_t);
+                                          const float *, const WindowPoly &, float *, int, int, bool, int, int64_t,
+                                          int64_t, cudaStream_t);
 template cudaError_t launch_spread<double>(const SpreadItem *, int, CellGrid, int, const int *, const void *,
                                            const double *, const WindowPoly64 &, double *, int, int,
-                                           bool, cudaStream_t);
+                                           bool, int, int64_t,
+                                           int64_t, cudaStream_t);
 template <typename real>
 cudaError_t launch_spread_direct(int64_t M, int m, const int *base, const void *frac, const real *q, Window<real> w,
                                  const WinPoly<real> &wp, real *grid, real *comp, int pitch, int n_a, bool kahan,
@@ -1071,24 +1088,25 @@ template <typename real>
 cudaError_t launch_interp_out(int64_t N, int m, const int *base, const void *frac, const WinPoly<real> &wp,
                               const real *grid, int pitch, real n_os, const real *phi_s, const real *grad_s,
                               const real *coinc, const int *perm, double shift, const double *q_sum, double s,
-                              void *phi_out, void *H_out, int out_is_f64, cudaStream_t st)
+                              void *phi_out, void *H_out, int out_is_f64, int nrhs, int64_t grid_stride, int64_t n_stride,
+                              cudaStream_t st)
 {
     if (N <= 0)
         return cudaSuccess;
     return with_width(m, [&](auto mc) {
         constexpr int M2 = decltype(mc)::value;
-        k_interp_out<real, M2><<<(unsigned)((N + 255) / 256), 256, 0, st>>>(
+        k_interp_out<real, M2><<<dim3((unsigned)((N + 255) / 256), (unsigned)nrhs), 256, 0, st>>>(
             N, base, (const real2_t<real> *)frac, wp, grid, pitch, n_os, phi_s, grad_s, coinc, perm, shift, q_sum, s,
-            phi_out, H_out, out_is_f64);
+            phi_out, H_out, out_is_f64, grid_stride, n_stride);
         return cudaGetLastError();
     });
 }
 template cudaError_t launch_interp_out<float>(int64_t, int, const int *, const void *, const WindowPoly &, const float *, int, float, const float *,
                                               const float *, const float *, const int *, double, const double *,
-                                              double, void *, void *, int, cudaStream_t);
+                                              double, void *, void *, int, int, int64_t, int64_t, cudaStream_t);
 template cudaError_t launch_interp_out<double>(int64_t, int, const int *, const void *, const WindowPoly64 &, const double *, int, double, const double *,
                                                const double *, const double *, const int *, double, const double *,
-                                               double, void *, void *, int, cudaStream_t);
+                                               double, void *, void *, int, int, int64_t, int64_t, cudaStream_t);
 
 // Raises the dynamic shared memory limit of the batched spreading kernel (outside graph capture).
 template <typename real> cudaError_t prepare_batch_spread(int m, int max_tile, bool kahan)

@@ -25,6 +25,7 @@ struct NearCell {
     int first, count;
 };
 constexpr int kSrcMajorItem = 64;   // sources per item of the source-major near field
+constexpr int kRhsGroup = 4;       // charge vectors a plan evaluates together at most
 constexpr int kSpreadChunk = 512;   // sources per spreading work item
 // 2D plans whose occupied spreading tiles hold fewer sources than this on average spread with
 // global atomics (the plan's choice in plan_init).  Zero: on GB300 the tiles won at every
@@ -103,8 +104,11 @@ struct fs_plan {
     void *grid = nullptr, *spec = nullptr;
     void *grid_comp = nullptr;        // direct spreading (FP32): compensation plane of the grid
     bool spread_direct = false;       // spread with global atomics instead of shared-memory tiles
-    void *phi_s = nullptr, *grad_s = nullptr, *coinc = nullptr;   // one allocation, at 0, sums_n and 3 sums_n
+    // grid, spec and the near field's sums hold rhs_cap charge vectors, evaluated together; the sums
+    // are one allocation: phi_s, grad_s from rhs_cap sums_n and coinc from 3 rhs_cap sums_n on
+    void *phi_s = nullptr, *grad_s = nullptr, *coinc = nullptr;
     int64_t sums_n = 0;
+    int rhs_cap = 1;
     // charges
     void *q_sorted = nullptr;
     double *q_sum = nullptr;

@@ -62,6 +62,28 @@ def test_fp64_pair_functions_by_degree(p):
         assert rel(a, torch.tensor(b)) <= 1e-12, (name, rel(a, torch.tensor(b)))
 
 
+@pytest.mark.parametrize("nrhs", [2, 3, 4, 5, 9])
+@pytest.mark.parametrize("precision,fem", [(32, False), (64, False), (32, True)])
+def test_charge_vectors_together(nrhs, precision, fem):
+    """Several charge vectors (groups of four and the remainders) against one at a time, which differ by the
+    rounding order alone: the FP32-vs-FP64 bar of small cases for FP32, 1e-12 for FP64."""
+    import paper_0807_2387_gb300 as fs
+    rng = np.random.default_rng(nrhs)
+    dev = torch.device("cuda", 0)
+    n_src, n_tgt = (3000, 700) if fem else (1500, 1301)      # FEM-like: the near field runs over source items
+    s, t = (torch.tensor(rng.uniform(-0.17, 0.17, (k, 2)), device=dev) for k in (n_src, n_tgt))
+    q = torch.tensor(rng.standard_normal((nrhs, n_src)), device=dev)
+    plan = fs.FastSum(s, t, 64, 2.0, 5, 4 / 64, precision=precision)
+    phi, H = plan.set_charges(q).field(dtype=torch.float64)
+    tol = 1e-12 if precision == 64 else 2e-5
+    for r in range(nrhs):
+        one = fs.FastSum(s, t, 64, 2.0, 5, 4 / 64, precision=precision)
+        phi1, H1 = one.set_charges(q[r].contiguous()).field(dtype=torch.float64)
+        assert rel(phi[r], phi1) <= tol and rel(H[r], H1) <= tol, (r, rel(phi[r], phi1), rel(H[r], H1))
+    phi0, H0 = plan.set_charges(q[0].contiguous()).field(dtype=torch.float64)
+    assert rel(phi0, phi[0]) <= tol and rel(H0, H[0]) <= tol
+
+
 @pytest.mark.parametrize("ns,n,lines", [(18000, 64, 2), (15000, 64, 3), (120000, 64, 2), (120000, 64, 4.4)])
 def test_3d_run_spreading(ns, n, lines):
     """3D spreading with the sources of a cell in runs of equal base lines: few and many to a run, items of
