@@ -61,15 +61,6 @@ __device__ __forceinline__ float warp_max(float v)
     return v;
 }
 
-// dx from hi parts (a = x_hi - y_hi by TwoSum), the exact cell step and the lo parts.
-__device__ __forceinline__ float refine_diff(float xh, float yh, float off, float xl, float yl)
-{
-    const float a = xh - yh;
-    const float bb = a - xh;
-    const float e = (xh - (a - bb)) + (-yh - bb);
-    return (a + off) + (e + (xl - yl));
-}
-
 // Single MUFU operations (approximate, flush-to-zero): log2 with ~2^-22 absolute error on
 // (0, 16), and the reciprocal with ~1 ulp error; both arguments here are normal numbers.
 __device__ __forceinline__ float lg2_approx(float x)
@@ -99,7 +90,6 @@ __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 min1(float2 w) { return make_float2(fminf(w.x, 1.f), fminf(w.y, 1.f)); }
 __device__ __forceinline__ float2 lg2_2(float2 w) { return make_float2(lg2_approx(w.x), lg2_approx(w.y)); }
 __device__ __forceinline__ float2 rcp_2(float2 w) { return make_float2(rcp_approx(w.x), rcp_approx(w.y)); }
 __device__ __forceinline__ float2 ex2_2(float2 w) { return make_float2(ex2_approx(w.x), ex2_approx(w.y)); }
@@ -525,112 +515,118 @@ template <class Op> cudaError_t launch_near_list(int64_t n_items, const int2 *it
 // ---- source-major forward near field (FP32), for plans with many more sources than targets
 //
 // FEM plans put several quadrature points around every node, so a cell holds few targets and
-// a target item's box spans the whole cell.  Here a warp takes an item of at most 64 sources
-// of one cell (compact) and keeps them in shared memory as packed pairs; it reads the targets
-// of the neighbour cells within eps_I of the sources' box 32 at a time, lists those within
-// reach (a second list for those within eps_I / 8 of the box), and each lane then takes one
-// listed target and sums the item's sources on it, two per packed operation; phi, grad phi and
-// the coincident charge are added to the target with atomics.  Close pairs are refined from
-// the hi and lo parts exactly as in the target-major traversal.
-constexpr int kSrcMajorCap = 128;   // listed targets per warp and list
+// a target item's box would be large.  Here a warp takes a piece of at most 64 sources of one
+// cell and keeps them in shared memory as packed pairs; it reads the targets of the 3 x 3 cells
+// around 32 at a time, lists those within reach of the sources' box (those within eps_I / 8 of it in a
+// second list, hi + lo), and each lane then takes one listed target and sums the item's sources
+// on it, two per packed operation; phi, grad phi and the coincident charge are added to the target
+// with atomics.  The pair arithmetic is NearFwd's.
+// Measured, disc mesh of 50,311 nodes and 301,086 quadrature points (p = 6): 101 us with runs of the
+// Morton order and a branch per close pair, 72 us here (items of 32 sources 76 us).
+constexpr int kSrcMajorCap = 128, kSrcMajorClose = 64;   // listed targets per warp
 
-template <int P, bool ALT = false>
-__device__ __forceinline__ void near_src_pair(const NearParams<float> &np, float2 r2, float2 dx, float2 dy,
-                                              float2 q2, float2 &phi, float2 &gx, float2 &gy)
+struct NearSources {
+    float4 xy[32];                    // (xa, xb, ya, yb) of the pairs, units of eps_I
+    float4 hi[32], lo[32];            // the same as hi and lo parts (torus units)
+    float2 q[32];
+    float4 far[kSrcMajorCap];         // listed targets: x, y (units of eps_I), index
+    float4 close[kSrcMajorClose];     // x, y as hi parts, then lo parts (torus units)
+    int close_k[kSrcMajorClose];
+};
+
+// The sums of a lane's target: phi in units of c_ln (P >= 2), the gradient of rcoef.
+struct NearSrcSums {
+    float2 phi, gx, gy;
+};
+
+template <int P>
+__device__ __forceinline__ void near_src_pair(const NearParams<float> &np, float2 w, float2 dx, float2 dy, float2 q2,
+                                              NearSrcSums &a)
 {
-    float2 w = mul2(r2, f2(np.inv_eps2));
-    if constexpr (P >= 2)
-        w = min1(w);                                      // f(1) = 0 and (w - 1)^(p-1) = 0: masked
-    const float2 val = near_f2<P>(np, w);
-    float2 coef;
-    if constexpr (P >= 2 && ALT) {
-        // the power form with the same sign, (1 - w)^(p-1) / w: the caller alternates the two
-        // forms between consecutive sources so that the FMA and MUFU pipes share the load
-        const float2 om = add2(w, f2(-1.f));
-        coef = mul2(ipow2<P - 1>(make_float2(-om.x, -om.y)), rcp_2(w));
-    } else if constexpr (P >= 2) {
-        // |w - 1|^(p-1) / w = 2^((p-1) log2(1 - w) - log2 w) (log2 w shared with val; the sign
-        // (-1)^(p-1) is applied at the store; w = 1 gives 2^-inf = 0)
-        const float2 lw = lg2_2(w);
-        const float2 om = add2(w, f2(-1.f));   // the value's w - 1: 1 - w = -om, no add of its own
-        const float2 lo = lg2_2(make_float2(-om.x, -om.y));
-        coef = ex2_2(fma2(f2((float)(P - 1)), lo, make_float2(-lw.x, -lw.y)));
+    float2 val, coef;
+    if constexpr (P >= 2) {
+        const float2 s = fma2(w, f2(-1.f), f2(1.f)), lw = lg2_2(w);
+        val = near_g2<P>(np, w, s, lw);
+        if constexpr (P >= 5)
+            coef = ex2_2(fma2(f2((float)(P - 1)), lg2_2(s), make_float2(-lw.x, -lw.y)));
+        else
+            coef = mul2(ipow2<P - 1>(s), rcp_2(w));
     } else {
+        val = near_f2<P>(np, w);
         coef = rcp_2(w);
+        q2 = select2(w, 1.f, q2);
     }
-    if constexpr (P == 1)
-        q2 = select2(r2, np.eps2, q2);
-    phi = fma2(q2, val, phi);
+    a.phi = fma2(q2, val, a.phi);
     const float2 tq = mul2(q2, coef);
-    gx = fma2(tq, dx, gx);
-    gy = fma2(tq, dy, gy);
+    a.gx = fma2(tq, dx, a.gx);
+    a.gy = fma2(tq, dy, a.gy);
 }
 
-// One round per 32 listed targets.  Far entries: (x, y) in the item's frame and the target
-// index; close entries: (hi x, hi y, lo x, lo y) and (cell step x, cell step y, index).
-template <int P, bool CLOSE>
-__device__ __forceinline__ void near_src_eval(const float4 *s_hi, const float4 *s_lo, const float2 *s_q,
-                                              const float4 *ta, const float4 *tb, int n, int lane,
-                                              const NearParams<float> &np, float rcoef, float *__restrict__ phi_s,
-                                              float *__restrict__ grad_s, float *__restrict__ coinc)
+template <int P>
+__device__ __forceinline__ void near_src_add(const NearSrcSums &a, int k, float cq, float rcoef,
+                                             float *__restrict__ phi_s, float *__restrict__ grad_s,
+                                             float *__restrict__ coinc)
+{
+    const float rc = (P >= 2 && (P - 1) % 2 == 1) ? -rcoef : rcoef;   // coef is |w - 1|^(p-1) / w
+    atomicAdd(phi_s + k, (P >= 2 ? kLnCoef : 1.f) * (a.phi.x + a.phi.y));
+    atomicAdd(grad_s + 2 * (int64_t)k, rc * (a.gx.x + a.gx.y));
+    atomicAdd(grad_s + 2 * (int64_t)k + 1, rc * (a.gy.x + a.gy.y));
+    if (cq != 0.f)
+        atomicAdd(coinc + k, cq);
+}
+
+template <int P>
+__device__ __forceinline__ void near_src_far(const NearSources &S, int n, int pairs, int lane,
+                                             const NearParams<float> &np, float rcoef, float *__restrict__ phi_s,
+                                             float *__restrict__ grad_s, float *__restrict__ coinc)
 {
     for (int base = 0; base < n; base += 32) {
-        const int e = base + lane;
-        const bool valid = e < n;
-        const float4 A = valid ? ta[e] : make_float4(1e6f, 1e6f, 0.f, 0.f);
-        const float4 B = (CLOSE && valid) ? tb[e] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const int k = __float_as_int(CLOSE ? B.z : A.z);
-        // frame position of the target (close entries carry hi parts and the cell step)
-        const float tx = CLOSE ? A.x + B.x : A.x, ty = CLOSE ? A.y + B.y : A.y;
-        const float2 X = f2(tx), Y = f2(ty);
-        float2 phi = f2(0.f), gx = f2(0.f), gy = f2(0.f);
+        const bool valid = base + lane < n;
+        const float4 T = valid ? S.far[base + lane] : make_float4(kPadPos, kPadPos, 0.f, 0.f);
+        NearSrcSums a;
+        a.phi = a.gx = a.gy = f2(0.f);
+#pragma unroll 8
+        for (int i = 0; i < pairs; ++i) {
+            const float4 s = S.xy[i];
+            const float2 dx = add2(f2(T.x), make_float2(-s.x, -s.y)), dy = add2(f2(T.y), make_float2(-s.z, -s.w));
+            near_src_pair<P>(np, near_w2(P >= 2, dx, dy), dx, dy, S.q[i], a);
+        }
+        if (valid)
+            near_src_add<P>(a, __float_as_int(T.z), 0.f, rcoef, phi_s, grad_s, coinc);
+    }
+}
+
+template <int P>
+__device__ __forceinline__ void near_src_close(const NearSources &S, int n, int pairs, int lane, float ie,
+                                               const NearParams<float> &np, float rcoef, float *__restrict__ phi_s,
+                                               float *__restrict__ grad_s, float *__restrict__ coinc)
+{
+    for (int base = 0; base < n; base += 32) {
+        const bool valid = base + lane < n;
+        const float4 T = valid ? S.close[base + lane] : make_float4(kPadPos, kPadPos, 0.f, 0.f);
+        NearSrcSums a;
+        a.phi = a.gx = a.gy = f2(0.f);
         float cq = 0.f;
-#pragma unroll 2
-        for (int i = 0; i < 32; ++i) {
-            const float4 sh = s_hi[i];                    // (xa, xb, ya, yb)
-            float2 q2 = s_q[i];
-            float2 dx = add2(X, make_float2(-sh.x, -sh.y));
-            float2 dy = add2(Y, make_float2(-sh.z, -sh.w));
-            float2 r2 = fma2(dy, dy, mul2(dx, dx));
-            if constexpr (CLOSE) {
-                const float4 sl = s_lo[i];
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    if (valid && (t == 0 ? r2.x : r2.y) < np.close2) {
-                        const float ex = refine_diff(A.x, t == 0 ? sh.x : sh.y, B.x, A.z, t == 0 ? sl.x : sl.y);
-                        const float ey = refine_diff(A.y, t == 0 ? sh.z : sh.w, B.y, A.w, t == 0 ? sl.z : sl.w);
-                        float e2 = ex * ex + ey * ey;
-                        if (ex == 0.f && ey == 0.f) {             // coincident: G(0) := 0
-                            const float qs = t == 0 ? q2.x : q2.y;
-                            add_comp(phi, t, -qs * np.beta[0]);
-                            cq += qs;
-                            e2 = np.eps2;                          // masked out: w = 1
-                        }
-                        if (t == 0) {
-                            dx.x = ex;
-                            dy.x = ey;
-                            r2.x = e2;
-                        } else {
-                            dx.y = ex;
-                            dy.y = ey;
-                            r2.y = e2;
-                        }
-                    }
-                }
+        for (int i = 0; i < pairs; ++i) {
+            const float4 h = S.hi[i], l = S.lo[i];
+            const float2 q2 = S.q[i];
+            const float2 ex = add2(add2(f2(T.x), make_float2(-h.x, -h.y)), add2(f2(T.z), make_float2(-l.x, -l.y)));
+            const float2 ey = add2(add2(f2(T.y), make_float2(-h.z, -h.w)), add2(f2(T.w), make_float2(-l.z, -l.w)));
+            const float2 dx = mul2(ex, f2(ie)), dy = mul2(ey, f2(ie));
+            float2 w = near_w2(P >= 2, dx, dy);
+            const bool z0 = ex.x == 0.f && ey.x == 0.f, z1 = ex.y == 0.f && ey.y == 0.f;
+            if (z0 || z1) {
+                // coincident: G(0) := 0; an idle second source has charge 0
+                const float qs = (z0 ? q2.x : 0.f) + (z1 ? q2.y : 0.f);
+                a.phi.x -= qs * (np.beta[0] / (P >= 2 ? kLnCoef : 1.f));
+                cq += qs;
+                w.x = z0 ? 1.f : w.x;
+                w.y = z1 ? 1.f : w.y;
             }
-            if (i & 1)
-                near_src_pair<P, true>(np, r2, dx, dy, q2, phi, gx, gy);
-            else
-                near_src_pair<P, false>(np, r2, dx, dy, q2, phi, gx, gy);
+            near_src_pair<P>(np, w, dx, dy, q2, a);
         }
-        if (valid) {
-            const float rc = (P >= 2 && (P - 1) % 2 == 1) ? -rcoef : rcoef;   // near_src_pair's coef is |w - 1|^(p-1) / w
-            atomicAdd(phi_s + k, phi.x + phi.y);
-            atomicAdd(grad_s + 2 * (int64_t)k, rc * (gx.x + gx.y));
-            atomicAdd(grad_s + 2 * (int64_t)k + 1, rc * (gy.x + gy.y));
-            if (CLOSE && cq != 0.f)
-                atomicAdd(coinc + k, cq);
-        }
+        if (valid)
+            near_src_add<P>(a, S.close_k[base + lane], cq, rcoef, phi_s, grad_s, coinc);
     }
 }
 
@@ -640,24 +636,25 @@ __global__ void __launch_bounds__(128) k_near_src32(int64_t n_items, const int2 
                                                     float *__restrict__ phi_s, float *__restrict__ grad_s,
                                                     float *__restrict__ coinc)
 {
-    __shared__ float4 s_hi_all[4][32], s_lo_all[4][32];
-    __shared__ float2 s_q_all[4][32];
-    __shared__ float4 far_all[4][kSrcMajorCap], ca_all[4][kSrcMajorCap], cb_all[4][kSrcMajorCap];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __shared__ NearSources all[4];
+    const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (warp >= n_items)
         return;                                   // whole warp past the end; no block-wide barrier follows
-    float4 *s_hi = s_hi_all[w], *s_lo = s_lo_all[w], *far = far_all[w], *ca = ca_all[w], *cb = cb_all[w];
-    float2 *s_q = s_q_all[w];
+    NearSources &S = all[threadIdx.x >> 5];
     const int2 item = items[warp];
-    // the item's sources (own side): slots a = lane, b = lane + 32; idle slots copy the first
+    // pair i: the item's sources i and i + pairs (own side); an idle second one copies the first
     // source with charge 0
-    const bool va = lane < item.y, vb = lane + 32 < item.y;
-    const int64_t ja = va ? item.x + lane : item.x, jb = vb ? item.x + 32 + lane : item.x;
+    const int pairs = (item.y + 1) / 2;
+    const int64_t ja = item.x + (lane < pairs ? lane : 0);
+    const bool vb = lane < pairs && lane + pairs < item.y;
+    const int64_t jb = vb ? ja + pairs : item.x;
     const float2 ha = sd.own_hi[ja], hb = sd.own_hi[jb], la = sd.own_lo[ja], lb = sd.own_lo[jb];
-    s_hi[lane] = make_float4(ha.x, hb.x, ha.y, hb.y);
-    s_lo[lane] = make_float4(la.x, lb.x, la.y, lb.y);
-    s_q[lane] = make_float2(va ? __ldg(q + ja) : 0.f, vb ? __ldg(q + jb) : 0.f);
+    const float ie = sqrtf(np.inv_eps2);
+    S.hi[lane] = make_float4(ha.x, hb.x, ha.y, hb.y);
+    S.lo[lane] = make_float4(la.x, lb.x, la.y, lb.y);
+    S.xy[lane] = make_float4(ha.x * ie, hb.x * ie, ha.y * ie, hb.y * ie);
+    S.q[lane] = make_float2(__ldg(q + ja), vb ? __ldg(q + jb) : 0.f);
     const int packed = sd.own_base[item.x];
     const int c1 = base1(packed) / cg.cell, c2 = base2(packed) / cg.cell;
     const float h = np.hcell, eps = sqrtf(np.eps2);
@@ -668,7 +665,7 @@ __global__ void __launch_bounds__(128) k_near_src32(int64_t n_items, const int2 
     const float reach = eps + margin, reach2 = reach * reach;
     const float close_reach = sqrtf(np.close2) + margin, close_reach2 = close_reach * close_reach;
     const unsigned below = (1u << lane) - 1u;
-    const float rcoef = np.rcoef;
+    const float rcoef = np.rcoef * eps;           // the differences are in units of eps_I
     __syncwarp();
     int nf = 0, nc = 0;
     for (int e1 = max(c1 - 1, 0); e1 <= min(c1 + 1, cg.n_c - 1); ++e1) {
@@ -683,46 +680,48 @@ __global__ void __launch_bounds__(128) k_near_src32(int64_t n_items, const int2 
             const int j0 = sd.oth_start[kbase], j1 = sd.oth_start[kbase + kSub];
             for (int jb0 = j0; jb0 < j1; jb0 += 32) {
                 const int j = jb0 + lane;
-                const bool in = j < j1;
                 float2 th = make_float2(0.f, 0.f);
-                if (in)
+                if (j < j1)
                     th = __ldg(sd.oth_hi + j);
-                const float tx = th.x + ox, ty = th.y + oy;
+                const float tx = ox + th.x, ty = oy + th.y;
                 const float dxb = fmaxf(0.f, fmaxf(tx - hx, lx - tx));
                 const float dyb = fmaxf(0.f, fmaxf(ty - hy, ly - ty));
-                const float g2 = dxb * dxb + dyb * dyb;
-                const bool keep = in && g2 <= reach2;
-                const bool close = keep && g2 <= close_reach2;
-                const unsigned mf = __ballot_sync(0xffffffffu, keep && !close);
-                const unsigned mc = __ballot_sync(0xffffffffu, close);
+                const float g2 = j < j1 ? dxb * dxb + dyb * dyb : 3e38f;
+                const bool keep = g2 <= reach2, close = g2 <= close_reach2;
+                const unsigned mc = __ballot_sync(0xffffffffu, close), mf = __ballot_sync(0xffffffffu, keep) & ~mc;
                 if (keep && !close)
-                    far[nf + __popc(mf & below)] = make_float4(tx, ty, __int_as_float(j), 0.f);
-                if (close) {
-                    const int at = nc + __popc(mc & below);
-                    const float2 tl = __ldg(sd.oth_lo + j);
-                    ca[at] = make_float4(th.x, th.y, tl.x, tl.y);
-                    cb[at] = make_float4(ox, oy, __int_as_float(j), 0.f);
-                }
+                    S.far[nf + __popc(mf & below)] = make_float4(tx * ie, ty * ie, __int_as_float(j), 0.f);
                 nf += __popc(mf);
-                nc += __popc(mc);
                 if (nf > kSrcMajorCap - 32) {
                     __syncwarp();
-                    near_src_eval<P, false>(s_hi, s_lo, s_q, far, nullptr, nf, lane, np, rcoef, phi_s, grad_s, coinc);
+                    near_src_far<P>(S, nf, pairs, lane, np, rcoef, phi_s, grad_s, coinc);
                     nf = 0;
                     __syncwarp();
                 }
-                if (nc > kSrcMajorCap - 32) {
-                    __syncwarp();
-                    near_src_eval<P, true>(s_hi, s_lo, s_q, ca, cb, nc, lane, np, rcoef, phi_s, grad_s, coinc);
-                    nc = 0;
-                    __syncwarp();
+                if (mc) {
+                    if (close) {
+                        const int at = nc + __popc(mc & below);
+                        const float2 tl = __ldg(sd.oth_lo + j);
+                        // step + hi + lo as hi + lo (TwoSum of the step and hi)
+                        const float bx = tx - ox, by = ty - oy;
+                        S.close[at] = make_float4(tx, ty, ((ox - (tx - bx)) + (th.x - bx)) + tl.x,
+                                                  ((oy - (ty - by)) + (th.y - by)) + tl.y);
+                        S.close_k[at] = j;
+                    }
+                    nc += __popc(mc);
+                    if (nc > kSrcMajorClose - 32) {
+                        __syncwarp();
+                        near_src_close<P>(S, nc, pairs, lane, ie, np, rcoef, phi_s, grad_s, coinc);
+                        nc = 0;
+                        __syncwarp();
+                    }
                 }
             }
         }
     }
     __syncwarp();
-    near_src_eval<P, false>(s_hi, s_lo, s_q, far, nullptr, nf, lane, np, rcoef, phi_s, grad_s, coinc);
-    near_src_eval<P, true>(s_hi, s_lo, s_q, ca, cb, nc, lane, np, rcoef, phi_s, grad_s, coinc);
+    near_src_far<P>(S, nf, pairs, lane, np, rcoef, phi_s, grad_s, coinc);
+    near_src_close<P>(S, nc, pairs, lane, ie, np, rcoef, phi_s, grad_s, coinc);
 }
 
 // Calls f(std::integral_constant<int, P>) for the expansion degree p in 1..16.
