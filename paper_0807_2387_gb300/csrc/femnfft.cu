@@ -627,6 +627,11 @@ fs_status plan_init(fs_plan *pl, const double *src, int64_t M, const double *tgt
 
     // grids and per-target intermediates
     FS_TRY(pl->alloc_bytes(&pl->grid, (size_t)n_a * pl->pitch * sizeof(real)));
+    // the filtered grid is its own buffer so that the first one stays zeroed; without memory for it
+    // both are one and every spreading begins with a memset
+    if (pl->alloc_bytes(&pl->field, (size_t)n_a * pl->pitch * sizeof(real)) != FS_OK)
+        pl->field = pl->grid;
+    FS_CUDA(cudaMemsetAsync(pl->grid, 0, (size_t)n_a * pl->pitch * sizeof(real), st));
     if (pl->spread_direct && pl->kahan && sizeof(real) == 4)
         FS_TRY(pl->alloc_bytes(&pl->grid_comp, (size_t)n_a * pl->pitch * sizeof(real)));
     FS_TRY(pl->alloc_bytes(&pl->spec, (size_t)(pl->n / 2 + 1) * pl->ld * 2 * sizeof(real)));
@@ -740,13 +745,15 @@ template <typename real> fs_status reserve_rhs(fs_plan *pl, int nrhs)
     const size_t grid_bytes = (size_t)pl->n_a * pl->pitch * sizeof(real);
     const size_t spec_bytes = (size_t)(pl->n / 2 + 1) * pl->ld * 2 * sizeof(real);
     auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
-    const size_t spec_at = up(grid_bytes * want), sums_at = spec_at + up(spec_bytes * want);
+    const size_t field_at = up(grid_bytes * want), spec_at = 2 * field_at, sums_at = spec_at + up(spec_bytes * want);
     // one allocation; the single-vector buffers stay until the plan is destroyed (freeing them here
     // would wait for the device)
     unsigned char *p = nullptr;
     if (pl->alloc(&p, sums_at + (size_t)pl->sums_n * 4 * want * sizeof(real)) != FS_OK)
         return FS_OK;
     pl->grid = p;
+    pl->grid_dirty = true;
+    pl->field = p + field_at;
     pl->spec = p + spec_at;
     pl->phi_s = p + sums_at;
     pl->grad_s = (unsigned char *)pl->phi_s + (size_t)pl->sums_n * want * sizeof(real);
@@ -786,12 +793,27 @@ template <typename real> fs_status set_charges_t(fs_plan *pl, const void *q, fs_
     return FS_OK;
 }
 
-// Step (c): the grid is zeroed and the charges spread into it, through shared-memory tiles or
+// The grid zeroed for a spreading: the forward transform leaves it so, unless an evaluation stopped
+// between the two, or the grid is new, or the memset was only recorded into a graph.
+fs_status clear_grid(fs_plan *pl)
+{
+    pl->grid_recorded = false;
+    if (pl->grid_dirty) {
+        FS_CUDA(cudaMemsetAsync(pl->grid, 0, (size_t)pl->n_a * pl->pitch * pl->rsize() * pl->rhs_cap, pl->stream));
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        FS_CUDA(cudaStreamIsCapturing(pl->stream, &cs));
+        pl->grid_recorded = cs != cudaStreamCaptureStatusNone;
+    }
+    pl->grid_dirty = true;
+    return FS_OK;
+}
+
+// Step (c): the charges spread into the zero grid, through shared-memory tiles or
 // (sparse plans, FS_FLAG_SPREAD_DIRECT: one vector) with global atomics and a compensation plane.
 template <typename real> fs_status spread_forward(fs_plan *pl, const real *q, int nrhs, cudaStream_t st)
 {
     const int64_t grid_n = (int64_t)pl->n_a * pl->pitch;
-    FS_CUDA(cudaMemsetAsync(pl->grid, 0, (size_t)grid_n * nrhs * sizeof(real), st));
+    FS_TRY(clear_grid(pl));
     if (!pl->spread_direct) {
         FS_CUDA(launch_spread<real>(pl->items, pl->n_items, pl->cg, pl->m, pl->src_base, pl->src_frac, q,
                                     win_poly<real>(pl), (real *)pl->grid, pl->pitch, pl->n_a, pl->kahan, nrhs, pl->M,
@@ -852,11 +874,9 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
             FS_CUDA(cudaEventRecord(pl->ev[0], st));
         if (pl->overlap)
             FS_CUDA(cudaEventRecord(pl->ev_fork, st));   // the charges are in
-        FS_TRY(spread_forward<real>(pl, q, R, st));
-        if constexpr (sizeof(real) == 4) {
-            if (pl->overlap) {
-                // the near field (stored, not added) on the second stream, submitted after the
-                // spreading so that the spreading's blocks are scheduled first
+        // the near field (stored, not added) on the second stream
+        auto near_beside = [&]() -> fs_status {
+            if constexpr (sizeof(real) == 4) {
                 FS_CUDA(cudaStreamWaitEvent(pl->aux, pl->ev_fork, 0));
                 if (rec)
                     FS_CUDA(cudaEventRecord(pl->ev_n0, pl->aux));
@@ -865,11 +885,18 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
                     FS_CUDA(cudaEventRecord(pl->ev_n1, pl->aux));
                 FS_CUDA(cudaEventRecord(pl->ev_join, pl->aux));
             }
-        }
+            return FS_OK;
+        };
+        if (pl->overlap && pl->near_first())
+            FS_TRY(near_beside());
+        FS_TRY(spread_forward<real>(pl, q, R, st));
+        if (pl->overlap && !pl->near_first())
+            FS_TRY(near_beside());
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[1], st));
-        FS_CUDA(launch_fft_rows_fwd<real>((const real *)pl->grid, pl->pitch, pl->n_a, pl->n_os, pl->n / 2,
-                                          (C *)pl->spec, pl->ld, (const C *)pl->tw, R, grid_n, spec_n, st));
+        FS_CUDA(launch_fft_rows_fwd<real>((real *)pl->grid, pl->pitch, pl->n_a, pl->n_os, pl->n / 2, (C *)pl->spec,
+                                          pl->ld, (const C *)pl->tw, R, grid_n, spec_n, st));
+        pl->grid_dirty = pl->grid_recorded || pl->field == pl->grid;
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[2], st));
         FS_CUDA(launch_fft_cols<real>((C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n, (const real *)pl->mul,
@@ -877,7 +904,7 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[3], st));
         FS_CUDA(launch_fft_rows_inv<real>((const C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n / 2,
-                                          (real *)pl->grid, pl->pitch, (const C *)pl->tw, R, grid_n, spec_n, st));
+                                          (real *)pl->field, pl->pitch, (const C *)pl->tw, R, grid_n, spec_n, st));
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[4], st));
         auto out_phi = [&](int r) { return phi ? (unsigned char *)phi + (size_t)(r0 + r) * pl->N * osz : nullptr; };
@@ -889,7 +916,7 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
             // steps (f) and (h) in one pass: the far field added to the near field's sums and
             // written to the caller's buffers (the output stage's time is in the interpolation's)
             FS_CUDA(launch_interp_out<real>(pl->N, pl->m, pl->tgt_base, pl->tgt_frac, win_poly<real>(pl),
-                                            (const real *)pl->grid, pl->pitch, (real)pl->n_os,
+                                            (const real *)pl->field, pl->pitch, (real)pl->n_os,
                                             (const real *)pl->phi_s, (const real *)pl->grad_s,
                                             (const real *)pl->coinc, pl->tgt_perm, shift, pl->q_sum + r0, pl->s,
                                             out_phi(0), out_h(0), dtype == FS_F64, R, grid_n, pl->sums_n, st));
@@ -902,7 +929,7 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
         }
         for (int r = 0; r < R; ++r) {
             FS_CUDA(launch_interp<real>(pl->N, pl->m, pl->tgt_base, pl->tgt_frac, win_poly<real>(pl),
-                                        (const real *)pl->grid + r * grid_n, pl->pitch, (real)pl->n_os,
+                                        (const real *)pl->field + r * grid_n, pl->pitch, (real)pl->n_os,
                                         (real *)pl->phi_s, (real *)pl->grad_s, false, st));
             if (rec)
                 FS_CUDA(cudaEventRecord(pl->ev[5], st));
@@ -983,11 +1010,12 @@ template <typename real> fs_status spectral_pipeline(fs_plan *pl)
 {
     using C = typename Cplx<real>::type;
     cudaStream_t st = pl->stream;
-    FS_CUDA(launch_fft_rows_fwd<real>((const real *)pl->grid, pl->pitch, pl->n_a, pl->n_os, pl->n / 2, (C *)pl->spec,
+    FS_CUDA(launch_fft_rows_fwd<real>((real *)pl->grid, pl->pitch, pl->n_a, pl->n_os, pl->n / 2, (C *)pl->spec,
                                       pl->ld, (const C *)pl->tw, 1, 0, 0, st));
+    pl->grid_dirty = pl->grid_recorded || pl->field == pl->grid;
     FS_CUDA(launch_fft_cols<real>((C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n, (const real *)pl->mul,
                                   (const C *)pl->tw, 1, 0, st));
-    FS_CUDA(launch_fft_rows_inv<real>((const C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n / 2, (real *)pl->grid,
+    FS_CUDA(launch_fft_rows_inv<real>((const C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n / 2, (real *)pl->field,
                                       pl->pitch, (const C *)pl->tw, 1, 0, 0, st));
     return FS_OK;
 }
@@ -1014,7 +1042,6 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
     const NearParams<real> np = make_near<real>(pl);
     const double shift = std::log(pl->s) / (2.0 * kPi);
     const size_t isz = in_dtype == FS_F64 ? 8 : 4, osz = out_dtype == FS_F64 ? 8 : 4;
-    const size_t grid_bytes = (size_t)pl->n_a * pl->pitch * sizeof(real);
     for (int r = 0; r < pl->nrhs; ++r) {
         const real *q = (const real *)pl->q_sorted + (int64_t)r * M;
         const void *gp = g_phi ? (const unsigned char *)g_phi + (size_t)r * N * isz : nullptr;
@@ -1038,7 +1065,7 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
             FS_TRY(spectral_pipeline<real>(pl));
             if (ovl)
                 FS_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
-            FS_CUDA(launch_interp_hess<real>(N, pl->m, pl->tgt_base, pl->tgt_frac, win_poly<real>(pl), (const real *)pl->grid,
+            FS_CUDA(launch_interp_hess<real>(N, pl->m, pl->tgt_base, pl->tgt_frac, win_poly<real>(pl), (const real *)pl->field,
                                              pl->pitch, (real)pl->n_os, (real *)pl->grad_s, (real *)pl->adj_hess, ovl,
                                              st));
             if constexpr (sizeof(real) == 4) {
@@ -1066,14 +1093,14 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
                     FS_CUDA(cudaEventRecord(pl->ev_join, pl->aux));
                 }
             }
-            FS_CUDA(cudaMemsetAsync(pl->grid, 0, grid_bytes, st));
+            FS_TRY(clear_grid(pl));
             FS_CUDA(launch_spread_dip<real>(pl->tgt_items, pl->n_tgt_items, pl->cg, pl->m, pl->tgt_base, pl->tgt_frac,
                                             (const real *)pl->adj_c, pl->adj_df, win_poly<real>(pl), (real *)pl->grid,
                                             pl->pitch, pl->n_a, pl->kahan, st));
             FS_TRY(spectral_pipeline<real>(pl));
             if (ovl)
                 FS_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
-            FS_CUDA(launch_interp<real>(M, pl->m, pl->src_base, pl->src_frac, win_poly<real>(pl), (const real *)pl->grid,
+            FS_CUDA(launch_interp<real>(M, pl->m, pl->src_base, pl->src_frac, win_poly<real>(pl), (const real *)pl->field,
                                         pl->pitch, (real)pl->n_os, (real *)pl->adj_a, (real *)pl->adj_ga, ovl, st));
             if constexpr (sizeof(real) == 4) {
                 if (!ovl)

@@ -8,6 +8,9 @@
 
 namespace fs {
 
+// Dynamic shared memory a kernel may use without raising its limit first.
+constexpr size_t kSmemDefault = 48 * 1024;
+
 // Warps per spreading CTA; each holds a private padded tile in shared memory.
 constexpr int kSpreadWarps = 4;
 
@@ -396,7 +399,7 @@ __host__ __device__ constexpr int fft_pass_radix(int rest) { return rest % 8 == 
 // k = 0..Ns-1, hold exp(-2 pi i r k / (Ns R)); entry L - 1 is 1.  Computed in FP64.
 template <typename real> void fft_twiddle_table(int L, real *re_im);
 template <typename real>
-cudaError_t launch_fft_rows_fwd(const real *grid, int pitch, int n_a, int L, int n_half,
+cudaError_t launch_fft_rows_fwd(real *grid, int pitch, int n_a, int L, int n_half,
                                 typename Cplx<real>::type *spec, int ld, const typename Cplx<real>::type *tw,
                                 int nrhs, int64_t grid_stride, int64_t spec_stride, cudaStream_t st);
 template <typename real>

@@ -655,9 +655,10 @@ __host__ __device__ constexpr int fft_threads(int L) { return L / 4 > 256 ? 256 
 
 // The three 2D kernels.  LC > 0 fixes the line length at compile time (one instance per
 // length the plans use, 256 .. 4096 points), LC = 0 takes it at run time.
-// blockIdx.y: the charge vector (grids and spectra at their strides).
+// blockIdx.y: the charge vector (grids and spectra at their strides).  The forward kernel zeroes the
+// grid rows it has read, which saves the next spreading a memset of the grid in front of it.
 template <typename real, int LC>
-__global__ void __launch_bounds__(256) k_fft_rows_fwd(const real *__restrict__ grid, int pitch, int n_a, int L,
+__global__ void __launch_bounds__(256) k_fft_rows_fwd(real *__restrict__ grid, int pitch, int n_a, int L,
                                                       int n_half, cplx<real> *__restrict__ spec, int ld,
                                                       const cplx<real> *__restrict__ tw, int64_t grid_stride,
                                                       int64_t spec_stride)
@@ -666,8 +667,13 @@ __global__ void __launch_bounds__(256) k_fft_rows_fwd(const real *__restrict__ g
     extern __shared__ unsigned char smem_raw[];
     cplx<real> *a = reinterpret_cast<cplx<real> *>(smem_raw);
     cplx<real> *s_tw = stage_twiddles<real, LC, NT>(a + 2 * L, tw, L);   // published by the unit's first barrier
-    rows_fwd_unit<real, LC, NT>(blockIdx.x, grid + blockIdx.y * grid_stride, pitch, n_a, L, n_half,
-                                spec + blockIdx.y * spec_stride, ld, s_tw, a, a + L);
+    real *g = grid + blockIdx.y * grid_stride;
+    rows_fwd_unit<real, LC, NT>(blockIdx.x, g, pitch, n_a, L, n_half, spec + blockIdx.y * spec_stride, ld, s_tw, a, a + L);
+    // the block's rows are read (its last barrier lies after the reads): leave the grid zeroed for the
+    // next spreading
+    const int rows = min(2, n_a - 2 * (int)blockIdx.x);
+    for (int i = threadIdx.x; i < rows * pitch; i += blockDim.x)
+        g[2 * (int64_t)blockIdx.x * pitch + i] = real(0);
 }
 
 template <typename real, int LC>
@@ -1085,6 +1091,8 @@ __global__ void k_build_mul(const double2 *__restrict__ bhat, int n, const doubl
 
 template <typename K> cudaError_t set_smem(K kern, size_t bytes)
 {
+    if (bytes <= kSmemDefault)
+        return cudaSuccess;
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
@@ -1094,6 +1102,7 @@ template <typename K> cudaError_t set_smem(K kern, size_t bytes)
 template <typename F> cudaError_t with_line_length(int L, F &&f)
 {
     switch (L) {
+    case 128: return f(std::integral_constant<int, 128>{});
     case 256: return f(std::integral_constant<int, 256>{});
     case 512: return f(std::integral_constant<int, 512>{});
     case 1024: return f(std::integral_constant<int, 1024>{});
@@ -1104,7 +1113,7 @@ template <typename F> cudaError_t with_line_length(int L, F &&f)
 }
 
 template <typename real>
-cudaError_t launch_fft_rows_fwd(const real *grid, int pitch, int n_a, int L, int n_half, cplx<real> *spec, int ld,
+cudaError_t launch_fft_rows_fwd(real *grid, int pitch, int n_a, int L, int n_half, cplx<real> *spec, int ld,
                                 const cplx<real> *tw, int nrhs, int64_t grid_stride, int64_t spec_stride, cudaStream_t st)
 {
     const size_t smem = 3 * (size_t)L * sizeof(cplx<real>);   // two line buffers and the twiddles
@@ -1286,9 +1295,9 @@ template <typename real> void fft_twiddle_table(int L, real *re_im)
 template void fft_twiddle_table<float>(int, float *);
 template void fft_twiddle_table<double>(int, double *);
 
-template cudaError_t launch_fft_rows_fwd<float>(const float *, int, int, int, int, float2 *, int, const float2 *, int,
+template cudaError_t launch_fft_rows_fwd<float>(float *, int, int, int, int, float2 *, int, const float2 *, int,
                                                 int64_t, int64_t, cudaStream_t);
-template cudaError_t launch_fft_rows_fwd<double>(const double *, int, int, int, int, double2 *, int, const double2 *, int,
+template cudaError_t launch_fft_rows_fwd<double>(double *, int, int, int, int, double2 *, int, const double2 *, int,
                                                 int64_t, int64_t, cudaStream_t);
 template cudaError_t launch_fft_cols<float>(float2 *, int, int, int, int, const float *, const float2 *, int, int64_t,
                                             cudaStream_t);

@@ -821,9 +821,11 @@ cudaError_t spread_m(const SpreadItem *items, int n_items, CellGrid cg, const in
     const size_t smem = spread_smem_bytes<real>(P, M2, kahan);
     const real2_t<real> *fr = (const real2_t<real> *)frac;
     auto run = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess)
-            return e;
+        if (smem > kSmemDefault) {
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess)
+                return e;
+        }
         kern<<<dim3((unsigned)n_items, (unsigned)nrhs), kSpreadWarps * 32, smem, st>>>(items, cg, base, fr, q, wp, grid,
                                                                                      pitch, n_a, q_stride, grid_stride);
         return cudaGetLastError();

@@ -105,3 +105,25 @@ def test_3d_run_spreading(ns, n, lines):
     assert plan.info["spread_items"] > 0
     assert rel(got[32][0], got[64][0]) <= 5e-6, rel(got[32][0], got[64][0])
     assert rel(got[32][1], got[64][1]) <= 5e-6, rel(got[32][1], got[64][1])
+
+
+@pytest.mark.parametrize("precision,tol", [(32, 2e-5), (64, 1e-12)])
+@pytest.mark.parametrize("n", [64, 128])
+def test_grid_is_left_clean(n, precision, tol):
+    """Every evaluation starts from a zero grid: the same charges give the same field again after other
+    charge vectors, several at once, and an adjoint (transform lengths 128 and 256; the sums differ by the
+    order of the grid's atomic additions, within the bars of the parity gates)."""
+    import paper_0807_2387_gb300 as pkg
+    rng = np.random.default_rng(8)
+    dev = torch.device("cuda", 0)
+    pts = [torch.tensor(rng.uniform(-0.17, 0.17, (k, 2)), device=dev) for k in (700, 500)]
+    q = torch.tensor(rng.standard_normal((4, 700)), device=dev)
+    fs = pkg.FastSum(*pts, n, 2.0, 4, 4.0 / n, precision=precision)
+    first = fs.set_charges(q[0]).field(dtype=torch.float64)
+    g = torch.tensor(rng.standard_normal(500), device=dev)
+    for again in (lambda: fs.set_charges(q[1]).potential(), lambda: fs.set_charges(q[1:]).field(),
+                  lambda: fs.set_charges(q[2]).adjoint(g_phi=g)):
+        again()
+        for a, b in zip(fs.set_charges(q[0]).field(dtype=torch.float64), first):
+            assert float((a - b).norm() / b.norm()) <= tol
+    fs.close()
