@@ -326,7 +326,8 @@ def measure_batch(pkg, dev, steps, warmup, flush, instances=64):
             "value": 3 * total / (t_batch / 1e3), "unit": "point-solves/s", "ms_per_replay": round(t_batch, 4),
             "sequential_ms": round(t_seq, 4), "speedup_vs_sequential": round(t_seq / t_batch, 3),
             "sequential": f"{3 * len(cases)} x (fs_set_charges + fs_eval_field) on the same instance plans",
-            "launches_per_replay": 5, "memsets_per_replay": 3, "fft_blocks": info["fft_blocks"],
+            "launches_per_replay": 4 + len({c["n"] for c in cases}),   # the transform: one per line length
+            "memsets_per_replay": 3, "fft_blocks": info["fft_blocks"],
             "create_s_with_autotune": round(create_s, 3),
             "largest_instance_vs_fp64": {"phi_rel_l2": e_phi, "H_rel_l2": e_H}}
 

@@ -282,8 +282,8 @@ fs_status fs_plan_destroy(fs_plan *plan);
  * nrhs charge vectors per instance, and evaluates all of them with one launch per
  * stage (charges, spreading, FFT + multiply, interpolation, near field, output)
  * over all (instance, right-hand side, work unit) items, replayed as one CUDA
- * graph.  The FFT stage is one persistent launch whose blocks wait on each other
- * through counters; those waits are bounded and a wait that gives up sets an
+ * graph.  The FFT stage is one persistent launch per transform length whose blocks wait
+ * on each other through counters; those waits are bounded and a wait that gives up sets an
  * error word reported by fs_batch_sync_status as FS_ETIMEOUT.
  */
 typedef struct fs_batch fs_batch;
@@ -302,7 +302,7 @@ typedef struct {
     int64_t total_src, total_tgt;
     int spread_items;       /* spreading work items over all instances (x nrhs per launch) */
     int fft_units;          /* row pairs + columns + inverse row pairs, all instances and rhs */
-    int fft_blocks;         /* persistent blocks of the FFT launch */
+    int fft_blocks;         /* persistent blocks of the largest FFT launch */
     int64_t near_items;     /* FP32 near-field warp items over all instances */
     int64_t workspace_bytes;
 } fs_batch_facts;

@@ -1,14 +1,14 @@
 // Batched solves: many independent fast summations (one per instance, each with its own
 // grid size and near-field radius, shared window and oversampling) and several charge
-// vectors each, evaluated with one launch per stage over all (instance, right-hand side,
-// unit) work items and replayed as one CUDA graph.
+// vectors each, evaluated with one launch per stage (the FFT: per line length) over all (instance, right-hand
+// side, unit) work items and replayed as one CUDA graph.
 //
 // Each instance is an ordinary plan (binning, coefficient table, twiddles, work items); the
 // batch adds the buffers of every right-hand side, a device table of per-instance
 // descriptors (BatchInst) and the merged work lists:
 //   spreading  - the plans' tile items, largest first, x right-hand sides;
-//   FFT        - one persistent launch over row pairs, then columns, then inverse row pairs
-//                of every (instance, right-hand side), ordered by dependency (waits bounded);
+//   FFT        - one persistent launch per line length over row pairs, then columns, then inverse
+//                row pairs of its (instance, right-hand side)s, ordered by dependency (waits bounded);
 //   near field - the plans' warp items ordered by estimated pair work across all instances,
 //                every right-hand side in one traversal;
 //   per-point stages (charges, interpolation, output) - block maps over the instances.
@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -59,8 +60,9 @@ struct fs_batch {
     int4 *near_items = nullptr;
     int64_t n_near_items = 0;
     FftUnit *fft_units = nullptr;
-    int n_fft_units = 0, fft_blocks = 0, L_max = 0;
-    int *counters = nullptr;              // 2 * count * nrhs + 1
+    std::vector<FftRun> fft_runs;         // one launch per line length
+    int n_fft_units = 0, fft_blocks = 0;  // fft_blocks: of the largest launch
+    int *counters = nullptr;              // 2 * count * nrhs, and one queue head per launch
     int *err = nullptr;
     int *src_inst = nullptr, *src_first = nullptr, *tgt_inst = nullptr, *tgt_first = nullptr;
     int src_blocks = 0, tgt_blocks = 0;
@@ -260,7 +262,6 @@ template <typename real> fs_status batch_build(fs_batch *b, const fs_instance *i
         tot_n += up((size_t)std::max<int64_t>(pl->N, 1) * sizeof(real)) * R;
         b->total_src += pl->M;
         b->total_tgt += pl->N;
-        b->L_max = std::max(b->L_max, pl->n_os);
         b->max_tile = std::max(b->max_tile, pl->cg.T * pl->cg.cell);
     }
     unsigned char *grids, *specs, *qs, *phis, *grads, *coincs;
@@ -362,27 +363,31 @@ template <typename real> fs_status batch_build(fs_batch *b, const fs_instance *i
         if (!items.empty())
             FS_CUDA(cudaMemcpy(b->near_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice));
     }
-    // FFT units: all forward row pairs, then all columns, then all inverse row pairs; larger
-    // transforms first inside each phase
-    std::vector<int> order(K);
+    // FFT units by line length, the longest first; of a length all forward row pairs, then all
+    // columns, then all inverse row pairs
+    std::map<int, std::vector<int>, std::greater<int>> lengths;   // line length -> instances
     for (int i = 0; i < K; ++i)
-        order[i] = i;
-    std::stable_sort(order.begin(), order.end(),
-                     [&](int x, int y) { return b->plans[x]->n_os > b->plans[y]->n_os; });
+        lengths[b->plans[i]->n_os].push_back(i);
     std::vector<FftUnit> fu;
-    for (int kind = 0; kind < 3; ++kind)
-        for (int i : order)
-            for (int r = 0; r < R; ++r) {
-                const fs_plan *pl = b->plans[i];
-                const int units = kind == 1 ? pl->n / 2 + 1 : (pl->n_a + 1) / 2;
-                for (int u = 0; u < units; ++u)
-                    fu.push_back(FftUnit{i, r, kind, u});
-            }
+    for (const auto &[L, of_length] : lengths) {
+        FftRun run{L, (int)fu.size(), 0, 0};
+        for (int kind = 0; kind < 3; ++kind)
+            for (int i : of_length)
+                for (int r = 0; r < R; ++r) {
+                    const fs_plan *pl = b->plans[i];
+                    const int units = kind == 1 ? pl->n / 2 + 1 : (pl->n_a + 1) / 2;
+                    for (int u = 0; u < units; ++u)
+                        fu.push_back(FftUnit{i, r, kind, u});
+                }
+        run.n = (int)fu.size() - run.first;
+        FS_CUDA(batch_fft_blocks<real>(L, &run.blocks));
+        b->fft_blocks = std::max(b->fft_blocks, std::min(run.blocks, run.n));
+        b->fft_runs.push_back(run);
+    }
     b->n_fft_units = (int)fu.size();
     FS_TRY(b->alloc(&b->fft_units, fu.size()));
     FS_CUDA(cudaMemcpy(b->fft_units, fu.data(), fu.size() * sizeof(FftUnit), cudaMemcpyHostToDevice));
-    FS_CUDA(batch_fft_blocks<real>(b->L_max, &b->fft_blocks));
-    FS_TRY(b->alloc(&b->counters, 2 * (size_t)K * R + 1));
+    FS_TRY(b->alloc(&b->counters, 2 * (size_t)K * R + b->fft_runs.size()));
     FS_TRY(b->alloc(&b->err, 1));
     FS_CUDA(cudaMemset(b->err, 0, sizeof(int)));
     // block maps of the per-point stages
@@ -420,7 +425,7 @@ template <typename real> fs_status batch_enqueue(fs_batch *b, int q_f64, int out
     const BlockMap src_map{b->src_inst, b->src_first}, tgt_map{b->tgt_inst, b->tgt_first};
     FS_CUDA(cudaMemsetAsync(b->q_sum, 0, sizeof(double) * K * R, st));
     FS_CUDA(cudaMemsetAsync(b->grids, 0, b->grid_bytes, st));
-    FS_CUDA(cudaMemsetAsync(b->counters, 0, sizeof(int) * (2 * (size_t)K * R + 1), st));
+    FS_CUDA(cudaMemsetAsync(b->counters, 0, sizeof(int) * (2 * (size_t)K * R + b->fft_runs.size()), st));
     FS_CUDA(launch_batch_gather_charges<real>(inst, b->io, src_map, b->src_blocks, R, q_f64, st));
     if constexpr (sizeof(real) == 4) {
         // the near field first, storing its sums (every target lies in one item); the grids are
@@ -430,8 +435,9 @@ template <typename real> fs_status batch_enqueue(fs_batch *b, int q_f64, int out
     }
     FS_CUDA(launch_batch_spread<real>(b->spread_items, b->n_spread_items, R, inst, b->m, b->max_tile, win_poly<real>(p0),
                                       b->kahan, st));
-    FS_CUDA(launch_batch_fft<real>(inst, b->fft_units, b->n_fft_units, K, R, b->L_max, b->fft_blocks, b->counters,
-                                   b->err, kWaitSpins, st));
+    for (size_t k = 0; k < b->fft_runs.size(); ++k)
+        FS_CUDA(launch_batch_fft<real>(inst, b->fft_units, b->fft_runs[k], K, R, b->counters,
+                                       b->counters + 2 * (size_t)K * R + k, b->err, kWaitSpins, st));
     if constexpr (sizeof(real) == 4) {
         FS_CUDA(launch_batch_interp_out<real>(inst, b->io, tgt_map, b->tgt_blocks, R, b->m, win_poly<real>(p0), out_f64, st));
     } else {

@@ -8,8 +8,9 @@
 
 namespace fs {
 
-// Dynamic shared memory a kernel may use without raising its limit first.
-constexpr size_t kSmemDefault = 48 * 1024;
+// Dynamic shared memory a kernel may use without raising its limit first: 48 KB less what it may
+// declare statically.
+constexpr size_t kSmemDefault = 47 * 1024;
 
 // Warps per spreading CTA; each holds a private padded tile in shared memory.
 constexpr int kSpreadWarps = 4;
@@ -300,6 +301,11 @@ struct FftUnit {
     int inst, rhs, kind, index;
 };
 
+// The units of one line length L, units first .. first + n - 1, and the blocks that are resident at once.
+struct FftRun {
+    int L, first, n, blocks;
+};
+
 // Device-side wait budget of the persistent FFT (spins of ~0.1 us each before the wait
 // gives up and records a timeout).
 constexpr int kWaitSpins = 1 << 23;
@@ -319,12 +325,12 @@ cudaError_t launch_batch_interp(const BatchInst<real> *inst, BlockMap bm, int bl
 template <typename real>
 cudaError_t launch_batch_interp_out(const BatchInst<real> *inst, const BatchIO *io, BlockMap bm, int blocks, int nrhs,
                                     int m, const WinPoly<real> &wp, int out_is_f64, cudaStream_t st);
-// counters: 2 * n_inst * nrhs ints (rows done, columns done) plus the queue head, zeroed
+// counters: 2 * n_inst * nrhs ints (rows done, columns done), head: the run's queue head, all zeroed
 // before each launch; err: set to 1 when a wait ran out of spins
 template <typename real>
-cudaError_t launch_batch_fft(const BatchInst<real> *inst, const FftUnit *units, int n_units, int n_inst, int nrhs,
-                             int L_max, int grid_blocks, int *counters, int *err, int spins, cudaStream_t st);
-template <typename real> cudaError_t batch_fft_blocks(int L_max, int *blocks);
+cudaError_t launch_batch_fft(const BatchInst<real> *inst, const FftUnit *units, const FftRun &run, int n_inst, int nrhs,
+                             int *counters, int *head, int *err, int spins, cudaStream_t st);
+template <typename real> cudaError_t batch_fft_blocks(int L, int *blocks);
 // one bounded wait on a counter that nothing increments (the timeout path, for tests)
 cudaError_t launch_wait_selftest(int *counter, int *err, int spins, cudaStream_t st);
 // items: (first target, count, instance, lanes) per warp, count <= lanes (8, 16 or 32)

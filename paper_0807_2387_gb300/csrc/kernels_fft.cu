@@ -22,6 +22,7 @@
 // fft_twiddle_table), which the 2D kernels first copy into shared memory; the
 // buffers between two passes are stored with an XOR swizzle of the index so that
 // the strided writes of the early passes hit distinct banks.
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -424,12 +425,12 @@ __device__ __forceinline__ void rows_inv_fused(int rp, const cplx<real> *__restr
 
 // Two real rows (2 rp, 2 rp + 1) of the window -> half spectra, bins 0..n_half, written to
 // spec[l1 * ld + r].  a, b: 2 L complex values of shared memory.
-template <typename real, int LC = 0, int NT = 0, bool FUSED = true>
+template <typename real, int LC = 0, int NT = 0>
 __device__ __forceinline__ void rows_fwd_unit(int rp, const real *__restrict__ grid, int pitch, int n_a, int L_rt,
                                               int n_half, cplx<real> *__restrict__ spec, int ld,
                                               const cplx<real> *__restrict__ tw, cplx<real> *a, cplx<real> *b)
 {
-    if constexpr (LC > 0 && FUSED) {
+    if constexpr (LC > 0) {
         rows_fwd_fused<real, LC, NT>(rp, grid, pitch, n_a, n_half, spec, ld, tw, a, b);
         return;
     }
@@ -489,12 +490,12 @@ __device__ __forceinline__ void rows_fwd_unit(int rp, const real *__restrict__ g
 }
 
 // Column l1: forward FFT over rows, multiply, inverse FFT, keep the window rows.
-template <typename real, bool CG, int LC = 0, int NT = 0, bool FUSED = true>
+template <typename real, bool CG, int LC = 0, int NT = 0>
 __device__ __forceinline__ void cols_unit(int l1, cplx<real> *__restrict__ spec, int ld, int n_a, int L_rt, int n,
                                           const real *__restrict__ mul, const cplx<real> *__restrict__ tw,
                                           cplx<real> *a, cplx<real> *b)
 {
-    if constexpr (LC > 0 && FUSED) {
+    if constexpr (LC > 0) {
         cols_fused<real, CG, LC, NT>(l1, spec, ld, n_a, n, mul, tw, a, b);
         return;
     }
@@ -549,12 +550,12 @@ __device__ __forceinline__ void cols_unit(int l1, cplx<real> *__restrict__ spec,
 }
 
 // Hermitian-extended inverse of two rows (2 rp, 2 rp + 1): real outputs on the window columns.
-template <typename real, bool CG, int LC = 0, int NT = 0, bool FUSED = true>
+template <typename real, bool CG, int LC = 0, int NT = 0>
 __device__ __forceinline__ void rows_inv_unit(int rp, const cplx<real> *__restrict__ spec, int ld, int n_a, int L_rt,
                                               int n_half, real *__restrict__ grid, int pitch,
                                               const cplx<real> *__restrict__ tw, cplx<real> *a, cplx<real> *b)
 {
-    if constexpr (LC > 0 && FUSED) {
+    if constexpr (LC > 0) {
         rows_inv_fused<real, CG, LC, NT>(rp, spec, ld, n_a, n_half, grid, pitch, tw, a, b);
         return;
     }
@@ -650,8 +651,16 @@ __device__ __forceinline__ cplx<real> *stage_twiddles(cplx<real> *dst, const cpl
     return dst;
 }
 
-// Threads of the 2D transform kernels for a line of L points: a quarter of L, 32 to 256.
-__host__ __device__ constexpr int fft_threads(int L) { return L / 4 > 256 ? 256 : (L / 4 < 32 ? 32 : L / 4); }
+// Threads of the 2D transform kernels for a line of L points: one per radix-8 butterfly, 32 to 256
+// (twice as many idle in the radix-8 passes: 78 batched transforms of 1,024-point lines 340 -> 242 us,
+// a plan's own transforms up to 1 us).
+__host__ __device__ constexpr int fft_threads(int L) { return L / 8 > 256 ? 256 : (L / 8 < 32 ? 32 : L / 8); }
+
+// Blocks per SM that the batched transform's registers are limited for: 1,024 threads in FP32 (64 registers), 512 in FP64.
+template <typename real> constexpr int fft_batch_blocks(int LC)
+{
+    return std::min(32, (sizeof(real) == 4 ? 1024 : 512) / fft_threads(LC));
+}
 
 // The three 2D kernels.  LC > 0 fixes the line length at compile time (one instance per
 // length the plans use, 256 .. 4096 points), LC = 0 takes it at run time.
@@ -731,38 +740,30 @@ __device__ bool block_wait_geq(const int *ctr, int target, int *err, int spins)
     return s_ok != 0;
 }
 
-// One unit of the batched transform (256 threads) on a line of LC points (0: bi.L at run time).
-// The shared-memory sweeps stay (FUSED = false): the fused units' extra registers made this
-// kernel, which holds every line length, spill at five blocks per SM, for no measured gain.
-template <typename real, int LC>
-__device__ __forceinline__ void batch_unit(const FftUnit &fu, const BatchInst<real> &bi, cplx<real> *spec, real *grid,
-                                           cplx<real> *a, cplx<real> *b)
-{
-    const int L = bi.L, n_a = bi.n_a, n = bi.n;
-    if (fu.kind == 0)
-        rows_fwd_unit<real, LC, 256, false>(fu.index, grid, bi.pitch, n_a, L, n / 2, spec, bi.ld, bi.tw, a, b);
-    else if (fu.kind == 1)
-        cols_unit<real, true, LC, 256, false>(fu.index, spec, bi.ld, n_a, L, n, bi.mul, bi.tw, a, b);
-    else
-        rows_inv_unit<real, true, LC, 256, false>(fu.index, spec, bi.ld, n_a, L, n / 2, grid, bi.pitch, bi.tw, a, b);
-}
-
-// Batched transform of all instances and right-hand sides in one persistent launch.  Blocks
-// take units from a queue in which every row pair precedes every column and every column
-// precedes every inverse row pair; a column waits until all forward row pairs of its
+// Batched transform of the instances (and right-hand sides) of one line length in one persistent
+// launch; LC > 0 fixes the length at compile time.  Blocks
+// take units from a queue in which a transform's row pairs precede its columns and its columns
+// its inverse row pairs; a column waits until all forward row pairs of its
 // (instance, right-hand side) are done, an inverse row pair until all its columns are.  The
 // units a block waits for were taken earlier by blocks that are running and never wait on
 // later units, so the waits end; each is bounded all the same (error word on timeout).
-template <typename real>
-__global__ void __launch_bounds__(256, sizeof(real) == 4 ? 5 : 3) k_batch_fft(const BatchInst<real> *__restrict__ inst,
-                                                   const FftUnit *__restrict__ units, int n_units, int n_inst,
-                                                   int nrhs, int L_max, int *counters, int *err, int spins)
+// One launch per length: with all lengths in one kernel of 256 threads the unfused units were all
+// that its registers allowed, short lines left most of the threads idle, and the twiddles, the
+// same for every instance of a length, came from global memory (64 instances of 256 to 2,048 lines,
+// three right-hand sides: 1,125 -> 776 us).  2,048-point lines take 1,500 SM cycles each, of which
+// the shared-memory sweeps need 1,000; queueing the transforms in groups that fit into L2 gave nothing.
+template <typename real, int LC>
+__global__ void __launch_bounds__(fft_threads(LC ? LC : 2048), fft_batch_blocks<real>(LC ? LC : 2048))
+    k_batch_fft(const BatchInst<real> *__restrict__ inst, const FftUnit *__restrict__ units, int n_units, int n_inst,
+                int nrhs, int L_rt, int *counters, int *head, int *err, int spins)
 {
+    constexpr int NT = LC ? fft_threads(LC) : 0;
     extern __shared__ unsigned char smem_raw[];
+    const int L = LC ? LC : L_rt;
     cplx<real> *a = reinterpret_cast<cplx<real> *>(smem_raw);
-    cplx<real> *b = a + L_max;
+    cplx<real> *b = a + L;
+    const cplx<real> *tw = stage_twiddles<real, LC, NT>(b + L, inst[units[0].inst].tw, L);
     __shared__ int s_unit;
-    int *head = counters + 2 * n_inst * nrhs;
     for (;;) {
         if (threadIdx.x == 0)
             s_unit = atomicAdd(head, 1);
@@ -775,7 +776,7 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 5 : 3) k_batch_fft(co
         const int slot = fu.inst * nrhs + fu.rhs;
         int *rows_done = counters + slot;
         int *cols_done = counters + n_inst * nrhs + slot;
-        const int L = bi.L, n_a = bi.n_a, n = bi.n;
+        const int n_a = bi.n_a, n = bi.n;
         cplx<real> *spec = bi.spec + (int64_t)fu.rhs * bi.spec_stride;
         real *grid = bi.grid + (int64_t)fu.rhs * bi.grid_stride;
         bool ok = true;
@@ -784,13 +785,12 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 5 : 3) k_batch_fft(co
         else if (fu.kind == 2)
             ok = block_wait_geq(cols_done, n / 2 + 1, err, spins);
         if (ok) {
-            switch (L) {   // the line lengths of the instances' plans, as compile-time constants
-            case 256: batch_unit<real, 256>(fu, bi, spec, grid, a, b); break;
-            case 512: batch_unit<real, 512>(fu, bi, spec, grid, a, b); break;
-            case 1024: batch_unit<real, 1024>(fu, bi, spec, grid, a, b); break;
-            case 2048: batch_unit<real, 2048>(fu, bi, spec, grid, a, b); break;
-            default: batch_unit<real, 0>(fu, bi, spec, grid, a, b); break;
-            }
+            if (fu.kind == 0)
+                rows_fwd_unit<real, LC, NT>(fu.index, grid, bi.pitch, n_a, L, n / 2, spec, bi.ld, tw, a, b);
+            else if (fu.kind == 1)
+                cols_unit<real, true, LC, NT>(fu.index, spec, bi.ld, n_a, L, n, bi.mul, tw, a, b);
+            else
+                rows_inv_unit<real, true, LC, NT>(fu.index, spec, bi.ld, n_a, L, n / 2, grid, bi.pitch, tw, a, b);
         }
         __syncthreads();
         if (threadIdx.x == 0 && fu.kind < 2) {
@@ -1160,33 +1160,35 @@ cudaError_t launch_fft_rows_inv(const cplx<real> *spec, int ld, int n_a, int L, 
     });
 }
 
-template <typename real> cudaError_t batch_fft_blocks(int L_max, int *blocks)
+template <typename real> cudaError_t batch_fft_blocks(int L, int *blocks)
 {
-    const size_t smem = 2 * (size_t)L_max * sizeof(cplx<real>);
-    cudaError_t e = set_smem(k_batch_fft<real>, smem);
-    if (e != cudaSuccess)
-        return e;
+    const size_t smem = 3 * (size_t)L * sizeof(cplx<real>);   // two line buffers and the twiddles
     int dev = 0, sms = 0, per_sm = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess)
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-        return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_fft<real>, 256, smem)) != cudaSuccess)
-        return e;
+    e = with_line_length(L, [&](auto lc) {
+        constexpr int LC = decltype(lc)::value;
+        const cudaError_t e = set_smem(k_batch_fft<real, LC>, smem);
+        if (e != cudaSuccess)
+            return e;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_fft<real, LC>, fft_threads(LC ? LC : 2048), smem);
+    });
     *blocks = sms * (per_sm > 0 ? per_sm : 1);
-    return cudaSuccess;
+    return e;
 }
 
 template <typename real>
-cudaError_t launch_batch_fft(const BatchInst<real> *inst, const FftUnit *units, int n_units, int n_inst, int nrhs,
-                             int L_max, int grid_blocks, int *counters, int *err, int spins, cudaStream_t st)
+cudaError_t launch_batch_fft(const BatchInst<real> *inst, const FftUnit *units, const FftRun &run, int n_inst, int nrhs,
+                             int *counters, int *head, int *err, int spins, cudaStream_t st)
 {
-    if (n_units <= 0)
-        return cudaSuccess;
-    const size_t smem = 2 * (size_t)L_max * sizeof(cplx<real>);
-    k_batch_fft<real><<<(unsigned)grid_blocks, 256, smem, st>>>(inst, units, n_units, n_inst, nrhs, L_max, counters,
-                                                                err, spins);
-    return cudaGetLastError();
+    const size_t smem = 3 * (size_t)run.L * sizeof(cplx<real>);
+    return with_line_length(run.L, [&](auto lc) {
+        constexpr int LC = decltype(lc)::value;
+        k_batch_fft<real, LC><<<(unsigned)std::min(run.blocks, run.n), fft_threads(LC ? LC : 2048), smem, st>>>(
+            inst, units + run.first, run.n, n_inst, nrhs, run.L, counters, head, err, spins);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_wait_selftest(int *counter, int *err, int spins, cudaStream_t st)
@@ -1312,10 +1314,10 @@ template cudaError_t launch_build_mul<double>(const double2 *, int, const double
 
 template cudaError_t batch_fft_blocks<float>(int, int *);
 template cudaError_t batch_fft_blocks<double>(int, int *);
-template cudaError_t launch_batch_fft<float>(const BatchInst<float> *, const FftUnit *, int, int, int, int, int, int *,
-                                             int *, int, cudaStream_t);
-template cudaError_t launch_batch_fft<double>(const BatchInst<double> *, const FftUnit *, int, int, int, int, int,
-                                              int *, int *, int, cudaStream_t);
+template cudaError_t launch_batch_fft<float>(const BatchInst<float> *, const FftUnit *, const FftRun &, int, int, int *, int *,
+                                               int *, int, cudaStream_t);
+template cudaError_t launch_batch_fft<double>(const BatchInst<double> *, const FftUnit *, const FftRun &, int, int, int *, int *,
+                                               int *, int, cudaStream_t);
 
 template cudaError_t launch_fft3<float>(float *, int, int, int, float2 *, float2 *, const float *, const float2 *,
                                         cudaStream_t);

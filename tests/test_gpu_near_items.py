@@ -127,3 +127,26 @@ def test_grid_is_left_clean(n, precision, tol):
         for a, b in zip(fs.set_charges(q[0]).field(dtype=torch.float64), first):
             assert float((a - b).norm() / b.norm()) <= tol
     fs.close()
+
+
+@pytest.mark.parametrize("precision,tol", [(32, 2e-5), (64, 1e-12)])
+def test_batch_of_every_line_length(precision, tol):
+    """Transform lengths 64 (run-time length) to 1024, several instances of one length, two charge
+    vectors: the batch against its instances as plans, which differ by the order of the sums."""
+    import paper_0807_2387_gb300 as pkg
+    rng = np.random.default_rng(5)
+    dev = torch.device("cuda", 0)
+    inst, q = [], []
+    for k, n in enumerate((64, 32, 128, 64, 512, 32, 256)):
+        s, t = (torch.tensor(rng.uniform(-0.17, 0.17, (c, 2)), device=dev) for c in (300 + 70 * k, 200 + 90 * k))
+        inst.append((s, t, n, 4.0 / n))
+        q.append(torch.tensor(rng.standard_normal((2, len(s))), device=dev))
+    batch = pkg.FastSumBatch(inst, 2.0, 4, 2, precision=precision)
+    for _ in range(2):
+        phi, H = batch.eval(q, dtype=torch.float64)
+    for k, (s, t, n, eps) in enumerate(inst):
+        fs = pkg.FastSum(s, t, n, 2.0, 4, eps, precision=precision)
+        for a, b in zip((phi[k], H[k]), fs.set_charges(q[k]).field(dtype=torch.float64)):
+            assert rel(a, b) <= tol, (n, rel(a, b))
+        fs.close()
+    batch.close()
