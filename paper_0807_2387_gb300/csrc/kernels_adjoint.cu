@@ -191,18 +191,29 @@ template <int P> struct NearHess32 {
     static constexpr int kR = 1;
     __device__ __forceinline__ void fetch(int j, float (&v)[1]) const { v[0] = __ldg(q + j); }
     __device__ __forceinline__ void set_q(const float2 (&v)[1]) { qj = v[0]; }
+    // the sums of the clamped form over c and c' carry these signs
+    static constexpr float kC = kSat && P % 2 == 0 ? -1.f : 1.f, kCp = kSat && P % 2 != 0 ? -1.f : 1.f;
     __device__ __forceinline__ void coincident(const NearParams<float> &, int t)
     {
-        add_comp(sI, t, -comp(qj, t) * self_c);
+        add_comp(sI, t, -comp(qj, t) * (kC * self_c));
     }
     __device__ __forceinline__ void pair2(const NearParams<float> &np, float2 w, float2 dx, float2 dy)
     {
-        float2 c, cp;
-        near_c_cp2<P>(w, c, cp);
-        float2 qq = qj;
-        if constexpr (!kSat)
-            qq = select2(w, np.eps2, qq);
-        const float2 qc = mul2(qq, c), k = mul2(qq, cp);
+        float2 qc, k;
+        if constexpr (kSat) {
+            const float2 s = fma2(w, f2(-1.f), f2(1.f));
+            float2 b, h;
+            near_b2<P>(w, s, b, h);
+            const float2 qb = mul2(qj, b);
+            qc = mul2(qb, s);
+            k = mul2(qb, h);
+        } else {
+            float2 c, cp;
+            near_c_cp2<P>(w, c, cp);
+            const float2 qq = select2(w, np.eps2, qj);
+            qc = mul2(qq, c);
+            k = mul2(qq, cp);
+        }
         gx = fma2(qc, dx, gx);
         gy = fma2(qc, dy, gy);
         sI = add2(sI, qc);
@@ -226,9 +237,9 @@ template <int P> struct NearHess32 {
     __device__ __forceinline__ void store(int64_t k)
     {
         // (a select, not a product with 0: the stored-to buffers may hold anything, NaN included)
-        const float i0 = sI.x, rg = rcoef * geps;
-        const float v[5] = {rg * gx.x, rg * gy.x, rcoef * fmaf(2.f, sxx.x, i0), rcoef * 2.f * sxy.x,
-                            rcoef * fmaf(2.f, syy.x, i0)};
+        const float i0 = kC * sI.x, rg = kC * rcoef * geps;
+        const float v[5] = {rg * gx.x, rg * gy.x, rcoef * fmaf(2.f * kCp, sxx.x, i0), rcoef * (2.f * kCp) * sxy.x,
+                            rcoef * fmaf(2.f * kCp, syy.x, i0)};
         grad_s[2 * k] = assign ? v[0] : grad_s[2 * k] + v[0];
         grad_s[2 * k + 1] = assign ? v[1] : grad_s[2 * k + 1] + v[1];
         hess_s[3 * k] = assign ? v[2] : hess_s[3 * k] + v[2];
@@ -254,7 +265,10 @@ template <int P> struct NearAdj32 {
     float *__restrict__ cg_s;
     float rcoef, geps, inv_eps, self_c;   // rc, eps_I, 1 / eps_I, self_c = Hess T_I(0) / rc
     bool assign;                           // store instead of adding (the far part is added later)
-    float2 gp, dn1, dn2;                   // of the pair of candidates
+    // f is summed in units of c_ln (near_g2); the sums of the clamped form over c and c' carry signs
+    static constexpr float kF = kSat ? kLnCoef : 1.f;
+    static constexpr float kC = kSat && P % 2 == 0 ? -1.f : 1.f, kCp = kSat && P % 2 != 0 ? -1.f : 1.f;
+    float2 gp, dn1, dn2;                   // of the pair of candidates: gphi and -n'
     float2 af, ac, gxc, gyc, gxk, gyk, gco;
 
     __device__ __forceinline__ void init() { af = ac = gxc = gyc = gxk = gyk = gco = f2(0.f); }
@@ -264,8 +278,8 @@ template <int P> struct NearAdj32 {
     {
         const float2 d = __ldg(dnw + i);
         v[0] = __ldg(cw + i);
-        v[1] = d.x * inv_eps;
-        v[2] = d.y * inv_eps;
+        v[1] = -d.x * inv_eps;
+        v[2] = -d.y * inv_eps;
     }
     __device__ __forceinline__ void set_q(const float2 (&v)[3])
     {
@@ -275,28 +289,34 @@ template <int P> struct NearAdj32 {
     }
     __device__ __forceinline__ void coincident(const NearParams<float> &np, int t)
     {
-        add_comp(af, t, -comp(gp, t) * np.beta[0]);
+        add_comp(af, t, -comp(gp, t) * (np.beta[0] / kF));
         add_comp(gco, t, comp(gp, t));
-        add_comp(gxc, t, self_c * comp(dn1, t));
-        add_comp(gyc, t, self_c * comp(dn2, t));
+        add_comp(gxc, t, -(kC * self_c) * comp(dn1, t));
+        add_comp(gyc, t, -(kC * self_c) * comp(dn2, t));
     }
     __device__ __forceinline__ void pair2(const NearParams<float> &np, float2 w, float2 dx, float2 dy)
     {
-        float2 c, cp;
-        near_c_cp2<P>(w, c, cp);
-        const float2 f = near_f2<P>(np, w);
-        float2 g = gp, n1 = dn1, n2 = dn2;
-        if constexpr (!kSat) {
+        float2 c, f, kd, g = gp, n1 = dn1, n2 = dn2;
+        if constexpr (kSat) {
+            const float2 s = fma2(w, f2(-1.f), f2(1.f));
+            float2 b, h;
+            near_b2<P>(w, s, b, h);
+            c = mul2(b, s);
+            f = near_g2<P>(np, w, s, lg2_2(w));
+            kd = mul2(b, h);
+        } else {
+            near_c_cp2<P>(w, c, kd);
+            f = near_f2<P>(np, w);
             g = select2(w, np.eps2, g);
             n1 = select2(w, np.eps2, n1);
             n2 = select2(w, np.eps2, n2);
         }
-        const float2 dD = fma2(n1, dx, mul2(n2, dy));
+        const float2 dD = fma2(n1, dx, mul2(n2, dy));   // -(n'.d')
         af = fma2(g, f, af);
         ac = fma2(dD, c, ac);
-        gxc = fma2(c, fma2(g, dx, mul2(f2(-1.f), n1)), gxc);
-        gyc = fma2(c, fma2(g, dy, mul2(f2(-1.f), n2)), gyc);
-        const float2 k = mul2(cp, dD);
+        gxc = fma2(c, fma2(g, dx, n1), gxc);
+        gyc = fma2(c, fma2(g, dy, n2), gyc);
+        const float2 k = mul2(kd, dD);
         gxk = fma2(k, dx, gxk);
         gyk = fma2(k, dy, gyk);
     }
@@ -315,9 +335,9 @@ template <int P> struct NearAdj32 {
     __device__ __forceinline__ void store(int64_t k)
     {
         const float rg = rcoef * geps;
-        const float va = fmaf(-rg * geps, ac.x, af.x);
-        const float vx = rg * fmaf(-2.f, gxk.x, gxc.x);
-        const float vy = rg * fmaf(-2.f, gyk.x, gyc.x);
+        const float va = fmaf(kC * rg * geps, ac.x, kF * af.x);
+        const float vx = rg * fmaf(2.f * kCp, gxk.x, kC * gxc.x);
+        const float vy = rg * fmaf(2.f * kCp, gyk.x, kC * gyc.x);
         a_s[k] = assign ? va : a_s[k] + va;
         ga_s[2 * k] = assign ? vx : ga_s[2 * k] + vx;
         ga_s[2 * k + 1] = assign ? vy : ga_s[2 * k + 1] + vy;
