@@ -193,6 +193,11 @@ template <int DEG, typename real> __device__ __forceinline__ real poly_eval(cons
     return acc;
 }
 
+// Launch chaining: from here on the stream's next kernel, if launched to allow it, may start its blocks
+// (once every block of this one got here); and the wait of such a kernel for the previous one's end.
+__device__ __forceinline__ void next_kernel_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Even and odd parts of sum_i c[i] t^i as polynomials in s = t^2: e = sum_j c[2j] s^j,
 // o = sum_j c[2j+1] s^j, so that the polynomial at +-t is e +- t o.
 template <int DEG, typename real> __device__ __forceinline__ void poly_even_odd(const real *c, real s, real &e, real &o)

@@ -894,17 +894,18 @@ template <typename real> fs_status eval_t(fs_plan *pl, void *phi, void *H, fs_dt
             FS_TRY(near_beside());
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[1], st));
+        const bool chain = pl->chained(pl->n_items, R);
         FS_CUDA(launch_fft_rows_fwd<real>((real *)pl->grid, pl->pitch, pl->n_a, pl->n_os, pl->n / 2, (C *)pl->spec,
-                                          pl->ld, (const C *)pl->tw, R, grid_n, spec_n, st));
+                                          pl->ld, (const C *)pl->tw, R, grid_n, spec_n, chain, st));
         pl->grid_dirty = pl->grid_recorded || pl->field == pl->grid;
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[2], st));
         FS_CUDA(launch_fft_cols<real>((C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n, (const real *)pl->mul,
-                                      (const C *)pl->tw, R, spec_n, st));
+                                      (const C *)pl->tw, R, spec_n, chain, st));
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[3], st));
         FS_CUDA(launch_fft_rows_inv<real>((const C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n / 2,
-                                          (real *)pl->field, pl->pitch, (const C *)pl->tw, R, grid_n, spec_n, st));
+                                          (real *)pl->field, pl->pitch, (const C *)pl->tw, R, grid_n, spec_n, chain, st));
         if (rec)
             FS_CUDA(cudaEventRecord(pl->ev[4], st));
         auto out_phi = [&](int r) { return phi ? (unsigned char *)phi + (size_t)(r0 + r) * pl->N * osz : nullptr; };
@@ -1006,17 +1007,17 @@ fs_status boundary_edges(const std::vector<int> &tris, int64_t Nt, int64_t Nv, s
 }
 
 // Far-field pipeline on the plan's grid: spread (given launcher) -> FFT rows -> columns x mul -> inverse rows.
-template <typename real> fs_status spectral_pipeline(fs_plan *pl)
+template <typename real> fs_status spectral_pipeline(fs_plan *pl, bool chained)
 {
     using C = typename Cplx<real>::type;
     cudaStream_t st = pl->stream;
     FS_CUDA(launch_fft_rows_fwd<real>((real *)pl->grid, pl->pitch, pl->n_a, pl->n_os, pl->n / 2, (C *)pl->spec,
-                                      pl->ld, (const C *)pl->tw, 1, 0, 0, st));
+                                      pl->ld, (const C *)pl->tw, 1, 0, 0, chained, st));
     pl->grid_dirty = pl->grid_recorded || pl->field == pl->grid;
     FS_CUDA(launch_fft_cols<real>((C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n, (const real *)pl->mul,
-                                  (const C *)pl->tw, 1, 0, st));
+                                  (const C *)pl->tw, 1, 0, chained, st));
     FS_CUDA(launch_fft_rows_inv<real>((const C *)pl->spec, pl->ld, pl->n_a, pl->n_os, pl->n / 2, (real *)pl->field,
-                                      pl->pitch, (const C *)pl->tw, 1, 0, 0, st));
+                                      pl->pitch, (const C *)pl->tw, 1, 0, 0, chained, st));
     return FS_OK;
 }
 
@@ -1062,7 +1063,7 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
                 }
             }
             FS_TRY(spread_forward<real>(pl, q, 1, st));
-            FS_TRY(spectral_pipeline<real>(pl));
+            FS_TRY(spectral_pipeline<real>(pl, pl->chained(pl->n_items, 1)));
             if (ovl)
                 FS_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
             FS_CUDA(launch_interp_hess<real>(N, pl->m, pl->tgt_base, pl->tgt_frac, win_poly<real>(pl), (const real *)pl->field,
@@ -1097,7 +1098,7 @@ fs_status adjoint_t(fs_plan *pl, const void *g_phi, const void *g_H, fs_dtype in
             FS_CUDA(launch_spread_dip<real>(pl->tgt_items, pl->n_tgt_items, pl->cg, pl->m, pl->tgt_base, pl->tgt_frac,
                                             (const real *)pl->adj_c, pl->adj_df, win_poly<real>(pl), (real *)pl->grid,
                                             pl->pitch, pl->n_a, pl->kahan, st));
-            FS_TRY(spectral_pipeline<real>(pl));
+            FS_TRY(spectral_pipeline<real>(pl, pl->chained(pl->n_tgt_items, 1)));
             if (ovl)
                 FS_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
             FS_CUDA(launch_interp<real>(M, pl->m, pl->src_base, pl->src_frac, win_poly<real>(pl), (const real *)pl->field,

@@ -407,15 +407,15 @@ template <typename real> void fft_twiddle_table(int L, real *re_im);
 template <typename real>
 cudaError_t launch_fft_rows_fwd(real *grid, int pitch, int n_a, int L, int n_half,
                                 typename Cplx<real>::type *spec, int ld, const typename Cplx<real>::type *tw,
-                                int nrhs, int64_t grid_stride, int64_t spec_stride, cudaStream_t st);
+                                int nrhs, int64_t grid_stride, int64_t spec_stride, bool chained, cudaStream_t st);
 template <typename real>
 cudaError_t launch_fft_cols(typename Cplx<real>::type *spec, int ld, int n_a, int L, int n,
                             const real *mul, const typename Cplx<real>::type *tw, int nrhs, int64_t spec_stride,
-                            cudaStream_t st);
+                            bool chained, cudaStream_t st);
 template <typename real>
 cudaError_t launch_fft_rows_inv(const typename Cplx<real>::type *spec, int ld, int n_a, int L, int n_half,
                                 real *grid, int pitch, const typename Cplx<real>::type *tw, int nrhs, int64_t grid_stride,
-                                int64_t spec_stride, cudaStream_t st);
+                                int64_t spec_stride, bool chained, cudaStream_t st);
 cudaError_t launch_kernel_samples(double2 *samp, int n, KernelParams kp, cudaStream_t st);
 cudaError_t launch_fft_lines_c64(double2 *data, int lines, int L, const double2 *tw, cudaStream_t st);
 cudaError_t launch_transpose_c64(const double2 *in, double2 *out, int n, cudaStream_t st);

@@ -676,6 +676,8 @@ __global__ void __launch_bounds__(256) k_fft_rows_fwd(real *__restrict__ grid, i
     extern __shared__ unsigned char smem_raw[];
     cplx<real> *a = reinterpret_cast<cplx<real> *>(smem_raw);
     cplx<real> *s_tw = stage_twiddles<real, LC, NT>(a + 2 * L, tw, L);   // published by the unit's first barrier
+    next_kernel_may_start();
+    wait_previous_kernel();
     real *g = grid + blockIdx.y * grid_stride;
     rows_fwd_unit<real, LC, NT>(blockIdx.x, g, pitch, n_a, L, n_half, spec + blockIdx.y * spec_stride, ld, s_tw, a, a + L);
     // the block's rows are read (its last barrier lies after the reads): leave the grid zeroed for the
@@ -694,6 +696,8 @@ __global__ void __launch_bounds__(256) k_fft_cols(cplx<real> *__restrict__ spec,
     extern __shared__ unsigned char smem_raw[];
     cplx<real> *a = reinterpret_cast<cplx<real> *>(smem_raw);
     cplx<real> *s_tw = stage_twiddles<real, LC, NT>(a + 2 * L, tw, L);
+    next_kernel_may_start();
+    wait_previous_kernel();
     cols_unit<real, false, LC, NT>(blockIdx.x, spec + blockIdx.y * spec_stride, ld, n_a, L, n, mul, s_tw, a, a + L);
 }
 
@@ -707,6 +711,7 @@ __global__ void __launch_bounds__(256) k_fft_rows_inv(const cplx<real> *__restri
     extern __shared__ unsigned char smem_raw[];
     cplx<real> *a = reinterpret_cast<cplx<real> *>(smem_raw);
     cplx<real> *s_tw = stage_twiddles<real, LC, NT>(a + 2 * L, tw, L);
+    wait_previous_kernel();
     rows_inv_unit<real, false, LC, NT>(blockIdx.x, spec + blockIdx.y * spec_stride, ld, n_a, L, n_half,
                                        grid + blockIdx.y * grid_stride, pitch, s_tw, a, a + L);
 }
@@ -1089,6 +1094,25 @@ __global__ void k_build_mul(const double2 *__restrict__ bhat, int n, const doubl
 }
 
 
+// A launch whose blocks may start while the stream's previous kernel (one of this library's that
+// calls next_kernel_may_start) still runs; the kernel calls wait_previous_kernel before it touches
+// anything another kernel writes or reads.
+template <typename... P, typename... A>
+cudaError_t launch_chained(bool chained, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 template <typename K> cudaError_t set_smem(K kern, size_t bytes)
 {
     if (bytes <= kSmemDefault)
@@ -1114,7 +1138,8 @@ template <typename F> cudaError_t with_line_length(int L, F &&f)
 
 template <typename real>
 cudaError_t launch_fft_rows_fwd(real *grid, int pitch, int n_a, int L, int n_half, cplx<real> *spec, int ld,
-                                const cplx<real> *tw, int nrhs, int64_t grid_stride, int64_t spec_stride, cudaStream_t st)
+                                const cplx<real> *tw, int nrhs, int64_t grid_stride, int64_t spec_stride, bool chained,
+                                cudaStream_t st)
 {
     const size_t smem = 3 * (size_t)L * sizeof(cplx<real>);   // two line buffers and the twiddles
     return with_line_length(L, [&](auto lc) {
@@ -1122,15 +1147,14 @@ cudaError_t launch_fft_rows_fwd(real *grid, int pitch, int n_a, int L, int n_hal
         cudaError_t e = set_smem(k_fft_rows_fwd<real, LC>, smem);
         if (e != cudaSuccess)
             return e;
-        k_fft_rows_fwd<real, LC><<<dim3((n_a + 1) / 2, nrhs), fft_threads(L), smem, st>>>(grid, pitch, n_a, L, n_half, spec,
-                                                                                            ld, tw, grid_stride, spec_stride);
-        return cudaGetLastError();
+        return launch_chained(chained, k_fft_rows_fwd<real, LC>, dim3((n_a + 1) / 2, nrhs), fft_threads(L), smem, st, grid,
+                              pitch, n_a, L, n_half, spec, ld, tw, grid_stride, spec_stride);
     });
 }
 
 template <typename real>
 cudaError_t launch_fft_cols(cplx<real> *spec, int ld, int n_a, int L, int n, const real *mul, const cplx<real> *tw,
-                            int nrhs, int64_t spec_stride, cudaStream_t st)
+                            int nrhs, int64_t spec_stride, bool chained, cudaStream_t st)
 {
     const size_t smem = 3 * (size_t)L * sizeof(cplx<real>);   // two line buffers and the twiddles
     return with_line_length(L, [&](auto lc) {
@@ -1138,15 +1162,15 @@ cudaError_t launch_fft_cols(cplx<real> *spec, int ld, int n_a, int L, int n, con
         cudaError_t e = set_smem(k_fft_cols<real, LC>, smem);
         if (e != cudaSuccess)
             return e;
-        k_fft_cols<real, LC><<<dim3(n / 2 + 1, nrhs), fft_threads(L), smem, st>>>(spec, ld, n_a, L, n, mul, tw, spec_stride);
-        return cudaGetLastError();
+        return launch_chained(chained, k_fft_cols<real, LC>, dim3(n / 2 + 1, nrhs), fft_threads(L), smem, st, spec, ld, n_a, L,
+                              n, mul, tw, spec_stride);
     });
 }
 
 template <typename real>
 cudaError_t launch_fft_rows_inv(const cplx<real> *spec, int ld, int n_a, int L, int n_half, real *grid, int pitch,
                                 const cplx<real> *tw, int nrhs, int64_t grid_stride, int64_t spec_stride,
-                                cudaStream_t st)
+                                bool chained, cudaStream_t st)
 {
     const size_t smem = 3 * (size_t)L * sizeof(cplx<real>);   // two line buffers and the twiddles
     return with_line_length(L, [&](auto lc) {
@@ -1154,9 +1178,8 @@ cudaError_t launch_fft_rows_inv(const cplx<real> *spec, int ld, int n_a, int L, 
         cudaError_t e = set_smem(k_fft_rows_inv<real, LC>, smem);
         if (e != cudaSuccess)
             return e;
-        k_fft_rows_inv<real, LC><<<dim3((n_a + 1) / 2, nrhs), fft_threads(L), smem, st>>>(spec, ld, n_a, L, n_half, grid,
-                                                                                            pitch, tw, grid_stride, spec_stride);
-        return cudaGetLastError();
+        return launch_chained(chained, k_fft_rows_inv<real, LC>, dim3((n_a + 1) / 2, nrhs), fft_threads(L), smem, st, spec, ld,
+                              n_a, L, n_half, grid, pitch, tw, grid_stride, spec_stride);
     });
 }
 
@@ -1298,17 +1321,17 @@ template void fft_twiddle_table<float>(int, float *);
 template void fft_twiddle_table<double>(int, double *);
 
 template cudaError_t launch_fft_rows_fwd<float>(float *, int, int, int, int, float2 *, int, const float2 *, int,
-                                                int64_t, int64_t, cudaStream_t);
+                                                int64_t, int64_t, bool, cudaStream_t);
 template cudaError_t launch_fft_rows_fwd<double>(double *, int, int, int, int, double2 *, int, const double2 *, int,
-                                                int64_t, int64_t, cudaStream_t);
+                                                int64_t, int64_t, bool, cudaStream_t);
 template cudaError_t launch_fft_cols<float>(float2 *, int, int, int, int, const float *, const float2 *, int, int64_t,
-                                            cudaStream_t);
+                                            bool, cudaStream_t);
 template cudaError_t launch_fft_cols<double>(double2 *, int, int, int, int, const double *, const double2 *, int, int64_t,
-                                            cudaStream_t);
+                                            bool, cudaStream_t);
 template cudaError_t launch_fft_rows_inv<float>(const float2 *, int, int, int, int, float *, int, const float2 *, int,
-                                                int64_t, int64_t, cudaStream_t);
+                                                int64_t, int64_t, bool, cudaStream_t);
 template cudaError_t launch_fft_rows_inv<double>(const double2 *, int, int, int, int, double *, int, const double2 *, int,
-                                                int64_t, int64_t, cudaStream_t);
+                                                int64_t, int64_t, bool, cudaStream_t);
 template cudaError_t launch_build_mul<float>(const double2 *, int, const double *, float *, cudaStream_t);
 template cudaError_t launch_build_mul<double>(const double2 *, int, const double *, double *, cudaStream_t);
 

@@ -300,6 +300,7 @@ __global__ void __launch_bounds__(kSpreadWarps * 32) k_spread(const SpreadItem *
                                                               real *__restrict__ grid, int pitch, int n_a,
                                                               int64_t q_stride, int64_t grid_stride)
 {
+    next_kernel_may_start();
     spread_item<real, M2, KAHAN, TGC>(items[blockIdx.x], cg, base, frac, q + blockIdx.y * q_stride, wp,
                                       grid + blockIdx.y * grid_stride, pitch, n_a);
 }
@@ -604,6 +605,7 @@ __global__ void __launch_bounds__(kSpreadWarps * 32) k_spread_dip(const SpreadIt
                                                                   WinPoly<real> wp, real *__restrict__ grid, int pitch,
                                                                   int n_a)
 {
+    next_kernel_may_start();
     constexpr int m = M2 / 2;
     constexpr int TAPS = M2 * M2;
     constexpr int PER = (TAPS + 31) / 32;

@@ -25,6 +25,7 @@ struct NearCell {
     int first, count;
 };
 constexpr int kSrcMajorItem = 64;   // sources per item of the source-major near field
+constexpr int kSms = 152;           // streaming multiprocessors of a GB300
 constexpr int kRhsGroup = 4;       // charge vectors a plan evaluates together at most
 constexpr int kSpreadChunk = 512;   // sources per spreading work item
 // 2D plans whose occupied spreading tiles hold fewer sources than this on average spread with
@@ -181,6 +182,15 @@ struct fs_plan {
     // makes no difference beyond 1.5 % (1,000 targets 40.7 us against 41.3 us with the near field first,
     // whose submission delays the longer chain); uniform 262,144 points have items of up to 5.7e4 pairs.
     bool near_first() const { return !near_cells_h.empty() && near_cells_h[0].work >= (1 << 16); }
+    // Whether the transform's kernels start before the kernel ahead of them has ended (launch_chained):
+    // where each of them and the spreading (n_items) has at most a block per SM.  There a launch's
+    // latency counts: evaluations of 1,000 and 4,096 points 35.8 -> 24.5 and 31.8 -> 24.6 us on the GPU.
+    // With more blocks the waiting ones keep slots that the spreading or the near field needs: 32,768 points in FP64
+    // 875 -> 992 us, the disc mesh 131 -> 145, a training step of 262,144 points 974 -> 988.
+    bool chained(int n_items, int nrhs) const
+    {
+        return n_items > 0 && n_items <= fs::kSms && (n_a + 1) / 2 * nrhs <= fs::kSms && !spread_direct;
+    }
     size_t rsize() const { return precision == 64 ? 8 : 4; }
 };
 
