@@ -45,22 +45,29 @@ def library_path() -> str:
     return LIB_PATH
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    # torch is imported at the first use; the module is kept, since small evaluations are a few
+    # microseconds of Python each
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _dev_ptr(t, dtype=None, name="tensor"):
-    torch = _torch()
     if t is None:
         return None
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+    if not isinstance(t, _torch().Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
     if dtype is not None and t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _dtype_code(dt):
@@ -241,7 +248,7 @@ def _ptr_array(tensors, name):
         return None
     arr = (ctypes.c_void_p * len(tensors))()
     for i, t in enumerate(tensors):
-        arr[i] = None if t is None else _dev_ptr(t, name=name).value
+        arr[i] = None if t is None else _dev_ptr(t, name=name)
     return arr
 
 
@@ -468,19 +475,19 @@ class FastSum:
     def potential(self, dtype=None):
         torch = _torch()
         dtype = dtype or (torch.float64 if self.info["precision"] == 64 else torch.float32)
-        phi = torch.empty((self.nrhs, self.info["n_tgt"]), dtype=dtype, device=self.device)
+        n = self.info["n_tgt"]
+        phi = torch.empty(n if self.nrhs == 1 else (self.nrhs, n), dtype=dtype, device=self.device)
         fs_eval_potential(self._h, phi)
-        return phi[0] if self.nrhs == 1 else phi
+        return phi
 
     def field(self, dtype=None, with_phi=True):
         torch = _torch()
         dtype = dtype or (torch.float64 if self.info["precision"] == 64 else torch.float32)
         n = self.info["n_tgt"]
-        phi = torch.empty((self.nrhs, n), dtype=dtype, device=self.device) if with_phi else None
-        H = torch.empty((self.nrhs, n, 2), dtype=dtype, device=self.device)
+        one = self.nrhs == 1                    # one vector: no leading axis
+        phi = torch.empty(n if one else (self.nrhs, n), dtype=dtype, device=self.device) if with_phi else None
+        H = torch.empty((n, 2) if one else (self.nrhs, n, 2), dtype=dtype, device=self.device)
         fs_eval_field(self._h, phi, H)
-        if self.nrhs == 1:
-            return (phi[0] if with_phi else None), H[0]
         return phi, H
 
     def adjoint(self, g_phi=None, g_H=None, want_q=True, want_src=False, want_tgt=False, dtype=None):
@@ -623,11 +630,10 @@ class FastSum3:
         torch = _torch()
         dtype = dtype or (torch.float64 if self.info["precision"] == 64 else torch.float32)
         n = self.info["n_tgt"]
-        phi = torch.empty((self.nrhs, n), dtype=dtype, device=self.device) if with_phi else None
-        H = torch.empty((self.nrhs, n, 3), dtype=dtype, device=self.device)
+        one = self.nrhs == 1                    # one vector: no leading axis
+        phi = torch.empty(n if one else (self.nrhs, n), dtype=dtype, device=self.device) if with_phi else None
+        H = torch.empty((n, 3) if one else (self.nrhs, n, 3), dtype=dtype, device=self.device)
         fs3_eval_field(self._h, phi, H)
-        if self.nrhs == 1:
-            return (phi[0] if with_phi else None), H[0]
         return phi, H
 
     def sync(self):
