@@ -150,3 +150,35 @@ def test_batch_of_every_line_length(precision, tol):
             assert rel(a, b) <= tol, (n, rel(a, b))
         fs.close()
     batch.close()
+
+
+@pytest.mark.parametrize("n,count", [(64, 900), (256, 40000)])
+def test_captured_evaluation(n, count):
+    """An evaluation recorded into a graph and replayed twice with new charges: plans whose transform
+    kernels are chained (n = 64) and plans without; against the same evaluations made directly."""
+    import paper_0807_2387_gb300 as pkg
+    rng = np.random.default_rng(6)
+    dev = torch.device("cuda", 0)
+    src = torch.tensor(rng.uniform(-0.17, 0.17, (count, 2)), device=dev)
+    qs = torch.tensor(rng.standard_normal((3, count)), device=dev)
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(st):
+        fs = pkg.FastSum(src, src, n, 2.0, 4, 4.0 / n, precision=32, stream=st)
+        ref = [[v.clone() for v in fs.set_charges(q).field()] for q in qs]
+        q = qs[0].clone()
+        phi, H = torch.empty(count, device=dev), torch.empty((count, 2), device=dev)
+        st.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            pkg.fs_set_charges(fs.handle, q)
+            pkg.fs_eval_field(fs.handle, phi, H)
+        for k in (2, 1):
+            q.copy_(qs[k])
+            graph.replay()
+            st.synchronize()
+            assert rel(phi, ref[k][0]) <= 2e-5 and rel(H, ref[k][1]) <= 2e-5
+        for a, b in zip(fs.set_charges(qs[0]).field(), ref[0]):   # and directly again
+            assert rel(a, b) <= 2e-5
+    st.synchronize()
+    fs.close()
