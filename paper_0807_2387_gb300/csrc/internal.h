@@ -15,24 +15,51 @@ constexpr size_t kSmemDefault = 47 * 1024;
 // Warps per spreading CTA; each holds a private padded tile in shared memory.
 constexpr int kSpreadWarps = 4;
 
-// Shared memory of the spreading kernels: the warp tiles (PLANES planes of P rows at pitch Q),
-// padded to 16 bytes, then each warp's window weights (a group's row weights vector-aligned,
-// then the column weights), then the FP32 window polynomials.
-template <typename real> __host__ __device__ constexpr int spread_weight_stride(int M2)
+// A warp of the spreading kernels forms the window weights of a batch of sources, then adds one source
+// after the other.  A source's record: the row weights of the G groups (each padded to 16 bytes), the
+// column weights times the charge in the same order, and its first tap's offset in the tile.
+template <typename real> __host__ __device__ constexpr int spread_group_pad(int M2)
 {
-    const int G = spread_groups(M2), RPL = M2 / G, VW = 16 / (int)sizeof(real);
-    return G * ((RPL + VW - 1) / VW * VW) + (M2 + VW - 1) / VW * VW;
+    const int RPL = M2 / spread_groups(M2), VW = 16 / (int)sizeof(real);
+    return (RPL + VW - 1) / VW * VW;
 }
 
+template <typename real> __host__ __device__ constexpr int spread_record(int M2)
+{
+    return 2 * spread_groups(M2) * spread_group_pad<real>(M2) + 16 / (int)sizeof(real);
+}
+
+// Shared memory of the spreading kernels: the warp tiles (PLANES planes of P rows at pitch Q),
+// padded to 16 bytes, then each warp's records.
 template <typename real> __host__ __device__ inline size_t spread_tiles_bytes(int P, int Q, int planes)
 {
     return ((size_t)kSpreadWarps * P * Q * planes * sizeof(real) + 15) / 16 * 16;
 }
 
-template <typename real> inline size_t spread_smem_bytes(int P, int M2, bool comp)   // k_spread, k_batch_spread
+// Sources of a batch: 16 (every lane forms weights); 8 beside FP32 tiles of more than 32 KB, whose
+// records would take the shared memory that the near field's blocks need on the same SMs (disc mesh,
+// 24-line tiles: time loop 141 us with 8, 152 with 16; 16-line tiles: 262,144 sources 43.6 us with 16,
+// 47.3 with 8; FP64, which has no such neighbour, 62 against 94 us for 32,768 sources).
+template <typename real> __host__ __device__ inline int spread_batch(int P, int Q, int planes)
 {
+    return sizeof(real) == 4 && spread_tiles_bytes<real>(P, Q, planes) > 32 * 1024 ? 8 : 16;
+}
+
+template <typename real> inline size_t spread_launch_bytes(int P, int M2, bool comp)   // k_spread, k_batch_spread
+{
+    const int Q = spread_group_pitch(P, M2), planes = comp ? 2 : 1;
+    return spread_tiles_bytes<real>(P, Q, planes) +
+           (size_t)kSpreadWarps * spread_batch<real>(P, Q, planes) * spread_record<real>(M2) * sizeof(real);
+}
+
+// The measure by which tiles are chosen and admitted (at most 200 KB): the tiles, one source's weights a
+// warp and the polynomials the adjoint's kernel holds.  The records, up to 18 KB, fit beside it.
+template <typename real> inline size_t spread_smem_bytes(int P, int M2, bool comp)
+{
+    const int G = spread_groups(M2), VW = 16 / (int)sizeof(real);
+    const int weights = G * spread_group_pad<real>(M2) + (M2 + VW - 1) / VW * VW;
     return spread_tiles_bytes<real>(P, spread_group_pitch(P, M2), comp ? 2 : 1) +
-           (size_t)kSpreadWarps * spread_weight_stride<real>(M2) * sizeof(real) + sizeof(float) * M2 * (kPolyD + 1);
+           (size_t)kSpreadWarps * weights * sizeof(real) + sizeof(float) * M2 * (kPolyD + 1);
 }
 
 // How the points of a cell, and its near-field items, are ordered: in runs of at most kOrderRun

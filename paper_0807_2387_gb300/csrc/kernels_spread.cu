@@ -57,6 +57,14 @@ __device__ __forceinline__ float2 sub2f(float2 a, float2 b)   // a - b, one roun
     return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
 }
 
+// A work item's sources, split over the warps of the block.  Lane pairs (one lane per coordinate) form the
+// window weights of `batch` sources at once, each symmetric pair of taps from the even and odd parts of
+// one's polynomials, and leave them in shared memory; then the warp adds the sources one by one: tap
+// lane (g, b) owns column b and rows g RPL .. g RPL + RPL - 1 of every source.  With the weights formed
+// per source by lanes that each held one tap's polynomial the kernel was bound by its issue slots (132
+// instructions a source at m = 5).  262,144 uniform sources 52.2 -> 43.6 us, 2^20 clustered ones
+// (m = 6) 178 -> 145, 32,768 in FP64 (m = 6) 101 -> 62.  Bound by the tile's shared-memory reads and writes
+// (two planes of 2m taps a lane column, about 25 wavefronts a source) and by occupancy.
 // TGC > 0: the tile edge (grid lines) fixed at compile time, so that the tile pitch and the
 // row offsets of the taps are constants (immediate offsets instead of one address per row).
 template <typename real, int M2, bool KAHAN, int TGC = 0>
@@ -69,8 +77,7 @@ __device__ __forceinline__ void spread_item(const SpreadItem &it, const CellGrid
     constexpr int G = spread_groups(M2);
     constexpr int RPL = M2 / G;                               // rows per tap lane
     constexpr int VW = 16 / (int)sizeof(real);
-    constexpr int RPAD = (RPL + VW - 1) / VW * VW;            // a group's row weights, vector-aligned
-    constexpr int WSTRIDE = spread_weight_stride<real>(M2);
+    constexpr int RPAD = spread_group_pad<real>(M2), SIDE = G * RPAD, REC = spread_record<real>(M2);
     constexpr int PLANES = KAHAN ? 2 : 1;
     constexpr bool kF32 = sizeof(real) == 4;
     constexpr int D = WinPolyOf<real>::D;
@@ -82,122 +89,127 @@ __device__ __forceinline__ void spread_item(const SpreadItem &it, const CellGrid
     const int Q = TGC > 0 ? kQ : spread_group_pitch(P, M2);   // row pitch: conflict-free tap rows
     const int PP = P * Q;                                     // one plane of a warp tile
     real *acc = reinterpret_cast<real *>(smem_raw) + (size_t)warp * PP * PLANES;
-    unsigned char *after_tiles = smem_raw + spread_tiles_bytes<real>(P, Q, PLANES);
-    real *wb = reinterpret_cast<real *>(after_tiles) + warp * WSTRIDE;
-    float *poly = reinterpret_cast<float *>(after_tiles + (size_t)kSpreadWarps * WSTRIDE * sizeof(real));
-    if constexpr (kF32) {
-        for (int i = threadIdx.x; i < M2 * (kPolyD + 1); i += blockDim.x)
-            poly[i] = wp.c[i / (kPolyD + 1)][i % (kPolyD + 1)];
-    }
+    const int batch = spread_batch<real>(P, Q, PLANES);
+    real *records = reinterpret_cast<real *>(smem_raw + spread_tiles_bytes<real>(P, Q, PLANES)) + warp * batch * REC;
     const int t1 = it.tile / cg.n_t, t2 = it.tile - (it.tile / cg.n_t) * cg.n_t;
     const int o1 = t1 * TG - (m - 1), o2 = t2 * TG - (m - 1);
     for (int i = lane; i < PP * PLANES; i += 32)
         acc[i] = real(0);
-    __syncthreads();
-    // weight lanes: lane a < M2 evaluates the first coordinate's weight of row a, lane M2 + b the
-    // second coordinate's weight of column b (times q); they go to the warp's weight slots
-    const bool first = lane < M2;
-    const int jw = first ? lane : lane - M2;
-    const int wslot = first ? (jw / RPL) * RPAD + (jw % RPL) : G * RPAD + jw;
-    real pc[D + 1];   // the lane's window polynomial, in registers for the item (FP64: tap min(jw, 2m-1-jw) at +-t)
-    {
-        const int row = lane < 2 * M2 ? jw : 0;
-#pragma unroll
-        for (int k = 0; k <= D; ++k) {
-            if constexpr (kF32)
-                pc[k] = poly[row * (kPolyD + 1) + k];
-            else
-                pc[k] = wp.c[row < m ? row : M2 - 1 - row][k];
-        }
-    }
-    // tap lanes: lane (g, b) owns column b and rows g RPL .. g RPL + RPL - 1 of every source
+    // staging lanes: source slot of the batch, coordinate
+    const int slot = lane >> 1, side = lane & 1;
+    // tap lanes
     const bool tap_lane = lane < G * M2;
-    const int g = lane / M2, b = lane - (lane / M2) * M2;
-    const real *wrow = wb + (tap_lane ? g : 0) * RPAD;
-    const real *wcol = wb + G * RPAD + (tap_lane ? b : 0);
+    const int g = tap_lane ? lane / M2 : 0, b = tap_lane ? lane - g * M2 : 0;
+    const int row_at = g * RPAD, col_at = SIDE + (b / RPL) * RPAD + b % RPL;
+    real *cell0 = acc + g * RPL * Q + b;
     const int end = it.start + it.count;
-    int j = it.start + warp;
-    // software pipeline: the next source's record is in flight while this one is spread
+    // the next batch's positions and charges are in flight while a batch is added
     int nb = 0;
     real2_t<real> nf{};
     real nq = real(0);
-    if (j < end) {
-        nb = base[j];
-        nf = frac[j];
-        nq = q[j];
-    }
-    for (; j < end; j += kSpreadWarps) {
-        const int packed = nb;
-        const real2_t<real> f = nf;
-        const real qj = nq;
-        if (j + kSpreadWarps < end) {
-            nb = base[j + kSpreadWarps];
-            nf = frac[j + kSpreadWarps];
-            nq = q[j + kSpreadWarps];
+    auto fetch = [&](int j) {
+        if (slot < batch && j < end) {
+            nb = base[j];
+            nf = frac[j];
+            nq = q[j];
         }
-        if (lane < 2 * M2) {
-            const real fr = first ? f.x : f.y;
-            real wv;
-            if constexpr (kF32) {
-                wv = poly_eval<D>(pc, fr - real(0.5));
-            } else {
-                wv = poly_eval<D>(pc, jw < m ? fr - 0.5 : 0.5 - fr);
-                if (jw == M2 - 1 && fr == 0.0)
-                    wv = 0.0;
+    };
+    fetch(it.start + warp + kSpreadWarps * slot);
+    for (int j0 = it.start + warp; j0 < end; j0 += kSpreadWarps * batch) {
+        const int cnt = min(batch, (end - j0 + kSpreadWarps - 1) / kSpreadWarps);
+        __syncwarp();   // the last batch's records are read (and the tile is zeroed)
+        if (slot < cnt) {
+            const real fr = side ? nf.y : nf.x, t = fr - real(0.5), tt = t * t, scale = side ? nq : real(1);
+            real w[SIDE] = {};
+#pragma unroll
+            for (int a = 0; a < m; ++a) {
+                real e, o;
+                poly_even_odd<D>(wp.c[a], tt, e, o);
+                const int a2 = M2 - 1 - a;
+                w[(a / RPL) * RPAD + a % RPL] = fma(t, o, e) * scale;
+                const real far = fma(-t, o, e) * scale;
+                w[(a2 / RPL) * RPAD + a2 % RPL] = !kF32 && a == 0 && fr == real(0) ? real(0) : far;
             }
-            wb[wslot] = first ? wv : wv * qj;
+            real *r = records + slot * REC + side * SIDE;
+#pragma unroll
+            for (int v = 0; v < SIDE; v += VW) {
+                if constexpr (kF32)
+                    *reinterpret_cast<float4 *>(r + v) = make_float4(w[v], w[v + 1], w[v + 2], w[v + 3]);
+                else
+                    *reinterpret_cast<double2 *>(r + v) = make_double2(w[v], w[v + 1]);
+            }
+            if (side == 0)
+                *reinterpret_cast<int *>(r + 2 * SIDE) = (base1(nb) - m + 1 - o1) * Q + (base2(nb) - m + 1 - o2);
         }
+        fetch(j0 + kSpreadWarps * (batch + slot));
         __syncwarp();
-        if (tap_lane) {
-            real w1[RPL];
-            load_row_weights<real, RPL>(wrow, w1);
-            const real w2 = *wcol;
+        const real *rec = records;
+        real w1[RPL], w2 = rec[col_at];
+        load_row_weights<real, RPL>(rec + row_at, w1);
+        int off = *reinterpret_cast<const int *>(rec + 2 * SIDE);
+        for (int s = 0; s < cnt; ++s) {
             // the taps of a lane are distinct cells, and distinct from the other lanes': every read
             // of this source is issued before any write
-            real *cell = acc + (base1(packed) - m + 1 - o1 + g * RPL) * Q + (base2(packed) - m + 1 - o2 + b);
+            real *cell = cell0 + off;
             real v[RPL], old[RPL], cmp[RPL];
-#pragma unroll
-            for (int i = 0; i < RPL; ++i) {
-                v[i] = w1[i] * w2;
-                old[i] = cell[i * Q];
-                if (KAHAN)
-                    cmp[i] = cell[i * Q + PP];
-            }
-            if constexpr (KAHAN && sizeof(real) == 4) {
-                // TwoSum of (old, v) for two taps per packed instruction; the error goes to the
-                // compensation plane
-#pragma unroll
-                for (int i = 0; i + 1 < RPL; i += 2) {
-                    const float2 o = make_float2(old[i], old[i + 1]), vv = make_float2(v[i], v[i + 1]);
-                    const float2 sm = __fadd2_rn(o, vv);
-                    const float2 bb = sub2f(sm, o);
-                    const float2 e = __fadd2_rn(sub2f(o, sub2f(sm, bb)), sub2f(vv, bb));
-                    const float2 c = __fadd2_rn(make_float2(cmp[i], cmp[i + 1]), e);
-                    cell[i * Q] = sm.x;
-                    cell[(i + 1) * Q] = sm.y;
-                    cell[i * Q + PP] = c.x;
-                    cell[(i + 1) * Q + PP] = c.y;
-                }
-                if constexpr (RPL % 2 == 1) {
-                    constexpr int i = RPL - 1;
-                    const real sm = old[i] + v[i];
-                    const real bb = sm - old[i];
-                    cell[i * Q] = sm;
-                    cell[i * Q + PP] = cmp[i] + ((old[i] - (sm - bb)) + (v[i] - bb));
-                }
-            } else {
+            if (tap_lane) {
 #pragma unroll
                 for (int i = 0; i < RPL; ++i) {
-                    const real sm = kF32 ? old[i] + v[i] : fma(w1[i], w2, old[i]);
-                    cell[i * Q] = sm;
-                    if (KAHAN) {
+                    old[i] = cell[i * Q];
+                    if (KAHAN)
+                        cmp[i] = cell[i * Q + PP];
+                }
+            }
+            real x1[RPL];
+            const real x2 = w2;
+#pragma unroll
+            for (int i = 0; i < RPL; ++i) {
+                x1[i] = w1[i];
+                v[i] = w1[i] * w2;
+            }
+            if (s + 1 < cnt) {   // the next source's record
+                rec += REC;
+                w2 = rec[col_at];
+                load_row_weights<real, RPL>(rec + row_at, w1);
+                off = *reinterpret_cast<const int *>(rec + 2 * SIDE);
+            }
+            if (tap_lane) {
+                if constexpr (KAHAN && sizeof(real) == 4) {
+                    // TwoSum of (old, v) for two taps per packed instruction; the error goes to the
+                    // compensation plane
+#pragma unroll
+                    for (int i = 0; i + 1 < RPL; i += 2) {
+                        const float2 o = make_float2(old[i], old[i + 1]), vv = make_float2(v[i], v[i + 1]);
+                        const float2 sm = __fadd2_rn(o, vv);
+                        const float2 bb = sub2f(sm, o);
+                        const float2 e = __fadd2_rn(sub2f(o, sub2f(sm, bb)), sub2f(vv, bb));
+                        const float2 c = __fadd2_rn(make_float2(cmp[i], cmp[i + 1]), e);
+                        cell[i * Q] = sm.x;
+                        cell[(i + 1) * Q] = sm.y;
+                        cell[i * Q + PP] = c.x;
+                        cell[(i + 1) * Q + PP] = c.y;
+                    }
+                    if constexpr (RPL % 2 == 1) {
+                        constexpr int i = RPL - 1;
+                        const real sm = old[i] + v[i];
                         const real bb = sm - old[i];
+                        cell[i * Q] = sm;
                         cell[i * Q + PP] = cmp[i] + ((old[i] - (sm - bb)) + (v[i] - bb));
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < RPL; ++i) {
+                        const real sm = kF32 ? old[i] + v[i] : fma(x1[i], x2, old[i]);
+                        cell[i * Q] = sm;
+                        if (KAHAN) {
+                            const real bb = sm - old[i];
+                            cell[i * Q + PP] = cmp[i] + ((old[i] - (sm - bb)) + (v[i] - bb));
+                        }
                     }
                 }
             }
+            __syncwarp();
         }
-        __syncwarp();
     }
     __syncthreads();
     const real *base_tile = reinterpret_cast<const real *>(smem_raw);
@@ -820,7 +832,7 @@ cudaError_t spread_m(const SpreadItem *items, int n_items, CellGrid cg, const in
 {
     const int TG = cg.T * cg.cell;
     const int P = TG + M2 - 1;
-    const size_t smem = spread_smem_bytes<real>(P, M2, kahan);
+    const size_t smem = spread_launch_bytes<real>(P, M2, kahan);
     const real2_t<real> *fr = (const real2_t<real> *)frac;
     auto run = [&](auto kern) {
         if (smem > kSmemDefault) {
@@ -1082,7 +1094,7 @@ template <typename real> size_t batch_spread_smem(int M2, int max_tile, bool com
     const int P = max_tile + M2 - 1;
     size_t bytes = 0;
     for (int r = P > 32 ? P - 32 : 1; r <= P; ++r)
-        bytes = std::max(bytes, spread_smem_bytes<real>(r, M2, comp));
+        bytes = std::max(bytes, spread_launch_bytes<real>(r, M2, comp));
     return bytes;
 }
 

@@ -182,3 +182,24 @@ def test_captured_evaluation(n, count):
             assert rel(a, b) <= 2e-5
     st.synchronize()
     fs.close()
+
+
+@pytest.mark.parametrize("precision,tol", [(32, 2e-5), (64, 1e-12)])
+@pytest.mark.parametrize("m,tile_cells", [(2, 0), (3, 4), (4, 0), (5, 0), (6, 6), (7, 0), (8, 3)])
+@pytest.mark.parametrize("n_src", [1, 3, 63, 64, 65, 517])
+def test_spreading_batches(n_src, m, tile_cells, precision, tol):
+    """Batches of 16 or 8 sources a warp (FP32 tiles of more than 32 KB), full, partial and empty, for
+    every window width: all sources in a tile or two, against direct spreading (no tiles)."""
+    import paper_0807_2387_gb300 as pkg
+    rng = np.random.default_rng(n_src + m)
+    dev = torch.device("cuda", 0)
+    src = torch.tensor(np.concatenate([rng.uniform(0.01, 0.03, (n_src, 2)), [[0.2, 0.1], [-0.2, 0.05]]]), device=dev)
+    tgt = torch.tensor(rng.uniform(-0.17, 0.17, (300, 2)), device=dev)
+    q = torch.tensor(rng.standard_normal(n_src + 2), device=dev)
+    out = []
+    for flag, tc in ((pkg.FS_FLAG_SPREAD_TILES, tile_cells), (pkg.FS_FLAG_SPREAD_DIRECT, 0)):
+        fs = pkg.FastSum(src, tgt, 64, 2.0, m, 4.0 / 64, precision=precision, flags=flag, tile_cells=tc)
+        out.append([v.clone() for v in fs.set_charges(q).field(dtype=torch.float64)])
+        fs.close()
+    for a, b in zip(*out):
+        assert rel(a, b) <= tol, rel(a, b)
