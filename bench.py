@@ -158,38 +158,14 @@ def algorithmic_bytes(info, n_points):
 
 
 # DRAM bytes per launch of the near-field kernel from an ncu capture, keyed by the SHA-256 of
-# the code it was taken on: the kernel sources (kernels_near.cu, near_warp.cuh) and the
+# the code it was taken on: the kernel sources (kernels_near.cu, near_fwd.cuh, near_warp.cuh) and the
 # function that forms its work items (build_near_items in femnfft.cu).  A changed kernel or
 # item layout reports null until it is re-captured.
 NEAR_TRAFFIC = {
-    # 21.48 MB per launch on the 2^19-point mixture (one-pass capture, -k regex:k_near_list -s 1 -c 1),
-    # scaled by the point count to the 2^20-point launch: the kernel reads per-point data once
-    "8be3b9f666b9503ab045cbff3e3a1e51f1dd16de3fa2435e939cb4183c6c3688": (
-        2 * 21484032, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
-    # 21.46 MB per launch on the 2^19-point mixture (same capture), differences in units of eps_I
-    "84ff42b81a248c29efae16affc7c55ecd8690f5eb8264ed13e62181d2b5db201": (
-        2 * 21455616, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
-    # 21.46 MB per launch on the 2^19-point mixture (same capture), exp2 form of the coefficient
-    "e656075e0636d17def29386190236016d48a29c2ca46fe0723d94bd36c4ba764": (
-        2 * 21455104, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
-    # 21.46 MB per launch on the 2^19-point mixture (same capture), log2(1 - w) from the value's w - 1
-    "43c5cc089aecb07f88b53eec773067e57d90b1e8aa98549d206e96811265ad37": (
-        2 * 21456128, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
-    # 21.46 MB per launch on the 2^19-point mixture (same capture), batched near field storing its sums
-    "f4aa79e81d4265ac184bfce8785142663845de7ff5a3c01b4dda5e37af254e87": (
-        2 * 21455104, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
-    # 21.46 MB per launch on the 2^19-point mixture (same capture), the coefficient's forms alternating
-    "6d78ca882bd0b1789f672b79907034e7cc0b8f3e469fde9f7a5af4bc86826020": (
-        2 * 21457664, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
-    # 21.46 MB per launch on the 2^19-point mixture (same capture), source-major kernel alternating too
-    "a33d24b40980e496e92b5144481c9df4a034abfa1b8aa6cf4fd355dca9d51a0f": (
-        2 * 21456128, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
-    # 21.46 MB per launch on the 2^19-point mixture (same capture), batched kernel's shared gradient vector
-    "b12c2c7150071a579c8f043241c69b6a9284e77f8901863be1001ae973bf37bd": (
-        2 * 21456896, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
-    # 21.46 MB per launch on the 2^19-point mixture (same capture), warps per block as a constant
-    "288ddfa52cfeaf9f265d07a52b5ca7a93974a7b356843dfe00170e01047d7a1d": (
-        2 * 21459712, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
+    # 21.52 MB per launch on the 2^19-point mixture (-k regex:"k_near_list|k_spread" -s 1 -c 4), scaled by
+    # the point count to the 2^20-point launch: the kernel reads per-point data once
+    "e3e5e531821030133171e60923f807789f605b49a43e5f2b8408724178913879": (
+        2 * 21524224, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
 }
 
 
@@ -197,7 +173,7 @@ def near_source_sha():
     import hashlib
     csrc = os.path.join(ROOT, "paper_0807_2387_gb300", "csrc")
     h = hashlib.sha256()
-    for name in ("kernels_near.cu", "near_warp.cuh"):
+    for name in ("kernels_near.cu", "near_fwd.cuh", "near_warp.cuh"):
         h.update(open(os.path.join(csrc, name), "rb").read())
     text = open(os.path.join(csrc, "femnfft.cu")).read()
     start = text.index("fs_status build_near_items(")

@@ -663,7 +663,7 @@ template <typename real> constexpr int fft_batch_blocks(int LC)
 }
 
 // The three 2D kernels.  LC > 0 fixes the line length at compile time (one instance per
-// length the plans use, 256 .. 4096 points), LC = 0 takes it at run time.
+// length the plans use, 128 .. 4096 points), LC = 0 takes it at run time.
 // blockIdx.y: the charge vector (grids and spectra at their strides).  The forward kernel zeroes the
 // grid rows it has read, which saves the next spreading a memset of the grid in front of it.
 template <typename real, int LC>

@@ -8,10 +8,9 @@
 // the gradient uses the analytic window slope psi'.
 //
 // Spreading: one CTA (kSpreadWarps warps) per work item (a tile of cells, or a
-// slice of a crowded tile).  A warp takes one source at a time: lanes 0..2m-1
-// evaluate the 2m window weights of the first coordinate, lanes 2m..4m-1 those
-// of the second (times q), and every lane owns a fixed subset of the (2m)^2
-// taps, fetching its two factors by shuffle.  Each warp accumulates into its
+// slice of a crowded tile).  A warp's lanes form the window weights of a batch of
+// sources into shared memory, then take one source at a time, every lane owning a
+// fixed subset of the (2m)^2 taps (spread_item).  Each warp accumulates into its
 // own padded copy of the tile in shared memory, so within a warp every tap
 // address is distinct and the read-modify-write needs no atomics; in FP32 each
 // addition's rounding error is recovered exactly (TwoSum) into a second,
@@ -63,8 +62,9 @@ __device__ __forceinline__ float2 sub2f(float2 a, float2 b)   // a - b, one roun
 // lane (g, b) owns column b and rows g RPL .. g RPL + RPL - 1 of every source.  With the weights formed
 // per source by lanes that each held one tap's polynomial the kernel was bound by its issue slots (132
 // instructions a source at m = 5).  262,144 uniform sources 52.2 -> 43.6 us, 2^20 clustered ones
-// (m = 6) 178 -> 145, 32,768 in FP64 (m = 6) 101 -> 62.  Bound by the tile's shared-memory reads and writes
-// (two planes of 2m taps a lane column, about 25 wavefronts a source) and by occupancy.
+// (m = 6) 178 -> 145, 32,768 in FP64 (m = 6) 101 -> 62.  The issue slots still bound it (125 instructions
+// a source at m = 6, 76 % of the slots), then the tile's reads and writes (two planes of 2m taps a lane
+// column, about 25 wavefronts a source).
 // TGC > 0: the tile edge (grid lines) fixed at compile time, so that the tile pitch and the
 // row offsets of the taps are constants (immediate offsets instead of one address per row).
 template <typename real, int M2, bool KAHAN, int TGC = 0>
