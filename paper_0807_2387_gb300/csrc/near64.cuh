@@ -33,22 +33,28 @@ struct Near64Tables {
             ln2[i] = t[2 * kLogTab + i];
         __syncthreads();
     }
-    // log of w in [2^-127, 1]; exactly 0 at 1
+    // log of w in (0, 1]; exactly 0 at 1.  The table of the exponent's multiples ends at 2^-127, a pair
+    // 7.7e-20 eps_I apart (such pairs are found near the origin alone, where doubles are that fine): below
+    // it CUDA's log, on a branch that ordinary warps do not take.
     __device__ __forceinline__ double ln(double w) const
     {
         const int hi = __double2hiint(w);
+        if (hi < (1024 - kLogExp) << 20)
+            return ::log(w);
         const double2 c = log[((hi & 0xfffff) + 0x1000) >> 13];
         const double r = fma(__hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(w)), c.x, -1.0);
         double t = fma(r, -1.0 / 6.0, 1.0 / 5.0);
         t = fma(r, t, -1.0 / 4.0);
         t = fma(r, t, 1.0 / 3.0);
         t = fma(r, t, -1.0 / 2.0);
-        return (ln2[(1023 - (hi >> 20)) & (kLogExp - 1)] + c.y) + fma(r * r, t, r);
+        return (ln2[1023 - (hi >> 20)] + c.y) + fma(r * r, t, r);
     }
 };
 
 __device__ __forceinline__ double near64_rcp(double w)
 {
+    if (__double2hiint(w) < 0x00100000)
+        return 1.0 / w;   // subnormal: the approximation would flush it
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(w));
     const double e = fma(-w, y, 1.0);

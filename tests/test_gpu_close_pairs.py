@@ -1,0 +1,58 @@
+"""Pairs much closer than eps_I: the near field at distances that only some places of the domain can hold
+(GPU).
+
+Doubles are finest near the coordinate origin, so distinct points there may be any distance apart.
+"""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+#: distances from the source at the origin, in the caller's units
+TINY = np.array([1e-17, 1e-19, 3e-20, 1e-20, 1e-21, 1e-22, 1e-30, 1e-45, 1e-60])
+
+
+def _around_the_origin(seed):
+    """A unit source at the origin, targets at TINY from it, and some ordinary points of both kinds."""
+    rng = np.random.default_rng(seed)
+    t = rng.uniform(0.0, 2.0 * np.pi, len(TINY))
+    near = TINY[:, None] * np.stack([np.cos(t), np.sin(t)], 1)
+    src = np.concatenate([[[0.0, 0.0]], rng.uniform(-0.17, 0.17, (60, 2)), [[0.25, 0.0]]])
+    tgt = np.concatenate([near, rng.uniform(-0.17, 0.17, (40, 2))])
+    return src, tgt, np.concatenate([[1.0], rng.standard_normal(len(src) - 1)])
+
+
+@pytest.mark.parametrize("p", [1, 2, 4])
+def test_fp64_log_of_very_close_pairs(p):
+    """phi, H and dL/dq of FP64 plans and phi of an FP64 batch at the targets a tiny distance from a
+    source, each within 1e-12 of the oracle's (the bar of the FP64 gates), element by element: phi grows
+    with the logarithm of the distance and H with its inverse.  (m = 8: the origin is a grid line, where the
+    narrower windows' edge values, 1e-9 of the peak at m = 5, are added or not by the last bit.)"""
+    import paper_0807_2387_gb300 as fs
+    from oracle import fastsum as F
+    from oracle import kernel as K
+    src, tgt, q = _around_the_origin(p)
+    eps, k = 4 / 64, len(TINY)
+    par = K.make_params(64, 2.0, 8, eps, p)
+    phi_o, H_o = F.fast_sum(src, tgt, q, par, "nfft")
+    dev = torch.device("cuda", 0)
+    s, t, qd = (torch.tensor(v, device=dev) for v in (src, tgt, q))
+    plan = fs.FastSum(s, t, 64, 2.0, 8, eps, precision=64, p=p)
+    phi, H = (v.cpu().numpy() for v in plan.set_charges(qd).field())
+    assert np.max(np.abs(phi - phi_o) / np.abs(phi_o).clip(0.1)) <= 1e-12
+    assert np.max(np.linalg.norm((H - H_o)[:k], axis=1) / np.linalg.norm(H_o[:k], axis=1)) <= 1e-12
+    batch = fs.FastSumBatch([(s, t, 64, eps)], 2.0, 8, 1, precision=64, p=p)
+    phi_b = batch.eval([qd[None]])[0][0].cpu().numpy().reshape(-1)
+    assert np.max(np.abs(phi_b - phi_o) / np.abs(phi_o).clip(0.1)) <= 1e-12
+    # dL/dq_0 for dL/dphi = 1 at one target is phi of a unit charge at the origin there
+    one = np.zeros(len(src))
+    one[0] = 1.0
+    unit, _ = F.fast_sum(src, tgt, one, par, "nfft")
+    for i in range(k):
+        g = torch.zeros(len(tgt), dtype=torch.float64, device=dev)
+        g[i] = 1.0
+        dq = plan.adjoint(g, None, want_q=True)[0]
+        assert abs(float(dq[0]) - unit[i]) <= 1e-12 * abs(unit[i]), (TINY[i], float(dq[0]), unit[i])
