@@ -173,7 +173,8 @@ __device__ __forceinline__ void kb_value_slope_curv(const Window<real> &w, real 
 // 2m-1-a at t is tap a at -t).  The tail of the Chebyshev series is below 1e-17 of a tap's largest
 // value for m <= 8 (degree 17 to 21 by m and oversampling), so they are as exact as the closed
 // form, whose exp, expm1 and square root cost over 100 FP64 instructions a tap against 21.  The
-// closed support edge (frac = 0, the last tap) is 0, as in the closed form.
+// closed support edge is 0, as in the closed form: the last tap at frac = 0, and the first at frac = 1,
+// which the fraction of a coordinate just below a grid line (0, where doubles are that fine) rounds to.
 constexpr int kPolyD64 = 21;
 struct WindowPoly64 {
     double c[kMaxM][kPolyD64 + 1];

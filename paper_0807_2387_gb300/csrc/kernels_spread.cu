@@ -126,8 +126,8 @@ __device__ __forceinline__ void spread_item(const SpreadItem &it, const CellGrid
                 real e, o;
                 poly_even_odd<D>(wp.c[a], tt, e, o);
                 const int a2 = M2 - 1 - a;
-                w[(a / RPL) * RPAD + a % RPL] = fma(t, o, e) * scale;
-                const real far = fma(-t, o, e) * scale;
+                const real near = fma(t, o, e) * scale, far = fma(-t, o, e) * scale;
+                w[(a / RPL) * RPAD + a % RPL] = !kF32 && a == 0 && fr == real(1) ? real(0) : near;
                 w[(a2 / RPL) * RPAD + a2 % RPL] = !kF32 && a == 0 && fr == real(0) ? real(0) : far;
             }
             real *r = records + slot * REC + side * SIDE;
@@ -416,17 +416,19 @@ __device__ __forceinline__ void interp_sums(int64_t k, const int *__restrict__ b
     }
     if (kEdge && f.y == real(0))
         w2[M2 - 1] = d2[M2 - 1] = real(0);
+    if (kEdge && f.y == real(1))
+        w2[0] = d2[0] = real(0);
 #pragma unroll
     for (int q = 0; q < m; ++q) {
         const int a = m - 1 - q, a2 = M2 - 1 - a;
         real e, o, de, dd;
         poly_even_odd<D>(wp.c[a], s1, e, o);
         poly_even_odd<D - 1>(wp.d[a], s1, de, dd);
-        const bool edge = kEdge && a == 0 && f.x == real(0);
-        interp_row<real, M2, kRef>(grid + (int64_t)(row0 + a) * pitch + col0, w2, d2, fma(t1, o, e), fma(t1, dd, de),
-                                   q == 0, rs_ref, phi, g1, g2);
-        interp_row<real, M2, kRef>(grid + (int64_t)(row0 + a2) * pitch + col0, w2, d2, edge ? real(0) : fma(-t1, o, e),
-                                   edge ? real(0) : fma(t1, dd, -de), false, rs_ref, phi, g1, g2);
+        const bool first = kEdge && a == 0 && f.x == real(1), last = kEdge && a == 0 && f.x == real(0);
+        interp_row<real, M2, kRef>(grid + (int64_t)(row0 + a) * pitch + col0, w2, d2, first ? real(0) : fma(t1, o, e),
+                                   first ? real(0) : fma(t1, dd, de), q == 0, rs_ref, phi, g1, g2);
+        interp_row<real, M2, kRef>(grid + (int64_t)(row0 + a2) * pitch + col0, w2, d2, last ? real(0) : fma(-t1, o, e),
+                                   last ? real(0) : fma(t1, dd, -de), false, rs_ref, phi, g1, g2);
     }
 }
 
@@ -684,7 +686,7 @@ __global__ void __launch_bounds__(kSpreadWarps * 32) k_spread_dip(const SpreadIt
             if constexpr (!kF32) {
                 if (jw >= m)
                     wd = -wd;
-                if (jw == M2 - 1 && fr == 0.0)
+                if ((jw == M2 - 1 && fr == 0.0) || (jw == 0 && fr == 1.0))
                     wv = wd = 0.0;
             }
         }
@@ -783,6 +785,10 @@ __global__ void __launch_bounds__(256) k_interp_hess(int64_t N, const int *__res
         w1[M2 - 1] = d1[M2 - 1] = e1[M2 - 1] = real(0);
     if (sizeof(real) == 8 && f.y == real(0))
         w2[M2 - 1] = d2[M2 - 1] = e2[M2 - 1] = real(0);
+    if (sizeof(real) == 8 && f.x == real(1))
+        w1[0] = d1[0] = e1[0] = real(0);
+    if (sizeof(real) == 8 && f.y == real(1))
+        w2[0] = d2[0] = e2[0] = real(0);
     const int row0 = base1(packed) - m + 1;
     const int col0 = base2(packed) - m + 1;
     real rs[M2], rd[M2];

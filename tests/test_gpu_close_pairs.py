@@ -56,3 +56,31 @@ def test_fp64_log_of_very_close_pairs(p):
         g[i] = 1.0
         dq = plan.adjoint(g, None, want_q=True)[0]
         assert abs(float(dq[0]) - unit[i]) <= 1e-12 * abs(unit[i]), (TINY[i], float(dq[0]), unit[i])
+
+
+@pytest.mark.parametrize("m", [2, 3, 4, 5])
+def test_fp64_points_just_below_a_grid_line(m):
+    """FP64 plans with coordinates a negative fraction of the last place from 0, a grid line: the fraction
+    to the line below rounds to 1, and the first tap then lies on the window's (open) edge, where it counts
+    nothing.  Field, gradients and Hessian against the oracle within 1e-12, the bar of the FP64 gates; the
+    edge's closed value is 1e-3 (m = 2) to 1e-9 (m = 5) of the peak."""
+    import paper_0807_2387_gb300 as fs
+    from oracle import adjoint as A
+    from oracle import fastsum as F
+    from oracle import kernel as K
+    rng = np.random.default_rng(m)
+    src, tgt = (rng.uniform(-0.17, 0.17, (k, 2)) for k in (60, 50))
+    for pts in (src, tgt):
+        pts[:10, 0] = -1e-22 * rng.uniform(1.0, 9.0, 10)
+        pts[10:20, 1] = -1e-25 * rng.uniform(1.0, 9.0, 10)
+    src, tgt = np.concatenate([src, [[0.25, 0.0]]]), np.concatenate([tgt, [[0.0, 0.25]]])
+    q, gp, gh = rng.standard_normal(len(src)), rng.standard_normal(len(tgt)), rng.standard_normal((len(tgt), 2))
+    par = K.make_params(64, 2.0, m, 4 / 64)
+    dev = torch.device("cuda", 0)
+    s, t, qd, gpd, ghd = (torch.tensor(v, device=dev) for v in (src, tgt, q, gp, gh))
+    plan = fs.FastSum(s, t, 64, 2.0, m, 4 / 64, precision=64)
+    got = (*plan.set_charges(qd).field(), *plan.adjoint(gpd, ghd, True, True, True))
+    want = (*F.fast_sum(src, tgt, q, par, "nfft"), *A.fast_sum_adjoint(src, tgt, q, gp, gh, par))
+    for name, a, b in zip(("phi", "H", "dq", "dsrc", "dtgt"), got, want):
+        a = a.cpu().numpy()
+        assert np.max(np.abs(a - b)) <= 1e-12 * np.max(np.abs(b)), (name, np.max(np.abs(a - b)) / np.max(np.abs(b)))
