@@ -15,7 +15,7 @@ cudaError_t launch_near32_rhs(int64_t n_items, const int2 *items, int lanes, con
     const NearSides sd{tgt_base, tgt_hi, tgt_lo, src_hi, src_lo, src_start};
     return with_degree(np.p, [&](auto pc) {
         auto run = [&](auto rc) {
-            NearFwd<decltype(pc)::value, decltype(rc)::value, true> op{};
+            NearFwd<decltype(pc)::value, decltype(rc)::value> op{};
             op.q = q;
             op.phi_s = phi_s;
             op.grad_s = grad_s;

@@ -8,19 +8,25 @@ namespace fs {
 // Forward correction at the targets for R right-hand sides at once (the pair geometry, the
 // log and the gradient coefficient are shared): phi += q f, grad += q c d for two candidates per
 // packed operation; the factor c_ln of f (near_g2) and rc eps_I of c are applied once at the
-// store (d arrives in units of eps_I).  With one right-hand side the sums are split into partial
-// sums per list evaluation; with several the registers go to the extra accumulators instead.
+// store (d arrives in units of eps_I).  A plan's sums are split into partial sums per list evaluation,
+// for any number of right-hand sides, so that a vector's rounding error does not depend on the vectors
+// beside it: 12,000 sources of one sign around 6,000 targets in a cell (p = 4), RMS error against FP64
+// 1.2e-7 of phi and 1.9e-7 of H, alone and together; with one running sum a vector 3.1e-7 and 9.5e-7.
+// 100,003 sources and 65,537 targets, an evaluation of 2 / 3 / 4 vectors 107.5 / 129 / 158 us (running sums
+// 107.7 / 127.4 / 152.3 us).  Four vectors need up to 168 registers and run at three blocks per SM: 20,000 points at p = 8
+// 50.6 us against 61 us with spills at four blocks.  The batched kernel, which reads its constants from
+// memory, keeps running sums where it holds several right-hand sides.
 // Right-hand side r reads q + r q_stride and writes at r n_stride.
 template <int P, int R, bool BATCH = false> struct NearFwd {
-    static constexpr int kMinBlocks = (R == 1 && !BATCH) ? 6 : 4;   // of four warps per SM: up to 80 and 128 registers
-    static constexpr int kUnroll = BATCH ? 4 : 2;
+    static constexpr int kMinBlocks = BATCH ? 4 : (R == 1 ? 6 : (R == 4 ? 3 : 4));   // of four warps per SM
+    static constexpr int kUnroll = (R == 1 && !BATCH) ? 2 : 4;
     // |w - 1|^(p-1) / w, the gradient coefficient over rc up to the sign (-1)^(p-1) (applied at the
     // store), as 2^((p-1) log2(1 - w) - log2 w) (log2 w is shared with the value; w = 1 gives 2^-inf):
     // four MUFU operations and one FMA a pair of candidates, against two and the power's
     // multiplications.  2.26 -> 2.19 ms at 2^20 points (p = 8) against alternating the two.  Several
     // right-hand sides add FMA work that hides the difference (batched replay the same either way).
-    static constexpr bool kExp2 = P >= 5 && !BATCH;
-    static constexpr bool kRows = R == 1;
+    static constexpr bool kExp2 = P >= 5 && R == 1 && !BATCH;
+    static constexpr bool kRows = R == 1 || !BATCH;
     static constexpr bool kSat = P >= 2;   // f(1) = 0 and (w - 1)^(p-1) = 0: clamping w masks a pair
     static constexpr float kPhi = P >= 2 ? kLnCoef : 1.f;   // unit of the phi sums
     const float *__restrict__ q;
@@ -35,9 +41,9 @@ template <int P, int R, bool BATCH = false> struct NearFwd {
     float qc[R];
     float2 rphi[kRows ? R : 1], rgx[kRows ? R : 1], rgy[kRows ? R : 1];
 
-    __device__ __forceinline__ float2 &acc_phi(int r) { return kRows ? rphi[0] : phi[r]; }
-    __device__ __forceinline__ float2 &acc_gx(int r) { return kRows ? rgx[0] : gx[r]; }
-    __device__ __forceinline__ float2 &acc_gy(int r) { return kRows ? rgy[0] : gy[r]; }
+    __device__ __forceinline__ float2 &acc_phi(int r) { return kRows ? rphi[kRows ? r : 0] : phi[r]; }
+    __device__ __forceinline__ float2 &acc_gx(int r) { return kRows ? rgx[kRows ? r : 0] : gx[r]; }
+    __device__ __forceinline__ float2 &acc_gy(int r) { return kRows ? rgy[kRows ? r : 0] : gy[r]; }
 
     __device__ __forceinline__ void init()
     {
@@ -110,15 +116,19 @@ template <int P, int R, bool BATCH = false> struct NearFwd {
     __device__ __forceinline__ void row_begin()
     {
         if constexpr (kRows)
-            rphi[0] = rgx[0] = rgy[0] = f2(0.f);
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                rphi[r] = rgx[r] = rgy[r] = f2(0.f);
     }
     __device__ __forceinline__ void row_end()
     {
-        if constexpr (kRows) {
-            phi[0] = add2(phi[0], rphi[0]);
-            gx[0] = add2(gx[0], rgx[0]);
-            gy[0] = add2(gy[0], rgy[0]);
-        }
+        if constexpr (kRows)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                phi[r] = add2(phi[r], rphi[r]);
+                gx[r] = add2(gx[r], rgx[r]);
+                gy[r] = add2(gy[r], rgy[r]);
+            }
     }
     __device__ __forceinline__ void fold()
     {
