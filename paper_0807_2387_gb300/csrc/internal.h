@@ -181,6 +181,25 @@ struct CellSplit3 {
     __host__ __device__ static int strip_first(int k, int n, int i) { return (int)((int64_t)n * strip_piece(k, i) / k); }
 };
 
+// Pairs of the FP32 3D near field closer than this part of eps_I take their difference from the FP64
+// positions: the hi + lo difference, good to 2^-45 of a cell edge, is 2^6 times finer than FP32's 2^-24
+// here (cells are one eps_I wide, rounded up to grid lines) and would fall short of it below 2^-21.
+constexpr float kNear3Exact = 0x1p-15f, kNear3Exact2 = 0x1p-30f;
+
+// The point sets of the FP32 3D near field in sorted order.
+struct Near3Targets {
+    const int *base;
+    float4 *hi;            // offset in the cell; w = 1: the target has sources closer than kNear3Exact at other positions
+    const float4 *lo;
+    const double *pos;
+};
+struct Near3Others {
+    const float4 *hi, *lo;
+    const double *pos;
+    const int *start;
+    double inv_eps;        // 1 / eps_I
+};
+
 // FP32 3D near field (distances in units of eps_I, w = |d|^2 / eps_I^2):
 //   f(w)       = c1 w^(-1/2) - P(w),             c1 = 1 / (4 pi eps_I), P(w) = T_I = sum beta_k w^k
 //   grad_x f   = -(1/eps_I) (c1 w^(-3/2) + 2 P'(w)) d,   d in units of eps_I
@@ -250,23 +269,23 @@ cudaError_t launch_near3_f64(int64_t N, const int *tgt_base, const double *tgt_p
 // FP32 near field over warp items {first target, count <= lanes} of one cell each (sorted order; lanes 8,
 // 16 or 32); coincident pairs (equal positions) are listed per target in coinc_start / coinc_src
 // (assign: store phi_s / grad_s instead of adding, for the near field run beside the far field)
-cudaError_t launch_near3_warp(const int2 *items, int n_items, int lanes, const int *tgt_base, const float4 *tgt_hi,
-                              const float4 *tgt_lo, const float4 *src_hi, const float4 *src_lo, const float *q,
-                              const int *src_start, CellGrid3 cg, const Near3Params &np, const int *coinc_start,
-                              const int *coinc_src, float *phi_s, float *grad_s, bool assign, cudaStream_t st);
+cudaError_t launch_near3_warp(const int2 *items, int n_items, int lanes, const Near3Targets &tgt, const Near3Others &src,
+                              const float *q, CellGrid3 cg, const Near3Params &np, int64_t N, const int *coinc_start,
+                              const int *coinc_src, bool any_marked, float *phi_s, float *grad_s, bool assign,
+                              cudaStream_t st);
 // Source-major FP32 near field (many more sources than targets): items of at most 64 sources of
 // one cell; phi and grad phi are added to the targets with atomics, then the coincident pairs'
-// -q T_I(0) when any_coincident
-cudaError_t launch_near3_src(const int2 *items, int n_items, const int *src_base, const float4 *src_hi,
-                             const float4 *src_lo, const float4 *tgt_hi, const float4 *tgt_lo, const float *q,
-                             const int *tgt_start, CellGrid3 cg, const Near3Params &np, int64_t N,
-                             const int *coinc_start, const int *coinc_src, bool any_coincident, float *phi_s,
-                             float *grad_s, cudaStream_t st);
-// per target: count of sources at the same FP64 position (same cell) when coinc_src is null, or
-// their sorted indices from coinc_start (coinc_src given)
-cudaError_t launch_coincident3(int64_t N, const int *tgt_base, const double *tgt_pos, const double *src_pos,
-                               const int *src_start, CellGrid3 cg, int *count, const int *coinc_start, int *coinc_src,
-                               cudaStream_t st);
+// -q T_I(0) and the pairs of marked targets when any_touching
+cudaError_t launch_near3_src(const int2 *items, int n_items, const int *src_base, const Near3Others &src,
+                             const Near3Targets &tgt, const int *tgt_start, const float *q, CellGrid3 cg,
+                             const Near3Params &np, int64_t N, const int *coinc_start, const int *coinc_src,
+                             bool any_touching, float *phi_s, float *grad_s, cudaStream_t st);
+// per target: count of sources at the same FP64 position when coinc_src is null, with the mark of
+// Near3Targets::hi and *touching = 1 where a target gets it; or their sorted indices from coinc_start
+// (coinc_src given).  source_frame: for the source-major kernel's differences
+cudaError_t launch_coincident3(int64_t N, const Near3Targets &tgt, const Near3Others &src, CellGrid3 cg,
+                               const Near3Params &np, bool source_frame, int *count, const int *coinc_start, int *coinc_src,
+                               int *touching, cudaStream_t st);
 template <typename real>
 cudaError_t launch_unpermute3(int64_t N, const real *phi_s, const real *grad_s, const int *perm, double s,
                               void *phi_out, void *H_out, int out_f64, cudaStream_t st);

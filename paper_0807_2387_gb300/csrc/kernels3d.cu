@@ -106,8 +106,8 @@ __global__ void k_gather_points3(const double *__restrict__ xyz, const int *__re
     }
     base[k] = b[0] | (b[1] << 10) | (b[2] << 20);
     if (hi) {
-        // offset from the lower corner of the point's cell as hi + lo: 48 bits of at most a cell's width
-        // reach the last place of a torus coordinate
+        // offset from the lower corner of the point's cell as hi + lo: 48 bits of at most a cell's width,
+        // which end some bits above or below the coordinate's last place
         float o[3], l[3];
         for (int d = 0; d < 3; ++d) {
             const double corner = (double)((b[d] / cell) * cell + window_lo) / n_os - 0.5;
@@ -739,10 +739,13 @@ __global__ void __launch_bounds__(256) k_near3_f64(int64_t N, const int *__restr
 // 27 cells around 32 at a time, keeps those within eps_I of the piece's box, and appends them to
 // lists in shared memory, negated in the piece's frame and in units of eps_I, which all lanes
 // evaluate two candidates to a packed operation.  Pairs beyond eps_I get charge 0.  Sources within
-// eps_I / 8 of the box go to a second list with hi + lo coordinates, whose differences keep full FP32
-// relative accuracy however small they are, without the FP64 differences taken before (a 64th of
-// the FP32 rate: half of the source-major kernel's time).  Coincident pairs (difference 0) get charge 0
-// and are accounted from the per-target lists built with the plan.
+// eps_I / 8 of the box go to a second list with hi + lo coordinates.  Their differences are good to
+// 2^-45 of a cell edge (a few roundings of the low words), FP32's relative accuracy and better down to
+// kNear3Exact eps_I.  Pairs closer than that get charge 0 in the lists: the coincident ones (equal
+// FP64 positions) are accounted from the per-target lists built with the plan, and targets that have
+// others, marked when the plan is built, take those from the FP64 positions at the end
+// (near3_touching).  FP64 differences of all close pairs, at a 64th of the FP32 rate, were half of the
+// source-major kernel's time.
 // Measured, 2^18 points of a ball (41 per cell, p = 3): 380 us with items of 64 targets (two per lane,
 // the box a whole cell: 0.13 of the pair slots useful) and FP64 close pairs, 249 us here; list building
 // is the larger part of it.
@@ -796,18 +799,19 @@ __device__ __forceinline__ void near3_pair(const Near3Params &np, float2 w, floa
     a.gz = fma2(qc, dz, a.gz);
 }
 
-// A pair that may coincide (w = 0): charge 0 and a finite w (the per-target lists account for it).
+// A pair of candidates close to the item's box: charge 0 below kNear3Exact2 (near3_touching and the lists of
+// coincident pairs account for those).
 template <int P>
 __device__ __forceinline__ void near3_pair_close(const Near3Params &np, float2 dx, float2 dy, float2 dz, float2 qq,
                                                  Near3Sums &a)
 {
     float2 w = near3_w(dx, dy, dz);
-    if (w.x == 0.f)
+    if (w.x < kNear3Exact2)
         qq.x = 0.f;
-    if (w.y == 0.f)
+    if (w.y < kNear3Exact2)
         qq.y = 0.f;
-    w.x = fmaxf(w.x, 1e-20f);   // (w^-3/2 stays finite; distinct points give w >= ~1e-14)
-    w.y = fmaxf(w.y, 1e-20f);
+    w.x = fmaxf(w.x, kNear3Exact2);
+    w.y = fmaxf(w.y, kNear3Exact2);
     near3_pair<P>(np, w, dx, dy, dz, qq, a);
 }
 
@@ -1236,42 +1240,129 @@ __global__ void __launch_bounds__(kNear3Warps * 32) k_near3_src(const int2 *__re
     near3_src_eval_close<P>(S, nc, pairs, np, phi_s, grad_s, lane);
 }
 
-// Coincident pairs for the source-major kernel: phi -= T_I(0) (sum of the coincident charges).
-__global__ void k_coincident3_apply(int64_t N, const int *__restrict__ coinc_start, const int *__restrict__ coinc_src,
-                                    const float *__restrict__ q, float beta0, float *__restrict__ phi_s)
+// Calls f(j) for the sources j whose pair with a target (tgt_hi entry X, tgt_lo entry XL) gets charge 0 in
+// near3_pair_close, that is, for w < kNear3Exact2 of the difference that it forms, in the target's or (SRC) the
+// source's frame, bit by bit the same.  Such sources lie in the target's cell, or across a face that is
+// no farther.
+template <bool SRC, class F>
+__device__ __forceinline__ void near3_touching(const Near3Params &np, const CellGrid3 &cg, int packed, float4 X, float4 XL,
+                                               const Near3Others &src, F &&f)
 {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= N)
-        return;
-    float self = 0.f;
-    for (int c = coinc_start[k]; c < coinc_start[k + 1]; ++c)
-        self += q[coinc_src[c]];
-    if (self != 0.f)
-        phi_s[k] -= beta0 * self;
-}
-
-// Coincident pairs: sources of the target's own cell at the same (FP64) position.
-__global__ void k_coincident3(int64_t N, const int *__restrict__ tgt_base, const double *__restrict__ tgt_pos,
-                              const double *__restrict__ src_pos, const int *__restrict__ src_start, CellGrid3 cg,
-                              int *__restrict__ count, const int *__restrict__ coinc_start, int *__restrict__ coinc_src)
-{
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= N)
-        return;
-    const int packed = tgt_base[k];
-    const int key = cg.key(b3x(packed) / cg.cell, b3y(packed) / cg.cell, b3z(packed) / cg.cell);
-    const double tx = tgt_pos[3 * k], ty = tgt_pos[3 * k + 1], tz = tgt_pos[3 * k + 2];
-    const int S3 = cg.sub3();
-    int c = 0, at = coinc_src ? coinc_start[k] : 0;
-    for (int j = src_start[key * S3]; j < src_start[(key + 1) * S3]; ++j) {
-        if (src_pos[3 * (int64_t)j] == tx && src_pos[3 * (int64_t)j + 1] == ty && src_pos[3 * (int64_t)j + 2] == tz) {
-            if (coinc_src)
-                coinc_src[at++] = j;
-            ++c;
+    const float lim = 1.05f * kNear3Exact / np.inv_eps;
+    auto diff = [&](float x, float xl, float y, float yl, float off) {   // off: step from the source's cell to the target's
+        const float a = SRC ? -off - x : off - y;
+        const float d = SRC ? (-a - y) + (-neg_lo(-off, x, xl, a) - yl) : (x + a) + (xl + neg_lo(off, y, yl, a));
+        return d * np.inv_eps;
+    };
+    for (int c = 0; c < 27; ++c) {
+        const int d1 = c / 9 - 1, d2 = c / 3 % 3 - 1, d3 = c % 3 - 1;
+        const int e1 = b3x(packed) / cg.cell + d1, e2 = b3y(packed) / cg.cell + d2, e3 = b3z(packed) / cg.cell + d3;
+        auto far = [&](int d, float x) { return d < 0 ? x > lim : (d > 0 && np.h - x > lim); };
+        if (far(d1, X.x) || far(d2, X.y) || far(d3, X.z) || min(min(e1, e2), e3) < 0 || max(max(e1, e2), e3) >= cg.n_c)
+            continue;
+        const float ox = -(float)d1 * np.h, oy = -(float)d2 * np.h, oz = -(float)d3 * np.h;
+        const int64_t key = (int64_t)cg.key(e1, e2, e3) * cg.sub3();
+        for (int j = src.start[key]; j < src.start[key + cg.sub3()]; ++j) {
+            const float4 y = src.hi[j];
+            if (fabsf(X.x + (ox - y.x)) > lim || fabsf(X.y + (oy - y.y)) > lim || fabsf(X.z + (oz - y.z)) > lim)
+                continue;
+            const float4 yl = src.lo[j];
+            const float2 dx = f2(diff(X.x, XL.x, y.x, yl.x, ox)), dy = f2(diff(X.y, XL.y, y.y, yl.y, oy)),
+                         dz = f2(diff(X.z, XL.z, y.z, yl.z, oz));
+            if (near3_w(dx, dy, dz).x < kNear3Exact2)
+                f(j);
         }
     }
-    if (!coinc_src)
-        count[k] = c;
+}
+
+// The differences of those pairs from the FP64 positions, in place of the hi + lo ones; nothing for a
+// coincident pair.  Adds to phi and the three components of grad.
+template <int P, bool SRC>
+__device__ __forceinline__ void near3_add_touching(const Near3Params &np, const CellGrid3 &cg, int k, int packed, float4 X,
+                                                   float4 XL, const Near3Others &src, const double *__restrict__ tgt_pos,
+                                                   const float *__restrict__ q, float (&add)[4])
+{
+    Near3Sums a;
+    a.phi = a.gx = a.gy = a.gz = f2(0.f);
+    const double tx = tgt_pos[3 * (int64_t)k], ty = tgt_pos[3 * (int64_t)k + 1], tz = tgt_pos[3 * (int64_t)k + 2];
+    near3_touching<SRC>(np, cg, packed, X, XL, src, [&](int j) {
+        const double *s = src.pos + 3 * (int64_t)j;
+        const double ex = tx - s[0], ey = ty - s[1], ez = tz - s[2];
+        if (ex == 0.0 && ey == 0.0 && ez == 0.0)
+            return;
+        const float2 dx = f2((float)(ex * src.inv_eps)), dy = f2((float)(ey * src.inv_eps)),
+                     dz = f2((float)(ez * src.inv_eps));
+        const float w = fmaxf(near3_w(dx, dy, dz).x, 1e-20f);   // (w^-3/2 stays finite)
+        near3_pair<P>(np, f2(w), dx, dy, dz, make_float2(q[j], 0.f), a);
+    });
+    add[0] = a.phi.x;
+    add[1] = -np.inv_eps * a.gx.x;
+    add[2] = -np.inv_eps * a.gy.x;
+    add[3] = -np.inv_eps * a.gz.x;
+}
+
+// The pairs that the kernels above leave out: those of the marked targets, and for the source-major kernel
+// the coincident ones (coinc_start given), phi -= T_I(0) (sum of their charges).
+template <int P, bool SRC>
+__global__ void k_touching3(int64_t N, const int *__restrict__ coinc_start, const int *__restrict__ coinc_src,
+                            const int *__restrict__ tgt_base, const float4 *__restrict__ tgt_hi,
+                            const float4 *__restrict__ tgt_lo, const double *__restrict__ tgt_pos, Near3Others src,
+                            const float *__restrict__ q, CellGrid3 cg, Near3Params np, float *__restrict__ phi_s,
+                            float *__restrict__ grad_s)
+{
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k >= N)
+        return;
+    if (coinc_start) {
+        float self = 0.f;
+        for (int c = coinc_start[k]; c < coinc_start[k + 1]; ++c)
+            self += q[coinc_src[c]];
+        if (self != 0.f)
+            phi_s[k] -= np.beta0 * self;
+    }
+    const float4 X = tgt_hi[k];
+    if (X.w == 0.f)
+        return;
+    float add[4];
+    near3_add_touching<P, SRC>(np, cg, (int)k, tgt_base[k], X, tgt_lo[k], src, tgt_pos, q, add);
+    phi_s[k] += add[0];
+    for (int d = 0; d < 3; ++d)
+        grad_s[3 * k + d] += add[1 + d];
+}
+
+// Per target, the number of its coincident sources (equal FP64 positions, so of its own cell), with
+// tgt_hi[k].w = 1 and *touching = 1 if it has other sources that close; or (coinc_src given) those
+// sources.
+template <bool SRC>
+__global__ void k_coincident3(int64_t N, const int *__restrict__ tgt_base, float4 *__restrict__ tgt_hi,
+                              const float4 *__restrict__ tgt_lo, const double *__restrict__ tgt_pos, Near3Others src,
+                              CellGrid3 cg, Near3Params np, int *__restrict__ count, const int *__restrict__ coinc_start,
+                              int *__restrict__ coinc_src, int *__restrict__ touching)
+{
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k >= N)
+        return;
+    const double tx = tgt_pos[3 * k], ty = tgt_pos[3 * k + 1], tz = tgt_pos[3 * k + 2];
+    const float4 X = tgt_hi[k];
+    int c = 0, at = coinc_src ? coinc_start[k] : 0;
+    bool other = false;
+    near3_touching<SRC>(np, cg, tgt_base[k], X, tgt_lo[k], src, [&](int j) {
+        const double *s = src.pos + 3 * (int64_t)j;
+        if (s[0] != tx || s[1] != ty || s[2] != tz) {
+            other = true;
+            return;
+        }
+        if (coinc_src)
+            coinc_src[at++] = j;
+        ++c;
+    });
+    if (coinc_src)
+        return;
+    count[k] = c;
+    if (other) {
+        tgt_hi[k] = make_float4(X.x, X.y, X.z, 1.f);
+        *touching = 1;
+    }
 }
 
 template <typename real>
@@ -1480,55 +1571,62 @@ cudaError_t launch_cell_order3(const int *start, CellGrid3 cg, int cap, const do
     return cudaGetLastError();
 }
 
-cudaError_t launch_near3_warp(const int2 *items, int n_items, int lanes, const int *tgt_base, const float4 *tgt_hi,
-                              const float4 *tgt_lo, const float4 *src_hi, const float4 *src_lo, const float *q,
-                              const int *src_start, CellGrid3 cg, const Near3Params &np, const int *coinc_start,
-                              const int *coinc_src, float *phi_s, float *grad_s, bool assign, cudaStream_t st)
+cudaError_t launch_near3_warp(const int2 *items, int n_items, int lanes, const Near3Targets &tgt, const Near3Others &src,
+                              const float *q, CellGrid3 cg, const Near3Params &np, int64_t N, const int *coinc_start,
+                              const int *coinc_src, bool any_marked, float *phi_s, float *grad_s, bool assign,
+                              cudaStream_t st)
 {
     if (n_items <= 0)
         return cudaSuccess;
     const unsigned blocks = (unsigned)((n_items + kNear3Warps - 1) / kNear3Warps);
     return with_degree(np.p, [&](auto pc) {
         constexpr int P = decltype(pc)::value;
-        k_near3_warp<P><<<blocks, kNear3Warps * 32, 0, st>>>(items, n_items, lanes, tgt_base, tgt_hi, tgt_lo, src_hi,
-                                                             src_lo, q, src_start, cg, np, coinc_start, coinc_src,
-                                                             phi_s, grad_s, assign);
+        k_near3_warp<P><<<blocks, kNear3Warps * 32, 0, st>>>(items, n_items, lanes, tgt.base, tgt.hi, tgt.lo, src.hi, src.lo,
+                                                             q, src.start, cg, np, coinc_start, coinc_src, phi_s, grad_s,
+                                                             assign);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess || !any_marked)
+            return e;
+        k_touching3<P, false><<<nblk(N, 256), 256, 0, st>>>(N, nullptr, nullptr, tgt.base, tgt.hi, tgt.lo, tgt.pos, src, q, cg,
+                                                            np, phi_s, grad_s);
         return cudaGetLastError();
     });
 }
 
-cudaError_t launch_near3_src(const int2 *items, int n_items, const int *src_base, const float4 *src_hi,
-                             const float4 *src_lo, const float4 *tgt_hi, const float4 *tgt_lo, const float *q,
-                             const int *tgt_start, CellGrid3 cg, const Near3Params &np, int64_t N,
-                             const int *coinc_start, const int *coinc_src, bool any_coincident, float *phi_s,
-                             float *grad_s, cudaStream_t st)
+cudaError_t launch_near3_src(const int2 *items, int n_items, const int *src_base, const Near3Others &src,
+                             const Near3Targets &tgt, const int *tgt_start, const float *q, CellGrid3 cg,
+                             const Near3Params &np, int64_t N, const int *coinc_start, const int *coinc_src,
+                             bool any_touching, float *phi_s, float *grad_s, cudaStream_t st)
 {
-    if (n_items > 0) {
-        const unsigned blocks = (unsigned)((n_items + kNear3Warps - 1) / kNear3Warps);
-        const cudaError_t e = with_degree(np.p, [&](auto pc) {
-            constexpr int P = decltype(pc)::value;
-            k_near3_src<P><<<blocks, kNear3Warps * 32, 0, st>>>(items, n_items, src_base, src_hi, src_lo, tgt_hi, tgt_lo,
-                                                                q, tgt_start, cg, np, phi_s, grad_s);
-            return cudaGetLastError();
-        });
-        if (e != cudaSuccess)
-            return e;
-    }
-    if (any_coincident && N > 0) {
-        k_coincident3_apply<<<nblk(N, 256), 256, 0, st>>>(N, coinc_start, coinc_src, q, np.beta0, phi_s);
+    return with_degree(np.p, [&](auto pc) {
+        constexpr int P = decltype(pc)::value;
+        if (n_items > 0) {
+            const unsigned blocks = (unsigned)((n_items + kNear3Warps - 1) / kNear3Warps);
+            k_near3_src<P><<<blocks, kNear3Warps * 32, 0, st>>>(items, n_items, src_base, src.hi, src.lo, tgt.hi, tgt.lo, q,
+                                                                tgt_start, cg, np, phi_s, grad_s);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess)
+                return e;
+        }
+        if (any_touching && N > 0)
+            k_touching3<P, true><<<nblk(N, 256), 256, 0, st>>>(N, coinc_start, coinc_src, tgt.base, tgt.hi, tgt.lo, tgt.pos,
+                                                               src, q, cg, np, phi_s, grad_s);
         return cudaGetLastError();
-    }
-    return cudaSuccess;
+    });
 }
 
-cudaError_t launch_coincident3(int64_t N, const int *tgt_base, const double *tgt_pos, const double *src_pos,
-                               const int *src_start, CellGrid3 cg, int *count, const int *coinc_start, int *coinc_src,
-                               cudaStream_t st)
+cudaError_t launch_coincident3(int64_t N, const Near3Targets &tgt, const Near3Others &src, CellGrid3 cg,
+                               const Near3Params &np, bool source_frame, int *count, const int *coinc_start, int *coinc_src,
+                               int *touching, cudaStream_t st)
 {
     if (N <= 0)
         return cudaSuccess;
-    k_coincident3<<<nblk(N, 256), 256, 0, st>>>(N, tgt_base, tgt_pos, src_pos, src_start, cg, count, coinc_start,
-                                                coinc_src);
+    if (source_frame)
+        k_coincident3<true><<<nblk(N, 256), 256, 0, st>>>(N, tgt.base, tgt.hi, tgt.lo, tgt.pos, src, cg, np, count, coinc_start,
+                                                          coinc_src, touching);
+    else
+        k_coincident3<false><<<nblk(N, 256), 256, 0, st>>>(N, tgt.base, tgt.hi, tgt.lo, tgt.pos, src, cg, np, count,
+                                                           coinc_start, coinc_src, touching);
     return cudaGetLastError();
 }
 

@@ -55,7 +55,7 @@ struct fs3_plan {
     bool src_major = false;
     int2 *src_items = nullptr;
     int n_src_items = 0;
-    int n_coinc = 0;
+    bool coincident = false, marked = false;   // some targets have coincident sources, and marks (Near3Targets)
     // FP32: the near field on a second stream beside spreading and the transform
     cudaStream_t aux = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -159,6 +159,7 @@ template <typename real> fs_status twiddles3(fs3_plan *pl, int L, void **out)
 }
 
 fs_status near_setup3(fs3_plan *pl);
+Near3Params make_near3_f32(const fs3_plan *pl);
 
 // Plans spread in run order (launch_spread3_runs) when the occupied cells are many enough to fill the
 // GPU with a block each and hold enough sources to pay for a tile's zeroing and flush.
@@ -369,6 +370,9 @@ fs_status plan3_init(fs3_plan *pl, const double *src, int64_t M, const double *t
     return FS_OK;
 }
 
+Near3Targets near3_targets(const fs3_plan *pl) { return {pl->tgt_base, pl->tgt_hi, pl->tgt_lo, pl->tgt_pos}; }
+Near3Others near3_others(const fs3_plan *pl) { return {pl->src_hi, pl->src_lo, pl->src_pos, pl->src_start, 1.0 / pl->eps_I}; }
+
 // FP32 near field: warp items (at most 64 consecutive targets of one cell, split evenly) and,
 // per target, the sources at exactly the same FP32 offsets (coincident pairs).
 fs_status near_setup3(fs3_plan *pl)
@@ -469,23 +473,27 @@ fs_status near_setup3(fs3_plan *pl)
         FS_TRY(make_items(pl->tgt_cells, pl->tgt_cap, &pl->near_items, &pl->n_near_items));
     // coincident sources: count, scan, fill
     const int64_t N = pl->N;
+    const Near3Params np = make_near3_f32(pl);
     int *count = nullptr, *tmp = nullptr;
-    FS_TRY(pl->alloc(&count, (size_t)std::max<int64_t>(N, 1)));
+    FS_TRY(pl->alloc(&count, (size_t)N + 1));   // the counts, and the mark
     FS_TRY(pl->alloc(&pl->coinc_start, (size_t)N + 1));
     FS_TRY(pl->alloc(&tmp, (size_t)N / 4096 + 2));
     FS_CUDA(cudaMemsetAsync(pl->coinc_start, 0, sizeof(int) * ((size_t)N + 1), st));
-    FS_CUDA(launch_coincident3(N, pl->tgt_base, pl->tgt_pos, pl->src_pos, pl->src_start, pl->cg, count, nullptr,
-                               nullptr, st));
+    FS_CUDA(cudaMemsetAsync(count + N, 0, sizeof(int), st));
+    FS_CUDA(launch_coincident3(N, near3_targets(pl), near3_others(pl), pl->cg, np, pl->src_major, count, nullptr, nullptr,
+                               count + N, st));
     if (N > 0)
         FS_CUDA(launch_exclusive_scan(count, pl->coinc_start, (int)N, tmp, st));
-    int total = 0;
+    int total = 0, marked = 0;
     FS_CUDA(cudaMemcpyAsync(&total, pl->coinc_start + N, sizeof(int), cudaMemcpyDeviceToHost, st));
+    FS_CUDA(cudaMemcpyAsync(&marked, count + N, sizeof(int), cudaMemcpyDeviceToHost, st));
     FS_CUDA(cudaStreamSynchronize(st));
-    pl->n_coinc = total;
+    pl->coincident = total > 0;
+    pl->marked = marked != 0;
     FS_TRY(pl->alloc(&pl->coinc_src, (size_t)std::max(total, 1)));
     if (total > 0)
-        FS_CUDA(launch_coincident3(N, pl->tgt_base, pl->tgt_pos, pl->src_pos, pl->src_start, pl->cg, nullptr,
-                                   pl->coinc_start, pl->coinc_src, st));
+        FS_CUDA(launch_coincident3(N, near3_targets(pl), near3_others(pl), pl->cg, np, pl->src_major, nullptr,
+                                   pl->coinc_start, pl->coinc_src, nullptr, st));
     FS_CUDA(cudaStreamSynchronize(st));
     pl->release(count);
     pl->release(tmp);
@@ -631,15 +639,15 @@ template <typename real> fs_status eval3_t(fs3_plan *pl, void *phi, void *H, fs_
                 if (pl->src_major) {
                     FS_CUDA(cudaMemsetAsync(pl->phi_s, 0, sizeof(float) * (size_t)pl->N, sa));
                     FS_CUDA(cudaMemsetAsync(pl->grad_s, 0, sizeof(float) * 3 * (size_t)pl->N, sa));
-                    FS_CUDA(launch_near3_src(pl->src_items, pl->n_src_items, pl->src_base, pl->src_hi, pl->src_lo,
-                                             pl->tgt_hi, pl->tgt_lo, (const float *)q, pl->tgt_start, pl->cg, np32,
-                                             pl->N, pl->coinc_start, pl->coinc_src, pl->n_coinc > 0,
-                                             (float *)pl->phi_s, (float *)pl->grad_s, sa));
+                    FS_CUDA(launch_near3_src(pl->src_items, pl->n_src_items, pl->src_base, near3_others(pl),
+                                             near3_targets(pl), pl->tgt_start, (const float *)q, pl->cg, np32, pl->N,
+                                             pl->coinc_start, pl->coinc_src, pl->coincident || pl->marked, (float *)pl->phi_s,
+                                             (float *)pl->grad_s, sa));
                 } else {
-                    FS_CUDA(launch_near3_warp(pl->near_items, pl->n_near_items, pl->tgt_cap, pl->tgt_base, pl->tgt_hi,
-                                              pl->tgt_lo, pl->src_hi, pl->src_lo, (const float *)q, pl->src_start,
-                                              pl->cg, np32, pl->coinc_start, pl->coinc_src, (float *)pl->phi_s,
-                                              (float *)pl->grad_s, true, sa));
+                    FS_CUDA(launch_near3_warp(pl->near_items, pl->n_near_items, pl->tgt_cap, near3_targets(pl),
+                                              near3_others(pl), (const float *)q, pl->cg, np32, pl->N, pl->coinc_start,
+                                              pl->coinc_src, pl->marked, (float *)pl->phi_s, (float *)pl->grad_s, true,
+                                              sa));
                 }
                 FS_CUDA(cudaEventRecord(pl->ev_join, sa));
             }

@@ -84,3 +84,50 @@ def test_fp64_points_just_below_a_grid_line(m):
     for name, a, b in zip(("phi", "H", "dq", "dsrc", "dtgt"), got, want):
         a = a.cpu().numpy()
         assert np.max(np.abs(a - b)) <= 1e-12 * np.max(np.abs(b)), (name, np.max(np.abs(a - b)) / np.max(np.abs(b)))
+
+
+#: distances of FP32 3D pairs in torus units: above the FP32 kernels' floor of w (1e-10 eps_I), and below it
+CLOSE3 = 10.0 ** np.linspace(-10.3, -5.0, 22)
+TOUCHING3 = np.array([1e-15, 3e-16, 1e-16])
+
+
+@pytest.mark.parametrize("source_major", [False, True])
+def test_3d_fp32_close_pairs(source_major):
+    """3D FP32 plans, point pairs at CLOSE3: phi and H of each target (its pair dominates them) against the
+    FP64 plan within 5e-6, the bar of the 3D gates.  Pairs at TOUCHING3 are a few units in the last place
+    apart, distinct all the same: not taken for coincident ones, whose charge is left out (phi at least
+    that of a pair at the floor of w)."""
+    import paper_0807_2387_gb300 as fs
+    rng = np.random.default_rng(7 + source_major)
+    n, eps = 32, 4 / 32
+    scale = (0.25 - eps / 2) / 0.25          # of caller's units to torus units; the rim below fixes it
+    dist = np.concatenate([np.repeat(CLOSE3, 8), np.repeat(TOUCHING3, 40)])
+    d = rng.standard_normal((len(dist), 3))
+    d *= (dist / scale / np.linalg.norm(d, axis=1))[:, None]
+    # the pairs lie eps_I / 4 and more from each other, a charge of 1 each, the rest a thousandth
+    g = np.stack(np.meshgrid(*[np.linspace(-0.13, 0.13, 9)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    at = g[rng.permutation(len(g))[: len(dist)]] + rng.uniform(-0.003, 0.003, (len(dist), 3))
+    tgt = at + d
+    rim = 0.25 * np.concatenate([np.eye(3), -np.eye(3)])
+    more = rng.uniform(-0.12, 0.12, (4 * len(tgt) if source_major else 40, 3))
+    src = np.concatenate([at, rim, more])
+    q = np.concatenate([np.ones(len(at)), np.zeros(len(rim)), 1e-3 * rng.standard_normal(len(more))])
+    keep = np.any(tgt != at, axis=1)         # a difference below the last place would be no difference
+    assert keep[: 8 * len(CLOSE3)].all() and keep.mean() > 0.8
+    dev = torch.device("cuda", 0)
+    s, t, qd = (torch.tensor(v, device=dev) for v in (src, tgt, q))
+    got = {}
+    for precision in (64, 32):
+        plan = fs.FastSum3(s, t, n, 2.0, 4, eps, precision=precision, p=3)
+        got[precision] = [v.cpu().numpy() for v in plan.set_charges(qd).field(dtype=torch.float64)]
+        plan.sync()
+        factor = plan.info["scale"]
+    assert abs(factor - scale) < 1e-6
+    k = 8 * len(CLOSE3)
+    (phi, H), (phi0, H0) = got[32], got[64]
+    e_phi, e_h = np.abs(phi - phi0)[:k] / phi0[:k], np.linalg.norm(H - H0, axis=1)[:k] / np.linalg.norm(H0, axis=1)[:k]
+    assert e_phi.max() <= 5e-6, (e_phi.max(), dist[e_phi.argmax()])
+    assert e_h.max() <= 5e-6, (e_h.max(), dist[e_h.argmax()])
+    floor = factor / (4 * np.pi * 1e-10 * eps)
+    assert (phi[k:][keep[k:]] >= 0.99 * floor).all(), (phi[k:][keep[k:]].min(), floor)
+    assert (phi[k:][~keep[k:]] < 1e-3 * floor).all()
