@@ -629,7 +629,8 @@ fs_status plan_init(fs_plan *pl, const double *src, int64_t M, const double *tgt
     FS_TRY(pl->alloc_bytes(&pl->grid, (size_t)n_a * pl->pitch * sizeof(real)));
     // the filtered grid is its own buffer so that the first one stays zeroed; without memory for it
     // both are one and every spreading begins with a memset
-    if (pl->alloc_bytes(&pl->field, (size_t)n_a * pl->pitch * sizeof(real)) != FS_OK)
+    pl->field = pl->try_alloc((size_t)n_a * pl->pitch * sizeof(real));
+    if (!pl->field)
         pl->field = pl->grid;
     FS_CUDA(cudaMemsetAsync(pl->grid, 0, (size_t)n_a * pl->pitch * sizeof(real), st));
     if (pl->spread_direct && pl->kahan && sizeof(real) == 4)
@@ -746,18 +747,25 @@ template <typename real> fs_status reserve_rhs(fs_plan *pl, int nrhs)
     const size_t spec_bytes = (size_t)(pl->n / 2 + 1) * pl->ld * 2 * sizeof(real);
     auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
     const size_t field_at = up(grid_bytes * want), spec_at = 2 * field_at, sums_at = spec_at + up(spec_bytes * want);
-    // one allocation; the single-vector buffers stay until the plan is destroyed (freeing them here
-    // would wait for the device)
-    unsigned char *p = nullptr;
-    if (pl->alloc(&p, sums_at + (size_t)pl->sums_n * 4 * want * sizeof(real)) != FS_OK)
+    // one allocation, given back when a larger one replaces it; the single-vector buffers stay until the
+    // plan is destroyed (four cudaFree calls would add 120 us to the first evaluation of several vectors,
+    // 334 us for three at 100,003 sources).  FP64 near fields run one vector at a time, on those sums.
+    constexpr bool kSums = sizeof(real) == 4;
+    const size_t sums_bytes = kSums ? (size_t)pl->sums_n * 4 * want * sizeof(real) : 0;
+    unsigned char *p = static_cast<unsigned char *>(pl->try_alloc(sums_at + sums_bytes));
+    if (!p)
         return FS_OK;
+    pl->release(pl->rhs_block);
+    pl->rhs_block = p;
     pl->grid = p;
     pl->grid_dirty = true;
     pl->field = p + field_at;
     pl->spec = p + spec_at;
-    pl->phi_s = p + sums_at;
-    pl->grad_s = (unsigned char *)pl->phi_s + (size_t)pl->sums_n * want * sizeof(real);
-    pl->coinc = (unsigned char *)pl->phi_s + (size_t)pl->sums_n * 3 * want * sizeof(real);
+    if (kSums) {
+        pl->phi_s = p + sums_at;
+        pl->grad_s = p + sums_at + (size_t)pl->sums_n * want * sizeof(real);
+        pl->coinc = p + sums_at + (size_t)pl->sums_n * 3 * want * sizeof(real);
+    }
     pl->rhs_cap = want;
     return FS_OK;
 }

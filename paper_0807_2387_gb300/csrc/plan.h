@@ -107,11 +107,12 @@ struct fs_plan {
     bool grid_dirty = false, grid_recorded = false;
     void *grid_comp = nullptr;        // direct spreading (FP32): compensation plane of the grid
     bool spread_direct = false;       // spread with global atomics instead of shared-memory tiles
-    // grid, spec and the near field's sums hold rhs_cap charge vectors, evaluated together; the sums
-    // are one allocation: phi_s, grad_s from rhs_cap sums_n and coinc from 3 rhs_cap sums_n on
+    // grid, field, spec and (FP32) the near field's sums hold rhs_cap charge vectors, evaluated together; the
+    // sums are phi_s, grad_s from rhs_cap sums_n and coinc from 3 rhs_cap sums_n on (FP64: of one vector)
     void *phi_s = nullptr, *grad_s = nullptr, *coinc = nullptr;
     int64_t sums_n = 0;
     int rhs_cap = 1;
+    void *rhs_block = nullptr;        // their allocation for rhs_cap > 1
     // charges
     void *q_sorted = nullptr;
     double *q_sum = nullptr;
@@ -140,22 +141,29 @@ struct fs_plan {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaEvent_t ev_n0 = nullptr, ev_n1 = nullptr, ev_j = nullptr;   // timing of the overlapped stages
 
-    template <typename T> fs_status alloc(T **out, size_t count)
+    // Memory the plan can do without (null, and no error text, if there is none).
+    void *try_alloc(size_t nbytes, cudaError_t *error = nullptr)
     {
-        *out = nullptr;
-        if (count == 0)
-            count = 1;
         void *p_ = nullptr;
-        const size_t nbytes = count * sizeof(T);
-        cudaError_t e = cudaMalloc(&p_, nbytes);
+        const cudaError_t e = cudaMalloc(&p_, nbytes);
+        if (error)
+            *error = e;
         if (e != cudaSuccess) {
             cudaGetLastError();
-            return fs::fail(FS_ENOMEM, "cudaMalloc of " + std::to_string(nbytes) + " bytes failed: " +
-                                       cudaGetErrorString(e));
+            return nullptr;
         }
         allocs.push_back(p_);
         bytes += (int64_t)nbytes;
-        *out = static_cast<T *>(p_);
+        return p_;
+    }
+    template <typename T> fs_status alloc(T **out, size_t count)
+    {
+        const size_t nbytes = std::max<size_t>(count, 1) * sizeof(T);
+        cudaError_t e = cudaSuccess;
+        *out = static_cast<T *>(try_alloc(nbytes, &e));
+        if (!*out)
+            return fs::fail(FS_ENOMEM, "cudaMalloc of " + std::to_string(nbytes) + " bytes failed: " +
+                                       cudaGetErrorString(e));
         return FS_OK;
     }
     fs_status alloc_bytes(void **out, size_t nbytes)
