@@ -232,6 +232,7 @@ template <typename real> fs_status batch_build(fs_batch *b, const fs_instance *i
         if ((o.flags & FS_FLAG_AUTOTUNE) && o.cell == 0 && o.tile_cells == 0)
             FS_TRY(tune_instance(in[i], b->sigma, b->m, oi, &oi.tile_cells, &oi.cell));
         fs_plan *pl = new fs_plan;
+        pl->member = true;
         fs_status s = plan_create_common(in[i].src_xy, in[i].M, in[i].tgt_xy, in[i].N, in[i].n_grid, b->sigma, b->m,
                                          in[i].eps_I, &oi, pl);
         if (s != FS_OK) {

@@ -241,6 +241,13 @@ namespace {
 // the 2^18-point adjoint step at 181 1256 / 1064 / 1050 us; 2^20 clustered points 3.23 / 2.46 / 2.26 ms.
 int near_item_lanes(double per_cell) { return per_cell < 25.0 ? 8 : (per_cell < 100.0 ? 16 : 32); }
 
+// The filtered grid in a buffer of its own, where there is memory for it.
+template <typename real> void reserve_field(fs_plan *pl)
+{
+    if (void *f = pl->try_alloc((size_t)pl->n_a * pl->pitch * sizeof(real)))
+        pl->field = f;
+}
+
 // Bin one point set: keys, counting sort, order within the cells (pieces of at most *cap points, chosen
 // here unless given), per-point records; `cells`: the cells' first points.
 template <typename real>
@@ -629,9 +636,9 @@ fs_status plan_init(fs_plan *pl, const double *src, int64_t M, const double *tgt
     FS_TRY(pl->alloc_bytes(&pl->grid, (size_t)n_a * pl->pitch * sizeof(real)));
     // the filtered grid is its own buffer so that the first one stays zeroed; without memory for it
     // both are one and every spreading begins with a memset
-    pl->field = pl->try_alloc((size_t)n_a * pl->pitch * sizeof(real));
-    if (!pl->field)
-        pl->field = pl->grid;
+    pl->field = pl->grid;
+    if (!pl->member)
+        reserve_field<real>(pl);
     FS_CUDA(cudaMemsetAsync(pl->grid, 0, (size_t)n_a * pl->pitch * sizeof(real), st));
     if (pl->spread_direct && pl->kahan && sizeof(real) == 4)
         FS_TRY(pl->alloc_bytes(&pl->grid_comp, (size_t)n_a * pl->pitch * sizeof(real)));
@@ -781,6 +788,8 @@ template <typename real> fs_status reserve_charges(fs_plan *pl, int nrhs)
         FS_TRY(pl->alloc_bytes(&pl->q_sorted, (size_t)std::max<int64_t>(pl->M, 1) * nrhs * sizeof(real)));
         FS_TRY(pl->alloc(&pl->q_sum, nrhs));
         pl->nrhs_cap = nrhs;
+        if (pl->member && pl->field == pl->grid)
+            reserve_field<real>(pl);
         FS_TRY(reserve_rhs<real>(pl, nrhs));
     }
     return FS_OK;

@@ -103,7 +103,8 @@ struct fs_plan {
     bool src_major = false;           // FP32 forward near field over source items (many more sources than targets)
     void *mul = nullptr, *tw = nullptr;
     void *grid = nullptr, *spec = nullptr;   // grid: zero between evaluations (grid_dirty: not known to be)
-    void *field = nullptr;            // the filtered grid
+    void *field = nullptr;            // the filtered grid (without memory for it, the grid)
+    bool member = false;              // of a batch, which has its own grids: field is not allocated before the first charges
     bool grid_dirty = false, grid_recorded = false;
     void *grid_comp = nullptr;        // direct spreading (FP32): compensation plane of the grid
     bool spread_direct = false;       // spread with global atomics instead of shared-memory tiles

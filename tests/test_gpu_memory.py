@@ -36,3 +36,27 @@ def test_growing_number_of_charge_vectors(precision):
     assert held["growing"] <= held["at once"] + 8 * 2 ** 20, held
     err = float((out["growing"] - out["at once"]).norm() / out["at once"].norm())
     assert err <= (1e-12 if precision == 64 else 2e-5), err
+
+
+@pytest.mark.parametrize("precision,tol", [(32, 2e-5), (64, 1e-12)])
+def test_instances_of_a_batch_hold_one_grid(precision, tol):
+    """A batch's instances are evaluated in the batch's buffers: their plans hold no second grid, until one
+    is solved on its own, which gives what the batch gives (sums in another order), call after call."""
+    import paper_0807_2387_gb300 as fs
+    rng = np.random.default_rng(4)
+    dev = torch.device("cuda", 0)
+    pts = torch.tensor(rng.uniform(-0.17, 0.17, (3000, 2)), device=dev)
+    q = torch.tensor(rng.standard_normal((2, 3000)), device=dev)
+    batch = fs.FastSumBatch([(pts, pts, 512, 4 / 512)], 2.0, 4, 2, precision=precision)
+    alone = fs.FastSum(pts, pts, 512, 2.0, 4, 4 / 512, precision=precision)
+    member = batch.plan(0)
+    grid = 512 * 512 * precision // 8
+    assert member.info["workspace_bytes"] <= alone.info["workspace_bytes"] - grid
+    H = batch.eval([q])[1][0].double()
+    for charges, want in ((q[0], H[0]), (q, H), (q[1], H[1])):
+        got = member.set_charges(charges).field()[1].double()
+        assert float((got - want).norm() / want.norm()) <= tol
+    H2 = batch.eval([q])[1][0].double()
+    assert float((H2 - H).norm() / H.norm()) <= tol
+    for plan in (member, alone, batch):
+        plan.close()
