@@ -666,9 +666,12 @@ template <typename real> constexpr int fft_batch_blocks(int LC)
 // length the plans use, 128 .. 4096 points), LC = 0 takes it at run time.
 // blockIdx.y: the charge vector (grids and spectra at their strides).  The forward kernel zeroes the
 // grid rows it has read, which saves the next spreading a memset of the grid in front of it.
+// Grids and spectra come as plain pointers: a chained launch is resident while the kernel ahead of it
+// still writes them, which __restrict__ would rule out for the whole kernel (the units, called after
+// the wait, may have it).
 template <typename real, int LC>
-__global__ void __launch_bounds__(256) k_fft_rows_fwd(real *__restrict__ grid, int pitch, int n_a, int L,
-                                                      int n_half, cplx<real> *__restrict__ spec, int ld,
+__global__ void __launch_bounds__(256) k_fft_rows_fwd(real *grid, int pitch, int n_a, int L,
+                                                      int n_half, cplx<real> *spec, int ld,
                                                       const cplx<real> *__restrict__ tw, int64_t grid_stride,
                                                       int64_t spec_stride)
 {
@@ -688,7 +691,7 @@ __global__ void __launch_bounds__(256) k_fft_rows_fwd(real *__restrict__ grid, i
 }
 
 template <typename real, int LC>
-__global__ void __launch_bounds__(256) k_fft_cols(cplx<real> *__restrict__ spec, int ld, int n_a, int L, int n,
+__global__ void __launch_bounds__(256) k_fft_cols(cplx<real> *spec, int ld, int n_a, int L, int n,
                                                   const real *__restrict__ mul, const cplx<real> *__restrict__ tw,
                                                   int64_t spec_stride)
 {
@@ -702,8 +705,8 @@ __global__ void __launch_bounds__(256) k_fft_cols(cplx<real> *__restrict__ spec,
 }
 
 template <typename real, int LC>
-__global__ void __launch_bounds__(256) k_fft_rows_inv(const cplx<real> *__restrict__ spec, int ld, int n_a, int L,
-                                                      int n_half, real *__restrict__ grid, int pitch,
+__global__ void __launch_bounds__(256) k_fft_rows_inv(const cplx<real> *spec, int ld, int n_a, int L,
+                                                      int n_half, real *grid, int pitch,
                                                       const cplx<real> *__restrict__ tw, int64_t grid_stride,
                                                       int64_t spec_stride)
 {
@@ -1096,7 +1099,7 @@ __global__ void k_build_mul(const double2 *__restrict__ bhat, int n, const doubl
 
 // A launch whose blocks may start while the stream's previous kernel (one of this library's that
 // calls next_kernel_may_start) still runs; the kernel calls wait_previous_kernel before it touches
-// anything another kernel writes or reads.
+// anything another kernel writes or reads, and takes none of that as a __restrict__ parameter.
 template <typename... P, typename... A>
 cudaError_t launch_chained(bool chained, void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
 {
