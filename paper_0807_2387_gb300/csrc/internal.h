@@ -223,7 +223,7 @@ cudaError_t launch_point_keys3(const double *xyz, int64_t n, double s, int n_os,
 template <typename real>
 cudaError_t launch_gather_points3(const double *xyz, const int *perm, int64_t n, double s, int n_os, int window_lo,
                                   int n_a, int m, int cell, double *pos, real *frac, int *base,
-                                  float4 *hi, float4 *lo, int *status, cudaStream_t st);
+                                  float4 *hi, float4 *lo, cudaStream_t st);
 // the points of each cell into the order of CellSplit3 (pieces of at most cap)
 cudaError_t launch_cell_order3(const int *start, CellGrid3 cg, int cap, const double *xyz, double s, int n_os,
                                int window_lo, int n_a, int m, int *perm, cudaStream_t st);

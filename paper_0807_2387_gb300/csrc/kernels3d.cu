@@ -47,17 +47,17 @@ __global__ void k_rmax3(const double *__restrict__ xyz, int64_t n, unsigned long
 }
 
 // Window grid line of torus coordinate s x: floor(n_os s x) + n_os/2 - window_lo, and the
-// fraction n_os s x - floor(n_os s x); status 1 when the taps leave the active window (the
+// fraction n_os s x - floor(n_os s x); `outside` is set when the taps leave the active window (the
 // point lies beyond the admissible radius).
 __device__ __forceinline__ int grid_line3(double x, double s, int n_os, int window_lo, int m, int n_a, double &frac,
-                                          int *status)
+                                          bool &outside)
 {
     const double v = (double)n_os * (s * x);
     const double fl = floor(v);
     frac = v - fl;
     int b = (int)fl + n_os / 2 - window_lo;
     if (b - m + 1 < 0 || b + m > n_a - 1) {
-        atomicExch(status, 1);
+        outside = true;
         b = b - m + 1 < 0 ? m - 1 : n_a - 1 - m;
         frac = 0.0;
     }
@@ -71,13 +71,16 @@ __global__ void k_point_keys3(const double *__restrict__ xyz, int64_t n, double 
     if (k >= n)
         return;
     int b[3], sc[3];
+    bool outside = false;
     for (int d = 0; d < 3; ++d) {
         double f;
-        b[d] = grid_line3(xyz[3 * k + d], s, n_os, window_lo, m, n_a, f, status);
+        b[d] = grid_line3(xyz[3 * k + d], s, n_os, window_lo, m, n_a, f, outside);
         // sub-cell from the offset inside the cell, (b mod cell + frac) / cell in [0, 1)
         const int sidx = (int)(((double)(b[d] % cg.cell) + f) * cg.sub / cg.cell);
         sc[d] = sidx < cg.sub ? sidx : cg.sub - 1;
     }
+    if (outside)
+        atomicExch(status, 1);
     int morton = 0;
     for (int bit = 0; bit < 2; ++bit)
         morton |= (((sc[2] >> bit) & 1) << (3 * bit)) | (((sc[1] >> bit) & 1) << (3 * bit + 1)) |
@@ -91,7 +94,7 @@ template <typename real>
 __global__ void k_gather_points3(const double *__restrict__ xyz, const int *__restrict__ perm, int64_t n, double s,
                                  int n_os, int window_lo, int n_a, int m, int cell,
                                  double *__restrict__ pos, real *__restrict__ frac, int *__restrict__ base,
-                                 float4 *__restrict__ hi, float4 *__restrict__ lo, int *status)
+                                 float4 *__restrict__ hi, float4 *__restrict__ lo)
 {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= n)
@@ -99,8 +102,9 @@ __global__ void k_gather_points3(const double *__restrict__ xyz, const int *__re
     const int64_t i = perm[k];
     int b[3];
     double fr[3];
+    bool outside;   // k_point_keys3 reports it
     for (int d = 0; d < 3; ++d) {
-        b[d] = grid_line3(xyz[3 * i + d], s, n_os, window_lo, m, n_a, fr[d], status);
+        b[d] = grid_line3(xyz[3 * i + d], s, n_os, window_lo, m, n_a, fr[d], outside);
         pos[3 * k + d] = s * xyz[3 * i + d];
         frac[3 * k + d] = (real)fr[d];
     }
@@ -133,7 +137,7 @@ __global__ void __launch_bounds__(kOrder3Threads) k_cell_order3(const int *__res
     const int a = start[(int64_t)blockIdx.x * S3], count = start[(int64_t)(blockIdx.x + 1) * S3] - a;
     if (count <= cap)
         return;
-    int ignored = 0;
+    bool outside;   // k_point_keys3 reports it
     for (int r = 0; r < CellSplit::runs(count); ++r) {
         const int first = a + CellSplit::run_first(count, r), n = a + CellSplit::run_first(count, r + 1) - first;
         const CellSplit3 split(n, cap);
@@ -147,7 +151,7 @@ __global__ void __launch_bounds__(kOrder3Threads) k_cell_order3(const int *__res
                 const int i = perm[first + t];
                 for (int d = 0; d < 3; ++d) {
                     double f;
-                    const int b = grid_line3(xyz[3 * (int64_t)i + d], s, n_os, window_lo, m, n_a, f, &ignored);
+                    const int b = grid_line3(xyz[3 * (int64_t)i + d], s, n_os, window_lo, m, n_a, f, outside);
                     q[d][t] = (unsigned)((((double)(b % cg.cell) + f) / cg.cell) * 4194304.0);   // 22 bits
                 }
                 idx[t] = i;
@@ -1429,12 +1433,12 @@ cudaError_t launch_point_keys3(const double *xyz, int64_t n, double s, int n_os,
 template <typename real>
 cudaError_t launch_gather_points3(const double *xyz, const int *perm, int64_t n, double s, int n_os, int window_lo,
                                   int n_a, int m, int cell, double *pos, real *frac, int *base,
-                                  float4 *hi, float4 *lo, int *status, cudaStream_t st)
+                                  float4 *hi, float4 *lo, cudaStream_t st)
 {
     if (n <= 0)
         return cudaSuccess;
     k_gather_points3<real><<<nblk(n, 256), 256, 0, st>>>(xyz, perm, n, s, n_os, window_lo, n_a, m, cell, pos, frac,
-                                                         base, hi, lo, status);
+                                                         base, hi, lo);
     return cudaGetLastError();
 }
 
@@ -1642,7 +1646,7 @@ cudaError_t launch_unpermute3(int64_t N, const real *phi_s, const real *grad_s, 
 
 #define FS_INST3(real)                                                                                            \
     template cudaError_t launch_gather_points3<real>(const double *, const int *, int64_t, double, int, int, int, \
-                                                     int, int, double *, real *, int *, float4 *, float4 *, int *,  \
+                                                     int, int, double *, real *, int *, float4 *, float4 *,  \
                                                      cudaStream_t);                                               \
     template cudaError_t launch_spread3<real>(int64_t, int, const int *, const real *, const real *, Window<real>, \
                                               const WindowPoly &, real *, int, cudaStream_t);                     \

@@ -233,7 +233,7 @@ fs_status bin3(fs3_plan *pl, const double *xyz, int64_t n, int **perm, int **bas
         FS_CUDA(launch_cell_order3(*start, pl->cg, *cap, xyz, pl->s, pl->n_os, pl->window_lo, pl->n_a, pl->m, *perm, st));
     }
     FS_CUDA(launch_gather_points3<real>(xyz, *perm, n, pl->s, pl->n_os, pl->window_lo, pl->n_a, pl->m, pl->cg.cell,
-                                        *pos, fr, *base, *hi, *lo, pl->status, st));
+                                        *pos, fr, *base, *hi, *lo, st));
     FS_CUDA(cudaStreamSynchronize(st));
     pl->release(key);
     pl->release(count);
