@@ -254,20 +254,30 @@ template <typename real>
 fs_status bin_points(fs_plan *pl, const double *xy, int64_t n, int **perm, int **base, void **frac, double2 **pos,
                      float2 **pos32, float2 **lo32, int **start, int *cap, std::vector<int> *cells)
 {
-    FS_TRY(pl->alloc(perm, n));
-    FS_TRY(pl->alloc(base, n));
-    FS_TRY(pl->alloc_bytes(frac, (size_t)std::max<int64_t>(n, 1) * 2 * sizeof(real)));
-    FS_TRY(pl->alloc(pos, n));
-    FS_TRY(pl->alloc(pos32, n));   // FP64 plans: for the near field's test of reach
-    *lo32 = nullptr;
-    if (pl->precision == 32)
-        FS_TRY(pl->alloc(lo32, n));
-    FS_TRY(pl->alloc(start, (size_t)pl->n_keys + 1));
+    unsigned char *kept = nullptr, *scratch = nullptr;
+    real *fr = nullptr;
     int *key = nullptr, *count = nullptr, *fill = nullptr, *tmp = nullptr;
-    FS_TRY(pl->alloc(&key, n));
-    FS_TRY(pl->alloc(&count, pl->n_keys));
-    FS_TRY(pl->alloc(&fill, (size_t)pl->n_keys + 1));
-    FS_TRY(pl->alloc(&tmp, (size_t)pl->n_keys / 4096 + 2));
+    *lo32 = nullptr;
+    for (int pass = 0; pass < 2; ++pass) {
+        Parts k{kept}, t{scratch};
+        k.take(perm, n);
+        k.take(base, n);
+        k.take(&fr, 2 * (size_t)n);
+        k.take(pos, n);
+        k.take(pos32, n);   // FP64 plans: for the near field's test of reach
+        if (pl->precision == 32)
+            k.take(lo32, n);
+        k.take(start, (size_t)pl->n_keys + 1);
+        t.take(&key, n);
+        t.take(&count, pl->n_keys);
+        t.take(&fill, (size_t)pl->n_keys + 1);
+        t.take(&tmp, (size_t)pl->n_keys / 4096 + 2);
+        if (pass == 0) {
+            FS_TRY(pl->alloc(&kept, k.used));
+            FS_TRY(pl->alloc(&scratch, t.used));
+        }
+    }
+    *frac = fr;
     cudaStream_t st = pl->stream;
     FS_CUDA(cudaMemsetAsync(count, 0, sizeof(int) * pl->n_keys, st));
     FS_CUDA(cudaMemsetAsync(*start, 0, sizeof(int) * ((size_t)pl->n_keys + 1), st));
@@ -296,10 +306,7 @@ fs_status bin_points(fs_plan *pl, const double *xy, int64_t n, int **perm, int *
     FS_CUDA(launch_gather_points<real>(xy, *perm, n, pl->s, pl->n_os, pl->window_lo, pl->n_a, pl->m, pl->cg.cell, *pos,
                                        *frac, *base, *pos32, *lo32, st));
     FS_CUDA(cudaStreamSynchronize(st));
-    pl->release(key);
-    pl->release(count);
-    pl->release(fill);
-    pl->release(tmp);
+    pl->release(scratch);
     return FS_OK;
 }
 

@@ -18,6 +18,19 @@ fs_status fail(fs_status st, const std::string &msg);
 
 constexpr int kStages = 8;
 
+// Several arrays in one allocation (a cudaMalloc takes about 30 us where arrays are some megabytes large, and
+// so does a cudaFree): take() each with no base to add the sizes up, then again with the allocation as
+// the base for the pointers.
+struct Parts {
+    unsigned char *base = nullptr;
+    size_t used = 0;
+    template <typename T> void take(T **out, size_t count)
+    {
+        *out = base ? reinterpret_cast<T *>(base + used) : nullptr;
+        used += (count * sizeof(T) + 255) / 256 * 256;
+    }
+};
+
 // A cell's run of near-field items: `count` items of one size from item `first` on, and the
 // estimated pair work of each.
 struct NearCell {

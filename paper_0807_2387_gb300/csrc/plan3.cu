@@ -192,23 +192,31 @@ fs_status bin3(fs3_plan *pl, const double *xyz, int64_t n, int **perm, int **bas
 {
     cudaStream_t st = pl->stream;
     const int n_keys = pl->cg.n_keys();
-    FS_TRY(pl->alloc(perm, n));
-    FS_TRY(pl->alloc(base, n));
+    unsigned char *kept = nullptr, *scratch = nullptr;
     real *fr = nullptr;
-    FS_TRY(pl->alloc(&fr, 3 * (size_t)std::max<int64_t>(n, 1)));
-    *frac = fr;
-    FS_TRY(pl->alloc(pos, 3 * (size_t)std::max<int64_t>(n, 1)));
-    *hi = *lo = nullptr;
-    if (pl->precision == 32) {
-        FS_TRY(pl->alloc(hi, n));
-        FS_TRY(pl->alloc(lo, n));
-    }
-    FS_TRY(pl->alloc(start, (size_t)n_keys + 1));
     int *key = nullptr, *count = nullptr, *fill = nullptr, *tmp = nullptr;
-    FS_TRY(pl->alloc(&key, n));
-    FS_TRY(pl->alloc(&count, n_keys));
-    FS_TRY(pl->alloc(&fill, (size_t)n_keys + 1));
-    FS_TRY(pl->alloc(&tmp, (size_t)n_keys / 4096 + 2));
+    *hi = *lo = nullptr;
+    for (int pass = 0; pass < 2; ++pass) {
+        Parts k{kept}, t{scratch};
+        k.take(perm, n);
+        k.take(base, n);
+        k.take(&fr, 3 * (size_t)n);
+        k.take(pos, 3 * (size_t)n);
+        if (pl->precision == 32) {
+            k.take(hi, n);
+            k.take(lo, n);
+        }
+        k.take(start, (size_t)n_keys + 1);
+        t.take(&key, n);
+        t.take(&count, n_keys);
+        t.take(&fill, (size_t)n_keys + 1);
+        t.take(&tmp, (size_t)n_keys / 4096 + 2);
+        if (pass == 0) {
+            FS_TRY(pl->alloc(&kept, k.used));
+            FS_TRY(pl->alloc(&scratch, t.used));
+        }
+    }
+    *frac = fr;
     FS_CUDA(cudaMemsetAsync(count, 0, sizeof(int) * n_keys, st));
     FS_CUDA(cudaMemsetAsync(*start, 0, sizeof(int) * ((size_t)n_keys + 1), st));
     FS_CUDA(launch_point_keys3(xyz, n, pl->s, pl->n_os, pl->window_lo, pl->n_a, pl->m, pl->cg, key, count, pl->status,
@@ -235,10 +243,7 @@ fs_status bin3(fs3_plan *pl, const double *xyz, int64_t n, int **perm, int **bas
     FS_CUDA(launch_gather_points3<real>(xyz, *perm, n, pl->s, pl->n_os, pl->window_lo, pl->n_a, pl->m, pl->cg.cell,
                                         *pos, fr, *base, *hi, *lo, st));
     FS_CUDA(cudaStreamSynchronize(st));
-    pl->release(key);
-    pl->release(count);
-    pl->release(fill);
-    pl->release(tmp);
+    pl->release(scratch);
     return FS_OK;
 }
 
@@ -426,14 +431,22 @@ fs_status near_setup3(fs3_plan *pl)
                            (runs && occupied >= kSpread3RunMinCells && pl->M >= kSpread3RunMinPerCell * occupied);
         if (pl->spread_tiles && runs) {
             const int n_lines = n_cells * c3;
+            unsigned char *kept = nullptr, *scratch = nullptr;
             int *key = nullptr, *count = nullptr, *first = nullptr, *tmp = nullptr;
-            FS_TRY(pl->alloc(&pl->run_order, pl->M));
-            FS_TRY(pl->alloc(&pl->run_base, pl->M));
-            FS_TRY(pl->alloc(&pl->run_frac, 3 * (size_t)pl->M));
-            FS_TRY(pl->alloc(&key, pl->M));
-            FS_TRY(pl->alloc(&count, n_lines));
-            FS_TRY(pl->alloc(&first, (size_t)n_lines + 1));
-            FS_TRY(pl->alloc(&tmp, (size_t)n_lines / 4096 + 2));
+            for (int pass = 0; pass < 2; ++pass) {
+                Parts k{kept}, t{scratch};
+                k.take(&pl->run_order, pl->M);
+                k.take(&pl->run_base, pl->M);
+                k.take(&pl->run_frac, 3 * (size_t)pl->M);
+                t.take(&key, pl->M);
+                t.take(&count, n_lines);
+                t.take(&first, (size_t)n_lines + 1);
+                t.take(&tmp, (size_t)n_lines / 4096 + 2);
+                if (pass == 0) {
+                    FS_TRY(pl->alloc(&kept, k.used));
+                    FS_TRY(pl->alloc(&scratch, t.used));
+                }
+            }
             FS_CUDA(cudaMemsetAsync(count, 0, sizeof(int) * (size_t)n_lines, st));
             FS_CUDA(launch_spread3_keys(pl->M, pl->src_base, pl->cg, key, count, st));
             FS_CUDA(launch_exclusive_scan(count, first, n_lines, tmp, st));
@@ -441,8 +454,7 @@ fs_status near_setup3(fs3_plan *pl)
             FS_CUDA(launch_spread3_gather(pl->M, pl->run_order, pl->src_base, (const float *)pl->src_frac, pl->run_base,
                                           pl->run_frac, st));
             FS_CUDA(cudaStreamSynchronize(st));
-            for (int *p : {key, count, first, tmp})
-                pl->release(p);
+            pl->release(scratch);
         }
     }
     if (pl->spread_tiles) {
@@ -474,10 +486,16 @@ fs_status near_setup3(fs3_plan *pl)
     // coincident sources: count, scan, fill
     const int64_t N = pl->N;
     const Near3Params np = make_near3_f32(pl);
+    unsigned char *scratch = nullptr;
     int *count = nullptr, *tmp = nullptr;
-    FS_TRY(pl->alloc(&count, (size_t)N + 1));   // the counts, and the mark
+    for (int pass = 0; pass < 2; ++pass) {
+        Parts t{scratch};
+        t.take(&count, (size_t)N + 1);   // the counts, and the mark
+        t.take(&tmp, (size_t)N / 4096 + 2);
+        if (pass == 0)
+            FS_TRY(pl->alloc(&scratch, t.used));
+    }
     FS_TRY(pl->alloc(&pl->coinc_start, (size_t)N + 1));
-    FS_TRY(pl->alloc(&tmp, (size_t)N / 4096 + 2));
     FS_CUDA(cudaMemsetAsync(pl->coinc_start, 0, sizeof(int) * ((size_t)N + 1), st));
     FS_CUDA(cudaMemsetAsync(count + N, 0, sizeof(int), st));
     FS_CUDA(launch_coincident3(N, near3_targets(pl), near3_others(pl), pl->cg, np, pl->src_major, count, nullptr, nullptr,
@@ -495,8 +513,7 @@ fs_status near_setup3(fs3_plan *pl)
         FS_CUDA(launch_coincident3(N, near3_targets(pl), near3_others(pl), pl->cg, np, pl->src_major, nullptr,
                                    pl->coinc_start, pl->coinc_src, nullptr, st));
     FS_CUDA(cudaStreamSynchronize(st));
-    pl->release(count);
-    pl->release(tmp);
+    pl->release(scratch);
     return FS_OK;
 }
 
