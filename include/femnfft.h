@@ -133,7 +133,9 @@ typedef struct {
  *  opts    NULL for defaults
  *  out     receives the plan
  * Returns FS_EINVAL on a bad argument, FS_ENOMEM, FS_ECUDA.  Synchronises the
- * plan's stream (it reads the binning counts back to the host).
+ * plan's stream (it reads the binning counts back to the host).  Creation sorts the
+ * points and allocates: about twice the time of an evaluation (2^18 points 1.6 ms,
+ * 2^20 4.1 ms), which counts where points move at every step.
  */
 fs_status fs_plan_create(const double *src_xy, int64_t M, const double *tgt_xy, int64_t N,
                          int n_grid, double sigma_os, int m_window, double eps_I,

@@ -30,7 +30,7 @@ using namespace fs;
 namespace {
 
 constexpr int kPointBlock = 256;   // threads (= points) per block of the per-point batched kernels
-constexpr size_t kMaxTileSmem = 56 * 1024;   // spreading tiles of tuned batches: >= 4 CTAs per SM
+constexpr size_t kMaxTileSmem = 56 * 1024;   // spreading tiles of tuned batches (spread_smem_bytes): 3 CTAs and more per SM
 constexpr int kMaxRhs = 4;
 
 struct GraphEntry {

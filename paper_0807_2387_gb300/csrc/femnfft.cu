@@ -129,10 +129,6 @@ long double window_value(long double b, int m, long double x)
     return (long double)m * b * expl(-b * x * x / (tau + m)) * -expm1l(-2 * z) / (z * -expm1l(-2 * b * m));
 }
 
-// Per-tap polynomial form of the normalised window for the FP32 kernels: for tap a the
-// function frac -> psi(frac + m - 1 - a) on [0, 1) is interpolated at kPolyD + 1 Chebyshev
-// points in FP64 and rewritten in monomials of t = frac - 1/2; the slope polynomial is its
-// exact derivative.
 }  // namespace
 
 // As build_window_poly, of degree kPolyD64 for the taps a < m, in extended precision throughout.
@@ -182,6 +178,10 @@ void fs::build_window_poly64(double sigma, int m, WindowPoly64 *wp)
         known[{sigma, m}] = *wp;
 }
 
+// Per-tap polynomial form of the normalised window for the FP32 kernels: for tap a the
+// function frac -> psi(frac + m - 1 - a) on [0, 1) is interpolated at kPolyD + 1 Chebyshev
+// points in FP64 and rewritten in monomials of t = frac - 1/2; the slope polynomial is its
+// exact derivative.
 void fs::build_window_poly(double sigma, int m, WindowPoly *wp)
 {
     const double b = kPi * (2.0 - 1.0 / sigma);

@@ -52,8 +52,9 @@ template <typename real> inline size_t spread_launch_bytes(int P, int M2, bool c
            (size_t)kSpreadWarps * spread_batch<real>(P, Q, planes) * spread_record<real>(M2) * sizeof(real);
 }
 
-// The measure by which tiles are chosen and admitted (at most 200 KB): the tiles, one source's weights a
-// warp and the polynomials the adjoint's kernel holds.  The records, up to 18 KB, fit beside it.
+// The measure by which tiles are chosen and admitted (at most 200 KB; 56 KB for the tuned tiles of batches):
+// the tiles, one source's weights a warp and the polynomials the adjoint's kernel holds.  A launch
+// asks for spread_launch_bytes, whose records take 5 to 18 KB in place of the last two.
 template <typename real> inline size_t spread_smem_bytes(int P, int M2, bool comp)
 {
     const int G = spread_groups(M2), VW = 16 / (int)sizeof(real);

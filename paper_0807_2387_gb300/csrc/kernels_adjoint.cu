@@ -18,7 +18,7 @@
 // removes those: -q beta_0 in phi, -q (2 beta_1 / eps_I^2) I in the Hessian and, in
 // the source gradient of the adjoint potential, +(2 beta_1 / eps_I^2) dn.
 //
-// FP64: one thread per point (the comparison path).  FP32: warp items over the
+// FP64: one warp per point (near64.cuh).  FP32: warp items over the
 // cells (near_warp.cuh), the Hessian over the forward's target items and
 // the adjoint potential over items of sources against the targets.
 #include <cmath>

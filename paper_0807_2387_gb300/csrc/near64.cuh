@@ -14,7 +14,7 @@
 //   1/w: the 20-bit hardware approximation y and one third-order step y (1 + e + e^2), e = 1 - w y;
 //   T_I: the two polynomials Ptilde and P' of the far field's own coefficients.
 // Measured (32,768 points, n = 256, 10.0e6 pairs within eps_I, p = 6): 3.03 ms with a thread per
-// target, 0.63 ms here; the FP64 pipe's bound for the pairs is 0.53 ms.
+// target, 0.67 ms here; the FP64 pipe's bound for the pairs is 0.53 ms.
 #pragma once
 
 #include "near_warp.cuh"

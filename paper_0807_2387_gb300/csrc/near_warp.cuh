@@ -32,21 +32,6 @@
 
 namespace fs {
 
-template <int E> __device__ __forceinline__ float ipow(float x)
-{
-    if constexpr (E == 0) {
-        return 1.0f;
-    } else if constexpr (E == 1) {
-        return x;
-    } else {
-        const float h = ipow<E / 2>(x);
-        if constexpr (E % 2 == 0)
-            return h * h;
-        else
-            return h * h * x;
-    }
-}
-
 __device__ __forceinline__ float warp_min(float v)
 {
     for (int o = 16; o > 0; o >>= 1)

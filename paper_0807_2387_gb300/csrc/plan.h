@@ -205,8 +205,8 @@ struct fs_plan {
     // whose submission delays the longer chain); uniform 262,144 points have items of up to 5.7e4 pairs.
     bool near_first() const { return !near_cells_h.empty() && near_cells_h[0].work >= (1 << 16); }
     // Whether the transform's kernels start before the kernel ahead of them has ended (launch_chained):
-    // where each of them and the spreading (n_items) has at most a block per SM.  There a launch's
-    // latency counts: evaluations of 1,000 and 4,096 points 35.8 -> 24.5 and 31.8 -> 24.6 us on the GPU.
+    // where the row kernels (over all vectors; the columns are about as many) and the spreading of one
+    // vector (n_items) have at most a block per SM.  There a launch's latency counts: evaluations of 1,000 and 4,096 points 35.8 -> 24.5 and 31.8 -> 24.6 us on the GPU.
     // With more blocks the waiting ones keep slots that the spreading or the near field needs: 32,768
     // points in FP64 875 -> 992 us, the disc mesh 131 -> 145, a training step of 262,144 points 974 -> 988.
     bool chained(int n_items, int nrhs) const

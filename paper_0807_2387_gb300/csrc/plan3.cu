@@ -163,7 +163,8 @@ Near3Params make_near3_f32(const fs3_plan *pl);
 
 // Plans spread in run order (launch_spread3_runs) when the occupied cells are many enough to fill the
 // GPU with a block each and hold enough sources to pay for a tile's zeroing and flush.
-constexpr int64_t kScanMost = 4096 * 4096;   // launch_exclusive_scan's range
+// (Only where launch_exclusive_scan takes a key per grid line: not on grids of n = 256, 264^3 lines.)
+constexpr int64_t kScanMost = 4096 * 4096;
 constexpr int64_t kSpread3RunMinCells = 304, kSpread3RunMinPerCell = 8;
 
 template <typename real> NearParams<real> make_near3(const fs3_plan *pl)
@@ -378,8 +379,8 @@ fs_status plan3_init(fs3_plan *pl, const double *src, int64_t M, const double *t
 Near3Targets near3_targets(const fs3_plan *pl) { return {pl->tgt_base, pl->tgt_hi, pl->tgt_lo, pl->tgt_pos}; }
 Near3Others near3_others(const fs3_plan *pl) { return {pl->src_hi, pl->src_lo, pl->src_pos, pl->src_start, 1.0 / pl->eps_I}; }
 
-// FP32 near field: warp items (at most 64 consecutive targets of one cell, split evenly) and,
-// per target, the sources at exactly the same FP32 offsets (coincident pairs).
+// FP32 near field: warp items (the pieces of the cells, at most 32 targets or 64 sources) and,
+// per target, the sources at the same FP64 position (coincident pairs).
 fs_status near_setup3(fs3_plan *pl)
 {
     cudaStream_t st = pl->stream;
