@@ -158,14 +158,15 @@ def algorithmic_bytes(info, n_points):
 
 
 # DRAM bytes per launch of the near-field kernel from an ncu capture, keyed by the SHA-256 of
-# the code it was taken on: the kernel sources (kernels_near.cu, near_fwd.cuh, near_warp.cuh) and the
-# function that forms its work items (build_near_items in femnfft.cu).  A changed kernel or
-# item layout reports null until it is re-captured.
+# the code it was taken on: the kernel sources (kernels_near.cu, near_fwd.cuh, near_warp.cuh), the order of
+# a cell's points (CellSplit in internal.h, k_cell_order in kernels_bin.cu, sort_shared.cuh) and the
+# functions that choose and form its work items (near_item_lanes, bin_points and build_near_items in
+# femnfft.cu).  A changed kernel or item layout reports null until it is re-captured.
 NEAR_TRAFFIC = {
-    # 21.52 MB per launch on the 2^19-point mixture (-k regex:"k_near_list|k_spread" -s 1 -c 4), scaled by
+    # 21.52 MB per launch on the 2^19-point mixture (-k regex:"k_near_list" -s 1 -c 3), scaled by
     # the point count to the 2^20-point launch: the kernel reads per-point data once
-    "e3e5e531821030133171e60923f807789f605b49a43e5f2b8408724178913879": (
-        2 * 21524224, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
+    "cadf6ae34e9f6e77226b807b9873f14995786f00ecf9d607b3c3ee0e51349551": (
+        2 * 21521152, "captured at 2^19 points on this source and item layout, scaled x2 to 2^20"),
 }
 
 
@@ -173,11 +174,16 @@ def near_source_sha():
     import hashlib
     csrc = os.path.join(ROOT, "paper_0807_2387_gb300", "csrc")
     h = hashlib.sha256()
-    for name in ("kernels_near.cu", "near_fwd.cuh", "near_warp.cuh"):
+    for name in ("kernels_near.cu", "near_fwd.cuh", "near_warp.cuh", "sort_shared.cuh"):
         h.update(open(os.path.join(csrc, name), "rb").read())
-    text = open(os.path.join(csrc, "femnfft.cu")).read()
-    start = text.index("fs_status build_near_items(")
-    h.update(text[start:text.index("\n}\n", start)].encode())
+    for name, first, last in (("internal.h", "constexpr int kOrderRun", "\n};\n"),             # with CellSplit
+                              ("kernels_bin.cu", "constexpr int kOrderThreads", "\n}\n"),      # with k_cell_order
+                              ("femnfft.cu", "int near_item_lanes(", "\n"),
+                              ("femnfft.cu", "fs_status bin_points(", "\n}\n"),
+                              ("femnfft.cu", "fs_status build_near_items(", "\n}\n")):
+        text = open(os.path.join(csrc, name)).read()
+        start = text.index(first)
+        h.update(text[start:text.index(last, start)].encode())
     return h.hexdigest()
 
 
